@@ -216,16 +216,28 @@ struct RegDft<T2, 5, SIGN> {
     }
 };
 
-// Registers per thread of a Stockham pass: ceil(16 / RD) items of RD values
-// with TPR = ceil(H / 16) threads per row: 16 for power-of-two radices, 20
-// once radix 3 or 5 passes occur (MIXED; compiled separately so that the
-// power-of-two kernels keep their smaller register footprint).
-template <bool MIXED> struct PassRegs { static constexpr int n = MIXED ? 20 : 16; };
-__host__ __device__ inline int row_tpr(int H) { return (H + 15) / 16; }
+// A thread of a Stockham pass holds V values (V = 16 or 4): ceil(V / RD) items
+// of radix RD <= V, with TPR = ceil(H / V) threads per row.  Registers: V for
+// power-of-two radices, up to 20 (V = 16) or 6 (V = 4) once radix 3 or 5
+// passes occur (MIXED; compiled separately so that the power-of-two kernels
+// keep their smaller register footprint).
+template <bool MIXED, int V = 16> struct PassRegs { static constexpr int n = !MIXED ? V : (V == 16 ? 20 : 6); };
+template <int V = 16> __host__ __device__ inline int row_tpr(int H) { return (H + V - 1) / V; }
+
+// Values per thread.  FP32: 16, two radix-16 passes with few barriers.  FP64 up
+// to H = 1024 (512 threads for two rows): 4.  The FP64 pipe takes a warp
+// instruction every ~64 cycles per SM quarter, so a row spread over four times
+// the threads keeps all four quarters busy where a launch has few rows, at the
+// same instruction count (radix 4: 28 FP64 instructions per 4 points and pass,
+// four passes; radix 16: 228 per 16 points, two passes).  One field of 256 x 512
+// points: 51 / 54 us with 16 values and 8 pairs per CTA (16 CTAs), 28 / 27 us
+// with one pair per CTA, 10.2 / 10.3 us with 4 values; 16 fields of 512 x 1024:
+// 373 / 417 -> 334 / 360 us (synthesis / analysis).
+template <typename T> inline int fft_values(int H) { return sizeof(T) == 8 && H <= 1024 ? 4 : 16; }
 
 // One Stockham pass of radix RD over a row of length H held in `row` (padded
 // indices) or, for the first/last pass, in global memory.  Each thread owns
-// up to ceil(16 / RD) items j = t + it * TPR; item j reads x[j + r H/RD],
+// up to ceil(V / RD) items j = t + it * TPR; item j reads x[j + r H/RD],
 // applies the twiddle W^(r (j mod Ns) H/(Ns RD)), runs the RD-point DFT and
 // writes y[(j / Ns) Ns RD + j mod Ns + r Ns].
 // log2 of a power of two
@@ -234,11 +246,11 @@ __device__ __forceinline__ int lg2(int v) { return __popc(v - 1); }
 // P2: every length involved is a power of two, so the index arithmetic is
 // masks and shifts (a division by a run-time value is a long instruction
 // sequence on the integer pipe, which the FFT kernels are short of).
-template <typename T2, int RD, int SIGN, int NR, bool P2>
+template <typename T2, int RD, int SIGN, int NR, bool P2, int V = 16>
 __device__ __forceinline__ void stockham_load(const T2 *src, bool global_src, int t, int TPR, int H, int Ns,
                                               const T2 *__restrict__ wtab, T2 (&v)[NR])
 {
-    constexpr int IT = (16 + RD - 1) / RD;
+    constexpr int IT = (V + RD - 1) / RD;
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
         const int j = t + it * TPR;
@@ -271,10 +283,10 @@ __device__ __forceinline__ int stockham_out(int j, int r, int Ns)
     return (j / Ns) * Ns * RD + (j % Ns) + r * Ns;
 }
 
-template <typename T2, int RD, int NR, bool P2>
+template <typename T2, int RD, int NR, bool P2, int V = 16>
 __device__ __forceinline__ void stockham_store_smem(T2 *row, int t, int TPR, int H, int Ns, const T2 (&v)[NR])
 {
-    constexpr int IT = (16 + RD - 1) / RD;
+    constexpr int IT = (V + RD - 1) / RD;
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
         const int j = t + it * TPR;
@@ -284,36 +296,46 @@ __device__ __forceinline__ void stockham_store_smem(T2 *row, int t, int TPR, int
     }
 }
 
-// Runs a pass of the given radix (run-time selected).
-template <typename T2, int SIGN, bool MIXED>
+// Runs a pass of the given radix (run-time selected, at most V).
+template <typename T2, int SIGN, bool MIXED, int V = 16>
 __device__ __forceinline__ void pass_load(int rd, const T2 *src, bool g, int t, int TPR, int H, int Ns,
-                                          const T2 *wtab, T2 (&v)[PassRegs<MIXED>::n])
+                                          const T2 *wtab, T2 (&v)[PassRegs<MIXED, V>::n])
 {
-    constexpr int NR = PassRegs<MIXED>::n;
+    constexpr int NR = PassRegs<MIXED, V>::n;
     constexpr bool P2 = !MIXED;
-    if (MIXED && rd == 3) { stockham_load<T2, 3, SIGN, NR, P2>(src, g, t, TPR, H, Ns, wtab, v); return; }
-    if (MIXED && rd == 5) { stockham_load<T2, 5, SIGN, NR, P2>(src, g, t, TPR, H, Ns, wtab, v); return; }
-    switch (rd) {
-    case 2: stockham_load<T2, 2, SIGN, NR, P2>(src, g, t, TPR, H, Ns, wtab, v); break;
-    case 4: stockham_load<T2, 4, SIGN, NR, P2>(src, g, t, TPR, H, Ns, wtab, v); break;
-    case 8: stockham_load<T2, 8, SIGN, NR, P2>(src, g, t, TPR, H, Ns, wtab, v); break;
-    default: stockham_load<T2, 16, SIGN, NR, P2>(src, g, t, TPR, H, Ns, wtab, v); break;
+    if (MIXED && rd == 3) { stockham_load<T2, 3, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v); return; }
+    if (MIXED && rd == 5) { stockham_load<T2, 5, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v); return; }
+    if constexpr (V == 4) {
+        if (rd == 2) stockham_load<T2, 2, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v);
+        else stockham_load<T2, 4, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v);
+    } else {
+        switch (rd) {
+        case 2: stockham_load<T2, 2, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v); break;
+        case 4: stockham_load<T2, 4, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v); break;
+        case 8: stockham_load<T2, 8, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v); break;
+        default: stockham_load<T2, 16, SIGN, NR, P2, V>(src, g, t, TPR, H, Ns, wtab, v); break;
+        }
     }
 }
 
-template <typename T2, bool MIXED>
+template <typename T2, bool MIXED, int V = 16>
 __device__ __forceinline__ void pass_store(int rd, T2 *row, int t, int TPR, int H, int Ns,
-                                           const T2 (&v)[PassRegs<MIXED>::n])
+                                           const T2 (&v)[PassRegs<MIXED, V>::n])
 {
-    constexpr int NR = PassRegs<MIXED>::n;
+    constexpr int NR = PassRegs<MIXED, V>::n;
     constexpr bool P2 = !MIXED;
-    if (MIXED && rd == 3) { stockham_store_smem<T2, 3, NR, P2>(row, t, TPR, H, Ns, v); return; }
-    if (MIXED && rd == 5) { stockham_store_smem<T2, 5, NR, P2>(row, t, TPR, H, Ns, v); return; }
-    switch (rd) {
-    case 2: stockham_store_smem<T2, 2, NR, P2>(row, t, TPR, H, Ns, v); break;
-    case 4: stockham_store_smem<T2, 4, NR, P2>(row, t, TPR, H, Ns, v); break;
-    case 8: stockham_store_smem<T2, 8, NR, P2>(row, t, TPR, H, Ns, v); break;
-    default: stockham_store_smem<T2, 16, NR, P2>(row, t, TPR, H, Ns, v); break;
+    if (MIXED && rd == 3) { stockham_store_smem<T2, 3, NR, P2, V>(row, t, TPR, H, Ns, v); return; }
+    if (MIXED && rd == 5) { stockham_store_smem<T2, 5, NR, P2, V>(row, t, TPR, H, Ns, v); return; }
+    if constexpr (V == 4) {
+        if (rd == 2) stockham_store_smem<T2, 2, NR, P2, V>(row, t, TPR, H, Ns, v);
+        else stockham_store_smem<T2, 4, NR, P2, V>(row, t, TPR, H, Ns, v);
+    } else {
+        switch (rd) {
+        case 2: stockham_store_smem<T2, 2, NR, P2, V>(row, t, TPR, H, Ns, v); break;
+        case 4: stockham_store_smem<T2, 4, NR, P2, V>(row, t, TPR, H, Ns, v); break;
+        case 8: stockham_store_smem<T2, 8, NR, P2, V>(row, t, TPR, H, Ns, v); break;
+        default: stockham_store_smem<T2, 16, NR, P2, V>(row, t, TPR, H, Ns, v); break;
+        }
     }
 }
 
@@ -335,10 +357,10 @@ __device__ __forceinline__ void fill_wtab(T2 *wtab, const T2 *__restrict__ tw, i
 }
 
 // Writes the last Stockham pass's outputs y[j + r H/RD] of a thread's items.
-template <int RD, int NR, typename T2, typename F>
+template <int RD, int NR, int V = 16, typename T2, typename F>
 __device__ __forceinline__ void last_pass_out(const T2 (&v)[NR], int t, int TPR, int H, const F &put)
 {
-    constexpr int IT = (16 + RD - 1) / RD;
+    constexpr int IT = (V + RD - 1) / RD;
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
         const int jj = t + it * TPR;
@@ -347,18 +369,23 @@ __device__ __forceinline__ void last_pass_out(const T2 (&v)[NR], int t, int TPR,
         for (int rr = 0; rr < RD; ++rr) put(jj + rr * (H / RD), v[it * RD + rr]);
     }
 }
-template <bool MIXED, typename T2, typename F>
-__device__ __forceinline__ void last_pass_out(int rd, const T2 (&v)[PassRegs<MIXED>::n], int t, int TPR, int H,
+template <bool MIXED, int V = 16, typename T2, typename F>
+__device__ __forceinline__ void last_pass_out(int rd, const T2 (&v)[PassRegs<MIXED, V>::n], int t, int TPR, int H,
                                               const F &put)
 {
-    constexpr int NR = PassRegs<MIXED>::n;
-    if (MIXED && rd == 3) { last_pass_out<3, NR>(v, t, TPR, H, put); return; }
-    if (MIXED && rd == 5) { last_pass_out<5, NR>(v, t, TPR, H, put); return; }
-    switch (rd) {
-    case 2: last_pass_out<2, NR>(v, t, TPR, H, put); break;
-    case 4: last_pass_out<4, NR>(v, t, TPR, H, put); break;
-    case 8: last_pass_out<8, NR>(v, t, TPR, H, put); break;
-    default: last_pass_out<16, NR>(v, t, TPR, H, put); break;
+    constexpr int NR = PassRegs<MIXED, V>::n;
+    if (MIXED && rd == 3) { last_pass_out<3, NR, V>(v, t, TPR, H, put); return; }
+    if (MIXED && rd == 5) { last_pass_out<5, NR, V>(v, t, TPR, H, put); return; }
+    if constexpr (V == 4) {
+        if (rd == 2) last_pass_out<2, NR, V>(v, t, TPR, H, put);
+        else last_pass_out<4, NR, V>(v, t, TPR, H, put);
+    } else {
+        switch (rd) {
+        case 2: last_pass_out<2, NR, V>(v, t, TPR, H, put); break;
+        case 4: last_pass_out<4, NR, V>(v, t, TPR, H, put); break;
+        case 8: last_pass_out<8, NR, V>(v, t, TPR, H, put); break;
+        default: last_pass_out<16, NR, V>(v, t, TPR, H, put); break;
+        }
     }
 }
 
@@ -369,13 +396,14 @@ __device__ __forceinline__ void last_pass_out(int rd, const T2 (&v)[PassRegs<MIX
 // One tile (field b, pairs p0 .. p0+G-1) of the synthesis FFT, run by the
 // whole CTA (blockDim.x >= 2 G max(1, H/16)); smem_raw holds the twiddle table
 // and the 2G padded rows.
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, int V = 16>
 __device__ __forceinline__ void fft_synth_tile(const PlanView<T> &pv, const T *__restrict__ eo, T *__restrict__ grid,
-                                               int b, int p0, int G, int op, unsigned char *smem_raw)
+                                               int b, int p0, int G, int op, unsigned long long plan,
+                                               unsigned char *smem_raw)
 {
     using T2 = typename Vec2<T>::type;
     const int H = pv.nphi / 2, R = 2 * G;
-    const int TPR = row_tpr(H);
+    const int TPR = row_tpr<V>(H);
     const int ld = padi(H) + 1;
     T2 *wtab = reinterpret_cast<T2 *>(smem_raw);
     T2 *buf = wtab + H;
@@ -399,7 +427,9 @@ __device__ __forceinline__ void fft_synth_tile(const PlanView<T> &pv, const T *_
         buf[(2 * i + 1) * ld + padi(m)] = XS;
     }
     __syncthreads();
-    // 2. pre-twiddle: Z_k = (X_k + conj X_{H-k}) + i W^k (X_k - conj X_{H-k}), X_H = 0
+    // 2. pre-twiddle: with A = X_k + conj X_{H-k} and P = W^k (X_k - conj X_{H-k}),
+    //    W = e^{2 pi i / (2H)}: Z_k = A + i P and, since W^{H-k} = -conj W^k,
+    //    Z_{H-k} = conj A + i conj P (one product for both positions); X_H = 0
     for (int q = threadIdx.x; q < R * (H / 2 + 1); q += blockDim.x) {
         const int r = q / (H / 2 + 1), k = q - r * (H / 2 + 1);
         T2 *row = buf + r * ld;
@@ -410,8 +440,9 @@ __device__ __forceinline__ void fft_synth_tile(const PlanView<T> &pv, const T *_
         }
         const int k2 = H - k;
         const T2 Xa = row[padi(k)], Xb = row[padi(k2)];
-        row[padi(k)] = cadd(cadd(Xa, conj_(Xb)), mul_i(cmul(pv.tw[k], csub(Xa, conj_(Xb)))));
-        if (k2 != k) row[padi(k2)] = cadd(cadd(Xb, conj_(Xa)), mul_i(cmul(pv.tw[k2], csub(Xb, conj_(Xa)))));
+        const T2 A = cadd(Xa, conj_(Xb)), P = cmul(pv.tw[k], csub(Xa, conj_(Xb)));
+        row[padi(k)] = cadd(A, mul_i(P));
+        if (k2 != k) row[padi(k2)] = cadd(conj_(A), mul_i(conj_(P)));
     }
     __syncthreads();
     // 3. inverse complex FFT of length H by Stockham passes; the last one writes the grid
@@ -419,65 +450,77 @@ __device__ __forceinline__ void fft_synth_tile(const PlanView<T> &pv, const T *_
     const int p = p0 + (r >> 1);
     const int j = (r & 1) ? nlat - 1 - p : p;
     const bool live_row = r < R && p < npairs && !((r & 1) && j == p);
+    const bool scaled = op == OP_ANALYS_ADJ;
     T scale = T(1);
-    if (op == OP_ANALYS_ADJ && p < npairs) scale = T(kTwoPiD) / T(pv.nphi) * pv.wq[p];
+    if (scaled && p < npairs) scale = T(kTwoPiD) / T(pv.nphi) * pv.wq[p];
     T2 *row = buf + (r < R ? r : 0) * ld;
     T2 *out = reinterpret_cast<T2 *>(grid) + ((size_t)b * nlat + (live_row ? j : 0)) * H;
     if (H == 1) {
         if (threadIdx.x < R && live_row) {
             T2 z = row[0];
-            z.x *= scale; z.y *= scale;
+            if (scaled) { z.x *= scale; z.y *= scale; }
             out[0] = z;
         }
         return;
     }
     int Ns = 1;
-    T2 v[PassRegs<MIXED>::n];
+    T2 v[PassRegs<MIXED, V>::n];
     for (int ps = 0;; ++ps) {
-        const int rd = fft_plan_radix(pv.fftplan, ps);
-        if (r < R) pass_load<T2, 1, MIXED>(rd, row, false, t, TPR, H, Ns, wtab, v);
+        const int rd = fft_plan_radix(plan, ps);
+        if (r < R) pass_load<T2, 1, MIXED, V>(rd, row, false, t, TPR, H, Ns, wtab, v);
         const bool last = Ns * rd == H;
         __syncthreads();
         if (last) {
             // last pass: y[j + r' H/RD] for item j -- contiguous over threads
             if (live_row)
-                last_pass_out<MIXED>(rd, v, t, TPR, H, [&](int idx, T2 z) {
-                    z.x *= scale; z.y *= scale;
+                last_pass_out<MIXED, V>(rd, v, t, TPR, H, [&](int idx, T2 z) {
+                    if (scaled) { z.x *= scale; z.y *= scale; }
                     out[idx] = z;
                 });
             break;
         }
-        if (r < R) pass_store<T2, MIXED>(rd, row, t, TPR, H, Ns, v);
+        if (r < R) pass_store<T2, MIXED, V>(rd, row, t, TPR, H, Ns, v);
         __syncthreads();
         Ns *= rd;
     }
 }
 
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, int V>
 __global__ void __launch_bounds__(512)
-k_fft_synth(PlanView<T> pv, const T *__restrict__ eo, T *__restrict__ grid, int G, int op)
+k_fft_synth(PlanView<T> pv, const T *__restrict__ eo, T *__restrict__ grid, int G, int op, unsigned long long plan)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fft_synth_tile<T, MIXED>(pv, eo, grid, blockIdx.y, blockIdx.x * G, G, op, smem_raw);
+    fft_synth_tile<T, MIXED, V>(pv, eo, grid, blockIdx.y, blockIdx.x * G, G, op, plan, smem_raw);
 }
 
 // ---------------------------------------------------------------------------
 // Analysis: grid [batch][nlat][nphi] -> SD [batch][mmax+1][npairs][2]
 // ---------------------------------------------------------------------------
 // One tile (field b, pairs p0 .. p0+G-1) of the analysis FFT (see fft_synth_tile).
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, int V = 16>
 __device__ __forceinline__ void fft_analys_tile(const PlanView<T> &pv, const T *__restrict__ grid, T *__restrict__ sd,
-                                                int b, int p0, int G, int op, int vector, unsigned char *smem_raw)
+                                                int b, int p0, int G, int op, int vector, unsigned long long plan,
+                                                unsigned char *smem_raw)
 {
     using T2 = typename Vec2<T>::type;
     const int H = pv.nphi / 2, R = 2 * G;
-    const int TPR = row_tpr(H);
+    const int TPR = row_tpr<V>(H);
     const int ld = padi(H) + 1;
     T2 *wtab = reinterpret_cast<T2 *>(smem_raw);
     T2 *buf = wtab + H;
+    T *s_w = reinterpret_cast<T *>(buf + R * ld);   // per pair: the factor of the folds
     const int mmax = pv.mmax, npairs = pv.npairs, nlat = pv.nlat;
 
     fill_wtab(wtab, pv.tw, H);
+    for (int i = threadIdx.x; i < G; i += blockDim.x) {
+        const int pp = p0 + i;
+        T wf = (op == OP_ANALYS) ? T(kTwoPiD) / T(pv.nphi) : T(1);
+        if (pp < npairs) {
+            if (op == OP_ANALYS) wf *= pv.wq[pp];
+            if (vector) wf /= pv.st[pp];
+        }
+        s_w[i] = wf * T(0.5);   // the halves of E and O below
+    }
     __syncthreads();
     const int r = threadIdx.x / TPR, t = threadIdx.x - r * TPR;
     const int p = p0 + (r >> 1);
@@ -491,50 +534,35 @@ __device__ __forceinline__ void fft_analys_tile(const PlanView<T> &pv, const T *
     } else {
         // forward complex FFT of length H; the first pass reads the grid row
         int Ns = 1;
-        T2 v[PassRegs<MIXED>::n];
-        const int npass = fft_plan_npass(pv.fftplan);
+        T2 v[PassRegs<MIXED, V>::n];
+        const int npass = fft_plan_npass(plan);
         for (int ps = 0; ps < npass; ++ps) {
-            const int rd = fft_plan_radix(pv.fftplan, ps);
+            const int rd = fft_plan_radix(plan, ps);
             if (r < R) {
                 if (ps == 0) {
                     if (live_row) {
-                        pass_load<T2, -1, MIXED>(rd, in, true, t, TPR, H, Ns, wtab, v);
+                        pass_load<T2, -1, MIXED, V>(rd, in, true, t, TPR, H, Ns, wtab, v);
                     } else {
 #pragma unroll
-                        for (int q = 0; q < PassRegs<MIXED>::n; ++q) v[q] = mk<T2>(T(0), T(0));
+                        for (int q = 0; q < PassRegs<MIXED, V>::n; ++q) v[q] = mk<T2>(T(0), T(0));
                     }
                 } else {
-                    pass_load<T2, -1, MIXED>(rd, row, false, t, TPR, H, Ns, wtab, v);
+                    pass_load<T2, -1, MIXED, V>(rd, row, false, t, TPR, H, Ns, wtab, v);
                 }
             }
             __syncthreads();
-            if (r < R) pass_store<T2, MIXED>(rd, row, t, TPR, H, Ns, v);
+            if (r < R) pass_store<T2, MIXED, V>(rd, row, t, TPR, H, Ns, v);
             __syncthreads();
             Ns *= rd;
         }
     }
     __syncthreads();
-    // post-twiddle, scale, fold north/south, weight
+    // post-twiddle, fold north/south, weight.  Positions m and H - m share their
+    // terms: with E = Z_m + conj Z_{H-m}, Od = (Z_m - conj Z_{H-m}) / i and
+    // P = W^{-m} Od (W = e^{2 pi i / (2H)}), 2 X_m = E + P and 2 X_{H-m} = conj(E - P).
     T2 *sd2 = reinterpret_cast<T2 *>(sd);
-    const T fscale = (op == OP_ANALYS) ? T(kTwoPiD) / T(pv.nphi) : T(1);
-    for (int q = threadIdx.x; q < G * (mmax + 1); q += blockDim.x) {
-        const int m = q / G, i = q - m * G;
-        const int pp = p0 + i;
-        if (pp >= npairs) continue;
-        T2 X[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const T2 *rw = buf + (2 * i + h) * ld;
-            const T2 Zk = rw[padi(m)];
-            const T2 Zc = conj_(rw[padi(MIXED ? (H - m) % H : (H - m) & (H - 1))]);
-            T2 E = cadd(Zk, Zc), O = csub(Zk, Zc);
-            E.x *= T(0.5); E.y *= T(0.5);
-            const T2 Od = mk<T2>(O.y * T(0.5), -O.x * T(0.5));  // O / (2i)
-            X[h] = cadd(E, cmul(conj_(pv.tw[m]), Od));
-        }
-        T wf = fscale;
-        if (op == OP_ANALYS) wf *= pv.wq[pp];
-        if (vector) wf /= pv.st[pp];
+    const auto emit = [&](int m, int i, int pp, const T2 (&X)[2]) {
+        const T wf = s_w[i];
         const bool equator = (nlat & 1) && pp == npairs - 1;
         T2 s, d;
         if (equator) {
@@ -547,15 +575,37 @@ __device__ __forceinline__ void fft_analys_tile(const PlanView<T> &pv, const T *
         const size_t o = (((size_t)b * (mmax + 1) + m) * npairs + pp) * 2;
         sd2[o] = s;
         sd2[o + 1] = d;
+    };
+    const int mhalf = min(H / 2, mmax);
+    for (int q = threadIdx.x; q < G * (mhalf + 1); q += blockDim.x) {
+        const int m = q / G, i = q - m * G;
+        const int pp = p0 + i;
+        if (pp >= npairs) continue;
+        const int m2 = H - m;   // its partner, when it is another position and an order of the plan
+        const bool two = m2 != m && m2 < H && m2 <= mmax;
+        T2 X[2], X2[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const T2 *rw = buf + (2 * i + h) * ld;
+            const T2 Zk = rw[padi(m)];
+            const T2 Zc = conj_(rw[padi(m == 0 ? 0 : m2)]);
+            const T2 E = cadd(Zk, Zc), O = csub(Zk, Zc);
+            const T2 P = cmul(conj_(pv.tw[m]), mk<T2>(O.y, -O.x));
+            X[h] = cadd(E, P);
+            X2[h] = conj_(csub(E, P));
+        }
+        emit(m, i, pp, X);
+        if (two) emit(m2, i, pp, X2);
     }
 }
 
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, int V>
 __global__ void __launch_bounds__(512)
-k_fft_analys(PlanView<T> pv, const T *__restrict__ grid, T *__restrict__ sd, int G, int op, int vector)
+k_fft_analys(PlanView<T> pv, const T *__restrict__ grid, T *__restrict__ sd, int G, int op, int vector,
+             unsigned long long plan)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fft_analys_tile<T, MIXED>(pv, grid, sd, blockIdx.y, blockIdx.x * G, G, op, vector, smem_raw);
+    fft_analys_tile<T, MIXED, V>(pv, grid, sd, blockIdx.y, blockIdx.x * G, G, op, vector, plan, smem_raw);
 }
 
 // ---------------------------------------------------------------------------
@@ -1335,25 +1385,43 @@ cudaError_t launch_rows_dispatch(int logH, bool synth, const PlanView<float> &pv
 inline int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 inline bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
+// SMs of the current device.
+inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 152;
+    return sms;
+}
+
 // Threads per row and pairs per CTA: TPR = ceil(H/16) threads per row and
 // enough rows for 256 threads, capped so the CTA's buffer stays <= 96 KB.
 // (512-thread CTAs read the intermediate in longer runs but fit one CTA per
 // SM and measured slower: the kernel is latency-bound, not DRAM-bound.)
+// A launch of few rows takes fewer pairs per CTA, down to one 32-byte sector
+// of the intermediate per order (1 pair in FP64, 2 in FP32), until there are
+// kFftCtasPerSm CTAs per SM: the tile's work is a serial chain of passes (FP64
+// arithmetic above all), so a few full CTAs leave the other SMs idle.
+constexpr int kFftCtasPerSm = 4;
 template <typename T>
-void fft_shape(int H, int npairs, int &G, int &threads, size_t &smem)
+void fft_shape(int H, int V, int npairs, int batch, int &G, int &threads, size_t &smem)
 {
     using T2 = typename Vec2<T>::type;
-    const int TPR = row_tpr(H);
+    const int TPR = (H + V - 1) / V;
     int rows = 256 / TPR;
     if (rows < 2) rows = 2;
     const size_t row_bytes = (size_t)((H + (H >> 4)) + 1) * sizeof(T2);
     while (rows > 2 && (size_t)rows * row_bytes > 96 * 1024) rows /= 2;
     G = rows / 2;
     if (G > npairs) G = npairs < 1 ? 1 : npairs;
+    constexpr int Gmin = sizeof(T) == 8 ? 1 : 2;
+    const long want = (long)kFftCtasPerSm * sm_count();
+    while (G > Gmin && (long)((npairs + G - 1) / G) * batch < want) G = G / 2 < Gmin ? Gmin : G / 2;
     threads = 2 * G * TPR;
-    if (threads < 32) threads = 32;
+    if (threads < 64) threads = 64;   // the phases around the passes have 2 G H / 2 items
     threads = (threads + 31) & ~31;
-    smem = (size_t)H * sizeof(T2) + (size_t)2 * G * row_bytes;
+    smem = (size_t)H * sizeof(T2) + (size_t)2 * G * row_bytes + (size_t)G * sizeof(T);
 }
 
 template <typename K>
@@ -1365,6 +1433,39 @@ cudaError_t set_smem(K kernel, size_t bytes)
 
 }  // namespace
 
+namespace {
+
+template <typename T, bool MIXED, int V>
+cudaError_t synth_tiles(const PlanView<T> &pv, const T *eo, T *grid, int batch, Op op, cudaStream_t s)
+{
+    const int H = pv.nphi / 2;
+    int G, threads;
+    size_t smem;
+    fft_shape<T>(H, V, pv.npairs, batch, G, threads, smem);
+    cudaError_t e = set_smem(k_fft_synth<T, MIXED, V>, smem);
+    if (e != cudaSuccess) return e;
+    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
+    k_fft_synth<T, MIXED, V><<<gridd, threads, smem, s>>>(pv, eo, grid, G, (int)op, fft_plan_of(H, V == 4 ? 2 : 4));
+    return cudaGetLastError();
+}
+
+template <typename T, bool MIXED, int V>
+cudaError_t analys_tiles(const PlanView<T> &pv, const T *grid, T *sd, int batch, Op op, bool vector, cudaStream_t s)
+{
+    const int H = pv.nphi / 2;
+    int G, threads;
+    size_t smem;
+    fft_shape<T>(H, V, pv.npairs, batch, G, threads, smem);
+    cudaError_t e = set_smem(k_fft_analys<T, MIXED, V>, smem);
+    if (e != cudaSuccess) return e;
+    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
+    k_fft_analys<T, MIXED, V><<<gridd, threads, smem, s>>>(pv, grid, sd, G, (int)op, vector ? 1 : 0,
+                                                           fft_plan_of(H, V == 4 ? 2 : 4));
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 template <typename T>
 cudaError_t launch_fft_synth(const PlanView<T> &pv, const T *eo, T *grid, int batch, Op op, cudaStream_t s)
 {
@@ -1372,18 +1473,13 @@ cudaError_t launch_fft_synth(const PlanView<T> &pv, const T *eo, T *grid, int ba
     if constexpr (sizeof(T) == 4) {
         if (pow2(H) && logH <= kRowLogMax) return launch_rows_dispatch(logH, true, pv, eo, grid, batch, op, false, s);
     }
-    int G, threads;
-    size_t smem;
-    fft_shape<T>(H, pv.npairs, G, threads, smem);
-    const bool mixed = !pow2(H);
-    cudaError_t e = mixed ? set_smem(k_fft_synth<T, true>, smem) : set_smem(k_fft_synth<T, false>, smem);
-    if (e != cudaSuccess) return e;
-    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
-    if (mixed)
-        k_fft_synth<T, true><<<gridd, threads, smem, s>>>(pv, eo, grid, G, (int)op);
-    else
-        k_fft_synth<T, false><<<gridd, threads, smem, s>>>(pv, eo, grid, G, (int)op);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        if (fft_values<T>(H) == 4)
+            return pow2(H) ? synth_tiles<T, false, 4>(pv, eo, grid, batch, op, s)
+                           : synth_tiles<T, true, 4>(pv, eo, grid, batch, op, s);
+    }
+    return pow2(H) ? synth_tiles<T, false, 16>(pv, eo, grid, batch, op, s)
+                   : synth_tiles<T, true, 16>(pv, eo, grid, batch, op, s);
 }
 
 template <typename T>
@@ -1395,18 +1491,13 @@ cudaError_t launch_fft_analys(const PlanView<T> &pv, const T *grid, T *sd, int b
         if (pow2(H) && logH <= kRowLogMax)
             return launch_rows_dispatch(logH, false, pv, grid, sd, batch, op, vector, s);
     }
-    int G, threads;
-    size_t smem;
-    fft_shape<T>(H, pv.npairs, G, threads, smem);
-    const bool mixed = !pow2(H);
-    cudaError_t e = mixed ? set_smem(k_fft_analys<T, true>, smem) : set_smem(k_fft_analys<T, false>, smem);
-    if (e != cudaSuccess) return e;
-    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
-    if (mixed)
-        k_fft_analys<T, true><<<gridd, threads, smem, s>>>(pv, grid, sd, G, (int)op, vector ? 1 : 0);
-    else
-        k_fft_analys<T, false><<<gridd, threads, smem, s>>>(pv, grid, sd, G, (int)op, vector ? 1 : 0);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        if (fft_values<T>(H) == 4)
+            return pow2(H) ? analys_tiles<T, false, 4>(pv, grid, sd, batch, op, vector, s)
+                           : analys_tiles<T, true, 4>(pv, grid, sd, batch, op, vector, s);
+    }
+    return pow2(H) ? analys_tiles<T, false, 16>(pv, grid, sd, batch, op, vector, s)
+                   : analys_tiles<T, true, 16>(pv, grid, sd, batch, op, vector, s);
 }
 
 cudaError_t launch_fft_synth_df(const PlanView<double> &pv, const double *eo, double *grid, int batch, Op op,
@@ -1415,7 +1506,7 @@ cudaError_t launch_fft_synth_df(const PlanView<double> &pv, const double *eo, do
     if (!pv.twdf) return cudaErrorInvalidValue;
     int G, threads;
     size_t smem;
-    fft_shape<double>(pv.nphi / 2, pv.npairs, G, threads, smem);
+    fft_shape<double>(pv.nphi / 2, 16, pv.npairs, batch, G, threads, smem);
     smem += df_extra_smem(G);
     const bool mixed = !pow2(pv.nphi / 2), h1024 = pv.nphi == 2048;
     cudaError_t e = mixed ? set_smem(k_fft_synth_df<true>, smem)
@@ -1437,7 +1528,7 @@ cudaError_t launch_fft_analys_df(const PlanView<double> &pv, const double *grid,
     if (!pv.twdf) return cudaErrorInvalidValue;
     int G, threads;
     size_t smem;
-    fft_shape<double>(pv.nphi / 2, pv.npairs, G, threads, smem);
+    fft_shape<double>(pv.nphi / 2, 16, pv.npairs, batch, G, threads, smem);
     smem += df_extra_smem(G);
     const bool mixed = !pow2(pv.nphi / 2), h1024 = pv.nphi == 2048;
     cudaError_t e = mixed ? set_smem(k_fft_analys_df<true>, smem)
@@ -1485,9 +1576,9 @@ __global__ void __launch_bounds__(256, 2) k_batch_fft(int synth, const BatchFiel
             default: break;
             }
         } else if (synth) {
-            fft_synth_tile<float, true>(f.pv, f.inter, f.out, 0, tl.y, f.G, OP_SYNTH, smem_raw);
+            fft_synth_tile<float, true>(f.pv, f.inter, f.out, 0, tl.y, f.G, OP_SYNTH, f.pv.fftplan, smem_raw);
         } else {
-            fft_analys_tile<float, true>(f.pv, f.in, f.inter, 0, tl.y, f.G, OP_ANALYS, 0, smem_raw);
+            fft_analys_tile<float, true>(f.pv, f.in, f.inter, 0, tl.y, f.G, OP_ANALYS, 0, f.pv.fftplan, smem_raw);
         }
     }
 }
@@ -1510,7 +1601,7 @@ size_t batch_fft_smem(int H, int G)
 {
     if (pow2(H) && ilog2(H) <= kRowLogMax) return row_fft_smem(row_ld(ilog2(H)), row_pairs(ilog2(H)));
     const size_t row_bytes = (size_t)((H + (H >> 4)) + 1) * sizeof(float2);
-    return (size_t)H * sizeof(float2) + (size_t)2 * G * row_bytes;
+    return (size_t)H * sizeof(float2) + (size_t)2 * G * row_bytes + (size_t)G * sizeof(float);
 }
 
 cudaError_t batch_fft_prepare(size_t smem) { return set_smem(k_batch_fft, smem); }

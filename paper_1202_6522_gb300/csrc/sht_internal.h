@@ -90,10 +90,10 @@ __host__ __device__ inline long col_of_mres(int lmax, int k, int mres)
 
 // Pass plan of a mixed-radix FFT of length H = 2^a 3^b 5^c: bits 0-3 the
 // number of passes (none for H = 1), then 5 bits per pass radix (2, 4, 8, 16,
-// 3 or 5), the power-of-two part first.  kFftPlanBad if H has another prime
-// factor or needs more than 12 passes.
+// 3 or 5), the power-of-two part first, in radices of at most 2^max_log.
+// kFftPlanBad if H has another prime factor or needs more than 12 passes.
 constexpr unsigned long long kFftPlanBad = ~0ull;
-inline unsigned long long fft_plan_of(int H)
+inline unsigned long long fft_plan_of(int H, int max_log = 4)
 {
     if (H < 1) return kFftPlanBad;
     int a = 0, b = 0, c = 0, h = H;
@@ -102,8 +102,8 @@ inline unsigned long long fft_plan_of(int H)
     while (h % 5 == 0) { h /= 5; ++c; }
     if (h != 1) return kFftPlanBad;
     int rad[16], n = 0;
-    if (a % 4) rad[n++] = 1 << (a % 4);
-    for (int i = 0; i < a / 4; ++i) rad[n++] = 16;
+    if (a % max_log) rad[n++] = 1 << (a % max_log);
+    for (int i = 0; i < a / max_log; ++i) rad[n++] = 1 << max_log;
     for (int i = 0; i < b; ++i) rad[n++] = 3;
     for (int i = 0; i < c; ++i) rad[n++] = 5;
     if (n > 12) return kFftPlanBad;
