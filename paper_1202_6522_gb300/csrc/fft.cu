@@ -1401,9 +1401,10 @@ inline int sm_count()
 // SM and measured slower: the kernel is latency-bound, not DRAM-bound.)
 // A launch of few rows takes fewer pairs per CTA, down to one 32-byte sector
 // of the intermediate per order (1 pair in FP64, 2 in FP32), until there are
-// kFftCtasPerSm CTAs per SM: the tile's work is a serial chain of passes (FP64
-// arithmetic above all), so a few full CTAs leave the other SMs idle.
-constexpr int kFftCtasPerSm = 4;
+// four (FP64) or two (FP32) CTAs per SM: the tile's work is a serial chain of
+// passes (FP64 arithmetic above all), so a few full CTAs leave the other SMs
+// idle.  Powers of two only, which keep the pairs' sectors whole: 16 FP32 fields
+// of 256 x 540 took 21 us with 7 pairs (304 CTAs) and 33 us with 3.
 template <typename T>
 void fft_shape(int H, int V, int npairs, int batch, int &G, int &threads, size_t &smem)
 {
@@ -1416,8 +1417,12 @@ void fft_shape(int H, int V, int npairs, int batch, int &G, int &threads, size_t
     G = rows / 2;
     if (G > npairs) G = npairs < 1 ? 1 : npairs;
     constexpr int Gmin = sizeof(T) == 8 ? 1 : 2;
-    const long want = (long)kFftCtasPerSm * sm_count();
-    while (G > Gmin && (long)((npairs + G - 1) / G) * batch < want) G = G / 2 < Gmin ? Gmin : G / 2;
+    const long want = (sizeof(T) == 8 ? 4L : 2L) * sm_count();
+    while (G > Gmin && (long)((npairs + G - 1) / G) * batch < want) {
+        int g = Gmin;
+        while (2 * g < G) g *= 2;
+        G = g;
+    }
     threads = 2 * G * TPR;
     if (threads < 64) threads = 64;   // the phases around the passes have 2 G H / 2 items
     threads = (threads + 31) & ~31;
