@@ -503,6 +503,28 @@ void set_tuned(sht::Plan &p, int mode, int batch, const sht::TunedShape &t)
 
 template <typename T> constexpr int mode_of_type() { return sizeof(T) == 8 ? SHT_F64 : SHT_F32; }
 
+// The Legendre stage of one precision with a tuned shape.
+cudaError_t legendre_synth(const sht::PlanView<double> &pv, const double *spec, double *eo, int batch, sht::Op op,
+                           const sht::TunedShape &ts, cudaStream_t s)
+{
+    return sht::launch_synth64(pv, spec, eo, batch, op, ts.synth_lpt, ts.synth_bc, s);
+}
+cudaError_t legendre_synth(const sht::PlanView<float> &pv, const float *spec, float *eo, int batch, sht::Op op,
+                           const sht::TunedShape &ts, cudaStream_t s)
+{
+    return sht::launch_legendre_synth(pv, spec, eo, batch, op, ts.synth_lpt, ts.synth_bc, s);
+}
+cudaError_t legendre_analys(const sht::PlanView<double> &pv, const double *sd, double *spec, int batch, sht::Op op,
+                            const sht::TunedShape &ts, cudaStream_t s)
+{
+    return sht::launch_analys64(pv, sd, spec, batch, op, ts.analys_bc, s);
+}
+cudaError_t legendre_analys(const sht::PlanView<float> &pv, const float *sd, float *spec, int batch, sht::Op op,
+                            const sht::TunedShape &ts, cudaStream_t s)
+{
+    return sht::launch_legendre_analys(pv, sd, spec, batch, op, ts.analys_lpt, ts.analys_bc, s);
+}
+
 // The two directions of the scalar transform, parameterised by precision.
 template <typename T>
 int run_synth(sht::Plan &p, const sht::PlanView<T> &pv, const void *spec, void *grid, int batch, sht::Op op,
@@ -511,8 +533,7 @@ int run_synth(sht::Plan &p, const sht::PlanView<T> &pv, const void *spec, void *
     T *eo = static_cast<T *>(p.work);
     const sht::TunedShape ts = tuned_shape(p, mode_of_type<T>(), batch);
     int rc = timed(p, SHT_K_LEGENDRE_SYNTH, s, "legendre synthesis launch", [&] {
-        return sht::launch_legendre_synth_cfg<T>(pv, static_cast<const T *>(spec), eo, batch, op, ts.synth_lpt,
-                                                 ts.synth_bc, s);
+        return legendre_synth(pv, static_cast<const T *>(spec), eo, batch, op, ts, s);
     });
     if (rc) return rc;
     return timed(p, SHT_K_FFT_SYNTH, s, "fft synthesis launch", [&] {
@@ -531,9 +552,15 @@ int run_analys(sht::Plan &p, const sht::PlanView<T> &pv, const void *grid, void 
     if (rc) return rc;
     const sht::TunedShape ts = tuned_shape(p, mode_of_type<T>(), batch);
     return timed(p, SHT_K_LEGENDRE_ANALYS, s, "legendre analysis launch", [&] {
-        return sht::launch_legendre_analys_cfg<T>(pv, sd, static_cast<T *>(spec), batch, op, ts.analys_lpt,
-                                                  ts.analys_bc, s);
+        return legendre_analys(pv, sd, static_cast<T *>(spec), batch, op, ts, s);
     });
+}
+
+// Vector transforms on the CUDA cores: two intermediates (theta, phi) and, in
+// FP64, the spectra of the scalar form behind them.
+size_t vec_work_bytes(const sht::Plan &p, int batch, int mode)
+{
+    return 2 * inter_bytes(p, batch, mode) + (mode == SHT_F64 ? sht::vec64_spec_bytes(p.nlm, p.mmax, batch) : 0);
 }
 
 template <typename T>
@@ -543,8 +570,12 @@ int run_synth_vec(sht::Plan &p, const sht::PlanView<T> &pv, const void *S, const
     T *eot = static_cast<T *>(p.work);
     T *eop = eot + (size_t)batch * (p.mmax + 1) * p.npairs * 4;
     int rc = timed(p, SHT_K_LEGENDRE_SYNTH_VEC, s, "legendre vector synthesis launch", [&] {
-        return sht::launch_legendre_synth_vec<T>(pv, static_cast<const T *>(S), static_cast<const T *>(Tc), eot, eop,
-                                                 batch, op, s);
+        const T *Si = static_cast<const T *>(S), *Ti = static_cast<const T *>(Tc);
+        if constexpr (sizeof(T) == sizeof(double))
+            return sht::launch_synth_vec64(pv, Si, Ti, eop + (size_t)batch * (p.mmax + 1) * p.npairs * 4, eot, batch,
+                                           op, s);
+        else
+            return sht::launch_legendre_synth_vec(pv, Si, Ti, eot, eop, batch, op, s);
     });
     if (rc) return rc;
     rc = timed(p, SHT_K_FFT_SYNTH, s, "fft synthesis launch",
@@ -569,8 +600,12 @@ int run_analys_vec(sht::Plan &p, const sht::PlanView<T> &pv, const void *vt, con
     });
     if (rc) return rc;
     return timed(p, SHT_K_LEGENDRE_ANALYS_VEC, s, "legendre vector analysis launch", [&] {
-        return sht::launch_legendre_analys_vec<T>(pv, sdt, sdp, static_cast<T *>(S), static_cast<T *>(Tc), batch, op,
-                                                  s);
+        T *So = static_cast<T *>(S), *To = static_cast<T *>(Tc);
+        if constexpr (sizeof(T) == sizeof(double))
+            return sht::launch_analys_vec64(pv, sdt, sdp + (size_t)batch * (p.mmax + 1) * p.npairs * 4, So, To, batch,
+                                            op, s);
+        else
+            return sht::launch_legendre_analys_vec(pv, sdt, sdp, So, To, batch, op, s);
     });
 }
 
@@ -659,7 +694,8 @@ int vector_s2g(sht_handle h, const void *S, const void *T, void *vt, void *vp, i
         return run_synth_vec_tc(h->p, S, T, vt, vp, batch, op, s);
     }
     if (mode == SHT_F32 && (rc = ensure_seeds32(h->p))) return rc;
-    if ((rc = ensure_work(h->p, 2 * inter_bytes(h->p, batch, mode)))) return rc;
+    if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
+    if ((rc = ensure_work(h->p, vec_work_bytes(h->p, batch, mode)))) return rc;
     if (mode == SHT_F64) return run_synth_vec<double>(h->p, h->p.view64(), S, T, vt, vp, batch, op, s);
     return run_synth_vec<float>(h->p, h->p.view32(), S, T, vt, vp, batch, op, s);
 }
@@ -678,7 +714,8 @@ int vector_g2s(sht_handle h, const void *vt, const void *vp, void *S, void *T, i
         return run_analys_vec_tc(h->p, vt, vp, S, T, batch, op, s);
     }
     if (mode == SHT_F32 && (rc = ensure_seeds32(h->p))) return rc;
-    if ((rc = ensure_work(h->p, 2 * inter_bytes(h->p, batch, mode)))) return rc;
+    if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
+    if ((rc = ensure_work(h->p, vec_work_bytes(h->p, batch, mode)))) return rc;
     if (mode == SHT_F64) return run_analys_vec<double>(h->p, h->p.view64(), vt, vp, S, T, batch, op, s);
     return run_analys_vec<float>(h->p, h->p.view32(), vt, vp, S, T, batch, op, s);
 }
@@ -978,7 +1015,7 @@ int sht_reserve(sht_handle h, int batch, int mode)
     }
     if ((mode == SHT_F32 || mode == SHT_F32_AUTO) && (rc = ensure_seeds32(h->p))) return rc;
     if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
-    return ensure_work(h->p, 2 * inter_bytes(h->p, batch, mode));
+    return ensure_work(h->p, vec_work_bytes(h->p, batch, mode));
 }
 
 int sht_synth(sht_handle h, const void *spec, void *grid, int batch, int mode, void *stream)
@@ -1242,36 +1279,35 @@ extern "C" int sht_tune(sht_handle h, int batch, int mode, double *report, void 
     sht::TunedShape best;
     double best_syn = 1e30, best_ana = 1e30;
     const int reps = 3;
-    const int lpts_s[3] = {1, 2, 4}, bcs_s[4] = {1, 2, 4, 8};
-    for (int li = 0; li < 3; ++li)
-        for (int bi = 0; bi < 4; ++bi) {
-            const int lpt = lpts_s[li], bc = bcs_s[bi];
+    const int widths[5] = {1, 2, 4, 8, 16};   // fields per CTA (FP32: up to 4 and 2)
+    const int lpts_s[4] = {1, 2, 4, 8}, lpts_a[3] = {2, 4, 8};
+    for (int li = 0; li < 4; ++li)
+        for (int bi = 0; bi < 5; ++bi) {
+            const int lpt = lpts_s[li], bc = widths[bi];   // FP64: lpt warps per CTA
             if (bc > batch && bc > 1) continue;
-            if (bc == 8 && (shape_mode != SHT_F64 || lpt > 2)) continue;
+            if (shape_mode == SHT_F64 ? (bc == 16 && lpt == 8) : (lpt > 4 || bc > 4)) continue;
             bool ok = false;
             double ms;
             if (shape_mode == SHT_F64)
-                ms = time_ms([&] { return sht::launch_legendre_synth_cfg<double>(p.view64(), (const double *)spec, (double *)p.work, batch, sht::OP_SYNTH, lpt, bc, s); }, s, reps, ok);
+                ms = time_ms([&] { return sht::launch_synth64(p.view64(), (const double *)spec, (double *)p.work, batch, sht::OP_SYNTH, lpt, bc, s); }, s, reps, ok);
             else
-                ms = time_ms([&] { return sht::launch_legendre_synth_cfg<float>(p.view32(), (const float *)spec, (float *)p.work, batch, sht::OP_SYNTH, lpt, bc, s); }, s, reps, ok);
+                ms = time_ms([&] { return sht::launch_legendre_synth(p.view32(), (const float *)spec, (float *)p.work, batch, sht::OP_SYNTH, lpt, bc, s); }, s, reps, ok);
             if (ok && ms < best_syn) { best_syn = ms; best.synth_lpt = lpt; best.synth_bc = bc; }
         }
-    const int lpts_a[4] = {2, 4, 8, sht::kAnalysSeg}, bcs_a[4] = {1, 2, 4, 8};
-    for (int li = 0; li < 4; ++li)
-        for (int bi = 0; bi < 4; ++bi) {
-            const int lpt = lpts_a[li], bc = bcs_a[bi];
+    for (int li = 0; li < 3; ++li)
+        for (int bi = 0; bi < 5; ++bi) {
+            const int lpt = lpts_a[li], bc = widths[bi];
             if (bc > batch && bc > 1) continue;
-            if (lpt == sht::kAnalysSeg
-                    ? (shape_mode != SHT_F64 || p.npairs > 2048 || (p.npairs > 1024 && bc > 2) ||
-                       (p.npairs > 512 && bc > 4))
+            if (shape_mode == SHT_F64
+                    ? li > 0
                     : (bc > 2 || (p.npairs + 32 * lpt - 1) / (32 * lpt) > 8))
                 continue;
             bool ok = false;
             double ms;
             if (shape_mode == SHT_F64)
-                ms = time_ms([&] { return sht::launch_legendre_analys_cfg<double>(p.view64(), (const double *)p.work, (double *)spec, batch, sht::OP_ANALYS, lpt, bc, s); }, s, reps, ok);
+                ms = time_ms([&] { return sht::launch_analys64(p.view64(), (const double *)p.work, (double *)spec, batch, sht::OP_ANALYS, bc, s); }, s, reps, ok);
             else
-                ms = time_ms([&] { return sht::launch_legendre_analys_cfg<float>(p.view32(), (const float *)p.work, (float *)spec, batch, sht::OP_ANALYS, lpt, bc, s); }, s, reps, ok);
+                ms = time_ms([&] { return sht::launch_legendre_analys(p.view32(), (const float *)p.work, (float *)spec, batch, sht::OP_ANALYS, lpt, bc, s); }, s, reps, ok);
             if (ok && ms < best_ana) { best_ana = ms; best.analys_lpt = lpt; best.analys_bc = bc; }
         }
     cudaGetLastError();
@@ -1396,8 +1432,7 @@ extern "C" int sht_synth_static(sht_handle h, const void *spec, void *grid, int 
     if (mode == SHT_F64) {
         const sht::PlanView<double> pv = h->p.view64();
         double *eo = static_cast<double *>(scratch);
-        rc = launched(sht::launch_legendre_synth<double>(pv, static_cast<const double *>(spec), eo, batch,
-                                                         sht::OP_SYNTH, s),
+        rc = launched(sht::launch_synth64(pv, static_cast<const double *>(spec), eo, batch, sht::OP_SYNTH, 0, 0, s),
                       "legendre synthesis launch");
         if (rc) return rc;
         return launched(sht::launch_fft_synth<double>(pv, eo, static_cast<double *>(grid), batch, sht::OP_SYNTH, s),
@@ -1405,7 +1440,7 @@ extern "C" int sht_synth_static(sht_handle h, const void *spec, void *grid, int 
     }
     const sht::PlanView<float> pv = h->p.view32();
     float *eo = static_cast<float *>(scratch);
-    rc = launched(sht::launch_legendre_synth<float>(pv, static_cast<const float *>(spec), eo, batch, sht::OP_SYNTH, s),
+    rc = launched(sht::launch_legendre_synth(pv, static_cast<const float *>(spec), eo, batch, sht::OP_SYNTH, 0, 0, s),
                   "legendre synthesis launch");
     if (rc) return rc;
     return launched(sht::launch_fft_synth<float>(pv, eo, static_cast<float *>(grid), batch, sht::OP_SYNTH, s),

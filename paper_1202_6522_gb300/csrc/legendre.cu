@@ -147,14 +147,11 @@ __device__ __forceinline__ unsigned live_groups(const int (&gf)[LPT], int seg)
     return r;
 }
 
-// The scalar kernels need the restart states and the first-live table (both
-// precisions); the vector kernels need the restart states in FP32 only.  A
-// plan without them is refused rather than run on other arithmetic.
-template <typename T> bool seeds_ok(const PlanView<T> &pv, bool scalar)
+// The kernels need the restart states, the scalar ones the first-live table
+// too.  A plan without them is refused rather than run on other arithmetic.
+bool seeds_ok(const PlanView<float> &pv, bool scalar)
 {
-    if (sizeof(T) == sizeof(float))
-        return pv.segoff != nullptr && pv.seeds != nullptr && (!scalar || pv.live != nullptr);
-    return !scalar || (pv.segoff != nullptr && pv.seeds64 != nullptr && pv.seeds64k != nullptr && pv.live != nullptr);
+    return pv.segoff != nullptr && pv.seeds != nullptr && (!scalar || pv.live != nullptr);
 }
 
 // Warp butterfly that sums V values (V a multiple of 32) over the 32 lanes and
@@ -487,277 +484,6 @@ k_analys(PlanView<T> pv, const T *__restrict__ sd, T *__restrict__ spec, int bat
 }
 
 // ---------------------------------------------------------------------------
-// Scalar analysis, one warp per segment (FP64; npairs <= 32 PPL).
-// grid.x = m (heaviest first), grid.y = field group of BC.  The CTA stages
-// the folds s, d of its BC fields for all pairs in shared memory; each of its
-// kSegWarps warps then takes kSeedSeg-degree segments from a shared counter,
-// restarts the recurrence from the stored state and sums over every pair on
-// its own: PPL pairs per lane, then one warp butterfly per K = 16 / BC
-// degrees.  There is no CTA-wide barrier inside the sums, the recurrence is
-// shared by BC fields, and the cross-lane reduction costs 1/PPL of the sums;
-// the order of every sum is fixed, so results are bitwise reproducible.
-// Groups of 32 pairs with no live pair in a segment (static polar
-// optimisation, Sec. 3.1) run neither the recurrence nor the sums.
-// ---------------------------------------------------------------------------
-constexpr int kSegWarps = 8;
-
-template <typename T, int PPL, int BC>
-__global__ void __launch_bounds__(kSegWarps * 32, 1)
-k_analys_seg(PlanView<T> pv, const T *__restrict__ sd, T *__restrict__ spec, int batch, int op)
-{
-    using T2 = typename Vec2<T>::type;
-    constexpr int K = 16 / BC;        // degrees per butterfly: 2 K BC = 32 values
-    constexpr int R = 32 * PPL;       // staged row: the pairs, zero-padded
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2 *s_v = reinterpret_cast<T2 *>(smem_raw);   // [BC][parity][R]: s (n - m even), d (odd)
-    __shared__ int s_next;
-    __shared__ int s_gfirst[PPL];                 // first live segment of each group of 32 pairs
-
-    const int m = blockIdx.x, b0 = blockIdx.y * BC;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int npairs = pv.npairs;
-    const int L = pv.lmax - m * pv.mres + 1;   // order index m is the order m mres
-    const long col = col_of_mres(pv.lmax, m, pv.mres);
-    const int nseg = (L + kSeedSeg - 1) / kSeedSeg;
-
-    const T2 *sd2 = reinterpret_cast<const T2 *>(sd);
-    for (int idx = threadIdx.x; idx < BC * 2 * R; idx += blockDim.x) {
-        const int b = idx / (2 * R), r = idx - b * 2 * R;
-        T2 v;
-        v.x = T(0); v.y = T(0);
-        if (r < 2 * npairs && b0 + b < batch) v = sd2[((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs * 2 + r];
-        s_v[(b * 2 + (r & 1)) * R + (r >> 1)] = v;
-    }
-    for (int g = warp; g < PPL; g += kSegWarps) {
-        const int pp = g * 32 + lane;
-        const int f = pp < npairs ? (int)pv.live[(size_t)m * npairs + pp] : 0xffff;
-        const int gm = __reduce_min_sync(kFull, f);
-        if (lane == 0) s_gfirst[g] = gm;
-    }
-    if (threadIdx.x == 0) s_next = kSegWarps;
-    __syncthreads();
-
-    const T outsc = (op == OP_SYNTH_ADJ && m > 0) ? T(2) : T(1);   // c_m for the adjoint of synthesis
-    T2 *spec2 = reinterpret_cast<T2 *>(spec);
-    int p[PPL];
-    T x[PPL];
-#pragma unroll
-    for (int i = 0; i < PPL; ++i) {
-        p[i] = lane + 32 * i;
-        x[i] = p[i] < npairs ? pv.x[p[i]] : T(0);
-    }
-    // value `lane` of the butterfly: degree t0 + kx, field b, real/imaginary part
-    const int okx = lane / (2 * BC), ob = (lane >> 1) % BC, opart = lane & 1;
-
-    for (int seg = warp; seg < nseg;) {
-        const int nn0 = seg * kSeedSeg, cnt = min(kSeedSeg, L - nn0);
-        unsigned live = 0;
-#pragma unroll
-        for (int i = 0; i < PPL; ++i)
-            if (s_gfirst[i] <= seg) live |= 1u << i;
-        if (live == 0) {
-            for (int q = lane; q < cnt * 2 * BC; q += 32) {
-                const int kx = q / (2 * BC), b = (q >> 1) % BC;
-                if (b0 + b < batch)
-                    reinterpret_cast<T *>(&spec2[(size_t)(b0 + b) * pv.nlm + col + nn0 + kx])[q & 1] = T(0);
-            }
-        } else {
-            T y1[PPL], y2[PPL];
-            int k[PPL];
-#pragma unroll
-            for (int i = 0; i < PPL; ++i) {
-                y1[i] = y2[i] = T(0);
-                k[i] = 0;
-            }
-            reseed<T, PPL>(pv, m, seg, p, y1, y2, k);
-            unsigned scaled = 0;
-#pragma unroll
-            for (int i = 0; i < PPL; ++i)
-                if (__any_sync(kFull, k[i] > 0)) scaled |= 1u << i;
-            for (int t0 = 0; t0 < cnt; t0 += K) {
-                T acc[32];
-#pragma unroll
-                for (int q = 0; q < 32; ++q) acc[q] = T(0);
-#pragma unroll
-                for (int kx = 0; kx < K; ++kx) {
-                    if (t0 + kx >= cnt) break;
-                    const T2 ab = __ldg(&pv.ab[col + nn0 + t0 + kx]);
-                    const T2 *vrow = s_v + ((t0 + kx) & 1) * R;   // nn0 is even
-#pragma unroll
-                    for (int i = 0; i < PPL; ++i) {
-                        if (!((live >> i) & 1)) continue;
-                        const T yn = fma(ab.x * x[i], y1[i], ab.y * y2[i]);
-                        y2[i] = y1[i];
-                        y1[i] = yn;
-                        T c = yn;
-                        if ((scaled >> i) & 1) {
-                            if (k[i] > 0 && abs_ge_one(yn)) {
-                                y1[i] *= down_scale<T>();
-                                y2[i] *= down_scale<T>();
-                                k[i] -= 1;
-                            }
-                            c = (k[i] == 0) ? y1[i] : T(0);
-                        }
-#pragma unroll
-                        for (int b = 0; b < BC; ++b) {
-                            const T2 v = vrow[b * 2 * R + p[i]];
-                            acc[(kx * BC + b) * 2] = fma(c, v.x, acc[(kx * BC + b) * 2]);
-                            acc[(kx * BC + b) * 2 + 1] = fma(c, v.y, acc[(kx * BC + b) * 2 + 1]);
-                        }
-                    }
-                }
-                warp_transpose_reduce<T, 32>(acc, lane);
-                if (t0 + okx < cnt && b0 + ob < batch) {
-                    T val = acc[0] * outsc;
-                    if (m == 0 && opart == 1) val = T(0);
-                    reinterpret_cast<T *>(&spec2[(size_t)(b0 + ob) * pv.nlm + col + nn0 + t0 + okx])[opart] = val;
-                }
-            }
-        }
-        int nx = 0;
-        if (lane == 0) nx = atomicAdd(&s_next, 1);
-        seg = __shfl_sync(kFull, nx, 0);
-    }
-}
-
-// More pairs than a warp holds (npairs <= 32 PPL TEAM): a team of TEAM warps
-// takes each segment, every warp summing its own 32 PPL pairs; per butterfly
-// the warps' partial sums meet in shared memory (double-buffered by
-// butterfly, one named barrier per team each time) and the team's first warp
-// adds them in a fixed order and writes the coefficients.  Teams take the
-// segments t, t + teams, ... of the order.
-template <typename T, int PPL, int BC, int TEAM>
-__global__ void __launch_bounds__(kSegWarps * 32, 1)
-k_analys_seg_team(PlanView<T> pv, const T *__restrict__ sd, T *__restrict__ spec, int batch, int op)
-{
-    using T2 = typename Vec2<T>::type;
-    constexpr int K = 16 / BC;           // degrees per butterfly: 2 K BC = 32 values
-    constexpr int R = 32 * PPL * TEAM;   // staged row: the pairs, zero-padded
-    constexpr int NTEAM = kSegWarps / TEAM, NG = PPL * TEAM;
-    static_assert(kSegWarps % TEAM == 0, "whole teams");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2 *s_v = reinterpret_cast<T2 *>(smem_raw);   // [BC][parity][R]: s (n - m even), d (odd)
-    __shared__ int s_gfirst[NG];                  // first live segment of each group of 32 pairs
-    __shared__ T s_part[NTEAM][2][TEAM][32];      // the warps' partial sums
-
-    const int m = blockIdx.x, b0 = blockIdx.y * BC;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int team = warp / TEAM, wt = warp - team * TEAM;
-    const int npairs = pv.npairs;
-    const int L = pv.lmax - m * pv.mres + 1;   // order index m is the order m mres
-    const long col = col_of_mres(pv.lmax, m, pv.mres);
-    const int nseg = (L + kSeedSeg - 1) / kSeedSeg;
-
-    const T2 *sd2 = reinterpret_cast<const T2 *>(sd);
-    for (int idx = threadIdx.x; idx < BC * 2 * R; idx += blockDim.x) {
-        const int b = idx / (2 * R), r = idx - b * 2 * R;
-        T2 v;
-        v.x = T(0); v.y = T(0);
-        if (r < 2 * npairs && b0 + b < batch) v = sd2[((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs * 2 + r];
-        s_v[(b * 2 + (r & 1)) * R + (r >> 1)] = v;
-    }
-    for (int g = warp; g < NG; g += kSegWarps) {
-        const int pp = g * 32 + lane;
-        const int f = pp < npairs ? (int)pv.live[(size_t)m * npairs + pp] : 0xffff;
-        const int gm = __reduce_min_sync(kFull, f);
-        if (lane == 0) s_gfirst[g] = gm;
-    }
-    __syncthreads();
-
-    const T outsc = (op == OP_SYNTH_ADJ && m > 0) ? T(2) : T(1);   // c_m for the adjoint of synthesis
-    T2 *spec2 = reinterpret_cast<T2 *>(spec);
-    const int pbase = wt * 32 * PPL;
-    int p[PPL];
-    T x[PPL];
-#pragma unroll
-    for (int i = 0; i < PPL; ++i) {
-        p[i] = pbase + lane + 32 * i;
-        x[i] = p[i] < npairs ? pv.x[p[i]] : T(0);
-    }
-    const int okx = lane / (2 * BC), ob = (lane >> 1) % BC, opart = lane & 1;
-    unsigned kb = 0;   // butterflies done by this team (selects the partial buffer)
-
-    for (int seg = team; seg < nseg; seg += NTEAM) {
-        const int nn0 = seg * kSeedSeg, cnt = min(kSeedSeg, L - nn0);
-        unsigned live = 0;      // this warp's groups
-        bool team_live = false;
-#pragma unroll
-        for (int i = 0; i < PPL; ++i)
-            if (s_gfirst[wt * PPL + i] <= seg) live |= 1u << i;
-        for (int g = 0; g < NG; ++g) team_live |= s_gfirst[g] <= seg;
-        if (!team_live) {
-            if (wt == 0) {
-                for (int q = lane; q < cnt * 2 * BC; q += 32) {
-                    const int kx = q / (2 * BC), b = (q >> 1) % BC;
-                    if (b0 + b < batch)
-                        reinterpret_cast<T *>(&spec2[(size_t)(b0 + b) * pv.nlm + col + nn0 + kx])[q & 1] = T(0);
-                }
-            }
-            continue;
-        }
-        T y1[PPL], y2[PPL];
-        int k[PPL];
-#pragma unroll
-        for (int i = 0; i < PPL; ++i) {
-            y1[i] = y2[i] = T(0);
-            k[i] = 0;
-        }
-        if (live) reseed<T, PPL>(pv, m, seg, p, y1, y2, k);
-        unsigned scaled = 0;
-#pragma unroll
-        for (int i = 0; i < PPL; ++i)
-            if (__any_sync(kFull, k[i] > 0)) scaled |= 1u << i;
-        for (int t0 = 0; t0 < cnt; t0 += K, ++kb) {
-            T acc[32];
-#pragma unroll
-            for (int q = 0; q < 32; ++q) acc[q] = T(0);
-            if (live) {
-#pragma unroll
-                for (int kx = 0; kx < K; ++kx) {
-                    if (t0 + kx >= cnt) break;
-                    const T2 ab = __ldg(&pv.ab[col + nn0 + t0 + kx]);
-                    const T2 *vrow = s_v + ((t0 + kx) & 1) * R;   // nn0 is even
-#pragma unroll
-                    for (int i = 0; i < PPL; ++i) {
-                        if (!((live >> i) & 1)) continue;
-                        const T yn = fma(ab.x * x[i], y1[i], ab.y * y2[i]);
-                        y2[i] = y1[i];
-                        y1[i] = yn;
-                        T c = yn;
-                        if ((scaled >> i) & 1) {
-                            if (k[i] > 0 && abs_ge_one(yn)) {
-                                y1[i] *= down_scale<T>();
-                                y2[i] *= down_scale<T>();
-                                k[i] -= 1;
-                            }
-                            c = (k[i] == 0) ? y1[i] : T(0);
-                        }
-#pragma unroll
-                        for (int b = 0; b < BC; ++b) {
-                            const T2 v = vrow[b * 2 * R + p[i]];
-                            acc[(kx * BC + b) * 2] = fma(c, v.x, acc[(kx * BC + b) * 2]);
-                            acc[(kx * BC + b) * 2 + 1] = fma(c, v.y, acc[(kx * BC + b) * 2 + 1]);
-                        }
-                    }
-                }
-                warp_transpose_reduce<T, 32>(acc, lane);
-            }
-            s_part[team][kb & 1][wt][lane] = acc[0];
-            // the team's warps: named barrier 1 + team over 32 TEAM threads
-            asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * TEAM) : "memory");
-            if (wt == 0 && t0 + okx < cnt && b0 + ob < batch) {
-                T tot = s_part[team][kb & 1][0][lane];
-#pragma unroll
-                for (int w = 1; w < TEAM; ++w) tot += s_part[team][kb & 1][w][lane];
-                T val = tot * outsc;
-                if (m == 0 && opart == 1) val = T(0);
-                reinterpret_cast<T *>(&spec2[(size_t)(b0 + ob) * pv.nlm + col + nn0 + t0 + okx])[opart] = val;
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Vector synthesis.  With dP = sin(theta) dP/dtheta = n x P_n - dc_n P_{n-1}:
 //   sin * V_theta,m = sum [S dP - i m T P],   sin * V_phi,m = sum [i m S P + T dP].
 // dP has the opposite mirror parity of P.  Outputs E/O for theta and phi.
@@ -1086,36 +812,6 @@ cudaError_t analys_go(const PlanView<T> &pv, const T *sd, T *spec, int batch, Op
     return cudaGetLastError();
 }
 
-// Pairs per lane of the segment analysis kernel (0: too many pairs for one warp).
-inline int seg_ppl(int npairs) { return npairs <= 128 ? 4 : (npairs <= 256 ? 8 : (npairs <= 512 ? 16 : 0)); }
-
-// FP64 analysis with 512 < npairs <= 2048: teams of 2 or 4 warps of 16 pairs per lane.
-template <int TEAM, int BC>
-cudaError_t analys_team_go(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op,
-                           cudaStream_t s)
-{
-    const size_t smem = sizeof(double2) * BC * 2 * 32 * 16 * TEAM;
-    cudaError_t e = cudaFuncSetAttribute(k_analys_seg_team<double, 16, BC, TEAM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(pv.mmax + 1), (unsigned)((batch + BC - 1) / BC));
-    k_analys_seg_team<double, 16, BC, TEAM><<<grid, kSegWarps * 32, smem, s>>>(pv, sd, spec, batch, (int)op);
-    return cudaGetLastError();
-}
-
-template <typename T, int PPL, int BC>
-cudaError_t analys_seg_go(const PlanView<T> &pv, const T *sd, T *spec, int batch, Op op, cudaStream_t s)
-{
-    using T2 = typename Vec2<T>::type;
-    const size_t smem = sizeof(T2) * BC * 2 * 32 * PPL;
-    cudaError_t e = cudaFuncSetAttribute(k_analys_seg<T, PPL, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(pv.mmax + 1), (unsigned)((batch + BC - 1) / BC));
-    k_analys_seg<T, PPL, BC><<<grid, kSegWarps * 32, smem, s>>>(pv, sd, spec, batch, (int)op);
-    return cudaGetLastError();
-}
-
 template <typename T, int LPT, int BC>
 cudaError_t synth_vec_go(const PlanView<T> &pv, const T *S, const T *Tc, T *eot, T *eop, int batch, Op op,
                          cudaStream_t s)
@@ -1145,105 +841,51 @@ inline int analys_lpt(int npairs) { return npairs <= 64 ? 2 : (npairs <= 1024 ? 
 
 }  // namespace
 
-template <typename T>
-cudaError_t launch_legendre_synth_cfg(const PlanView<T> &pv, const T *spec, T *eo, int batch, Op op, int lpt, int bc,
-                                      cudaStream_t s)
+cudaError_t launch_legendre_synth(const PlanView<float> &pv, const float *spec, float *eo, int batch, Op op, int lpt,
+                                  int bc, cudaStream_t s)
 {
     if (!seeds_ok(pv, true)) return cudaErrorInvalidValue;
-    // default shape: 2 pairs per thread, up to 4 fields per CTA (FP64: 1 pair
-    // per thread, 8 fields, sharing each recurrence step among more sums)
-    if (lpt <= 0) lpt = (sizeof(T) == sizeof(double) && batch >= 8) ? 1 : 2;
-    if (bc <= 0) bc = (sizeof(T) == sizeof(double) && batch >= 8) ? 8 : pick_bc(batch);
-#define SHT_SYN(L, B) if (lpt == L && bc == B) return synth_go<T, L, B>(pv, spec, eo, batch, op, s);
+    // default shape: 2 pairs per thread, up to 4 fields per CTA
+    if (lpt <= 0) lpt = 2;
+    if (bc <= 0) bc = pick_bc(batch);
+#define SHT_SYN(L, B) if (lpt == L && bc == B) return synth_go<float, L, B>(pv, spec, eo, batch, op, s);
     SHT_SYN(1, 1) SHT_SYN(1, 2) SHT_SYN(1, 4)
     SHT_SYN(2, 1) SHT_SYN(2, 2) SHT_SYN(2, 4)
     SHT_SYN(4, 1) SHT_SYN(4, 2) SHT_SYN(4, 4)
 #undef SHT_SYN
-    if constexpr (sizeof(T) == sizeof(double)) {
-        if (lpt == 1 && bc == 8) return synth_go<T, 1, 8>(pv, spec, eo, batch, op, s);
-        if (lpt == 2 && bc == 8) return synth_go<T, 2, 8>(pv, spec, eo, batch, op, s);
-    }
     return cudaErrorInvalidValue;
 }
 
-template <typename T>
-cudaError_t launch_legendre_synth(const PlanView<T> &pv, const T *spec, T *eo, int batch, Op op, cudaStream_t s)
-{
-    return launch_legendre_synth_cfg<T>(pv, spec, eo, batch, op, 0, 0, s);
-}
-
-template <typename T>
-cudaError_t launch_legendre_analys_cfg(const PlanView<T> &pv, const T *sd, T *spec, int batch, Op op, int lpt, int bc,
-                                       cudaStream_t s)
+cudaError_t launch_legendre_analys(const PlanView<float> &pv, const float *sd, float *spec, int batch, Op op, int lpt,
+                                   int bc, cudaStream_t s)
 {
     if (!seeds_ok(pv, true)) return cudaErrorInvalidValue;
-    // default shape: FP64 up to 512 pairs, the segment kernel with up to 8
-    // fields per CTA; otherwise LPT from the pair count (<= 8 warps), 2 fields
-    // per CTA when batched
-    if (lpt <= 0)
-        lpt = (sizeof(T) == sizeof(double) && pv.npairs <= 2048) ? kAnalysSeg : analys_lpt(pv.npairs);
-    if (lpt == kAnalysSeg) {
-        if (sizeof(T) != sizeof(double)) return cudaErrorInvalidValue;
-        const int ppl = seg_ppl(pv.npairs);
-        if constexpr (sizeof(T) == sizeof(double)) {
-            if (ppl == 0) {
-                // teams: 2 warps and up to 4 fields per CTA, or 4 warps and 2 fields
-                // (128 KB of staged folds either way)
-                if (pv.npairs <= 1024) {
-                    if (bc <= 0) bc = batch >= 4 ? 4 : (batch >= 2 ? 2 : 1);
-                    if (bc == 4) return analys_team_go<2, 4>(pv, sd, spec, batch, op, s);
-                    if (bc == 2) return analys_team_go<2, 2>(pv, sd, spec, batch, op, s);
-                    if (bc == 1) return analys_team_go<2, 1>(pv, sd, spec, batch, op, s);
-                } else if (pv.npairs <= 2048) {
-                    if (bc <= 0) bc = batch >= 2 ? 2 : 1;
-                    if (bc == 2) return analys_team_go<4, 2>(pv, sd, spec, batch, op, s);
-                    if (bc == 1) return analys_team_go<4, 1>(pv, sd, spec, batch, op, s);
-                }
-                return cudaErrorInvalidValue;
-            }
-        }
-        if (bc <= 0) bc = batch >= 8 ? 8 : (batch >= 4 ? 4 : (batch >= 2 ? 2 : 1));
-        if constexpr (sizeof(T) == sizeof(double)) {
-#define SHT_SEG(P, B) if (ppl == P && bc == B) return analys_seg_go<T, P, B>(pv, sd, spec, batch, op, s);
-            SHT_SEG(4, 1) SHT_SEG(4, 2) SHT_SEG(4, 4) SHT_SEG(4, 8)
-            SHT_SEG(8, 1) SHT_SEG(8, 2) SHT_SEG(8, 4) SHT_SEG(8, 8)
-            SHT_SEG(16, 1) SHT_SEG(16, 2) SHT_SEG(16, 4) SHT_SEG(16, 8)
-#undef SHT_SEG
-        }
-        return cudaErrorInvalidValue;
-    }
+    // default shape: LPT from the pair count (<= 8 warps), 2 fields per CTA when batched
+    if (lpt <= 0) lpt = analys_lpt(pv.npairs);
     if (bc <= 0) bc = batch >= 2 ? 2 : 1;
     if (analys_warps(pv.npairs, lpt) > 8) return cudaErrorInvalidValue;
-#define SHT_ANA(L, B) if (lpt == L && bc == B) return analys_go<T, L, B>(pv, sd, spec, batch, op, s);
+#define SHT_ANA(L, B) if (lpt == L && bc == B) return analys_go<float, L, B>(pv, sd, spec, batch, op, s);
     SHT_ANA(2, 1) SHT_ANA(2, 2) SHT_ANA(4, 1) SHT_ANA(4, 2) SHT_ANA(8, 1) SHT_ANA(8, 2)
 #undef SHT_ANA
     return cudaErrorInvalidValue;
 }
 
-template <typename T>
-cudaError_t launch_legendre_analys(const PlanView<T> &pv, const T *sd, T *spec, int batch, Op op, cudaStream_t s)
-{
-    return launch_legendre_analys_cfg<T>(pv, sd, spec, batch, op, 0, 0, s);
-}
-
-template <typename T>
-cudaError_t launch_legendre_synth_vec(const PlanView<T> &pv, const T *S, const T *Tc, T *eot, T *eop, int batch,
-                                      Op op, cudaStream_t s)
+cudaError_t launch_legendre_synth_vec(const PlanView<float> &pv, const float *S, const float *Tc, float *eot,
+                                      float *eop, int batch, Op op, cudaStream_t s)
 {
     if (!seeds_ok(pv, false)) return cudaErrorInvalidValue;
-    if (batch >= 2) return synth_vec_go<T, 1, 2>(pv, S, Tc, eot, eop, batch, op, s);
-    return synth_vec_go<T, 1, 1>(pv, S, Tc, eot, eop, batch, op, s);
+    if (batch >= 2) return synth_vec_go<float, 1, 2>(pv, S, Tc, eot, eop, batch, op, s);
+    return synth_vec_go<float, 1, 1>(pv, S, Tc, eot, eop, batch, op, s);
 }
 
-template <typename T>
-cudaError_t launch_legendre_analys_vec(const PlanView<T> &pv, const T *sdt, const T *sdp, T *S, T *Tc, int batch,
-                                       Op op, cudaStream_t s)
+cudaError_t launch_legendre_analys_vec(const PlanView<float> &pv, const float *sdt, const float *sdp, float *S,
+                                       float *Tc, int batch, Op op, cudaStream_t s)
 {
     if (!seeds_ok(pv, false)) return cudaErrorInvalidValue;
     switch (analys_lpt(pv.npairs)) {
-    case 2: return analys_vec_go<T, 2, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
-    case 4: return analys_vec_go<T, 4, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
-    default: return analys_vec_go<T, 8, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
+    case 2: return analys_vec_go<float, 2, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
+    case 4: return analys_vec_go<float, 4, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
+    default: return analys_vec_go<float, 8, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
     }
 }
 
@@ -1303,7 +945,7 @@ cudaError_t launch_batch_legendre(bool synth, const BatchField *fields, const in
 // polar optimisation.  One thread per (order index m, pair): the FP64
 // recurrence of Sec. 3.2 from P_m^m, carried as y 2^(-240 k) (Sec. 3.5).  At
 // the start of every kSeedSeg-degree segment the state (y1, y2) =
-// (P_{n0-1}, P_{n0-2}) is stored, either as it is with k (FP64 plans) or
+// (P_{n0-1}, P_{n0-2}) is stored, either times 2^hseg with k (FP64 plans) or
 // rewritten in the FP32 form y' 2^(-64 k'): k' = 0 when the larger of the two
 // is at least 2^-63, else the k' that brings it into [2^-65, 1) -- the form in
 // which the FP32 kernels carry it.  live[m][pair] is the first segment that
@@ -1328,8 +970,8 @@ __device__ float4 fp32_state(double y1, double y2, int k)
 
 __global__ void __launch_bounds__(128)
 k_build_restarts(PlanView<double> pv, const unsigned long long *__restrict__ segoff, float4 *__restrict__ seeds32,
-                 double2 *__restrict__ seeds64, int *__restrict__ seeds64k, unsigned short *__restrict__ live,
-                 double thr)
+                 double2 *__restrict__ seeds64, int *__restrict__ seeds64k, const int *__restrict__ hseg,
+                 unsigned short *__restrict__ live, double thr)
 {
     const int m = blockIdx.y;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1346,7 +988,8 @@ k_build_restarts(PlanView<double> pv, const unsigned long long *__restrict__ seg
         const size_t o = (segoff[m] + s) * npairs + p;
         if (seeds32) seeds32[o] = fp32_state(y1, y2, k);
         if (seeds64) {
-            seeds64[o] = make_double2(y1, y2);
+            const int h = hseg[segoff[m] + s];
+            seeds64[o] = make_double2(scalbn(y1, h), scalbn(y2, h));
             seeds64k[o] = k;
         }
         for (int i = 0; i < kSeedSeg; ++i) {
@@ -1370,36 +1013,12 @@ k_build_restarts(PlanView<double> pv, const unsigned long long *__restrict__ seg
 }  // namespace
 
 cudaError_t launch_build_restarts(const PlanView<double> &pv, const unsigned long long *segoff, float4 *seeds32,
-                                  double2 *seeds64, int *seeds64k, unsigned short *live, double thr, cudaStream_t st)
+                                  double2 *seeds64, int *seeds64k, const int *hseg, unsigned short *live, double thr,
+                                  cudaStream_t st)
 {
     dim3 grid((unsigned)((pv.npairs + 127) / 128), (unsigned)(pv.mmax + 1));
-    k_build_restarts<<<grid, 128, 0, st>>>(pv, segoff, seeds32, seeds64, seeds64k, live, thr);
+    k_build_restarts<<<grid, 128, 0, st>>>(pv, segoff, seeds32, seeds64, seeds64k, hseg, live, thr);
     return cudaGetLastError();
 }
-
-template cudaError_t launch_legendre_synth_cfg<double>(const PlanView<double> &, const double *, double *, int, Op,
-                                                       int, int, cudaStream_t);
-template cudaError_t launch_legendre_synth_cfg<float>(const PlanView<float> &, const float *, float *, int, Op, int,
-                                                      int, cudaStream_t);
-template cudaError_t launch_legendre_analys_cfg<double>(const PlanView<double> &, const double *, double *, int, Op,
-                                                        int, int, cudaStream_t);
-template cudaError_t launch_legendre_analys_cfg<float>(const PlanView<float> &, const float *, float *, int, Op, int,
-                                                       int, cudaStream_t);
-template cudaError_t launch_legendre_synth<double>(const PlanView<double> &, const double *, double *, int, Op,
-                                                   cudaStream_t);
-template cudaError_t launch_legendre_synth<float>(const PlanView<float> &, const float *, float *, int, Op,
-                                                  cudaStream_t);
-template cudaError_t launch_legendre_analys<double>(const PlanView<double> &, const double *, double *, int, Op,
-                                                    cudaStream_t);
-template cudaError_t launch_legendre_analys<float>(const PlanView<float> &, const float *, float *, int, Op,
-                                                   cudaStream_t);
-template cudaError_t launch_legendre_synth_vec<double>(const PlanView<double> &, const double *, const double *,
-                                                       double *, double *, int, Op, cudaStream_t);
-template cudaError_t launch_legendre_synth_vec<float>(const PlanView<float> &, const float *, const float *, float *,
-                                                      float *, int, Op, cudaStream_t);
-template cudaError_t launch_legendre_analys_vec<double>(const PlanView<double> &, const double *, const double *,
-                                                        double *, double *, int, Op, cudaStream_t);
-template cudaError_t launch_legendre_analys_vec<float>(const PlanView<float> &, const float *, const float *, float *,
-                                                       float *, int, Op, cudaStream_t);
 
 }  // namespace sht

@@ -1,0 +1,727 @@
+// legendre64.cu -- the FP64 Legendre stage on the CUDA cores, scalar and vector.
+//
+// The sums and the mirror folding are those of legendre.cu; this file holds
+// what FP64 asks for on this GPU.  Its FP64 pipe takes one warp instruction
+// every ~19 cycles per SM (every ~64 per SM quarter), some seventy times fewer
+// than FP32, so a kernel's time is its count of FP64 instructions, provided
+// every SM quarter has a warp with work.
+//
+// * Recurrence in two instructions instead of three.  Within a segment of
+//   kSeedSeg degrees P_n^m = s_n Q_n with s_n = prod a_j over the segment's
+//   degrees up to n, and Q_n = x Q_{n-1} + beta_n Q_{n-2}, beta_n = b_n / (a_n a_{n-1})
+//   = -((n-1)^2 - m^2) / (4 (n-1)^2 - 1) (Sec. 3.2 divided by s_n; beta = b_n / a_n
+//   at the segment's first degree, whose two predecessors are the stored state).
+//   s_n goes into the spectral value once per degree and field, not per
+//   latitude.  A power of two per segment, taken into the stored state, centres
+//   the range of s on 1 (2^-70 .. 2^70 at order 2047).
+// * Vector transforms are scalar ones.  With eps_n = sqrt((n^2 - m^2) / (4 n^2 - 1)),
+//   sin(theta) dP_n/dtheta = n eps_{n+1} P_{n+1} - (n + 1) eps_n P_{n-1}, so
+//     sin V_theta = sum_k U_k P_k,  U_k = (k-1) eps_k S_{k-1} - (k+2) eps_{k+1} S_{k+1} - i m T_k,
+//     sin V_phi   = sum_k W_k P_k,  W_k = (k-1) eps_k T_{k-1} - (k+2) eps_{k+1} T_{k+1} + i m S_k
+//   for k = m .. lmax + 1: per field two complex sums per degree and pair
+//   instead of four, and no derivative to generate.  The differences multiply
+//   by n whatever is not smooth in n in the errors of P, near the poles above
+//   all, so here the recurrence is Sec. 3.2's own, the one whose states are
+//   stored (the Q_n agree with them to rounding only and would jump at every
+//   segment: errors 1.1 times as large, geometric mean over N = 33 .. 124, up
+//   to 5 times; with Sec. 3.2's the errors are those of the form with
+//   derivatives).  The analysis is the transpose: A_k, B_k = sum P_k fold(V_theta), fold(V_phi), then
+//     S_n = n eps_{n+1} A_{n+1} - (n+1) eps_n A_{n-1} - i m B_n,
+//     T_n = n eps_{n+1} B_{n+1} - (n+1) eps_n B_{n-1} + i m A_n.
+#include <cuda_runtime.h>
+
+#include "sht_internal.h"
+
+namespace sht {
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+constexpr double kDown = 0x1p-240;   // 2^-Scale<double>::S
+constexpr int kHiOne = 0x3ff00000;   // high word of 1.0
+constexpr int kMaxDeg = kSeedSeg + 2;   // degrees of a segment: kSeedSeg, one more at lmax + 1, padded to even
+
+// Orders' first index in a table or spectrum that runs to degree lmax + ext.
+__device__ __forceinline__ long col_ext(const PlanView<double> &pv, int m, int ext)
+{
+    return col_of_mres(pv.lmax + ext, m, pv.mres);
+}
+
+// CTAs that are all resident at once go to the SMs round robin; every second
+// round of `nsm` runs backwards, so that an SM with a heavy item of one round
+// takes a light one of the next (the items come heaviest first).
+__device__ __forceinline__ int snake(int i, int total, int nsm)
+{
+    const int r = i / nsm, first = r * nsm;
+    if (!(r & 1)) return i;
+    const int len = min(nsm, total - first);
+    return first + len - 1 - (i - first);
+}
+
+// One step of the recurrence, y_n = a x y_{n-1} + b y_{n-2}, and the factor s_n of
+// the value: (beta_n, s_n) of Q_n, where a = 1 is left out by the caller, or
+// (a_n, b_n) of P_n itself (`plain`).  Zeros past the order's last degree.
+struct Step { double a, b, s; };
+__device__ __forceinline__ Step step_of(const PlanView<double> &pv, long i, bool in, bool plain)
+{
+    Step r = {0.0, 0.0, 0.0};
+    if (!in) return r;
+    const double2 v = __ldg((plain ? pv.abx : pv.qs) + i);
+    if (plain) {
+        r.a = v.x;
+        r.b = v.y;
+        r.s = 1.0;
+    } else {
+        r.b = v.x;
+        r.s = v.y;
+    }
+    return r;
+}
+
+// The power of two that takes a segment's stored state back to P.
+__device__ __forceinline__ double seg_down(const PlanView<double> &pv, int m, int seg)
+{
+    return __hiloint2double((1023 - __ldg(pv.hseg + pv.segoff[m] + seg)) << 20, 0);
+}
+
+// |Q| s >= 1 to within the 2^-20 of the high words' sum (a rescaling test: see
+// Sec. 3.5; hs = high word of s less that of 1).
+__device__ __forceinline__ bool reaches_one(double q, int hs)
+{
+    return (__double2hiint(q) & 0x7fffffff) + hs >= kHiOne;
+}
+
+// ---------------------------------------------------------------------------
+// Scalar synthesis.  A CTA of W warps per (order m, 32 latitude pairs, BC
+// fields), one pair per lane; warp w takes the live segments w, w + W, ... and
+// the warps' sums meet in shared memory in a fixed order.  Splitting the
+// degrees over warps keeps the SMs busy where orders x pairs x fields are few
+// (one field at N = 255: 134 us with one CTA of 128 pairs per order, 43 us with
+// four warps per 32 pairs).  16 fields at N = 511: 1981 us with three
+// instructions per step and 8 fields, 1766 us with two and 16 fields (34 FP64
+// instructions per degree, pair and 16 fields; 0.86 of the pipe's rate).  vec: the
+// spectra run to degree lmax + 1, the recurrence is Sec. 3.2's, and the sums
+// are divided by sin(theta).
+// ---------------------------------------------------------------------------
+template <int BC, int W>
+__global__ void __launch_bounds__(32 * W)
+k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restrict__ eo, int batch, int ngroups,
+          int nchunk, int nsm, int vec, int op)
+{
+    extern __shared__ __align__(16) double2 s_mem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double2 *s_f = s_mem + w * 64 * BC;                                  // [BC][kMaxDeg]
+    __shared__ double s_a[W][kMaxDeg], s_beta[W][kMaxDeg];
+    __shared__ int s_hs[W][kMaxDeg];
+
+    const int item = snake(blockIdx.x, gridDim.x, nsm);
+    const int chunk = item % nchunk, rest = item / nchunk;
+    const int g = rest % ngroups, m = rest / ngroups;
+    const int b0 = chunk * BC;
+    const int npairs = pv.npairs, Ls = pv.lmax - m * pv.mres + 1, L = Ls + vec;
+    const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg;
+    const long colq = col_ext(pv, m, 1), col = col_ext(pv, m, vec);
+    const size_t nlm = (size_t)pv.nlm + (size_t)vec * (pv.mmax + 1);
+    const double2 *spec2 = reinterpret_cast<const double2 *>(spec);
+    const int p = g * 32 + lane;
+    const bool valid = p < npairs;
+    const double x = valid ? pv.x[p] : 0.0;
+    const int first = __reduce_min_sync(kFull, valid ? (int)pv.live[(size_t)m * npairs + p] : 0xffff);
+    const double insc = (op == OP_ANALYS_ADJ && m > 0) ? 0.5 : 1.0;   // adjoint of analysis: b / c_m
+
+    double er[BC], ei[BC], orr[BC], oi[BC];
+#pragma unroll
+    for (int b = 0; b < BC; ++b) er[b] = ei[b] = orr[b] = oi[b] = 0.0;
+
+    for (int seg = first + w; seg < nseg; seg += W) {
+        const int n0 = seg * kSeedSeg;
+        const int cnt = seg == nseg - 1 ? L - n0 : kSeedSeg;
+        double y1 = 0.0, y2 = 0.0;
+        int k = 0;
+        if (valid) {
+            const size_t o = (size_t)(pv.segoff[m] + seg) * npairs + p;
+            const double2 v = __ldg(pv.seeds64 + o);
+            const double down = vec ? seg_down(pv, m, seg) : 1.0;
+            y1 = v.x * down;
+            y2 = v.y * down;
+            k = __ldg(pv.seeds64k + o);
+        }
+        __syncwarp();
+        for (int t = lane; t < ((cnt + 1) & ~1); t += 32) {
+            const Step st = step_of(pv, colq + n0 + t, t < cnt, vec);
+            s_a[w][t] = st.a;
+            s_beta[w][t] = st.b;
+            s_hs[w][t] = __double2hiint(st.s) - kHiOne;
+            const double sc = st.s * insc;
+#pragma unroll
+            for (int b = 0; b < BC; ++b) {
+                double2 f = make_double2(0.0, 0.0);
+                if (t < cnt && b0 + b < batch) {
+                    f = __ldg(spec2 + (size_t)(b0 + b) * nlm + col + n0 + t);
+                    f.x *= sc;
+                    f.y = m == 0 ? 0.0 : f.y * sc;
+                }
+                s_f[b * kMaxDeg + t] = f;
+            }
+        }
+        __syncwarp();
+        if (!__any_sync(kFull, k > 0)) {
+            for (int t = 0; t < cnt; t += 2) {
+                y2 = fma(vec ? s_a[w][t] * x : x, y1, s_beta[w][t] * y2);
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    const double2 f = s_f[b * kMaxDeg + t];
+                    er[b] = fma(f.x, y2, er[b]);
+                    ei[b] = fma(f.y, y2, ei[b]);
+                }
+                y1 = fma(vec ? s_a[w][t + 1] * x : x, y2, s_beta[w][t + 1] * y1);
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    const double2 f = s_f[b * kMaxDeg + t + 1];
+                    orr[b] = fma(f.x, y1, orr[b]);
+                    oi[b] = fma(f.y, y1, oi[b]);
+                }
+            }
+        } else {
+            // some pair of the warp still carries a scaled value (Sec. 3.5)
+            for (int t = 0; t < cnt; ++t) {
+                double yn = fma(vec ? s_a[w][t] * x : x, y1, s_beta[w][t] * y2);
+                y2 = y1;
+                if (k > 0 && reaches_one(yn, s_hs[w][t])) {
+                    yn *= kDown;
+                    y2 *= kDown;
+                    k -= 1;
+                }
+                y1 = yn;
+                if (!__any_sync(kFull, k == 0)) continue;
+                const double c = k == 0 ? yn : 0.0;
+                const bool odd = t & 1;
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    const double2 f = s_f[b * kMaxDeg + t];
+                    if (odd) {
+                        orr[b] = fma(f.x, c, orr[b]);
+                        oi[b] = fma(f.y, c, oi[b]);
+                    } else {
+                        er[b] = fma(f.x, c, er[b]);
+                        ei[b] = fma(f.y, c, ei[b]);
+                    }
+                }
+            }
+        }
+    }
+
+    double2 *eo2 = reinterpret_cast<double2 *>(eo);
+    if (W == 1) {
+        if (!valid) return;
+        const double is = vec ? 1.0 / pv.st[p] : 1.0;
+#pragma unroll
+        for (int b = 0; b < BC; ++b) {
+            if (b0 + b >= batch) break;
+            const size_t o = (((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + p) * 2;
+            eo2[o] = make_double2(er[b] * is, ei[b] * is);
+            eo2[o + 1] = make_double2(orr[b] * is, oi[b] * is);
+        }
+        return;
+    }
+    // the warps' sums, [warp][field][pair][E, O]
+    __syncwarp();
+#pragma unroll
+    for (int b = 0; b < BC; ++b) {
+        s_f[(b * 32 + lane) * 2] = make_double2(er[b], ei[b]);
+        s_f[(b * 32 + lane) * 2 + 1] = make_double2(orr[b], oi[b]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < BC * 64; i += 32 * W) {
+        const int b = i >> 6, q = g * 32 + ((i & 63) >> 1);
+        if (b0 + b >= batch || q >= npairs) continue;
+        double2 v = s_mem[i];
+#pragma unroll
+        for (int u = 1; u < W; ++u) {
+            const double2 z = s_mem[u * 64 * BC + i];
+            v.x += z.x;
+            v.y += z.y;
+        }
+        if (vec) {
+            const double is = 1.0 / pv.st[q];
+            v.x *= is;
+            v.y *= is;
+        }
+        eo2[(((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + q) * 2 + (i & 1)] = v;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Scalar analysis.  A CTA of four warps (one per SM quarter) per (order m,
+// segment of kSeedSeg degrees, BC fields).  It takes the latitude pairs 128 at a
+// time: each warp generates P of the segment for 32 of them, one pair per lane,
+// into shared memory; then warp w sums degrees 8 w .. 8 w + 7 over all 128,
+// lane (slice, c) the products of component c (field, real/imaginary) over the
+// pairs of its slice, one accumulator per degree.  With C = 2 BC components there
+// are 32 / C slices, so the sum over latitudes needs one butterfly over the
+// slices per segment (none at 16 fields); a lane per pair instead needs an FP64
+// butterfly over all 32 lanes for every 16 / BC degrees -- with 96 pairs a third
+// on top of the sums -- and a warp per segment leaves SM quarters idle where
+// segments are few.  Every sum has a fixed order, so results are bitwise
+// reproducible.  The groups of 32 pairs before the first one with a live pair in
+// the segment (static polar optimisation, Sec. 3.1) are left out.
+//
+// blockIdx: x segment (with `vec`, see k_synth64, the degree lmax + 1 is one
+// more, alone in its block when the order's degrees fill their segments: it
+// continues the recurrence of the last segment), y order index, z field chunk.
+// ---------------------------------------------------------------------------
+constexpr int kAnaWarps = 4;
+
+template <int BC>
+__global__ void __launch_bounds__(32 * kAnaWarps)
+k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restrict__ spec, int batch, int vec, int op)
+{
+    constexpr int C = 2 * BC, SL = 32 / C, W = kAnaWarps, DB = kSeedSeg / W;
+    constexpr int NQ = W * 32 / SL;   // pairs of a slice per block of 128
+    __shared__ double s_P[W][kSeedSeg][33];
+    __shared__ double s_a[kSeedSeg + DB], s_beta[kSeedSeg + DB];
+    __shared__ int s_hs[kSeedSeg + DB];
+    __shared__ int s_g0;
+
+    const int m = blockIdx.y, b0 = blockIdx.z * BC, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int npairs = pv.npairs, ngroups = (npairs + 31) >> 5;
+    const int Ls = pv.lmax - m * pv.mres + 1, L = Ls + vec;
+    const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg;
+    const bool tail = (int)blockIdx.x == nseg;   // the degree lmax + 1 alone
+    const int seg = tail ? nseg - 1 : blockIdx.x;
+    const int n0 = blockIdx.x * kSeedSeg;        // first degree summed
+    if (n0 >= L) return;
+    const int cnt = min(kSeedSeg, L - n0);
+    const int nstep = tail ? kSeedSeg + 1 : (cnt + DB - 1) & ~(DB - 1);
+    const long colq = col_ext(pv, m, 1) + seg * kSeedSeg, col = col_ext(pv, m, vec) + n0;
+    const size_t nlm = (size_t)pv.nlm + (size_t)vec * (pv.mmax + 1);
+    if (threadIdx.x == 0) s_g0 = ngroups;
+    if (threadIdx.x < nstep) {
+        const int t = threadIdx.x;
+        const Step st = step_of(pv, colq + t, seg * kSeedSeg + t < L, vec);
+        s_a[t] = st.a;
+        s_beta[t] = st.b;
+        s_hs[t] = __double2hiint(st.s) - kHiOne;
+    }
+    if (tail)   // one degree: the rest of its block of DB is zero
+        for (int t = 1; t < DB; ++t) s_P[w][t][lane] = 0.0;
+    __syncthreads();
+    for (int g = w; g < ngroups; g += W) {
+        const int p = g * 32 + lane;
+        const int f = p < npairs ? (int)pv.live[(size_t)m * npairs + p] : 0xffff;
+        if (__any_sync(kFull, f <= seg)) {
+            if (lane == 0) atomicMin(&s_g0, g);
+            break;
+        }
+    }
+    __syncthreads();
+    const int g0 = s_g0;
+
+    // this lane's component and slice of the pairs, this warp's degrees
+    const int c = lane % C, slice = lane / C, b = b0 + (c >> 1), d0 = w * DB;
+    const double *fold = sd + ((size_t)b * (pv.mmax + 1) + m) * npairs * 4 + (c & 1);   // s at 4 q, d at 4 q + 2
+    const bool has = b < batch && d0 < cnt;
+    double acc[DB];
+#pragma unroll
+    for (int t = 0; t < DB; ++t) acc[t] = 0.0;
+
+    for (int gb = g0; gb < ngroups; gb += W) {
+        const int p = (gb + w) * 32 + lane;
+        const bool valid = p < npairs;
+        double x = 0.0, y1 = 0.0, y2 = 0.0;
+        int k = 0;
+        if (valid) {
+            const size_t o = (size_t)(pv.segoff[m] + seg) * npairs + p;
+            const double2 v = __ldg(pv.seeds64 + o);
+            x = pv.x[p];
+            const double down = vec ? seg_down(pv, m, seg) : 1.0;
+            y1 = v.x * down;
+            y2 = v.y * down;
+            k = __ldg(pv.seeds64k + o);
+        }
+        // the folds of the slice's pairs, two pairs ahead of the sums
+        const int q0 = gb * 32 + slice;
+        double sv[2], dv[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int q = q0 + u * SL;
+            sv[u] = has && q < npairs ? __ldg(fold + (size_t)q * 4) : 0.0;
+            dv[u] = has && q < npairs ? __ldg(fold + (size_t)q * 4 + 2) : 0.0;
+        }
+        __syncthreads();   // the last block's sums are done with s_P
+        if (gb + w < ngroups) {
+            const bool scaled = __any_sync(kFull, k > 0);
+            for (int t = 0; t < nstep; ++t) {
+                double yn = fma(vec ? s_a[t] * x : x, y1, s_beta[t] * y2);
+                y2 = y1;
+                double v = yn;
+                if (scaled) {   // some pair still carries a scaled value (Sec. 3.5)
+                    if (k > 0 && reaches_one(yn, s_hs[t])) {
+                        yn *= kDown;
+                        y2 *= kDown;
+                        k -= 1;
+                    }
+                    v = k == 0 ? yn : 0.0;
+                }
+                y1 = yn;
+                if (!tail) s_P[w][t][lane] = v;
+                else if (t == kSeedSeg) s_P[w][0][lane] = v;
+            }
+        }
+        __syncthreads();
+        if (d0 < cnt) {
+            const int nq = min(NQ, (npairs - gb * 32 + SL - 1) / SL);
+#pragma unroll 2
+            for (int j = 0; j < nq; ++j) {
+                const int r = j * SL + slice;   // pair within the block
+                const double *P = &s_P[r >> 5][d0][r & 31];
+                const double s = sv[j & 1], d = dv[j & 1];
+                const int q = q0 + (j + 2) * SL;
+                sv[j & 1] = has && j + 2 < nq && q < npairs ? __ldg(fold + (size_t)q * 4) : 0.0;
+                dv[j & 1] = has && j + 2 < nq && q < npairs ? __ldg(fold + (size_t)q * 4 + 2) : 0.0;
+#pragma unroll
+                for (int t = 0; t < DB; ++t) acc[t] = fma(P[t * 33], (t & 1) ? d : s, acc[t]);
+            }
+        }
+    }
+    // over the slices (lane bits C .. 16): while a lane holds several degrees it
+    // keeps half of them, then both lanes of a pair keep the sum
+#pragma unroll
+    for (int o = 16; o >= C; o >>= 1) {
+        const int h = DB * o / 32;   // degrees kept (0: one degree left, add)
+        if (h > 0) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int t = 0; t < h; ++t) {
+                const double send = up ? acc[t] : acc[t + h];
+                const double keep = up ? acc[t + h] : acc[t];
+                acc[t] = keep + __shfl_xor_sync(kFull, send, o);
+            }
+        } else {
+            acc[0] += __shfl_xor_sync(kFull, acc[0], o);
+        }
+    }
+    __syncthreads();
+    {
+        // degrees held: DB C / 32 (at least one) from the kept halves' offset
+        constexpr int V = DB * C / 32 > 0 ? DB * C / 32 : 1;
+        const int off = (lane & ~(C - 1)) * DB / 32 / V * V;
+#pragma unroll
+        for (int t = 0; t < V; ++t) s_P[0][d0 + off + t][c] = acc[t];
+    }
+    __syncthreads();
+    if (lane >= cnt) return;
+    // P_n = s_n Q_n; c_m for the adjoint of synthesis
+    const double sc = (vec ? 1.0 : __ldg(&pv.qs[colq + lane].y)) * ((op == OP_SYNTH_ADJ && m > 0) ? 2.0 : 1.0);
+    double2 *spec2 = reinterpret_cast<double2 *>(spec);
+    for (int i = w; i < BC && b0 + i < batch; i += W)
+        spec2[(size_t)(b0 + i) * nlm + col + lane] =
+            make_double2(s_P[0][lane][2 * i] * sc, m == 0 ? 0.0 : s_P[0][lane][2 * i + 1] * sc);
+}
+
+// ---------------------------------------------------------------------------
+// Vector transforms: spectra in and out of the scalar sums (see the head of
+// this file).  Thread per (degree, order index m = blockIdx.y, field blockIdx.z).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128)
+k_vec64_split(PlanView<double> pv, const double2 *__restrict__ S, const double2 *__restrict__ T,
+              double2 *__restrict__ uw, int batch, int op)
+{
+    const int m = blockIdx.y, b = blockIdx.z, dm = m * pv.mres;
+    const int L = pv.lmax - dm + 1;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // degree k = dm + i, up to lmax + 1
+    if (i > L) return;
+    const long col = col_ext(pv, m, 0), colx = col_ext(pv, m, 1);
+    const size_t nlmx = (size_t)pv.nlm + pv.mmax + 1;
+    const double2 *Sb = S + (size_t)b * pv.nlm + col, *Tb = T + (size_t)b * pv.nlm + col;
+    const double k = dm + i;
+    // adjoint of analysis: b / (c_m n (n + 1)), nothing at n = 0
+    const auto load = [&](const double2 *a, int j) {
+        if (j < 0 || j >= L) return make_double2(0.0, 0.0);
+        double2 v = a[j];
+        if (m == 0) v.y = 0.0;
+        if (op == OP_ANALYS_ADJ) {
+            const double n = dm + j, sc = n == 0.0 ? 0.0 : (m > 0 ? 0.5 : 1.0) / (n * (n + 1.0));
+            v.x *= sc;
+            v.y *= sc;
+        }
+        return v;
+    };
+    const double lo = (k - 1.0) * pv.eps[colx + i], hi = i < L ? (k + 2.0) * pv.eps[colx + i + 1] : 0.0;
+    const double2 Sl = load(Sb, i - 1), Sc = load(Sb, i), Sh = load(Sb, i + 1);
+    const double2 Tl = load(Tb, i - 1), Tc = load(Tb, i), Th = load(Tb, i + 1);
+    double2 U, W;
+    U.x = lo * Sl.x - hi * Sh.x + dm * Tc.y;
+    U.y = lo * Sl.y - hi * Sh.y - dm * Tc.x;
+    W.x = lo * Tl.x - hi * Th.x - dm * Sc.y;
+    W.y = lo * Tl.y - hi * Th.y + dm * Sc.x;
+    uw[(size_t)b * nlmx + colx + i] = U;
+    uw[(size_t)(batch + b) * nlmx + colx + i] = W;
+}
+
+__global__ void __launch_bounds__(128)
+k_vec64_join(PlanView<double> pv, const double2 *__restrict__ ab, double2 *__restrict__ S, double2 *__restrict__ T,
+             int batch, int op)
+{
+    const int m = blockIdx.y, b = blockIdx.z, dm = m * pv.mres;
+    const int L = pv.lmax - dm + 1;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // degree n = dm + i
+    if (i >= L) return;
+    const long col = col_ext(pv, m, 0), colx = col_ext(pv, m, 1);
+    const size_t nlmx = (size_t)pv.nlm + pv.mmax + 1;
+    const double2 *A = ab + (size_t)b * nlmx + colx, *B = ab + (size_t)(batch + b) * nlmx + colx;
+    const double n = dm + i;
+    const double hi = n * pv.eps[colx + i + 1], lo = i > 0 ? (n + 1.0) * pv.eps[colx + i] : 0.0;
+    const double2 Ah = A[i + 1], Ac = A[i], Bh = B[i + 1], Bc = B[i];
+    const double2 z = make_double2(0.0, 0.0), Al = i > 0 ? A[i - 1] : z, Bl = i > 0 ? B[i - 1] : z;
+    double sc;
+    if (op == OP_SYNTH_ADJ) sc = m > 0 ? 2.0 : 1.0;
+    else sc = n == 0.0 ? 0.0 : 1.0 / (n * (n + 1.0));
+    double2 s, t;
+    s.x = sc * (hi * Ah.x - lo * Al.x + dm * Bc.y);
+    s.y = sc * (hi * Ah.y - lo * Al.y - dm * Bc.x);
+    t.x = sc * (hi * Bh.x - lo * Bl.x - dm * Ac.y);
+    t.y = sc * (hi * Bh.y - lo * Bl.y + dm * Ac.x);
+    if (m == 0) s.y = t.y = 0.0;
+    S[(size_t)b * pv.nlm + col + i] = s;
+    T[(size_t)b * pv.nlm + col + i] = t;
+}
+
+// ---------------------------------------------------------------------------
+// Plan tables: (beta_n, s_n), (a_n, b_n) and eps_n of every degree m .. lmax + 1
+// of every order, and per segment the exponent h of its states' scale.  s_n^2 is
+// the product of (4 j^2 - 1) / (j^2 - m^2) over the segment, formed in
+// double-double arithmetic (Dekker 1971).  Thread per (segment, order index
+// blockIdx.y).
+// ---------------------------------------------------------------------------
+struct dd { double h, l; };
+__device__ __forceinline__ dd dd_norm(double h, double l)
+{
+    dd r;
+    r.h = h + l;
+    r.l = l - (r.h - h);
+    return r;
+}
+__device__ __forceinline__ dd dd_mul(dd a, double b)
+{
+    const double p = a.h * b;
+    return dd_norm(p, fma(a.l, b, fma(a.h, b, -p)));
+}
+// the quotient, rounded
+__device__ __forceinline__ double dd_div(dd a, dd b)
+{
+    const double q = a.h / b.h;
+    return q + (fma(-q, b.h, a.h) + (a.l - q * b.l)) / b.h;
+}
+
+__global__ void __launch_bounds__(64)
+k_build_qs(PlanView<double> pv, const unsigned long long *__restrict__ segoff, double2 *__restrict__ qs,
+           double2 *__restrict__ abx, double *__restrict__ eps, int *__restrict__ hseg)
+{
+    const int m = blockIdx.y, seg = blockIdx.x * blockDim.x + threadIdx.x;
+    const double dm = m * pv.mres;
+    const int Ls = pv.lmax - m * pv.mres + 1;
+    const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg;
+    if (seg >= nseg) return;
+    const long colx = col_ext(pv, m, 1), col = col_ext(pv, m, 0);
+    const int i0 = seg * kSeedSeg, i1 = seg == nseg - 1 ? Ls + 1 : i0 + kSeedSeg;
+    const auto factor = [&](int i, dd &num, dd &den) {   // into s^2 at degree dm + i
+        const double n = dm + i;
+        num = dd_mul(num, 4.0 * n * n - 1.0);
+        den = dd_mul(den, n * n - dm * dm);
+    };
+    dd num = {1.0, 0.0}, den = num;
+    for (int i = max(1, i0); i < min(Ls, i0 + kSeedSeg); ++i) factor(i, num, den);
+    const int h = ilogb(num.h / den.h) / 4;   // half of the growth of s
+    hseg[segoff[m] + seg] = h;
+    num.h = scalbn(1.0, -2 * h);
+    num.l = 0.0;
+    den.h = 1.0;
+    den.l = 0.0;
+    for (int i = i0; i < i1; ++i) {
+        const double n = dm + i, n1 = n - 1.0;
+        if (i == 0) {   // Q_m is the start value P_m^m, handed over as Q_{m-2}
+            qs[colx] = make_double2(1.0, scalbn(1.0, -h));
+            abx[colx] = make_double2(0.0, 1.0);
+            eps[colx] = 0.0;
+            continue;
+        }
+        factor(i, num, den);
+        const double bb = i == 1 ? 0.0 : (n1 * n1 - dm * dm) / (4.0 * n1 * n1 - 1.0);   // eps_{n-1}^2
+        qs[colx + i] = make_double2(i == i0 ? -sqrt(bb) : -bb, sqrt(dd_div(num, den)));
+        eps[colx + i] = sqrt((n * n - dm * dm) / (4.0 * n * n - 1.0));
+        double2 ab;
+        if (i < Ls)
+            ab = pv.ab[col + i];
+        else if (i == 1)
+            ab = make_double2(sqrt(2.0 * dm + 3.0), 0.0);
+        else
+            ab = make_double2(sqrt((4.0 * n * n - 1.0) / (n * n - dm * dm)),
+                              -sqrt((2.0 * n + 1.0) / (2.0 * n - 3.0) * (n1 * n1 - dm * dm) / (n * n - dm * dm)));
+        abx[colx + i] = ab;
+    }
+}
+
+inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 152;
+    return sms;
+}
+
+// Fields per CTA: the width whose CTAs issue the fewest FP64 instructions per
+// degree and pair, 2 + 2 BC each (unused fields of the last CTA count); the
+// larger of equals.
+inline int pick_bc64(int batch, int most)
+{
+    int best = 1;
+    for (int bc = 2; bc <= most; bc *= 2)
+        if ((long)((batch + bc - 1) / bc) * (2 + 2 * bc) <= (long)((batch + best - 1) / best) * (2 + 2 * best)) best = bc;
+    return best;
+}
+
+bool tables_ok(const PlanView<double> &pv)
+{
+    return pv.segoff && pv.seeds64 && pv.seeds64k && pv.live && pv.qs && pv.abx && pv.eps && pv.hseg;
+}
+
+// A launch of the synthesis with W warps per CTA.
+template <int BC, int W>
+cudaError_t synth64_go(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, bool vec,
+                       cudaStream_t s)
+{
+    const int ng = (pv.npairs + 31) / 32, nc = (batch + BC - 1) / BC;
+    const size_t smem = sizeof(double2) * 64 * BC * W;
+    if (smem > 40 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_synth64<BC, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    const long items = (long)(pv.mmax + 1) * ng * nc;
+    k_synth64<BC, W><<<(unsigned)items, 32 * W, smem, s>>>(pv, spec, eo, batch, ng, nc, sm_count(), vec ? 1 : 0,
+                                                          (int)op);
+    return cudaGetLastError();
+}
+
+// w: warps per CTA {1, 2, 4, 8} (0: enough for 16 warps per SM, at most one per
+// segment of order 0); bc: fields per CTA {1, 2, 4, 8, 16} (0: pick_bc64).
+cudaError_t synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int w, int bc,
+                    bool vec, cudaStream_t s)
+{
+    if (!tables_ok(pv)) return cudaErrorInvalidValue;
+    if (bc <= 0) bc = pick_bc64(batch, 16);
+    if (w <= 0) {
+        const long units = (long)(pv.mmax + 1) * ((pv.npairs + 31) / 32) * ((batch + bc - 1) / bc);
+        const int nseg = (pv.lmax + kSeedSeg) / kSeedSeg;
+        w = 1;
+        while (w < 8 && w < nseg && units * w < 16L * sm_count() && !(bc == 16 && w == 4)) w *= 2;
+    }
+#define SHT_SYN64(B, W_) if (bc == B && w == W_) return synth64_go<B, W_>(pv, spec, eo, batch, op, vec, s);
+    SHT_SYN64(1, 1) SHT_SYN64(1, 2) SHT_SYN64(1, 4) SHT_SYN64(1, 8)
+    SHT_SYN64(2, 1) SHT_SYN64(2, 2) SHT_SYN64(2, 4) SHT_SYN64(2, 8)
+    SHT_SYN64(4, 1) SHT_SYN64(4, 2) SHT_SYN64(4, 4) SHT_SYN64(4, 8)
+    SHT_SYN64(8, 1) SHT_SYN64(8, 2) SHT_SYN64(8, 4) SHT_SYN64(8, 8)
+    SHT_SYN64(16, 1) SHT_SYN64(16, 2) SHT_SYN64(16, 4)
+#undef SHT_SYN64
+    return cudaErrorInvalidValue;
+}
+
+template <int BC>
+cudaError_t analys64_go(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, bool vec,
+                        cudaStream_t s)
+{
+    const dim3 grid((unsigned)((pv.lmax + (vec ? 1 : 0) + kSeedSeg) / kSeedSeg), (unsigned)(pv.mmax + 1),
+                    (unsigned)((batch + BC - 1) / BC));
+    k_analys64<BC><<<grid, 32 * kAnaWarps, 0, s>>>(pv, sd, spec, batch, vec ? 1 : 0, (int)op);
+    return cudaGetLastError();
+}
+
+// Segments of all orders (orders k mres, degrees k mres .. lmax).
+inline long segments(const PlanView<double> &pv)
+{
+    long n = 0;
+    for (int k = 0; k <= pv.mmax; ++k) n += (pv.lmax - k * pv.mres + kSeedSeg) / kSeedSeg;
+    return n;
+}
+
+// bc: fields per CTA {1, 2, 4, 8, 16}; 0: the width with the shortest busiest
+// SM -- CTAs per SM, rounded up, times the FP64 instructions of one (2 per degree
+// and 32 pairs to generate P, 2 per field to sum).
+cudaError_t analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc, bool vec,
+                     cudaStream_t s)
+{
+    if (!tables_ok(pv)) return cudaErrorInvalidValue;
+    if (bc <= 0) {
+        const long sms = sm_count(), segs = segments(pv);
+        long best = 0;
+        for (int f = 16; f >= 1; f /= 2) {
+            const long ctas = segs * ((batch + f - 1) / f);
+            const long t = (ctas + sms - 1) / sms * (1 + f);
+            if (best == 0 || t < best) {
+                best = t;
+                bc = f;
+            }
+        }
+    }
+    switch (bc) {
+    case 1: return analys64_go<1>(pv, sd, spec, batch, op, vec, s);
+    case 2: return analys64_go<2>(pv, sd, spec, batch, op, vec, s);
+    case 4: return analys64_go<4>(pv, sd, spec, batch, op, vec, s);
+    case 8: return analys64_go<8>(pv, sd, spec, batch, op, vec, s);
+    case 16: return analys64_go<16>(pv, sd, spec, batch, op, vec, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_build_qs(const PlanView<double> &pv, const unsigned long long *segoff, double2 *qs, double2 *abx,
+                            double *eps, int *hseg, cudaStream_t st)
+{
+    const int nseg = (pv.lmax + kSeedSeg) / kSeedSeg;
+    k_build_qs<<<dim3((unsigned)((nseg + 63) / 64), (unsigned)(pv.mmax + 1)), 64, 0, st>>>(pv, segoff, qs, abx, eps,
+                                                                                       hseg);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int w, int bc,
+                           cudaStream_t s)
+{
+    return synth64(pv, spec, eo, batch, op, w, bc, false, s);
+}
+
+cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc,
+                            cudaStream_t s)
+{
+    return analys64(pv, sd, spec, batch, op, bc, false, s);
+}
+
+size_t vec64_spec_bytes(int nlm, int mmax, int batch)
+{
+    return (size_t)2 * batch * ((size_t)nlm + mmax + 1) * sizeof(double2);
+}
+
+cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *uw, double *eo,
+                               int batch, Op op, cudaStream_t s)
+{
+    if (!tables_ok(pv)) return cudaErrorInvalidValue;
+    const dim3 grid((unsigned)((pv.lmax + 2 + 127) / 128), (unsigned)(pv.mmax + 1), (unsigned)batch);
+    k_vec64_split<<<grid, 128, 0, s>>>(pv, reinterpret_cast<const double2 *>(S), reinterpret_cast<const double2 *>(Tc),
+                                       reinterpret_cast<double2 *>(uw), batch, (int)op);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return synth64(pv, uw, eo, 2 * batch, OP_SYNTH, 0, 0, true, s);
+}
+
+cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *ab, double *S, double *Tc,
+                                int batch, Op op, cudaStream_t s)
+{
+    cudaError_t e = analys64(pv, sd, ab, 2 * batch, OP_ANALYS, 0, true, s);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((pv.lmax + 1 + 127) / 128), (unsigned)(pv.mmax + 1), (unsigned)batch);
+    k_vec64_join<<<grid, 128, 0, s>>>(pv, reinterpret_cast<const double2 *>(ab), reinterpret_cast<double2 *>(S),
+                                      reinterpret_cast<double2 *>(Tc), batch, (int)op);
+    return cudaGetLastError();
+}
+
+}  // namespace sht

@@ -95,7 +95,7 @@ PlanView<double> Plan::view64() const
 {
     PlanView<double> v{lmax, mmax, nlat, nphi, npairs, nlm,
                        t64.ab, t64.dc, t64.x, t64.st, t64.wq, t64.pmm, t64.pmmk, t64.tw, t64.rtw, fft_plan_of(nphi / 2), mres, twdf,
-                       nullptr, d_seg32, seeds64, seeds64k, live64};
+                       nullptr, d_seg32, seeds64, seeds64k, live64, qs64, abx64, eps64, hseg64};
     return v;
 }
 
@@ -103,7 +103,7 @@ PlanView<float> Plan::view32() const
 {
     PlanView<float> v{lmax, mmax, nlat, nphi, npairs, nlm,
                       t32.ab, t32.dc, t32.x, t32.st, t32.wq, t32.pmm, t32.pmmk, t32.tw, t32.rtw, fft_plan_of(nphi / 2), mres, nullptr,
-                      seeds32, d_seg32, nullptr, nullptr, live32};
+                      seeds32, d_seg32, nullptr, nullptr, live32, nullptr, nullptr, nullptr, nullptr};
     return v;
 }
 
@@ -314,6 +314,18 @@ int plan_segments(Plan &p, std::string &err)
     return SHT_OK;
 }
 
+// seeds64 is the base of the allocation of all of these.
+void free_seeds64(Plan &p)
+{
+    cudaFree(p.seeds64);
+    p.seeds64 = nullptr;
+    p.seeds64k = nullptr;
+    p.live64 = nullptr;
+    p.qs64 = p.abx64 = nullptr;
+    p.eps64 = nullptr;
+    p.hseg64 = nullptr;
+}
+
 size_t plan_nseg(const Plan &p)
 {
     std::vector<unsigned long long> segoff;
@@ -331,7 +343,8 @@ int plan_seeds32(Plan &p, std::string &err)
     cudaError_t e = cudaMalloc(&p.seeds32, sizeof(float4) * nseg * (size_t)p.npairs);
     if (e == cudaSuccess) e = cudaMalloc(&p.live32, sizeof(unsigned short) * (size_t)(p.mmax + 1) * p.npairs);
     if (e == cudaSuccess)
-        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, p.live32, p.thr_cc32(), 0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, nullptr, p.live32, p.thr_cc32(),
+                                  0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -345,26 +358,36 @@ int plan_seeds32(Plan &p, std::string &err)
     return SHT_OK;
 }
 
+// One allocation for everything the FP64 CUDA-core kernels keep (a cudaMalloc
+// costs about as much as a small transform).
 int plan_seeds64(Plan &p, std::string &err)
 {
     if (p.seeds64) return SHT_OK;
     int rc = plan_segments(p, err);
     if (rc) return rc;
-    const size_t nseg = plan_nseg(p);
-    cudaError_t e = cudaMalloc(&p.seeds64, sizeof(double2) * nseg * (size_t)p.npairs);
-    if (e == cudaSuccess) e = cudaMalloc(&p.seeds64k, sizeof(int) * nseg * (size_t)p.npairs);
-    if (e == cudaSuccess) e = cudaMalloc(&p.live64, sizeof(unsigned short) * (size_t)(p.mmax + 1) * p.npairs);
+    const size_t nseg = plan_nseg(p), nstate = nseg * (size_t)p.npairs, norder = (size_t)(p.mmax + 1) * p.npairs;
+    const size_t nlmx = (size_t)p.nlm + p.mmax + 1;   // degrees to lmax + 1
+    DevArena ar;
+    ar.cap = padded<double2>(nstate) + padded<int>(nstate) + padded<unsigned short>(norder) +
+             2 * padded<double2>(nlmx) + padded<double>(nlmx) + padded<int>(nseg);
+    cudaError_t e = cudaMalloc(&ar.base, ar.cap);
+    if (e == cudaSuccess) {
+        p.seeds64 = ar.take<double2>(nstate);   // the allocation's base
+        p.seeds64k = ar.take<int>(nstate);
+        p.live64 = ar.take<unsigned short>(norder);
+        p.qs64 = ar.take<double2>(nlmx);
+        p.abx64 = ar.take<double2>(nlmx);
+        p.eps64 = ar.take<double>(nlmx);
+        p.hseg64 = ar.take<int>(nseg);
+        e = launch_build_qs(p.view64(), p.d_seg32, p.qs64, p.abx64, p.eps64, p.hseg64, 0);
+    }
     if (e == cudaSuccess)
-        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.live64, p.thr_cc64(), 0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.hseg64, p.live64,
+                                  p.thr_cc64(), 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(p.seeds64);
-        cudaFree(p.seeds64k);
-        cudaFree(p.live64);
-        p.seeds64 = nullptr;
-        p.seeds64k = nullptr;
-        p.live64 = nullptr;
+        free_seeds64(p);
         err = std::string("building FP64 recurrence seeds: ") + cudaGetErrorString(e);
         return SHT_ENOMEM;
     }
@@ -375,9 +398,11 @@ int plan_relive(Plan &p, std::string &err)
 {
     cudaError_t e = cudaSuccess;
     if (p.seeds32)
-        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, p.live32, p.thr_cc32(), 0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, nullptr, p.live32, p.thr_cc32(),
+                                  0);
     if (e == cudaSuccess && p.seeds64)
-        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.live64, p.thr_cc64(), 0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.hseg64, p.live64,
+                                  p.thr_cc64(), 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         err = std::string("rebuilding the polar tables: ") + cudaGetErrorString(e);
@@ -441,15 +466,11 @@ void plan_free(Plan &p)
 {
     cudaFree(p.seeds32);
     cudaFree(p.d_seg32);
-    cudaFree(p.seeds64);
-    cudaFree(p.seeds64k);
     cudaFree(p.live32);
-    cudaFree(p.live64);
+    free_seeds64(p);
     p.seeds32 = nullptr;
     p.d_seg32 = nullptr;
-    p.seeds64 = nullptr;
-    p.seeds64k = nullptr;
-    p.live32 = p.live64 = nullptr;
+    p.live32 = nullptr;
     for (cudaEvent_t e : p.timer.pool) cudaEventDestroy(e);
     p.timer.pool.clear();
     if (p.tables_base) cudaFree(p.tables_base);

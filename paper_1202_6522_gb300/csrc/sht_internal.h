@@ -64,13 +64,20 @@ struct PlanView {
     // float4 (y1, y2, k as int bits, 0), segments of order index m from segoff[m].
     const float4 *seeds;
     const unsigned long long *segoff;
-    // FP64 plans: the same states as (y1, y2) and k, [segment][npairs].
+    // FP64 plans: the same states as (y1, y2) 2^hseg and k, [segment][npairs].
     const double2 *seeds64;
     const int *seeds64k;
     // Static polar optimisation (Sec. 3.1): per (order index m, pair) the
     // first kSeedSeg-degree segment holding a |P_n^m| at or above the
     // threshold (the segment count when none does), [mmax+1][npairs].
     const unsigned short *live;
+    // FP64 plans: recurrences of legendre64.cu for degrees m .. lmax + 1 of every
+    // order, order index m from col_of_mres(lmax + 1, m, mres): (beta_n, s_n) of
+    // Q_n = P_n / s_n, (a_n, b_n) of P_n, eps_n; and the state scale of each segment.
+    const double2 *qs;
+    const double2 *abx;
+    const double *eps;
+    const int *hseg;
 };
 
 // The FP32 Legendre kernels restart the recurrence of Sec. 3.2 every kSeedSeg
@@ -78,8 +85,6 @@ struct PlanView {
 // carried in the exponent-scaled form of Sec. 3.5 (y * 2^(-64 k)), so that
 // FP32 rounding errors accumulate over at most kSeedSeg steps.
 constexpr int kSeedSeg = 32;
-// Analysis shape code (TunedShape::analys_lpt) of the FP64 warp-per-segment kernel.
-constexpr int kAnalysSeg = 32;
 
 // First packed index of order index k (order m = k mres): the degrees of the
 // orders before it, sum_{k' < k} (lmax - k' mres + 1).
@@ -122,7 +127,8 @@ enum Op {
     OP_ANALYS_ADJ = 3   // adjoint of analysis (a weighted synthesis of b / c_m)
 };
 
-// Kernel shapes chosen by sht_tune for one (precision, batch).
+// Kernel shapes chosen by sht_tune for one (precision, batch).  FP64: synth_lpt
+// is the warps per CTA, analys_lpt is not used (legendre64.cu).
 struct TunedShape {
     int synth_lpt = 0, synth_bc = 0, analys_lpt = 0, analys_bc = 0;
     int auto_mode = 1;           // SHT_F32_AUTO: the fastest of SHT_F32, SHT_TC_BF16X3, SHT_TC_OTF
@@ -176,6 +182,9 @@ struct Plan {
     unsigned long long *d_seg32 = nullptr;      // first kSeedSeg segment of each order index (both precisions)
     double2 *seeds64 = nullptr;                 // FP64 restart states (y1, y2) ...
     int *seeds64k = nullptr;                    // ... and their exponent counters
+    double2 *qs64 = nullptr, *abx64 = nullptr;  // ... with the recurrences of legendre64.cu to degree lmax + 1
+    double *eps64 = nullptr;
+    int *hseg64 = nullptr;
     unsigned short *live32 = nullptr, *live64 = nullptr;   // first live segment per (m, pair), per precision
     bool polar_thr_set = false;                 // sht_set_polar_threshold was called
     // thresholds of the static polar optimisation of the CUDA-core kernels:
@@ -209,33 +218,41 @@ int plan_relive(Plan &p, std::string &err);
 // Segment offsets of kSeedSeg degrees per order index; returns the total.
 size_t seed_segment_offsets(int lmax, int mmax, int mres, std::vector<unsigned long long> &segoff);
 // One thread per (m, pair): FP32 states (seeds32) or FP64 states (seeds64,
-// seeds64k), and the first segment holding |P| >= thr (thr <= 0: segment 0).
+// seeds64k, scaled by 2^hseg of their segment), and the first segment holding
+// |P| >= thr (thr <= 0: segment 0).
 cudaError_t launch_build_restarts(const PlanView<double> &pv, const unsigned long long *segoff, float4 *seeds32,
-                                  double2 *seeds64, int *seeds64k, unsigned short *live, double thr, cudaStream_t st);
+                                  double2 *seeds64, int *seeds64k, const int *hseg, unsigned short *live, double thr,
+                                  cudaStream_t st);
 
-// Launchers (legendre.cu, fft.cu).  `eo` / `sd` are intermediate buffers of
-// [batch][mmax+1][npairs][2] complex values of precision T.
-template <typename T>
-cudaError_t launch_legendre_synth(const PlanView<T> &pv, const T *spec, T *eo, int batch, Op op,
-                                  cudaStream_t s);
-template <typename T>
-cudaError_t launch_legendre_analys(const PlanView<T> &pv, const T *sd, T *spec, int batch, Op op,
-                                   cudaStream_t s);
-// Explicit kernel shapes (lpt pairs per thread, bc fields per CTA; 0 = default).
-// Synthesis: lpt in {1,2,4}, bc in {1,2,4}; analysis: lpt in {2,4,8}, bc in {1,2}.
-template <typename T>
-cudaError_t launch_legendre_synth_cfg(const PlanView<T> &pv, const T *spec, T *eo, int batch, Op op, int lpt,
-                                      int bc, cudaStream_t s);
-template <typename T>
-cudaError_t launch_legendre_analys_cfg(const PlanView<T> &pv, const T *sd, T *spec, int batch, Op op, int lpt,
-                                       int bc, cudaStream_t s);
-
-template <typename T>
-cudaError_t launch_legendre_synth_vec(const PlanView<T> &pv, const T *S, const T *Tc, T *eot,
-                                      T *eop, int batch, Op op, cudaStream_t s);
-template <typename T>
-cudaError_t launch_legendre_analys_vec(const PlanView<T> &pv, const T *sdt, const T *sdp, T *S,
-                                       T *Tc, int batch, Op op, cudaStream_t s);
+// Launchers (legendre.cu, legendre64.cu, fft.cu).  `eo` / `sd` are intermediate
+// buffers of [batch][mmax+1][npairs][2] complex values.
+// FP32.  Explicit kernel shapes (lpt pairs per thread, bc fields per CTA; 0 =
+// default).  Synthesis: lpt in {1,2,4}, bc in {1,2,4}; analysis: lpt in
+// {2,4,8}, bc in {1,2}.
+cudaError_t launch_legendre_synth(const PlanView<float> &pv, const float *spec, float *eo, int batch, Op op, int lpt,
+                                  int bc, cudaStream_t s);
+cudaError_t launch_legendre_analys(const PlanView<float> &pv, const float *sd, float *spec, int batch, Op op, int lpt,
+                                   int bc, cudaStream_t s);
+cudaError_t launch_legendre_synth_vec(const PlanView<float> &pv, const float *S, const float *Tc, float *eot,
+                                      float *eop, int batch, Op op, cudaStream_t s);
+cudaError_t launch_legendre_analys_vec(const PlanView<float> &pv, const float *sdt, const float *sdp, float *S,
+                                       float *Tc, int batch, Op op, cudaStream_t s);
+// FP64.  w: warps per CTA of the synthesis in {1,2,4,8}; bc: fields per CTA in
+// {1,2,4,8,16} (16 fields: w <= 4); 0 = default.
+cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int w, int bc,
+                           cudaStream_t s);
+cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc,
+                            cudaStream_t s);
+// Vector transforms as scalar ones of 2 batch fields: `uw` / `ab` are scratch
+// of vec64_spec_bytes; eo / sd hold the theta fields, then the phi fields.
+size_t vec64_spec_bytes(int nlm, int mmax, int batch);
+cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *uw, double *eo,
+                               int batch, Op op, cudaStream_t s);
+cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *ab, double *S, double *Tc,
+                                int batch, Op op, cudaStream_t s);
+// Fills the plan's qs, abx, eps and hseg tables (the view's are not used).
+cudaError_t launch_build_qs(const PlanView<double> &pv, const unsigned long long *segoff, double2 *qs, double2 *abx,
+                            double *eps, int *hseg, cudaStream_t st);
 template <typename T>
 cudaError_t launch_fft_synth(const PlanView<T> &pv, const T *eo, T *grid, int batch, Op op,
                              cudaStream_t s);
