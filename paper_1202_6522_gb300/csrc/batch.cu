@@ -359,7 +359,10 @@ int sht_batch_create_mode(int nfields, const int *lmax, const int *nlat, const i
                 const int np = std::min(sht::kBatchSynthPairs, p.npairs - pb * sht::kBatchSynthPairs);
                 syn.push_back({(double)(p.lmax - m + 1) * (np + 32), make_int4(f, m, pb, 0)});
             }
-            ana.push_back({(double)(p.lmax - m + 1) * (p.npairs + 32), make_int4(f, m, 0, 0)});
+            const int nseg = (p.lmax - m + sht::kSeedSeg) / sht::kSeedSeg;
+            for (int seg = 0; seg < nseg; seg += sht::kBatchAnalysSegs)
+                ana.push_back({(double)std::min(sht::kBatchAnalysSegs, nseg - seg) * (p.npairs + 32),
+                               make_int4(f, m, seg, 0)});
         }
         int logH = 0;
         while ((1 << logH) < p.nphi / 2) ++logH;
@@ -416,7 +419,7 @@ int sht_batch_create_mode(int nfields, const int *lmax, const int *nlat, const i
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
     b->ctas_legendre_syn = sms * 8;   // 128-thread CTAs
-    b->ctas_legendre_ana = sms * 4;   // 256-thread CTAs
+    b->ctas_legendre_ana = sms * 4;   // 128-thread CTAs of independent warps
     b->ctas_fft = sms * std::max(1, (int)std::min<size_t>(8, (200 * 1024) / std::max<size_t>(smem, 1)));
     cudaError_t e = cudaMallocHost(&b->h_fields, sizeof(sht::BatchField) * nfields);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_fields, sizeof(sht::BatchField) * nfields);

@@ -522,7 +522,7 @@ cudaError_t legendre_analys(const sht::PlanView<double> &pv, const double *sd, d
 cudaError_t legendre_analys(const sht::PlanView<float> &pv, const float *sd, float *spec, int batch, sht::Op op,
                             const sht::TunedShape &ts, cudaStream_t s)
 {
-    return sht::launch_legendre_analys(pv, sd, spec, batch, op, ts.analys_lpt, ts.analys_bc, s);
+    return sht::launch_legendre_analys(pv, sd, spec, batch, op, ts.analys_bc, s);
 }
 
 // The two directions of the scalar transform, parameterised by precision.
@@ -1280,12 +1280,12 @@ extern "C" int sht_tune(sht_handle h, int batch, int mode, double *report, void 
     double best_syn = 1e30, best_ana = 1e30;
     const int reps = 3;
     const int widths[5] = {1, 2, 4, 8, 16};   // fields per CTA (FP32: up to 4 and 2)
-    const int lpts_s[4] = {1, 2, 4, 8}, lpts_a[3] = {2, 4, 8};
+    const int lpts_s[4] = {1, 2, 4, 8};
     for (int li = 0; li < 4; ++li)
         for (int bi = 0; bi < 5; ++bi) {
             const int lpt = lpts_s[li], bc = widths[bi];   // FP64: lpt warps per CTA
             if (bc > batch && bc > 1) continue;
-            if (shape_mode == SHT_F64 ? (bc == 16 && lpt == 8) : (lpt > 4 || bc > 4)) continue;
+            if (shape_mode == SHT_F64 ? (bc == 16 && lpt == 8) : (lpt > 4 || bc > 4 || lpt * bc > 8)) continue;
             bool ok = false;
             double ms;
             if (shape_mode == SHT_F64)
@@ -1294,22 +1294,17 @@ extern "C" int sht_tune(sht_handle h, int batch, int mode, double *report, void 
                 ms = time_ms([&] { return sht::launch_legendre_synth(p.view32(), (const float *)spec, (float *)p.work, batch, sht::OP_SYNTH, lpt, bc, s); }, s, reps, ok);
             if (ok && ms < best_syn) { best_syn = ms; best.synth_lpt = lpt; best.synth_bc = bc; }
         }
-    for (int li = 0; li < 3; ++li)
-        for (int bi = 0; bi < 5; ++bi) {
-            const int lpt = lpts_a[li], bc = widths[bi];
-            if (bc > batch && bc > 1) continue;
-            if (shape_mode == SHT_F64
-                    ? li > 0
-                    : (bc > 2 || (p.npairs + 32 * lpt - 1) / (32 * lpt) > 8))
-                continue;
-            bool ok = false;
-            double ms;
-            if (shape_mode == SHT_F64)
-                ms = time_ms([&] { return sht::launch_analys64(p.view64(), (const double *)p.work, (double *)spec, batch, sht::OP_ANALYS, bc, s); }, s, reps, ok);
-            else
-                ms = time_ms([&] { return sht::launch_legendre_analys(p.view32(), (const float *)p.work, (float *)spec, batch, sht::OP_ANALYS, lpt, bc, s); }, s, reps, ok);
-            if (ok && ms < best_ana) { best_ana = ms; best.analys_lpt = lpt; best.analys_bc = bc; }
-        }
+    for (int bi = 0; bi < 5; ++bi) {
+        const int bc = widths[bi];
+        if ((bc > batch && bc > 1) || (shape_mode == SHT_F32 && bc > 2)) continue;
+        bool ok = false;
+        double ms;
+        if (shape_mode == SHT_F64)
+            ms = time_ms([&] { return sht::launch_analys64(p.view64(), (const double *)p.work, (double *)spec, batch, sht::OP_ANALYS, bc, s); }, s, reps, ok);
+        else
+            ms = time_ms([&] { return sht::launch_legendre_analys(p.view32(), (const float *)p.work, (float *)spec, batch, sht::OP_ANALYS, bc, s); }, s, reps, ok);
+        if (ok && ms < best_ana) { best_ana = ms; best.analys_bc = bc; }
+    }
     cudaGetLastError();
     set_tuned(p, shape_mode, batch, best);
     if (report) { report[0] = best_syn; report[1] = best_ana; report[2] = -1.0; }

@@ -1,4 +1,5 @@
-// legendre.cu -- the per-order Legendre stage of the Gauss-Legendre SHT.
+// legendre.cu -- the FP32 Legendre stage of the Gauss-Legendre SHT on the CUDA
+// cores, and the restart tables of both precisions (FP64: legendre64.cu).
 //
 // Synthesis (Sec. 2.2, Eq. synth_direct): for each order m and each latitude
 // pair (x, -x), sum over n the spectral coefficients times P_n^m, split by the
@@ -8,19 +9,24 @@
 // Analysis (Sec. 2.3, Eq. gauss): with s = w (F(x) + F(-x)), d = w (F(x) - F(-x))
 // prepared by the FFT kernel, f_n^m = sum_pairs P_n^m(x) (s if n-m even else d).
 //
-// P_n^m is generated on the fly by the recurrence of Sec. 3.2, held in
-// registers, one thread per latitude pair (LPT pairs per thread); the
-// coefficients (a_n^m, b_n^m) and the spectral values are staged through
-// shared memory and read as broadcasts.  Underflow is handled as in Sec. 3.5:
-// a value is y * 2^(-S k); while k > 0 it is left out of the sums and the
-// recurrence rescales y by 2^-S when it exceeds 1.  Warps in which every pair
-// is still scaled skip the accumulation (the dynamic polar optimisation).
+// P_n^m is generated on the fly by the recurrence of Sec. 3.2, one latitude
+// pair per lane, restarted at every segment of kSeedSeg degrees from the state
+// the FP64 recurrence computed once per plan (the FP32 recurrence alone loses
+// accuracy with n).  Underflow (Sec. 3.5) is taken care of per segment: where the
+// values entering it are below 2^-62, the state is stored times a power of two
+// that keeps the whole segment in the FP32 range, together with the factor that
+// takes it back (0 where no |P| of the segment reaches 2^-70), so the recurrence
+// itself tests nothing.  Since segments do not depend on one another, they are
+// what the kernels split over warps.
 //
-// Analysis reduces over latitudes without atomics: each thread sums its own
-// pairs in registers for K consecutive degrees, a warp-level transposing
-// butterfly leaves one partial per lane, and the warps' partials are added in
-// shared memory in a fixed order, so results are bitwise reproducible.
+// What bounds these kernels is instruction issue: 3 instructions of recurrence
+// per degree and pair and 2 per field and degree, on the FMA pipe, plus
+// whatever else the loops carry.  So a warp tests liveness and scaling once per
+// segment, not per degree, and the sums over latitudes are taken across lanes
+// once per segment of all pairs, not once per few degrees.
 #include <cuda_runtime.h>
+
+#include <climits>
 
 #include "sht_internal.h"
 
@@ -29,610 +35,544 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-template <typename T> __device__ __forceinline__ bool abs_ge_one(T y);
-template <> __device__ __forceinline__ bool abs_ge_one<double>(double y)
+// P_n = a x P_{n-1} + b P_{n-2}.
+__device__ __forceinline__ float next_p(float a, float b, float x, float y1, float y2)
 {
-    return (__double2hiint(y) & 0x7fffffff) >= 0x3ff00000;
-}
-template <> __device__ __forceinline__ bool abs_ge_one<float>(float y)
-{
-    return (__float_as_int(y) & 0x7fffffff) >= 0x3f800000;
+    return fmaf(a * x, y1, b * y2);
 }
 
-template <typename T> __device__ __forceinline__ T down_scale();
-template <> __device__ __forceinline__ double down_scale<double>() { return 0x1p-240; }
-template <> __device__ __forceinline__ float down_scale<float>() { return 0x1p-64f; }
-
-// One step of P_n = a x P_{n-1} + b P_{n-2} for LPT pairs.  With CHECK the
-// rescaling of Sec. 3.5 is applied and c[] receives the value entering the
-// sums (0 while k > 0); without it c[] is the value itself.  Pairs i whose
-// bit in `live` (warp-uniform) is clear are left as they are, with c[i] = 0.
-template <typename T, int LPT, bool CHECK>
-__device__ __forceinline__ void rec_step(T a, T b, const T (&x)[LPT], T (&y1)[LPT], T (&y2)[LPT],
-                                         int (&k)[LPT], T (&c)[LPT], unsigned live = ~0u)
+// 16 bytes from global to shared memory, asynchronously; zeros unless `in`.
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool in)
 {
-#pragma unroll
-    for (int i = 0; i < LPT; ++i) {
-        if (!((live >> i) & 1)) {
-            c[i] = T(0);
-            continue;
-        }
-        T yn = fma(a * x[i], y1[i], b * y2[i]);
-        y2[i] = y1[i];
-        y1[i] = yn;
-        if (CHECK) {
-            if (k[i] > 0 && abs_ge_one(yn)) {
-                y1[i] *= down_scale<T>();
-                y2[i] *= down_scale<T>();
-                k[i] -= 1;
-            }
-            c[i] = (k[i] == 0) ? y1[i] : T(0);
-        } else {
-            c[i] = yn;
-        }
-    }
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-template <typename T, int LPT>
-__device__ __forceinline__ int kmax_of(const int (&k)[LPT])
+// The kernels need the restart states and the tables of live groups.  A plan
+// without them is refused rather than run on other arithmetic.
+bool seeds_ok(const PlanView<float> &pv)
 {
-    int r = 0;
-#pragma unroll
-    for (int i = 0; i < LPT; ++i) r = max(r, k[i]);
-    return r;
+    return pv.segoff != nullptr && pv.seeds != nullptr && pv.glive != nullptr && pv.glive_vec != nullptr;
 }
 
-template <typename T, int LPT>
-__device__ __forceinline__ int kmin_of(const int (&k)[LPT])
+// Sums V values (a multiple of 32) over the 32 lanes and leaves lane l holding
+// the sums of values [l V/32, (l + 1) V/32) in v[0 .. V/32).  Step by step a lane
+// keeps half of its values and hands the other half to the lane O away.
+template <int V, int O = 16, int N>
+__device__ __forceinline__ void warp_transpose_reduce(float (&v)[N], int lane)
 {
-    int r = k[0];
-#pragma unroll
-    for (int i = 1; i < LPT; ++i) r = min(r, k[i]);
-    return r;
-}
-
-// Restart the recurrence of the LPT pairs p[] at segment `seg` (degrees
-// n - m in [kSeedSeg seg, kSeedSeg (seg + 1))) of order index m from the
-// state the FP64 recurrence computed once per plan: y1 = P_{n0-1},
-// y2 = P_{n0-2} and the exponent counter k of Sec. 3.5, in the precision's
-// own scaled form.  FP32 kernels restart every segment (the FP32 recurrence
-// alone loses accuracy with n); FP64 kernels restart where they skip dead
-// segments (the static polar optimisation).
-template <typename T, int LPT>
-__device__ __forceinline__ void reseed(const PlanView<T> &pv, int m, int seg, const int (&p)[LPT], T (&y1)[LPT],
-                                       T (&y2)[LPT], int (&k)[LPT])
-{
-    const size_t base = (size_t)(pv.segoff[m] + seg) * pv.npairs;
-#pragma unroll
-    for (int i = 0; i < LPT; ++i) {
-        if (p[i] < pv.npairs) {
-            if constexpr (sizeof(T) == sizeof(float)) {
-                const float4 v = __ldg(pv.seeds + base + p[i]);
-                y1[i] = v.x;
-                y2[i] = v.y;
-                k[i] = __float_as_int(v.z);
-            } else {
-                const double2 v = __ldg(pv.seeds64 + base + p[i]);
-                y1[i] = v.x;
-                y2[i] = v.y;
-                k[i] = __ldg(pv.seeds64k + base + p[i]);
-            }
-        }
-    }
-}
-
-// First live segment of each group i of 32 pairs (the warp's lanes' p[i];
-// no pair: past every segment), warp-uniform; returns the smallest.
-template <typename T, int LPT>
-__device__ __forceinline__ int group_first_live(const PlanView<T> &pv, int m, const int (&p)[LPT], int (&gf)[LPT])
-{
-    int r = 0xffff;
-#pragma unroll
-    for (int i = 0; i < LPT; ++i) {
-        const int f = p[i] < pv.npairs ? (int)__ldg(pv.live + (size_t)m * pv.npairs + p[i]) : 0xffff;
-        gf[i] = __reduce_min_sync(kFull, f);
-        r = min(r, gf[i]);
-    }
-    return r;
-}
-
-// Bit i set when group i has a live pair in segment seg.
-template <int LPT>
-__device__ __forceinline__ unsigned live_groups(const int (&gf)[LPT], int seg)
-{
-    unsigned r = 0;
-#pragma unroll
-    for (int i = 0; i < LPT; ++i)
-        if (seg >= gf[i]) r |= 1u << i;
-    return r;
-}
-
-// The kernels need the restart states, the scalar ones the first-live table
-// too.  A plan without them is refused rather than run on other arithmetic.
-bool seeds_ok(const PlanView<float> &pv, bool scalar)
-{
-    return pv.segoff != nullptr && pv.seeds != nullptr && (!scalar || pv.live != nullptr);
-}
-
-// Warp butterfly that sums V values (V a multiple of 32) over the 32 lanes and
-// leaves lane l holding the sums of values [l*V/32, (l+1)*V/32) in v[0..V/32).
-template <typename T, int V>
-__device__ __forceinline__ void warp_transpose_reduce(T (&v)[V], int lane)
-{
-#pragma unroll
-    for (int s = 0; s < 5; ++s) {
-        const int o = 16 >> s;
-        const int h = V >> (s + 1);
-        const bool up = (lane & o) != 0;
+    if constexpr (O > 0) {
+        constexpr int h = V / 2;
+        const bool up = (lane & O) != 0;
 #pragma unroll
         for (int q = 0; q < h; ++q) {
-            T send = up ? v[q] : v[q + h];
-            T keep = up ? v[q + h] : v[q];
-            v[q] = keep + __shfl_xor_sync(kFull, send, o);
+            const float send = up ? v[q] : v[q + h];
+            const float keep = up ? v[q + h] : v[q];
+            v[q] = keep + __shfl_xor_sync(kFull, send, O);
         }
+        warp_transpose_reduce<h, O / 2>(v, lane);
     }
 }
 
-// ---------------------------------------------------------------------------
-// Scalar synthesis.  grid.x = (m, pair block), heaviest m first; grid.y = field chunk.
-// ---------------------------------------------------------------------------
-constexpr int kSynthNch = 128;  // degrees staged per chunk (scalar synthesis)
-static_assert(kSynthNch % kSeedSeg == 0, "restart segments must not straddle staged chunks");
+constexpr int kWarps = 4;   // warps per CTA of the kernels below
 
-// One (order m, pair block pb, field chunk b0) tile of the scalar synthesis,
-// run by a whole CTA of NT threads; s_ab[kSynthNch], s_f[kSynthNch * BC] are
-// the CTA's staging buffers, *s_first a shared word.
+// Groups of 32 pairs of a plan.
+__device__ __forceinline__ int groups_of(int npairs) { return (npairs + 31) >> 5; }
+
+// ---------------------------------------------------------------------------
+// Synthesis.  A CTA of four warps per (order m, block of 32 LPT pairs, BC
+// fields): warp w sums the segments w, w + 4, ... over the block's pairs, LPT
+// pairs per lane, and the warps' sums meet in shared memory in a fixed order.
+// Which segments a warp takes does not depend on LPT, BC or the batch, nor does
+// any sum.  Static polar optimisation (Sec. 3.1): a group of 32 pairs (one per
+// lane) is left out of the segments before its first live one.
 //
-// Static polar optimisation (Sec. 3.1): the CTA starts at the first segment
-// in which one of its pairs is live; within a warp, a group of 32 pairs (one
-// p[i] per lane) runs neither the recurrence nor the sums over a segment in
-// which none of its pairs is live.  Each segment a warp runs restarts the
-// recurrence from the stored state.
-template <typename T, int LPT, int BC, int NT>
-__device__ __forceinline__ void synth_tile(const PlanView<T> &pv, const T *__restrict__ spec, T *__restrict__ eo,
-                                           int batch, int m, int pb, int b0, int op, typename Vec2<T>::type *s_ab,
-                                           typename Vec2<T>::type *s_f, int *s_first)
-{
-    using T2 = typename Vec2<T>::type;
-    constexpr int NCH = kSynthNch;
-    const int lmax = pv.lmax, npairs = pv.npairs;
-    const int L = lmax - m * pv.mres + 1;   // order index m is the order m mres
-    const long col = col_of_mres(lmax, m, pv.mres);
+// Per degree, LPT pairs and BC fields: 3 LPT + 2 BC LPT FMA-pipe instructions,
+// half a shared-memory load of (a, b) and BC / 2 of the spectral values, all
+// broadcasts.  N = 2047, 2 fields: 552 us (issue 72 %, FMA pipe 45 %) against 817
+// with a CTA of 256 pairs walking the degrees between barriers and testing each
+// pair's scale at every degree; N = 383, 3-fold, 6 fields: 61 -> 13.5 us.
+// ---------------------------------------------------------------------------
+template <int LPT, int BC>
+struct SynthSmem {
+    float4 ab[kWarps][kSeedSeg / 2];          // (a, b) of two degrees
+    float2 f[kWarps][kSeedSeg * BC];          // [degree][field]
+    float4 sum[kWarps][LPT * 32 * BC];        // [pair][field] (E, O)
+};
 
-    T x[LPT], y1[LPT], y2[LPT], c[LPT];
-    int k[LPT], p[LPT];
+template <int LPT, int BC>
+__device__ __forceinline__ void synth_tile(const PlanView<float> &pv, const float *__restrict__ spec,
+                                           float *__restrict__ eo, int batch, int m, int pb, int b0, int op,
+                                           SynthSmem<LPT, BC> &sm)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int npairs = pv.npairs, ng = groups_of(npairs);
+    const int L = pv.lmax - m * pv.mres + 1;   // order index m is the order m mres
+    const int nseg = (L + kSeedSeg - 1) / kSeedSeg;
+    const long col = col_of_mres(pv.lmax, m, pv.mres);
+    const float2 *spec2 = reinterpret_cast<const float2 *>(spec);
+    const float insc = (op == OP_ANALYS_ADJ && m > 0) ? 0.5f : 1.f;   // adjoint of analysis: b / c_m
+
+    int p[LPT], gf[LPT], first = 0xffff;
+    float x[LPT], er[LPT][BC], ei[LPT][BC], orr[LPT][BC], oi[LPT][BC];
 #pragma unroll
     for (int i = 0; i < LPT; ++i) {
-        p[i] = pb * NT * LPT + i * NT + threadIdx.x;
-        const bool v = p[i] < npairs;
-        const size_t o = (size_t)m * npairs + p[i];
-        x[i] = v ? pv.x[p[i]] : T(0);
-        y2[i] = v ? pv.pmm[o] : T(0);
-        k[i] = v ? pv.pmmk[o] : 0;
-        y1[i] = T(0);
+        const int g = pb * LPT + i;
+        p[i] = g * 32 + lane;
+        x[i] = p[i] < npairs ? pv.x[p[i]] : 0.f;
+        gf[i] = g < ng ? (int)pv.glive[(size_t)m * ng + g] : 0xffff;
+        first = min(first, gf[i]);
+#pragma unroll
+        for (int b = 0; b < BC; ++b) er[i][b] = ei[i][b] = orr[i][b] = oi[i][b] = 0.f;
     }
-    T er[LPT][BC], ei[LPT][BC], orr[LPT][BC], oi[LPT][BC];
+
+    // a segment's spectral values, (a, b) (lane = degree) and states (lane = pair),
+    // read one segment ahead through pointers that step with the warp's segments
+    int seg = first + ((w - first) & (kWarps - 1));   // the first one >= `first` of this warp
+    if (seg > nseg) seg = nseg;
+    const int nb = min(BC, batch - b0);
+    const float2 *pab = pv.ab + col + seg * kSeedSeg + lane;
+    const float2 *pf = spec2 + (size_t)b0 * pv.nlm + col + seg * kSeedSeg + lane;
+    const float4 *ps = pv.seeds + (pv.segoff[m] + seg) * npairs + p[0];
+    float2 nab, nf[BC];
+    float4 ns[LPT];
+    const auto fetch = [&](int sg) {
+        const bool in = sg * kSeedSeg + lane < L;
+        nab = in ? __ldg(pab) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int b = 0; b < BC; ++b) nf[b] = in && b < nb ? __ldg(pf + (size_t)b * pv.nlm) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < LPT; ++i)
+            ns[i] = sg < nseg && p[i] < npairs ? __ldg(ps + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        pab += kWarps * kSeedSeg;
+        pf += kWarps * kSeedSeg;
+        ps += (size_t)kWarps * npairs;
+    };
+    fetch(seg);
+    for (; seg < nseg; seg += kWarps) {
+        const int cnt = min(kSeedSeg, L - seg * kSeedSeg);
+        __syncwarp();   // the last segment's reads are done
+        reinterpret_cast<float2 *>(sm.ab[w])[lane] = nab;
+#pragma unroll
+        for (int b = 0; b < BC; ++b)
+            sm.f[w][lane * BC + b] = make_float2(nf[b].x * insc, m == 0 ? 0.f : nf[b].y * insc);
+        float y1[LPT], y2[LPT], sc[LPT];
+        bool all = true, scaled = false;
+#pragma unroll
+        for (int i = 0; i < LPT; ++i) {
+            y1[i] = ns[i].x;
+            y2[i] = ns[i].y;
+            sc[i] = ns[i].z;
+            all = all && seg >= gf[i];
+            scaled = scaled || (sc[i] != 1.f && p[i] < npairs);
+        }
+        fetch(seg + kWarps);
+        __syncwarp();
+        if (all && !__any_sync(kFull, scaled)) {
+#pragma unroll 1
+            for (int tb = 0; tb < cnt; tb += 8)   // rows past cnt are zero
+#pragma unroll
+            for (int t = tb; t < tb + 8; t += 2) {
+                const float4 ab = sm.ab[w][t >> 1];
+#pragma unroll
+                for (int i = 0; i < LPT; ++i) y2[i] = next_p(ab.x, ab.y, x[i], y1[i], y2[i]);
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    const float2 f = sm.f[w][t * BC + b];
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) {
+                        er[i][b] = fmaf(f.x, y2[i], er[i][b]);
+                        ei[i][b] = fmaf(f.y, y2[i], ei[i][b]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < LPT; ++i) y1[i] = next_p(ab.z, ab.w, x[i], y2[i], y1[i]);
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    const float2 f = sm.f[w][(t + 1) * BC + b];
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) {
+                        orr[i][b] = fmaf(f.x, y1[i], orr[i][b]);
+                        oi[i][b] = fmaf(f.y, y1[i], oi[i][b]);
+                    }
+                }
+            }
+        } else {
+            // a group not live yet, or a pair whose state is stored scaled
+#pragma unroll
+            for (int i = 0; i < LPT; ++i) {
+                if (seg < gf[i]) continue;
+#pragma unroll 2
+                for (int t = 0; t < cnt; t += 2) {
+                    const float4 ab = sm.ab[w][t >> 1];
+                    y2[i] = next_p(ab.x, ab.y, x[i], y1[i], y2[i]);
+                    const float c0 = sc[i] * y2[i];
+                    y1[i] = next_p(ab.z, ab.w, x[i], y2[i], y1[i]);
+                    const float c1 = sc[i] * y1[i];
+#pragma unroll
+                    for (int b = 0; b < BC; ++b) {
+                        const float2 f0 = sm.f[w][t * BC + b], f1 = sm.f[w][(t + 1) * BC + b];
+                        er[i][b] = fmaf(f0.x, c0, er[i][b]);
+                        ei[i][b] = fmaf(f0.y, c0, ei[i][b]);
+                        orr[i][b] = fmaf(f1.x, c1, orr[i][b]);
+                        oi[i][b] = fmaf(f1.y, c1, oi[i][b]);
+                    }
+                }
+            }
+        }
+    }
 #pragma unroll
     for (int i = 0; i < LPT; ++i)
 #pragma unroll
-        for (int b = 0; b < BC; ++b) er[i][b] = ei[i][b] = orr[i][b] = oi[i][b] = T(0);
-
-    // adjoint of analysis: synthesis of b / c_m
-    const T insc = (op == OP_ANALYS_ADJ && m > 0) ? T(0.5) : T(1);
-    const T2 *spec2 = reinterpret_cast<const T2 *>(spec);
-
-    int gf[LPT];
-    const int wfirst = group_first_live<T, LPT>(pv, m, p, gf);
-    if (threadIdx.x == 0) *s_first = 0xffff;
+        for (int b = 0; b < BC; ++b)
+            sm.sum[w][(b * LPT + i) * 32 + lane] = make_float4(er[i][b], ei[i][b], orr[i][b], oi[i][b]);
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) atomicMin(s_first, wfirst);
-    __syncthreads();
-    const int start = min(*s_first * kSeedSeg, L);
-
-    for (int n0 = start; n0 < L; n0 += NCH) {
-        const int cnt = min(NCH, L - n0);
-        __syncthreads();
-        for (int t = threadIdx.x; t < NCH; t += NT) {
-            T2 ab;
-            ab.x = T(0); ab.y = T(0);
-            if (t < cnt) ab = pv.ab[col + n0 + t];
-            s_ab[t] = ab;
+    float4 *eo4 = reinterpret_cast<float4 *>(eo);
+    for (int q = threadIdx.x; q < LPT * 32 * BC; q += 32 * kWarps) {
+        const int b = q / (LPT * 32), pp = pb * LPT * 32 + q % (LPT * 32);
+        if (b0 + b >= batch || pp >= npairs) continue;
+        float4 v = sm.sum[0][q];
 #pragma unroll
-            for (int b = 0; b < BC; ++b) {
-                T2 f;
-                f.x = T(0); f.y = T(0);
-                if (t < cnt && b0 + b < batch) {
-                    f = spec2[(size_t)(b0 + b) * pv.nlm + col + n0 + t];
-                    f.x *= insc;
-                    f.y = (m == 0) ? T(0) : f.y * insc;
-                }
-                s_f[t * BC + b] = f;
-            }
+        for (int u = 1; u < kWarps; ++u) {
+            const float4 z = sm.sum[u][q];
+            v.x += z.x; v.y += z.y; v.z += z.z; v.w += z.w;
         }
-        __syncthreads();
-        for (int s0 = 0; s0 < cnt; s0 += kSeedSeg) {
-            const unsigned gl = live_groups<LPT>(gf, (n0 + s0) / kSeedSeg);
-            if (gl == 0) continue;   // no live pair in this warp yet
-            reseed<T, LPT>(pv, m, (n0 + s0) / kSeedSeg, p, y1, y2, k);
-            const int s1 = min(cnt, s0 + kSeedSeg);
-            const bool scaled = __any_sync(kFull, kmax_of<T, LPT>(k) > 0);
-            if (!scaled) {
-                for (int t = s0; t < s1; t += 2) {
-                    T2 ab = s_ab[t];
-                    rec_step<T, LPT, false>(ab.x, ab.y, x, y1, y2, k, c, gl);
-#pragma unroll
-                    for (int b = 0; b < BC; ++b) {
-                        const T2 f = s_f[t * BC + b];
-#pragma unroll
-                        for (int i = 0; i < LPT; ++i) {
-                            if (!((gl >> i) & 1)) continue;
-                            er[i][b] = fma(f.x, c[i], er[i][b]);
-                            ei[i][b] = fma(f.y, c[i], ei[i][b]);
-                        }
-                    }
-                    ab = s_ab[t + 1];
-                    rec_step<T, LPT, false>(ab.x, ab.y, x, y1, y2, k, c, gl);
-#pragma unroll
-                    for (int b = 0; b < BC; ++b) {
-                        const T2 f = s_f[(t + 1) * BC + b];
-#pragma unroll
-                        for (int i = 0; i < LPT; ++i) {
-                            if (!((gl >> i) & 1)) continue;
-                            orr[i][b] = fma(f.x, c[i], orr[i][b]);
-                            oi[i][b] = fma(f.y, c[i], oi[i][b]);
-                        }
-                    }
-                }
-            } else {
-                for (int t = s0; t < s1; t += 2) {
-                    T2 ab = s_ab[t];
-                    rec_step<T, LPT, true>(ab.x, ab.y, x, y1, y2, k, c, gl);
-                    if (__any_sync(kFull, kmin_of<T, LPT>(k) == 0)) {
-#pragma unroll
-                        for (int b = 0; b < BC; ++b) {
-                            const T2 f = s_f[t * BC + b];
-#pragma unroll
-                            for (int i = 0; i < LPT; ++i) {
-                                if (!((gl >> i) & 1)) continue;
-                                er[i][b] = fma(f.x, c[i], er[i][b]);
-                                ei[i][b] = fma(f.y, c[i], ei[i][b]);
-                            }
-                        }
-                    }
-                    ab = s_ab[t + 1];
-                    rec_step<T, LPT, true>(ab.x, ab.y, x, y1, y2, k, c, gl);
-                    if (__any_sync(kFull, kmin_of<T, LPT>(k) == 0)) {
-#pragma unroll
-                        for (int b = 0; b < BC; ++b) {
-                            const T2 f = s_f[(t + 1) * BC + b];
-#pragma unroll
-                            for (int i = 0; i < LPT; ++i) {
-                                if (!((gl >> i) & 1)) continue;
-                                orr[i][b] = fma(f.x, c[i], orr[i][b]);
-                                oi[i][b] = fma(f.y, c[i], oi[i][b]);
-                            }
-                        }
-                    }
-                }
-            }
-        }
-    }
-
-    T2 *eo2 = reinterpret_cast<T2 *>(eo);
-#pragma unroll
-    for (int i = 0; i < LPT; ++i) {
-        if (p[i] >= npairs) continue;
-#pragma unroll
-        for (int b = 0; b < BC; ++b) {
-            if (b0 + b >= batch) continue;
-            const size_t o = (((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + p[i]) * 2;
-            T2 e, d;
-            e.x = er[i][b]; e.y = ei[i][b];
-            d.x = orr[i][b]; d.y = oi[i][b];
-            eo2[o] = e;
-            eo2[o + 1] = d;
-        }
+        eo4[((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + pp] = v;
     }
 }
 
-template <typename T, int LPT, int BC, int NT>
-__global__ void __launch_bounds__(NT)
-k_synth(PlanView<T> pv, const T *__restrict__ spec, T *__restrict__ eo, int batch, int npb, int op)
+// blockIdx.x = (m, pair block), heaviest m first; blockIdx.y = field chunk.
+template <int LPT, int BC>
+__global__ void __launch_bounds__(32 * kWarps)
+k_synth(PlanView<float> pv, const float *__restrict__ spec, float *__restrict__ eo, int batch, int npb, int op)
 {
-    using T2 = typename Vec2<T>::type;
-    __shared__ T2 s_ab[kSynthNch];
-    __shared__ T2 s_f[kSynthNch * BC];
-    __shared__ int s_first;
-    const int m = blockIdx.x / npb;
-    const int pb = blockIdx.x - m * npb;
-    synth_tile<T, LPT, BC, NT>(pv, spec, eo, batch, m, pb, blockIdx.y * BC, op, s_ab, s_f, &s_first);
+    __shared__ SynthSmem<LPT, BC> sm;
+    const int m = blockIdx.x / npb, pb = blockIdx.x - m * npb;
+    synth_tile<LPT, BC>(pv, spec, eo, batch, m, pb, blockIdx.y * BC, op, sm);
+}
+
+// First group of 32 pairs with a live pair in segment `seg` (the group count if
+// there is none), warp-uniform.  glive: first live segment of each group.
+__device__ __forceinline__ int first_live_group(const unsigned short *__restrict__ glive, int ng, int seg, int lane)
+{
+    for (int gb = 0; gb < ng; gb += 32) {
+        const bool lv = gb + lane < ng && (int)glive[gb + lane] <= seg;
+        const unsigned mk = __ballot_sync(kFull, lv);
+        if (mk) return gb + __ffs(mk) - 1;
+    }
+    return ng;
 }
 
 // ---------------------------------------------------------------------------
-// Scalar analysis.  grid.x = m (heaviest first), grid.y = field chunk; the CTA
-// covers all latitude pairs (NT * LPT >= npairs).
+// Analysis of one segment of order m by one warp, over all latitude pairs, BC
+// fields.  A lane takes the pairs lane, lane + 32, ... one after the other: it
+// restarts the recurrence and adds P_n (s or d) into one accumulator per
+// degree, field and part, 64 BC of them; one butterfly at the end sums them
+// over the lanes and leaves lane t the sums of degree t.  Per degree and pair 3
+// instructions of recurrence, 2 BC of sums and half a load of (a, b); the
+// butterfly (~4 instructions per accumulator) is shared by all pairs.  States and
+// folds come kRing pairs ahead by asynchronous copies into slots of the lane's
+// own (the accumulators leave 12 warps per SM, too few to cover a DRAM access
+// with one pair's sums).  Pairs come in a fixed order, so results are bitwise
+// reproducible.  N = 2047, 2 fields: 560 us (issue 67 %) against 2106 with a CTA
+// per order that reduced over its lanes and warps every 8 degrees; the same form
+// with plain loads one pair ahead took 1536.  N = 383, 3-fold, 6 fields: 89 -> 14 us.
 // ---------------------------------------------------------------------------
-constexpr int kAnalysNch = 128;  // degrees staged per chunk (scalar analysis)
-static_assert(kAnalysNch % kSeedSeg == 0 && kSeedSeg % 16 == 0, "restart segments must align with the chunks");
+constexpr int kRing = 4;
 
-// One (order m, field chunk b0) tile of the scalar analysis, run by the whole
-// CTA (blockDim.x * LPT >= npairs, at most 8 warps); s_ab[kAnalysNch] and
-// s_red[8 * 32] are the CTA's buffers.
-template <typename T, int LPT, int BC>
-__device__ __forceinline__ void analys_tile(const PlanView<T> &pv, const T *__restrict__ sd, T *__restrict__ spec,
-                                            int batch, int m, int b0, int op, typename Vec2<T>::type *s_ab,
-                                            T (*s_red)[32])
+template <int BC>
+struct AnalysSmem {
+    float4 ab[kSeedSeg / 2];          // (a, b) of two degrees
+    float4 ring[kRing][1 + BC][32];   // state; folds (s, d) of each field
+};
+
+template <int BC>
+__device__ __forceinline__ void analys_segment(const PlanView<float> &pv, const float *__restrict__ sd,
+                                               float *__restrict__ spec, int batch, int m, int seg, int b0, int op,
+                                               AnalysSmem<BC> &sm)
 {
-    using T2 = typename Vec2<T>::type;
-    constexpr int K = 16 / BC;   // degrees per reduction: 2*K*BC = 32 values
-    constexpr int NCH = kAnalysNch;  // multiple of K
+    constexpr int C = 2 * BC;
+    const int lane = threadIdx.x & 31;
+    const int npairs = pv.npairs, ng = groups_of(npairs);
+    const int L = pv.lmax - m * pv.mres + 1;
+    const int n0 = seg * kSeedSeg, cnt = min(kSeedSeg, L - n0);
+    const long col = col_of_mres(pv.lmax, m, pv.mres) + n0;
+    const float4 *sd4 = reinterpret_cast<const float4 *>(sd) + ((size_t)b0 * (pv.mmax + 1) + m) * npairs;
+    const size_t fstride = (size_t)(pv.mmax + 1) * npairs;
 
-    const int NT = blockDim.x;
-    const int nw = NT >> 5;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int lmax = pv.lmax, npairs = pv.npairs;
-    const int L = lmax - m * pv.mres + 1;   // order index m is the order m mres
-    const long col = col_of_mres(lmax, m, pv.mres);
+    const int g0 = first_live_group(pv.glive + (size_t)m * ng, ng, seg, lane);
+    // the next pair to fetch (pointers stop at the lane's last pair) and its slot
+    int p = g0 * 32 + lane, slot = 0;
+    const int q0 = min(p, npairs - 1), nb = min(BC, batch - b0);
+    const float4 *ps = pv.seeds + (pv.segoff[m] + seg) * npairs + q0, *pf = sd4 + q0;
+    const float *px = pv.x + q0;
+    const auto fetch = [&]() {   // one group of copies per call, also past the last pair
+        const bool in = p < npairs;
+        cp_async16(&sm.ring[slot][0][lane], ps, in);
+#pragma unroll
+        for (int b = 0; b < BC; ++b) cp_async16(&sm.ring[slot][1 + b][lane], pf + (b < nb ? b * fstride : 0), in && b < nb);
+        cp_async_commit();
+        p += 32;
+        slot = (slot + 1) & (kRing - 1);
+        const int step = p < npairs ? 32 : 0;
+        ps += step;
+        pf += step;
+    };
+#pragma unroll
+    for (int u = 0; u < kRing - 1; ++u) fetch();
+    __syncwarp();   // the last segment is done with sm.ab
+    reinterpret_cast<float2 *>(sm.ab)[lane] = lane < cnt ? __ldg(pv.ab + col + lane) : make_float2(0.f, 0.f);
+    __syncwarp();
 
-    T x[LPT], y1[LPT], y2[LPT], c[LPT];
-    int k[LPT], p[LPT];
-    T2 sv[LPT][BC], dv[LPT][BC];
-    const T2 *sd2 = reinterpret_cast<const T2 *>(sd);
+    float acc[kSeedSeg * C];
 #pragma unroll
-    for (int i = 0; i < LPT; ++i) {
-        p[i] = i * NT + threadIdx.x;
-        const bool v = p[i] < npairs;
-        const size_t o = (size_t)m * npairs + p[i];
-        x[i] = v ? pv.x[p[i]] : T(0);
-        y2[i] = v ? pv.pmm[o] : T(0);
-        k[i] = v ? pv.pmmk[o] : 0;
-        y1[i] = T(0);
+    for (int q = 0; q < kSeedSeg * C; ++q) acc[q] = 0.f;
+#pragma unroll 1
+    for (int g = g0; g < ng; ++g) {
+        const float x = __ldg(px);
+        px += (g + 1) * 32 + lane < npairs ? 32 : 0;
+        cp_async_wait<kRing - 2>();
+        const float4 (&r)[1 + BC][32] = sm.ring[(slot + 1) & (kRing - 1)];   // the oldest
+        const float4 st = r[0][lane];
+        float4 f[BC];
 #pragma unroll
-        for (int b = 0; b < BC; ++b) {
-            T2 z;
-            z.x = T(0); z.y = T(0);
-            sv[i][b] = z;
-            dv[i][b] = z;
-            if (v && b0 + b < batch) {
-                const size_t q = (((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + p[i]) * 2;
-                sv[i][b] = sd2[q];
-                dv[i][b] = sd2[q + 1];
+        for (int b = 0; b < BC; ++b) f[b] = r[1 + b][lane];
+        fetch();
+        float y1 = st.x, y2 = st.y;
+        if (__any_sync(kFull, st.z != 1.f)) {   // states stored scaled: the factor into the folds
+#pragma unroll
+            for (int b = 0; b < BC; ++b)
+                f[b] = make_float4(f[b].x * st.z, f[b].y * st.z, f[b].z * st.z, f[b].w * st.z);
+        }
+#pragma unroll
+        for (int tb = 0; tb < kSeedSeg; tb += 8) {
+            if (tb >= cnt) break;   // rows past cnt are zero
+#pragma unroll
+            for (int t = tb; t < tb + 8; t += 2) {
+                const float4 ab = sm.ab[t >> 1];
+                y2 = next_p(ab.x, ab.y, x, y1, y2);
+                y1 = next_p(ab.z, ab.w, x, y2, y1);
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    float *a = acc + t * C + 2 * b;
+                    a[0] = fmaf(y2, f[b].x, a[0]);
+                    a[1] = fmaf(y2, f[b].y, a[1]);
+                    a[C] = fmaf(y1, f[b].z, a[C]);
+                    a[C + 1] = fmaf(y1, f[b].w, a[C + 1]);
+                }
             }
         }
     }
-    // output scale: c_m for the adjoint of synthesis
-    const T outsc = (op == OP_SYNTH_ADJ && m > 0) ? T(2) : T(1);
-    T2 *spec2 = reinterpret_cast<T2 *>(spec);
-    int gf[LPT];
-    group_first_live<T, LPT>(pv, m, p, gf);
-
-    for (int n0 = 0; n0 < L; n0 += NCH) {
-        const int cnt = min(NCH, L - n0);
-        __syncthreads();
-        for (int t = threadIdx.x; t < NCH; t += NT) {
-            T2 ab;
-            ab.x = T(0); ab.y = T(0);
-            if (t < cnt) ab = pv.ab[col + n0 + t];
-            s_ab[t] = ab;
-        }
-        __syncthreads();
-        for (int t0 = 0; t0 < cnt; t0 += K) {
-            // static polar optimisation: groups of 32 pairs with no live pair
-            // in this segment run neither the recurrence nor the sums; a warp
-            // with none contributes zeros
-            const unsigned gl = live_groups<LPT>(gf, (n0 + t0) / kSeedSeg);
-            const bool wlive = gl != 0;
-            if (wlive && (n0 + t0) % kSeedSeg == 0) reseed<T, LPT>(pv, m, (n0 + t0) / kSeedSeg, p, y1, y2, k);
-            T acc[32];
+    cp_async_wait<0>();
+    warp_transpose_reduce<kSeedSeg * C>(acc, lane);
+    if (lane >= cnt) return;
+    const float outsc = (op == OP_SYNTH_ADJ && m > 0) ? 2.f : 1.f;   // c_m for the adjoint of synthesis
+    float2 *spec2 = reinterpret_cast<float2 *>(spec);
 #pragma unroll
-            for (int q = 0; q < 32; ++q) acc[q] = T(0);
-            const bool scaled = __any_sync(kFull, kmax_of<T, LPT>(k) > 0);
-            if (wlive) {
-#pragma unroll
-                for (int kx = 0; kx < K; ++kx) {
-                    const T2 ab = s_ab[t0 + kx];
-                    bool live = true;
-                    if (scaled) {
-                        rec_step<T, LPT, true>(ab.x, ab.y, x, y1, y2, k, c, gl);
-                        live = __any_sync(kFull, kmin_of<T, LPT>(k) == 0);
-                    } else {
-                        rec_step<T, LPT, false>(ab.x, ab.y, x, y1, y2, k, c, gl);
-                    }
-                    if (live) {
-#pragma unroll
-                        for (int b = 0; b < BC; ++b) {
-#pragma unroll
-                            for (int i = 0; i < LPT; ++i) {
-                                if (!((gl >> i) & 1)) continue;
-                                const T2 v = (kx & 1) ? dv[i][b] : sv[i][b];
-                                acc[(kx * BC + b) * 2] = fma(c[i], v.x, acc[(kx * BC + b) * 2]);
-                                acc[(kx * BC + b) * 2 + 1] = fma(c[i], v.y, acc[(kx * BC + b) * 2 + 1]);
-                            }
-                        }
-                    }
-                }
-                warp_transpose_reduce<T, 32>(acc, lane);
-            }
-            s_red[warp][lane] = acc[0];
-            __syncthreads();
-            if (threadIdx.x < 2 * K * BC) {
-                T tot = T(0);
-                for (int w = 0; w < nw; ++w) tot += s_red[w][threadIdx.x];
-                const int q = threadIdx.x;
-                const int kx = q / (2 * BC), b = (q >> 1) % BC, part = q & 1;
-                const int nn = n0 + t0 + kx;  // n - m
-                if (nn < L && b0 + b < batch) {
-                    T val = tot * outsc;
-                    if (m == 0 && part == 1) val = T(0);
-                    T *dst = reinterpret_cast<T *>(&spec2[(size_t)(b0 + b) * pv.nlm + col + nn]);
-                    dst[part] = val;
-                }
-            }
-            __syncthreads();
-        }
+    for (int b = 0; b < BC; ++b) {
+        if (b0 + b >= batch) break;
+        spec2[(size_t)(b0 + b) * pv.nlm + col + lane] =
+            make_float2(acc[2 * b] * outsc, m == 0 ? 0.f : acc[2 * b + 1] * outsc);
     }
 }
 
-template <typename T, int LPT, int BC>
-__global__ void __launch_bounds__(256)
-k_analys(PlanView<T> pv, const T *__restrict__ sd, T *__restrict__ spec, int batch, int op)
+// blockIdx: x four segments (a warp each; neighbours of one order share its
+// folds in L1), y order index, z field chunk.
+template <int BC>
+__global__ void __launch_bounds__(32 * kWarps)
+k_analys(PlanView<float> pv, const float *__restrict__ sd, float *__restrict__ spec, int batch, int op)
 {
-    using T2 = typename Vec2<T>::type;
-    __shared__ T2 s_ab[kAnalysNch];
-    __shared__ T s_red[8][32];
-    analys_tile<T, LPT, BC>(pv, sd, spec, batch, blockIdx.x, blockIdx.y * BC, op, s_ab, s_red);
+    __shared__ AnalysSmem<BC> sm[kWarps];
+    const int w = threadIdx.x >> 5, seg = blockIdx.x * kWarps + w, m = blockIdx.y;
+    if (seg * kSeedSeg > pv.lmax - m * pv.mres) return;
+    analys_segment<BC>(pv, sd, spec, batch, m, seg, blockIdx.z * BC, op, sm[w]);
 }
 
 // ---------------------------------------------------------------------------
 // Vector synthesis.  With dP = sin(theta) dP/dtheta = n x P_n - dc_n P_{n-1}:
 //   sin * V_theta,m = sum [S dP - i m T P],   sin * V_phi,m = sum [i m S P + T dP].
-// dP has the opposite mirror parity of P.  Outputs E/O for theta and phi.
+// dP has the opposite mirror parity of P, so a degree with n - m even adds its
+// P terms to E and its dP terms to O, an odd one the other way round: four
+// complex sums per pair and field (theta and phi, E and O), the factors -i m and
+// i m taken into the spectral values.  CTA and warps as in the scalar synthesis;
+// a group of 32 pairs is left out of the segments in which none of its values
+// reaches 2^-70.  Per degree and pair 6 instructions for P and dP and 8 per
+// field; N = 511, 8 fields: 193 -> 144 us (issue 63 %, FMA pipe 46 %).
 // ---------------------------------------------------------------------------
-template <typename T, int LPT, int BC, int NT>
-__global__ void __launch_bounds__(NT)
-k_synth_vec(PlanView<T> pv, const T *__restrict__ Sg, const T *__restrict__ Tg, T *__restrict__ eot,
-            T *__restrict__ eop, int batch, int npb, int op)
+template <int LPT, int BC>
+struct SynthVecSmem {
+    float4 rec[kWarps][kSeedSeg];                   // (a, b, dc, n)
+    float4 f[kWarps][kSeedSeg * BC][2];             // [degree][field] (S, T), (-i m T, i m S)
+    float4 sum[kWarps][LPT * 32 * BC];              // [pair][field] (E, O) of one component
+};
+
+// P and dP of the degree of r.
+__device__ __forceinline__ void vec_step(const float4 &r, float x, float &y1, float &y2, float &c, float &cd)
 {
-    using T2 = typename Vec2<T>::type;
-    constexpr int NCH = 64;
-    __shared__ T2 s_ab[NCH];
-    __shared__ T s_dc[NCH];
-    __shared__ T2 s_S[NCH * BC];
-    __shared__ T2 s_T[NCH * BC];
+    c = next_p(r.x, r.y, x, y1, y2);
+    y2 = y1;
+    y1 = c;
+    cd = fmaf(r.w * x, y1, -r.z * y2);
+}
 
-    const int m = blockIdx.x / npb;
-    const int pb = blockIdx.x - m * npb;
-    const int b0 = blockIdx.y * BC;
-    const int lmax = pv.lmax, npairs = pv.npairs;
-    const int L = lmax - m * pv.mres + 1;   // order index m is the order m mres
-    const long col = col_of_mres(lmax, m, pv.mres);
+// Adds one degree of one field to a pair's sums: P terms to the component of
+// the degree's parity, dP terms to the other.
+template <bool ODD>
+__device__ __forceinline__ void vec_add(const float4 (&f)[2], float c, float cd, float (&te)[2], float (&to)[2],
+                                        float (&pe)[2], float (&po)[2])
+{
+    float (&tp)[2] = ODD ? to : te, (&td)[2] = ODD ? te : to;
+    float (&pp)[2] = ODD ? po : pe, (&pd)[2] = ODD ? pe : po;
+    tp[0] = fmaf(f[1].x, c, tp[0]);
+    tp[1] = fmaf(f[1].y, c, tp[1]);
+    pp[0] = fmaf(f[1].z, c, pp[0]);
+    pp[1] = fmaf(f[1].w, c, pp[1]);
+    td[0] = fmaf(f[0].x, cd, td[0]);
+    td[1] = fmaf(f[0].y, cd, td[1]);
+    pd[0] = fmaf(f[0].z, cd, pd[0]);
+    pd[1] = fmaf(f[0].w, cd, pd[1]);
+}
 
-    T x[LPT], y1[LPT], y2[LPT], c[LPT];
-    int k[LPT], p[LPT];
+template <int LPT, int BC>
+__global__ void __launch_bounds__(32 * kWarps)
+k_synth_vec(PlanView<float> pv, const float *__restrict__ Sg, const float *__restrict__ Tg, float *__restrict__ eot,
+            float *__restrict__ eop, int batch, int npb, int op)
+{
+    __shared__ SynthVecSmem<LPT, BC> sm;
+    const int m = blockIdx.x / npb, pb = blockIdx.x - m * npb, b0 = blockIdx.y * BC;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int npairs = pv.npairs, ng = groups_of(npairs);
+    const int L = pv.lmax - m * pv.mres + 1;
+    const int nseg = (L + kSeedSeg - 1) / kSeedSeg;
+    const long col = col_of_mres(pv.lmax, m, pv.mres);
+    const float2 *S2 = reinterpret_cast<const float2 *>(Sg), *T2 = reinterpret_cast<const float2 *>(Tg);
+    const float cadj = (op == OP_ANALYS_ADJ && m > 0) ? 0.5f : 1.f, fm = (float)(m * pv.mres);
+
+    int p[LPT], gf[LPT], first = 0xffff;
+    float x[LPT], te[LPT][BC][2], to[LPT][BC][2], pe[LPT][BC][2], po[LPT][BC][2];   // theta and phi, E and O
 #pragma unroll
     for (int i = 0; i < LPT; ++i) {
-        p[i] = pb * NT * LPT + i * NT + threadIdx.x;
-        const bool v = p[i] < npairs;
-        const size_t o = (size_t)m * npairs + p[i];
-        x[i] = v ? pv.x[p[i]] : T(0);
-        y2[i] = v ? pv.pmm[o] : T(0);
-        k[i] = v ? pv.pmmk[o] : 0;
-        y1[i] = T(0);
-    }
-    // accumulators [pair][field][8 complex]: A_e A_o B_e B_o C_e C_o D_e D_o
-    //   A: S dP, B: T P, C: S P, D: T dP; e/o = even/odd function of x
-    T acc[LPT][BC][16];
-#pragma unroll
-    for (int i = 0; i < LPT; ++i)
+        const int g = pb * LPT + i;
+        p[i] = g * 32 + lane;
+        x[i] = p[i] < npairs ? pv.x[p[i]] : 0.f;
+        gf[i] = g < ng ? (int)pv.glive_vec[(size_t)m * ng + g] : 0xffff;
+        first = min(first, gf[i]);
 #pragma unroll
         for (int b = 0; b < BC; ++b)
 #pragma unroll
-            for (int q = 0; q < 16; ++q) acc[i][b][q] = T(0);
-
-    const T2 *S2 = reinterpret_cast<const T2 *>(Sg);
-    const T2 *T2p = reinterpret_cast<const T2 *>(Tg);
-    const T cadj = (op == OP_ANALYS_ADJ && m > 0) ? T(0.5) : T(1);
-
-    for (int n0 = 0; n0 < L; n0 += NCH) {
-        const int cnt = min(NCH, L - n0);
-        __syncthreads();
-        for (int t = threadIdx.x; t < NCH; t += NT) {
-            T2 ab;
-            ab.x = T(0); ab.y = T(0);
-            T dcv = T(0);
-            if (t < cnt) { ab = pv.ab[col + n0 + t]; dcv = pv.dc[col + n0 + t]; }
-            s_ab[t] = ab;
-            s_dc[t] = dcv;
-            const int n = m * pv.mres + n0 + t;
-            // adjoint of analysis: b / (c_m n(n+1)), nothing at n = 0
-            T sc = T(1);
-            if (op == OP_ANALYS_ADJ) sc = (n == 0) ? T(0) : cadj / (T(n) * T(n + 1));
+            for (int q = 0; q < 2; ++q) te[i][b][q] = to[i][b][q] = pe[i][b][q] = po[i][b][q] = 0.f;
+    }
+    for (int seg = first + ((w - first) & (kWarps - 1)); seg < nseg; seg += kWarps) {
+        const int cnt = min(kSeedSeg, L - seg * kSeedSeg), t0 = seg * kSeedSeg + lane, n = m * pv.mres + t0;
+        float y1[LPT], y2[LPT], fac[LPT];
+        bool all = true, scaled = false;
 #pragma unroll
-            for (int b = 0; b < BC; ++b) {
-                T2 fs, ft;
-                fs.x = fs.y = ft.x = ft.y = T(0);
-                if (t < cnt && b0 + b < batch) {
-                    fs = S2[(size_t)(b0 + b) * pv.nlm + col + n0 + t];
-                    ft = T2p[(size_t)(b0 + b) * pv.nlm + col + n0 + t];
-                    fs.x *= sc; fs.y = (m == 0) ? T(0) : fs.y * sc;
-                    ft.x *= sc; ft.y = (m == 0) ? T(0) : ft.y * sc;
-                }
-                s_S[t * BC + b] = fs;
-                s_T[t * BC + b] = ft;
-            }
+        for (int i = 0; i < LPT; ++i) {
+            const float4 s = p[i] < npairs ? __ldg(pv.seeds + (pv.segoff[m] + seg) * npairs + p[i])
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+            y1[i] = s.x;
+            y2[i] = s.y;
+            fac[i] = s.z;
+            all = all && seg >= gf[i];
+            scaled = scaled || (fac[i] != 1.f && p[i] < npairs);
         }
-        __syncthreads();
-        bool scaled = false;
-        for (int t = 0; t < cnt; t += 2) {
-            if (t % kSeedSeg == 0) {
-                if constexpr (sizeof(T) == sizeof(float)) reseed<T, LPT>(pv, m, (n0 + t) / kSeedSeg, p, y1, y2, k);
-                scaled = __any_sync(kFull, kmax_of<T, LPT>(k) > 0);
+        __syncwarp();
+        float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (lane < cnt) {
+            const float2 ab = __ldg(pv.ab + col + t0);
+            r = make_float4(ab.x, ab.y, __ldg(pv.dc + col + t0), (float)n);
+        }
+        sm.rec[w][lane] = r;
+        // adjoint of analysis: b / (c_m n(n+1)), nothing at n = 0
+        float sc = 1.f;
+        if (op == OP_ANALYS_ADJ) sc = (n == 0) ? 0.f : cadj / ((float)n * (float)(n + 1));
+#pragma unroll
+        for (int b = 0; b < BC; ++b) {
+            float2 s = make_float2(0.f, 0.f), t = s;
+            if (lane < cnt && b0 + b < batch) {
+                s = __ldg(S2 + (size_t)(b0 + b) * pv.nlm + col + t0);
+                t = __ldg(T2 + (size_t)(b0 + b) * pv.nlm + col + t0);
+                s = make_float2(s.x * sc, m == 0 ? 0.f : s.y * sc);
+                t = make_float2(t.x * sc, m == 0 ? 0.f : t.y * sc);
             }
+            sm.f[w][lane * BC + b][0] = make_float4(s.x, s.y, t.x, t.y);
+            sm.f[w][lane * BC + b][1] = make_float4(fm * t.y, -fm * t.x, -fm * s.y, fm * s.x);
+        }
+        __syncwarp();
+        if (all && !__any_sync(kFull, scaled)) {
+#pragma unroll 1
+            for (int tb = 0; tb < cnt; tb += 4)   // rows past cnt are zero
 #pragma unroll
-            for (int par = 0; par < 2; ++par) {
-                const int tt = t + par;
-                const T2 ab = s_ab[tt];
-                const T dcn = s_dc[tt];
-                const T nf = T(m * pv.mres + n0 + tt);
-                bool live = true;
-                if (scaled) {
-                    rec_step<T, LPT, true>(ab.x, ab.y, x, y1, y2, k, c);
-                    live = __any_sync(kFull, kmin_of<T, LPT>(k) == 0);
-                } else {
-                    rec_step<T, LPT, false>(ab.x, ab.y, x, y1, y2, k, c);
-                }
-                if (!live) continue;
-                T cd[LPT];
+            for (int t = tb; t < tb + 4; t += 2) {
+                float c[LPT], cd[LPT];
 #pragma unroll
-                for (int i = 0; i < LPT; ++i) {
-                    // dP = n x P_n - dc_n P_{n-1}; zero whenever P itself is dropped
-                    const T dpv = fma(nf * x[i], y1[i], -dcn * y2[i]);
-                    cd[i] = (scaled && k[i] > 0) ? T(0) : dpv;
-                }
+                for (int i = 0; i < LPT; ++i) vec_step(sm.rec[w][t], x[i], y1[i], y2[i], c[i], cd[i]);
 #pragma unroll
-                for (int b = 0; b < BC; ++b) {
-                    const T2 fs = s_S[tt * BC + b];
-                    const T2 ft = s_T[tt * BC + b];
+                for (int b = 0; b < BC; ++b)
 #pragma unroll
-                    for (int i = 0; i < LPT; ++i) {
-                        // n-m even (par 0): P even, dP odd.  n-m odd: P odd, dP even.
-                        const int iA = par == 0 ? 2 : 0;   // A_o : A_e
-                        const int iB = par == 0 ? 4 : 6;   // B_e : B_o
-                        const int iC = par == 0 ? 8 : 10;  // C_e : C_o
-                        const int iD = par == 0 ? 14 : 12; // D_o : D_e
-                        acc[i][b][iA] = fma(fs.x, cd[i], acc[i][b][iA]);
-                        acc[i][b][iA + 1] = fma(fs.y, cd[i], acc[i][b][iA + 1]);
-                        acc[i][b][iB] = fma(ft.x, c[i], acc[i][b][iB]);
-                        acc[i][b][iB + 1] = fma(ft.y, c[i], acc[i][b][iB + 1]);
-                        acc[i][b][iC] = fma(fs.x, c[i], acc[i][b][iC]);
-                        acc[i][b][iC + 1] = fma(fs.y, c[i], acc[i][b][iC + 1]);
-                        acc[i][b][iD] = fma(ft.x, cd[i], acc[i][b][iD]);
-                        acc[i][b][iD + 1] = fma(ft.y, cd[i], acc[i][b][iD + 1]);
-                    }
+                    for (int i = 0; i < LPT; ++i)
+                        vec_add<false>(sm.f[w][t * BC + b], c[i], cd[i], te[i][b], to[i][b], pe[i][b], po[i][b]);
+#pragma unroll
+                for (int i = 0; i < LPT; ++i) vec_step(sm.rec[w][t + 1], x[i], y1[i], y2[i], c[i], cd[i]);
+#pragma unroll
+                for (int b = 0; b < BC; ++b)
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i)
+                        vec_add<true>(sm.f[w][(t + 1) * BC + b], c[i], cd[i], te[i][b], to[i][b], pe[i][b], po[i][b]);
+            }
+        } else {
+            // a group not live yet, or a pair whose state is stored scaled
+#pragma unroll
+            for (int i = 0; i < LPT; ++i) {
+                if (seg < gf[i]) continue;
+                for (int t = 0; t < cnt; t += 2) {
+                    float c, cd;
+                    vec_step(sm.rec[w][t], x[i], y1[i], y2[i], c, cd);
+                    c *= fac[i];
+                    cd *= fac[i];
+#pragma unroll
+                    for (int b = 0; b < BC; ++b)
+                        vec_add<false>(sm.f[w][t * BC + b], c, cd, te[i][b], to[i][b], pe[i][b], po[i][b]);
+                    vec_step(sm.rec[w][t + 1], x[i], y1[i], y2[i], c, cd);
+                    c *= fac[i];
+                    cd *= fac[i];
+#pragma unroll
+                    for (int b = 0; b < BC; ++b)
+                        vec_add<true>(sm.f[w][(t + 1) * BC + b], c, cd, te[i][b], to[i][b], pe[i][b], po[i][b]);
                 }
             }
         }
     }
-
-    T2 *eot2 = reinterpret_cast<T2 *>(eot);
-    T2 *eop2 = reinterpret_cast<T2 *>(eop);
-    const T fm = T(m * pv.mres);
+    // the warps' sums, theta then phi, divided by sin(theta)
 #pragma unroll
-    for (int i = 0; i < LPT; ++i) {
-        if (p[i] >= npairs) continue;
-        const T is = T(1) / pv.st[p[i]];
+    for (int comp = 0; comp < 2; ++comp) {
+        __syncthreads();
 #pragma unroll
-        for (int b = 0; b < BC; ++b) {
-            if (b0 + b >= batch) continue;
-            const T *a = acc[i][b];
-            const size_t o = (((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + p[i]) * 2;
-            T2 v;
-            // theta: (A - i m B) / sin ; E uses A_e,B_e ; O uses A_o,B_o
-            v.x = (a[0] + fm * a[5]) * is; v.y = (a[1] - fm * a[4]) * is; eot2[o] = v;
-            v.x = (a[2] + fm * a[7]) * is; v.y = (a[3] - fm * a[6]) * is; eot2[o + 1] = v;
-            // phi: (i m C + D) / sin ; E uses C_e,D_e ; O uses C_o,D_o
-            v.x = (a[12] - fm * a[9]) * is; v.y = (a[13] + fm * a[8]) * is; eop2[o] = v;
-            v.x = (a[14] - fm * a[11]) * is; v.y = (a[15] + fm * a[10]) * is; eop2[o + 1] = v;
+        for (int i = 0; i < LPT; ++i)
+#pragma unroll
+            for (int b = 0; b < BC; ++b)
+                sm.sum[w][(b * LPT + i) * 32 + lane] =
+                    comp == 0 ? make_float4(te[i][b][0], te[i][b][1], to[i][b][0], to[i][b][1])
+                              : make_float4(pe[i][b][0], pe[i][b][1], po[i][b][0], po[i][b][1]);
+        __syncthreads();
+        float4 *eo4 = reinterpret_cast<float4 *>(comp == 0 ? eot : eop);
+        for (int q = threadIdx.x; q < LPT * 32 * BC; q += 32 * kWarps) {
+            const int b = q / (LPT * 32), pp = pb * LPT * 32 + q % (LPT * 32);
+            if (b0 + b >= batch || pp >= npairs) continue;
+            const float is = 1.f / pv.st[pp];
+            float4 v = sm.sum[0][q];
+#pragma unroll
+            for (int u = 1; u < kWarps; ++u) {
+                const float4 z = sm.sum[u][q];
+                v.x += z.x; v.y += z.y; v.z += z.z; v.w += z.w;
+            }
+            eo4[((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + pp] =
+                make_float4(v.x * is, v.y * is, v.z * is, v.w * is);
         }
     }
 }
@@ -641,265 +581,198 @@ k_synth_vec(PlanView<T> pv, const T *__restrict__ Sg, const T *__restrict__ Tg, 
 // Vector analysis.  With folds s/d of (w/sin) V_theta and V_phi:
 //   S_n = sum [dP * fold(V_theta) - i m P * fold(V_phi)] / (n(n+1))
 //   T_n = sum [i m P * fold(V_theta) + dP * fold(V_phi)] / (n(n+1))
-// where the fold is s for an even function and d for an odd one.
+// where the fold is s for an even function and d for an odd one.  A warp per
+// segment and field, as in the scalar analysis: four accumulators per degree
+// (S and T), the folds times m beside the folds.  N = 511, 8 fields: 452 -> 215 us.
 // ---------------------------------------------------------------------------
-template <typename T, int LPT, int BC>
-__global__ void __launch_bounds__(256)
-k_analys_vec(PlanView<T> pv, const T *__restrict__ sdt, const T *__restrict__ sdp, T *__restrict__ So,
-             T *__restrict__ To, int batch, int op)
+struct AnalysVecSmem {
+    float4 rec[kSeedSeg];         // (a, b, dc, n)
+    float4 ring[kRing][3][32];    // state; folds (s, d) of theta and phi
+};
+
+__global__ void __launch_bounds__(32 * kWarps)
+k_analys_vec(PlanView<float> pv, const float *__restrict__ sdt, const float *__restrict__ sdp, float *__restrict__ So,
+             float *__restrict__ To, int op)
 {
-    using T2 = typename Vec2<T>::type;
-    constexpr int K = 4 / BC;    // degrees per reduction: 8*K*BC = 32 values
-    constexpr int NCH = 64;      // multiple of K
-    static_assert(K % 2 == 0, "K must be even so that kx carries the parity of n - m");
-    __shared__ T2 s_ab[NCH];
-    __shared__ T s_dc[NCH];
-    __shared__ T s_red[8][32];
-
-    const int NT = blockDim.x;
-    const int nw = NT >> 5;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m = blockIdx.x;
-    const int b0 = blockIdx.y * BC;
-    const int lmax = pv.lmax, npairs = pv.npairs;
-    const int L = lmax - m * pv.mres + 1;   // order index m is the order m mres
-    const long col = col_of_mres(lmax, m, pv.mres);
-
-    T x[LPT], y1[LPT], y2[LPT], c[LPT];
-    int k[LPT], p[LPT];
-    T2 st_[LPT][BC], dt_[LPT][BC], sp_[LPT][BC], dp_[LPT][BC];
-    const T2 *sdt2 = reinterpret_cast<const T2 *>(sdt);
-    const T2 *sdp2 = reinterpret_cast<const T2 *>(sdp);
+    __shared__ AnalysVecSmem s_sm[kWarps];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int seg = blockIdx.x * kWarps + w, m = blockIdx.y, b = blockIdx.z;
+    const int npairs = pv.npairs, ng = groups_of(npairs);
+    const int L = pv.lmax - m * pv.mres + 1;
+    const int n0 = seg * kSeedSeg;
+    if (n0 >= L) return;
+    AnalysVecSmem &sm = s_sm[w];
+    const int cnt = min(kSeedSeg, L - n0), n = m * pv.mres + n0 + lane;
+    const long col = col_of_mres(pv.lmax, m, pv.mres) + n0;
+    const float fm = (float)(m * pv.mres);
+    const int g0 = first_live_group(pv.glive_vec + (size_t)m * ng, ng, seg, lane);
+    int p = g0 * 32 + lane, slot = 0;   // as in analys_segment
+    const int q0 = min(p, npairs - 1);
+    const float4 *ps = pv.seeds + (pv.segoff[m] + seg) * npairs + q0;
+    const size_t fo = ((size_t)b * (pv.mmax + 1) + m) * npairs + q0;
+    const float4 *ft = reinterpret_cast<const float4 *>(sdt) + fo, *fp = reinterpret_cast<const float4 *>(sdp) + fo;
+    const float *px = pv.x + q0;
+    const auto fetch = [&]() {
+        const bool in = p < npairs;
+        cp_async16(&sm.ring[slot][0][lane], ps, in);
+        cp_async16(&sm.ring[slot][1][lane], ft, in);
+        cp_async16(&sm.ring[slot][2][lane], fp, in);
+        cp_async_commit();
+        p += 32;
+        slot = (slot + 1) & (kRing - 1);
+        const int step = p < npairs ? 32 : 0;
+        ps += step;
+        ft += step;
+        fp += step;
+    };
 #pragma unroll
-    for (int i = 0; i < LPT; ++i) {
-        p[i] = i * NT + threadIdx.x;
-        const bool v = p[i] < npairs;
-        const size_t o = (size_t)m * npairs + p[i];
-        x[i] = v ? pv.x[p[i]] : T(0);
-        y2[i] = v ? pv.pmm[o] : T(0);
-        k[i] = v ? pv.pmmk[o] : 0;
-        y1[i] = T(0);
+    for (int u = 0; u < kRing - 1; ++u) fetch();
+    {
+        float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (lane < cnt) {
+            const float2 ab = __ldg(pv.ab + col + lane);
+            r = make_float4(ab.x, ab.y, __ldg(pv.dc + col + lane), (float)n);
+        }
+        sm.rec[lane] = r;
+    }
+    __syncwarp();
+
+    float acc[kSeedSeg * 4];   // per degree: S, T
 #pragma unroll
-        for (int b = 0; b < BC; ++b) {
-            T2 z;
-            z.x = T(0); z.y = T(0);
-            st_[i][b] = dt_[i][b] = sp_[i][b] = dp_[i][b] = z;
-            if (v && b0 + b < batch) {
-                const size_t q = (((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + p[i]) * 2;
-                st_[i][b] = sdt2[q];
-                dt_[i][b] = sdt2[q + 1];
-                sp_[i][b] = sdp2[q];
-                dp_[i][b] = sdp2[q + 1];
+    for (int q = 0; q < kSeedSeg * 4; ++q) acc[q] = 0.f;
+#pragma unroll 1
+    for (int g = g0; g < ng; ++g) {
+        const float x = __ldg(px);
+        px += (g + 1) * 32 + lane < npairs ? 32 : 0;
+        cp_async_wait<kRing - 2>();
+        const float4 (&r)[3][32] = sm.ring[(slot + 1) & (kRing - 1)];   // the oldest
+        const float4 st = r[0][lane];
+        float4 vt = r[1][lane], vp = r[2][lane];   // (s, d) of theta and phi
+        fetch();
+        float y1 = st.x, y2 = st.y;
+        if (__any_sync(kFull, st.z != 1.f)) {   // states stored scaled: the factor into the folds
+            vt = make_float4(vt.x * st.z, vt.y * st.z, vt.z * st.z, vt.w * st.z);
+            vp = make_float4(vp.x * st.z, vp.y * st.z, vp.z * st.z, vp.w * st.z);
+        }
+        const float4 mt = make_float4(fm * vt.x, fm * vt.y, fm * vt.z, fm * vt.w);
+        const float4 mp = make_float4(fm * vp.x, fm * vp.y, fm * vp.z, fm * vp.w);
+#pragma unroll
+        for (int tb = 0; tb < kSeedSeg; tb += 8) {
+            if (tb >= cnt) break;   // rows past cnt are zero
+#pragma unroll
+            for (int t = tb; t < tb + 8; ++t) {
+                float c, cd;
+                vec_step(sm.rec[t], x, y1, y2, c, cd);
+                // n - m even: P even -> s folds, dP odd -> d folds; odd: the other way round
+                const bool odd = t & 1;
+                float *a = acc + 4 * t;
+                a[0] = fmaf(cd, odd ? vt.x : vt.z, fmaf(c, odd ? mp.w : mp.y, a[0]));
+                a[1] = fmaf(cd, odd ? vt.y : vt.w, fmaf(-c, odd ? mp.z : mp.x, a[1]));
+                a[2] = fmaf(cd, odd ? vp.x : vp.z, fmaf(-c, odd ? mt.w : mt.y, a[2]));
+                a[3] = fmaf(cd, odd ? vp.y : vp.w, fmaf(c, odd ? mt.z : mt.x, a[3]));
             }
         }
     }
-    const T fm = T(m * pv.mres);
-    T2 *S2 = reinterpret_cast<T2 *>(So);
-    T2 *T2o = reinterpret_cast<T2 *>(To);
-
-    for (int n0 = 0; n0 < L; n0 += NCH) {
-        const int cnt = min(NCH, L - n0);
-        __syncthreads();
-        for (int t = threadIdx.x; t < NCH; t += NT) {
-            T2 ab;
-            ab.x = T(0); ab.y = T(0);
-            T dcv = T(0);
-            if (t < cnt) { ab = pv.ab[col + n0 + t]; dcv = pv.dc[col + n0 + t]; }
-            s_ab[t] = ab;
-            s_dc[t] = dcv;
-        }
-        __syncthreads();
-        for (int t0 = 0; t0 < cnt; t0 += K) {
-            if (sizeof(T) == sizeof(float) && (n0 + t0) % kSeedSeg == 0)
-                reseed<T, LPT>(pv, m, (n0 + t0) / kSeedSeg, p, y1, y2, k);
-            // per (kx, b): SA(2) SB(2) TA(2) TB(2)
-            T acc[32];
-#pragma unroll
-            for (int q = 0; q < 32; ++q) acc[q] = T(0);
-            const bool scaled = __any_sync(kFull, kmax_of<T, LPT>(k) > 0);
-#pragma unroll
-            for (int kx = 0; kx < K; ++kx) {
-                const T2 ab = s_ab[t0 + kx];
-                const T dcn = s_dc[t0 + kx];
-                const T nf = T(m * pv.mres + n0 + t0 + kx);
-                bool live = true;
-                if (scaled) {
-                    rec_step<T, LPT, true>(ab.x, ab.y, x, y1, y2, k, c);
-                    live = __any_sync(kFull, kmin_of<T, LPT>(k) == 0);
-                } else {
-                    rec_step<T, LPT, false>(ab.x, ab.y, x, y1, y2, k, c);
-                }
-                if (!live) continue;
-#pragma unroll
-                for (int i = 0; i < LPT; ++i) {
-                    const T dpv = fma(nf * x[i], y1[i], -dcn * y2[i]);
-                    const T cd = (scaled && k[i] > 0) ? T(0) : dpv;
-#pragma unroll
-                    for (int b = 0; b < BC; ++b) {
-                        // n-m even (kx even): P even -> s folds; dP odd -> d folds
-                        const T2 vt_dP = (kx & 1) ? st_[i][b] : dt_[i][b];
-                        const T2 vp_P = (kx & 1) ? dp_[i][b] : sp_[i][b];
-                        const T2 vt_P = (kx & 1) ? dt_[i][b] : st_[i][b];
-                        const T2 vp_dP = (kx & 1) ? sp_[i][b] : dp_[i][b];
-                        T *a = &acc[(kx * BC + b) * 8];
-                        a[0] = fma(cd, vt_dP.x, a[0]);
-                        a[1] = fma(cd, vt_dP.y, a[1]);
-                        a[2] = fma(c[i], vp_P.x, a[2]);
-                        a[3] = fma(c[i], vp_P.y, a[3]);
-                        a[4] = fma(c[i], vt_P.x, a[4]);
-                        a[5] = fma(c[i], vt_P.y, a[5]);
-                        a[6] = fma(cd, vp_dP.x, a[6]);
-                        a[7] = fma(cd, vp_dP.y, a[7]);
-                    }
-                }
-            }
-            warp_transpose_reduce<T, 32>(acc, lane);
-            s_red[warp][lane] = acc[0];
-            __syncthreads();
-            if (threadIdx.x < K * BC) {
-                T tot[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) tot[q] = T(0);
-                for (int w = 0; w < nw; ++w)
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) tot[q] += s_red[w][threadIdx.x * 8 + q];
-                const int kx = threadIdx.x / BC, b = threadIdx.x % BC;
-                const int nn = n0 + t0 + kx;
-                const int n = m * pv.mres + nn;
-                if (nn < L && b0 + b < batch) {
-                    T sc;
-                    if (op == OP_SYNTH_ADJ) sc = (m > 0) ? T(2) : T(1);
-                    else sc = (n == 0) ? T(0) : T(1) / (T(n) * T(n + 1));
-                    T2 sv, tv;
-                    // S = SA - i m SB ; T = i m TA + TB
-                    sv.x = sc * (tot[0] + fm * tot[3]);
-                    sv.y = sc * (tot[1] - fm * tot[2]);
-                    tv.x = sc * (tot[6] - fm * tot[5]);
-                    tv.y = sc * (tot[7] + fm * tot[4]);
-                    if (m == 0) { sv.y = T(0); tv.y = T(0); }
-                    S2[(size_t)(b0 + b) * pv.nlm + col + nn] = sv;
-                    T2o[(size_t)(b0 + b) * pv.nlm + col + nn] = tv;
-                }
-            }
-            __syncthreads();
-        }
-    }
+    cp_async_wait<0>();
+    warp_transpose_reduce<kSeedSeg * 4>(acc, lane);
+    if (lane >= cnt) return;
+    float sc;
+    if (op == OP_SYNTH_ADJ) sc = (m > 0) ? 2.f : 1.f;
+    else sc = (n == 0) ? 0.f : 1.f / ((float)n * (float)(n + 1));
+    const size_t o = (size_t)b * pv.nlm + col + lane;
+    reinterpret_cast<float2 *>(So)[o] = make_float2(sc * acc[0], m == 0 ? 0.f : sc * acc[1]);
+    reinterpret_cast<float2 *>(To)[o] = make_float2(sc * acc[2], m == 0 ? 0.f : sc * acc[3]);
 }
 
 // Field chunk per CTA for a batch.
 inline int pick_bc(int batch) { return batch >= 4 ? 4 : (batch >= 2 ? 2 : 1); }
 
-template <typename T, int LPT, int BC>
-cudaError_t synth_go(const PlanView<T> &pv, const T *spec, T *eo, int batch, Op op, cudaStream_t s)
+inline unsigned segment_ctas(const PlanView<float> &pv)
 {
-    constexpr int NT = 128;
-    const int npb = (pv.npairs + NT * LPT - 1) / (NT * LPT);
+    return (unsigned)((pv.lmax + kSeedSeg * kWarps) / (kSeedSeg * kWarps));
+}
+
+template <int LPT, int BC>
+cudaError_t synth_go(const PlanView<float> &pv, const float *spec, float *eo, int batch, Op op, cudaStream_t s)
+{
+    const int npb = (pv.npairs + 32 * LPT - 1) / (32 * LPT);
     dim3 grid((unsigned)((pv.mmax + 1) * npb), (unsigned)((batch + BC - 1) / BC));
-    k_synth<T, LPT, BC, NT><<<grid, NT, 0, s>>>(pv, spec, eo, batch, npb, (int)op);
+    k_synth<LPT, BC><<<grid, 32 * kWarps, 0, s>>>(pv, spec, eo, batch, npb, (int)op);
     return cudaGetLastError();
 }
 
-// Analysis CTAs hold every latitude pair of one order: nw warps of LPT pairs per thread.
-inline int analys_warps(int npairs, int lpt) { int nw = (npairs + 32 * lpt - 1) / (32 * lpt); return nw < 1 ? 1 : nw; }
-
-template <typename T, int LPT, int BC>
-cudaError_t analys_go(const PlanView<T> &pv, const T *sd, T *spec, int batch, Op op, cudaStream_t s)
+template <int BC>
+cudaError_t analys_go(const PlanView<float> &pv, const float *sd, float *spec, int batch, Op op, cudaStream_t s)
 {
-    const int nw = analys_warps(pv.npairs, LPT);
-    if (nw > 8) return cudaErrorInvalidConfiguration;
-    dim3 grid((unsigned)(pv.mmax + 1), (unsigned)((batch + BC - 1) / BC));
-    k_analys<T, LPT, BC><<<grid, nw * 32, 0, s>>>(pv, sd, spec, batch, (int)op);
+    dim3 grid(segment_ctas(pv), (unsigned)(pv.mmax + 1), (unsigned)((batch + BC - 1) / BC));
+    k_analys<BC><<<grid, 32 * kWarps, 0, s>>>(pv, sd, spec, batch, (int)op);
     return cudaGetLastError();
 }
 
-template <typename T, int LPT, int BC>
-cudaError_t synth_vec_go(const PlanView<T> &pv, const T *S, const T *Tc, T *eot, T *eop, int batch, Op op,
-                         cudaStream_t s)
+template <int LPT, int BC>
+cudaError_t synth_vec_go(const PlanView<float> &pv, const float *S, const float *Tc, float *eot, float *eop, int batch,
+                         Op op, cudaStream_t s)
 {
-    constexpr int NT = 128;
-    const int npb = (pv.npairs + NT * LPT - 1) / (NT * LPT);
+    const int npb = (pv.npairs + 32 * LPT - 1) / (32 * LPT);
     dim3 grid((unsigned)((pv.mmax + 1) * npb), (unsigned)((batch + BC - 1) / BC));
-    k_synth_vec<T, LPT, BC, NT><<<grid, NT, 0, s>>>(pv, S, Tc, eot, eop, batch, npb, (int)op);
+    k_synth_vec<LPT, BC><<<grid, 32 * kWarps, 0, s>>>(pv, S, Tc, eot, eop, batch, npb, (int)op);
     return cudaGetLastError();
 }
-
-template <typename T, int LPT, int BC>
-cudaError_t analys_vec_go(const PlanView<T> &pv, const T *sdt, const T *sdp, T *S, T *Tc, int batch, Op op,
-                          cudaStream_t s)
-{
-    const int nw = analys_warps(pv.npairs, LPT);
-    if (nw > 8) return cudaErrorInvalidConfiguration;
-    dim3 grid((unsigned)(pv.mmax + 1), (unsigned)((batch + BC - 1) / BC));
-    k_analys_vec<T, LPT, BC><<<grid, nw * 32, 0, s>>>(pv, sdt, sdp, S, Tc, batch, (int)op);
-    return cudaGetLastError();
-}
-
-// Pairs per thread for analysis: the cross-lane reduction costs ~1/LPT of the
-// sums, so use 4 pairs per thread once there are enough pairs, 8 beyond 1024
-// (at most 8 warps per CTA).
-inline int analys_lpt(int npairs) { return npairs <= 64 ? 2 : (npairs <= 1024 ? 4 : 8); }
 
 }  // namespace
 
 cudaError_t launch_legendre_synth(const PlanView<float> &pv, const float *spec, float *eo, int batch, Op op, int lpt,
                                   int bc, cudaStream_t s)
 {
-    if (!seeds_ok(pv, true)) return cudaErrorInvalidValue;
-    // default shape: 2 pairs per thread, up to 4 fields per CTA
+    if (!seeds_ok(pv)) return cudaErrorInvalidValue;
+    // default shape: 2 pairs per lane, up to 4 fields per CTA
     if (lpt <= 0) lpt = 2;
     if (bc <= 0) bc = pick_bc(batch);
-#define SHT_SYN(L, B) if (lpt == L && bc == B) return synth_go<float, L, B>(pv, spec, eo, batch, op, s);
+#define SHT_SYN(L, B) if (lpt == L && bc == B) return synth_go<L, B>(pv, spec, eo, batch, op, s);
     SHT_SYN(1, 1) SHT_SYN(1, 2) SHT_SYN(1, 4)
     SHT_SYN(2, 1) SHT_SYN(2, 2) SHT_SYN(2, 4)
-    SHT_SYN(4, 1) SHT_SYN(4, 2) SHT_SYN(4, 4)
+    SHT_SYN(4, 1) SHT_SYN(4, 2)
 #undef SHT_SYN
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_legendre_analys(const PlanView<float> &pv, const float *sd, float *spec, int batch, Op op, int lpt,
-                                   int bc, cudaStream_t s)
+cudaError_t launch_legendre_analys(const PlanView<float> &pv, const float *sd, float *spec, int batch, Op op, int bc,
+                                   cudaStream_t s)
 {
-    if (!seeds_ok(pv, true)) return cudaErrorInvalidValue;
-    // default shape: LPT from the pair count (<= 8 warps), 2 fields per CTA when batched
-    if (lpt <= 0) lpt = analys_lpt(pv.npairs);
+    if (!seeds_ok(pv)) return cudaErrorInvalidValue;
     if (bc <= 0) bc = batch >= 2 ? 2 : 1;
-    if (analys_warps(pv.npairs, lpt) > 8) return cudaErrorInvalidValue;
-#define SHT_ANA(L, B) if (lpt == L && bc == B) return analys_go<float, L, B>(pv, sd, spec, batch, op, s);
-    SHT_ANA(2, 1) SHT_ANA(2, 2) SHT_ANA(4, 1) SHT_ANA(4, 2) SHT_ANA(8, 1) SHT_ANA(8, 2)
-#undef SHT_ANA
+    if (bc == 1) return analys_go<1>(pv, sd, spec, batch, op, s);
+    if (bc == 2) return analys_go<2>(pv, sd, spec, batch, op, s);
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_legendre_synth_vec(const PlanView<float> &pv, const float *S, const float *Tc, float *eot,
                                       float *eop, int batch, Op op, cudaStream_t s)
 {
-    if (!seeds_ok(pv, false)) return cudaErrorInvalidValue;
-    if (batch >= 2) return synth_vec_go<float, 1, 2>(pv, S, Tc, eot, eop, batch, op, s);
-    return synth_vec_go<float, 1, 1>(pv, S, Tc, eot, eop, batch, op, s);
+    if (!seeds_ok(pv)) return cudaErrorInvalidValue;
+    if (batch >= 2) return synth_vec_go<2, 2>(pv, S, Tc, eot, eop, batch, op, s);
+    return synth_vec_go<2, 1>(pv, S, Tc, eot, eop, batch, op, s);
 }
 
 cudaError_t launch_legendre_analys_vec(const PlanView<float> &pv, const float *sdt, const float *sdp, float *S,
                                        float *Tc, int batch, Op op, cudaStream_t s)
 {
-    if (!seeds_ok(pv, false)) return cudaErrorInvalidValue;
-    switch (analys_lpt(pv.npairs)) {
-    case 2: return analys_vec_go<float, 2, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
-    case 4: return analys_vec_go<float, 4, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
-    default: return analys_vec_go<float, 8, 1>(pv, sdt, sdp, S, Tc, batch, op, s);
-    }
+    if (!seeds_ok(pv)) return cudaErrorInvalidValue;
+    dim3 grid(segment_ctas(pv), (unsigned)(pv.mmax + 1), (unsigned)batch);
+    k_analys_vec<<<grid, 32 * kWarps, 0, s>>>(pv, sdt, sdp, S, Tc, (int)op);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// Persistent kernels for uneven batches (FP32, one field per tile).
+// Persistent kernels for uneven batches (one field per tile).
 // ---------------------------------------------------------------------------
 namespace {
 
-__global__ void __launch_bounds__(128) k_batch_synth(const BatchField *__restrict__ fields,
-                                                     const int4 *__restrict__ tiles, int ntiles, int *counter)
+__global__ void __launch_bounds__(32 * kWarps) k_batch_synth(const BatchField *__restrict__ fields,
+                                                             const int4 *__restrict__ tiles, int ntiles, int *counter)
 {
-    __shared__ float2 s_ab[kSynthNch];
-    __shared__ float2 s_f[kSynthNch];
-    __shared__ int s_tile, s_first;
+    __shared__ SynthSmem<2, 1> sm;
+    __shared__ int s_tile;
     for (;;) {
         __syncthreads();  // the previous tile is done with the shared buffers
         if (threadIdx.x == 0) s_tile = atomicAdd(counter, 1);
@@ -908,25 +781,26 @@ __global__ void __launch_bounds__(128) k_batch_synth(const BatchField *__restric
         if (t >= ntiles) break;
         const int4 tl = tiles[t];
         const BatchField f = fields[tl.x];
-        synth_tile<float, 2, 1, 128>(f.pv, f.in, f.inter, 1, tl.y, tl.z, 0, OP_SYNTH, s_ab, s_f, &s_first);
+        synth_tile<2, 1>(f.pv, f.in, f.inter, 1, tl.y, tl.z, 0, OP_SYNTH, sm);
     }
 }
 
-__global__ void __launch_bounds__(256) k_batch_analys(const BatchField *__restrict__ fields,
-                                                      const int4 *__restrict__ tiles, int ntiles, int *counter)
+// A warp takes the next four segments of an order at a time.
+__global__ void __launch_bounds__(32 * kWarps) k_batch_analys(const BatchField *__restrict__ fields,
+                                                              const int4 *__restrict__ tiles, int ntiles, int *counter)
 {
-    __shared__ float2 s_ab[kAnalysNch];
-    __shared__ float s_red[8][32];
-    __shared__ int s_tile;
+    __shared__ AnalysSmem<1> sm[kWarps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_tile = atomicAdd(counter, 1);
-        __syncthreads();
-        const int t = s_tile;
+        int t = 0;
+        if (lane == 0) t = atomicAdd(counter, 1);
+        t = __shfl_sync(kFull, t, 0);
         if (t >= ntiles) break;
         const int4 tl = tiles[t];
         const BatchField f = fields[tl.x];
-        analys_tile<float, 2, 1>(f.pv, f.inter, f.out, 1, tl.y, 0, OP_ANALYS, s_ab, s_red);
+        const int nseg = (f.pv.lmax - tl.y * f.pv.mres + kSeedSeg) / kSeedSeg;
+        for (int seg = tl.z; seg < min(nseg, tl.z + kBatchAnalysSegs); ++seg)
+            analys_segment<1>(f.pv, f.inter, f.out, 1, tl.y, seg, 0, OP_ANALYS, sm[w]);
     }
 }
 
@@ -935,8 +809,8 @@ __global__ void __launch_bounds__(256) k_batch_analys(const BatchField *__restri
 cudaError_t launch_batch_legendre(bool synth, const BatchField *fields, const int4 *tiles, int ntiles, int *counter,
                                   int ctas, cudaStream_t s)
 {
-    if (synth) k_batch_synth<<<ctas, 128, 0, s>>>(fields, tiles, ntiles, counter);
-    else k_batch_analys<<<ctas, 256, 0, s>>>(fields, tiles, ntiles, counter);
+    if (synth) k_batch_synth<<<ctas, 32 * kWarps, 0, s>>>(fields, tiles, ntiles, counter);
+    else k_batch_analys<<<ctas, 32 * kWarps, 0, s>>>(fields, tiles, ntiles, counter);
     return cudaGetLastError();
 }
 
@@ -945,79 +819,103 @@ cudaError_t launch_batch_legendre(bool synth, const BatchField *fields, const in
 // polar optimisation.  One thread per (order index m, pair): the FP64
 // recurrence of Sec. 3.2 from P_m^m, carried as y 2^(-240 k) (Sec. 3.5).  At
 // the start of every kSeedSeg-degree segment the state (y1, y2) =
-// (P_{n0-1}, P_{n0-2}) is stored, either times 2^hseg with k (FP64 plans) or
-// rewritten in the FP32 form y' 2^(-64 k'): k' = 0 when the larger of the two
-// is at least 2^-63, else the k' that brings it into [2^-65, 1) -- the form in
-// which the FP32 kernels carry it.  live[m][pair] is the first segment that
-// holds a degree with |P_n^m| >= thr (all segments live when thr <= 0; the
-// segment count when none is).
+// (P_{n0-1}, P_{n0-2}) is stored: times 2^hseg with k (FP64 plans), or in the
+// form of the FP32 kernels, (y1, y2, factor) with P = factor y (fp32_state).
+// live[m][pair] is the first segment that holds a degree with |P_n^m| >= thr to
+// within 2^-20 of its value (all segments live when thr <= 0; the segment count
+// when none is), glive the smallest of each group of 32 pairs, and glive_vec the
+// group's first segment that holds a value the precision keeps (2^-70 in FP32; any
+// unscaled one in FP64): segments that contribute nothing at any threshold.
+// The kernel is bound by its FP64 instructions, three per degree: every test is
+// on the high words (22 -> 13 ms at N = 2047 with FP64 comparisons left out).
 // ---------------------------------------------------------------------------
 namespace {
 
-__device__ float4 fp32_state(double y1, double y2, int k)
+constexpr int kLeast32 = -70;   // FP32 leaves out segments with every |P| below 2^kLeast32
+
+// y 2^(-240 k) = P; emax: floor(log2) of the segment's largest |P|.  A state of
+// at least 2^-62 is stored as it is.  A smaller one can grow by up to 2^149 over
+// 32 degrees (order 4095): it is stored times the power of two that takes the
+// segment's largest value to about 2^50, which leaves every value and the factor
+// in FP32's normal range; the recurrence rounds the same at either scale.
+__device__ float4 fp32_state(double y1, double y2, int k, int emax)
 {
+    constexpr int kTop = 50;
     const double mx = fmax(fabs(y1), fabs(y2));
-    if (mx == 0.0) return make_float4(0.f, 0.f, __int_as_float(0), 0.f);
-    int ex = 0;
-    frexp(mx, &ex);
-    const long E = (long)ex - (long)Scale<double>::S * k;   // the larger value < 2^E
-    constexpr int S32 = Scale<float>::S;
-    long k32 = 0;
-    if (E < 1 - S32) k32 = (-E) / S32;
-    const int sh = (int)(-(long)Scale<double>::S * k + (long)S32 * k32);
-    return make_float4((float)scalbn(y1, sh), (float)scalbn(y2, sh), __int_as_float((int)k32), 0.f);
+    if (mx == 0.0 || emax < kLeast32) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const int down = -Scale<double>::S * k;
+    if (ilogb(mx) + down >= -63) return make_float4((float)scalbn(y1, down), (float)scalbn(y2, down), 1.f, 0.f);
+    const int e = kTop - emax;
+    return make_float4((float)scalbn(y1, down + e), (float)scalbn(y2, down + e), (float)scalbn(1.0, -e), 0.f);
 }
 
 __global__ void __launch_bounds__(128)
 k_build_restarts(PlanView<double> pv, const unsigned long long *__restrict__ segoff, float4 *__restrict__ seeds32,
                  double2 *__restrict__ seeds64, int *__restrict__ seeds64k, const int *__restrict__ hseg,
-                 unsigned short *__restrict__ live, double thr)
+                 unsigned short *__restrict__ live, unsigned short *__restrict__ glive,
+                 unsigned short *__restrict__ glive_vec, double thr)
 {
     const int m = blockIdx.y;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     const int npairs = pv.npairs;
-    if (p >= npairs) return;
+    const bool in = p < npairs;
     const int L = pv.lmax - m * pv.mres + 1;
     const int nseg = (L + kSeedSeg - 1) / kSeedSeg;
     const long col = col_of_mres(pv.lmax, m, pv.mres);
-    const double x = pv.x[p];
-    double y1 = 0.0, y2 = pv.pmm[(size_t)m * npairs + p];
-    int k = pv.pmmk[(size_t)m * npairs + p];
-    int first = thr > 0.0 ? nseg : 0;
-    for (int s = 0; s < nseg; ++s) {
+    const double x = in ? pv.x[p] : 0.0;
+    double y1 = 0.0, y2 = in ? pv.pmm[(size_t)m * npairs + p] : 0.0;
+    int k = in ? pv.pmmk[(size_t)m * npairs + p] : 0;
+    int first = thr > 0.0 ? nseg : 0, kept = nseg;
+    constexpr int kOne = 0x3ff00000, kStep = Scale<double>::S << 20;   // high words of 1 and of a step of k
+    const int hthr = __double2hiint(thr), hkeep = seeds32 ? kOne + kLeast32 * (1 << 20) : kOne - kStep;
+    for (int s = 0; s < nseg && in; ++s) {
         const size_t o = (segoff[m] + s) * npairs + p;
-        if (seeds32) seeds32[o] = fp32_state(y1, y2, k);
+        const double b1 = y1, b2 = y2;   // the state entering the segment
+        const int bk = k;
+        int top = INT_MIN;   // high word of the segment's largest |P|, k steps taken off
         if (seeds64) {
             const int h = hseg[segoff[m] + s];
             seeds64[o] = make_double2(scalbn(y1, h), scalbn(y2, h));
             seeds64k[o] = k;
         }
-        for (int i = 0; i < kSeedSeg; ++i) {
-            const int nn = kSeedSeg * s + i;
-            if (nn >= L) break;
-            const double2 ab = pv.ab[col + nn];
+        const int n1 = min(kSeedSeg, L - kSeedSeg * s);
+        for (int i = 0; i < n1; ++i) {
+            const double2 ab = pv.ab[col + kSeedSeg * s + i];
             const double yn = fma(ab.x * x, y1, ab.y * y2);
             y2 = y1;
             y1 = yn;
-            if (k > 0 && fabs(yn) >= 1.0) {
-                y1 *= down_scale<double>();
-                y2 *= down_scale<double>();
+            int hi = __double2hiint(yn) & 0x7fffffff;
+            if (k > 0 && hi >= kOne) {
+                y1 *= 0x1p-240;
+                y2 *= 0x1p-240;
                 k -= 1;
+                hi -= kStep;
             }
-            if (k == 0 && fabs(y1) >= thr && s < first) first = s;
+            top = max(top, hi - min(k, 3) * kStep);   // below 2^-700 all the same
         }
+        if (s < first && top >= hthr) first = s;
+        if (s < kept && top >= hkeep) kept = s;
+        if (seeds32) seeds32[o] = fp32_state(b1, b2, bk, (top >> 20) - 1023);
     }
-    live[(size_t)m * npairs + p] = (unsigned short)first;
+    if (in) live[(size_t)m * npairs + p] = (unsigned short)first;
+    first = __reduce_min_sync(kFull, in ? first : 0xffff);
+    kept = __reduce_min_sync(kFull, in ? kept : 0xffff);
+    if ((threadIdx.x & 31) == 0 && in) {   // the group's first pair
+        const size_t g = (size_t)m * groups_of(npairs) + (p >> 5);
+        glive[g] = (unsigned short)first;
+        glive_vec[g] = (unsigned short)kept;
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_build_restarts(const PlanView<double> &pv, const unsigned long long *segoff, float4 *seeds32,
-                                  double2 *seeds64, int *seeds64k, const int *hseg, unsigned short *live, double thr,
-                                  cudaStream_t st)
+                                  double2 *seeds64, int *seeds64k, const int *hseg, unsigned short *live,
+                                  unsigned short *glive, unsigned short *glive_vec, double thr, cudaStream_t st)
 {
     dim3 grid((unsigned)((pv.npairs + 127) / 128), (unsigned)(pv.mmax + 1));
-    k_build_restarts<<<grid, 128, 0, st>>>(pv, segoff, seeds32, seeds64, seeds64k, hseg, live, thr);
+    k_build_restarts<<<grid, 128, 0, st>>>(pv, segoff, seeds32, seeds64, seeds64k, hseg, live, glive, glive_vec,
+                                          thr);
     return cudaGetLastError();
 }
 

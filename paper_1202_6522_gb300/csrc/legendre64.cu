@@ -125,7 +125,7 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restri
     const int p = g * 32 + lane;
     const bool valid = p < npairs;
     const double x = valid ? pv.x[p] : 0.0;
-    const int first = __reduce_min_sync(kFull, valid ? (int)pv.live[(size_t)m * npairs + p] : 0xffff);
+    const int first = (vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g];
     const double insc = (op == OP_ANALYS_ADJ && m > 0) ? 0.5 : 1.0;   // adjoint of analysis: b / c_m
 
     double er[BC], ei[BC], orr[BC], oi[BC];
@@ -305,14 +305,11 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
     if (tail)   // one degree: the rest of its block of DB is zero
         for (int t = 1; t < DB; ++t) s_P[w][t][lane] = 0.0;
     __syncthreads();
-    for (int g = w; g < ngroups; g += W) {
-        const int p = g * 32 + lane;
-        const int f = p < npairs ? (int)pv.live[(size_t)m * npairs + p] : 0xffff;
-        if (__any_sync(kFull, f <= seg)) {
-            if (lane == 0) atomicMin(&s_g0, g);
+    for (int g = threadIdx.x; g < ngroups; g += 32 * W)
+        if ((vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g] <= seg) {
+            atomicMin(&s_g0, g);
             break;
         }
-    }
     __syncthreads();
     const int g0 = s_g0;
 
@@ -583,7 +580,7 @@ inline int pick_bc64(int batch, int most)
 
 bool tables_ok(const PlanView<double> &pv)
 {
-    return pv.segoff && pv.seeds64 && pv.seeds64k && pv.live && pv.qs && pv.abx && pv.eps && pv.hseg;
+    return pv.segoff && pv.seeds64 && pv.seeds64k && pv.glive && pv.glive_vec && pv.qs && pv.abx && pv.eps && pv.hseg;
 }
 
 // A launch of the synthesis with W warps per CTA.

@@ -89,13 +89,16 @@ struct DevArena {
 template <typename U>
 size_t padded(size_t count) { return (count * sizeof(U) + 255) & ~size_t(255); }
 
+// Groups of 32 pairs over all orders.
+size_t plan_groups(const Plan &p) { return (size_t)(p.mmax + 1) * ((p.npairs + 31) / 32); }
+
 }  // namespace
 
 PlanView<double> Plan::view64() const
 {
     PlanView<double> v{lmax, mmax, nlat, nphi, npairs, nlm,
                        t64.ab, t64.dc, t64.x, t64.st, t64.wq, t64.pmm, t64.pmmk, t64.tw, t64.rtw, fft_plan_of(nphi / 2), mres, twdf,
-                       nullptr, d_seg32, seeds64, seeds64k, live64, qs64, abx64, eps64, hseg64};
+                       nullptr, d_seg32, seeds64, seeds64k, live64, glive64, glive64 + plan_groups(*this), qs64, abx64, eps64, hseg64};
     return v;
 }
 
@@ -103,7 +106,7 @@ PlanView<float> Plan::view32() const
 {
     PlanView<float> v{lmax, mmax, nlat, nphi, npairs, nlm,
                       t32.ab, t32.dc, t32.x, t32.st, t32.wq, t32.pmm, t32.pmmk, t32.tw, t32.rtw, fft_plan_of(nphi / 2), mres, nullptr,
-                      seeds32, d_seg32, nullptr, nullptr, live32, nullptr, nullptr, nullptr, nullptr};
+                      seeds32, d_seg32, nullptr, nullptr, live32, glive32, glive32 + plan_groups(*this), nullptr, nullptr, nullptr, nullptr};
     return v;
 }
 
@@ -151,8 +154,8 @@ int plan_build(Plan &p, std::string &err)
     // Starting values P_m^m(x_j) = sqrt(1/4pi) prod_{k<=m} sqrt((2k+1)/(2k)) sin^m,
     // carried as mantissa * 2^e, then written as y * 2^(-S k) with y in [2^-S, 1)
     // when the value is below 2^-S (k > 0), else y = value, k = 0.
-    std::vector<double> pmm64((size_t)(mmax + 1) * npairs), pmm32d((size_t)(mmax + 1) * npairs);
-    std::vector<int> k64((size_t)(mmax + 1) * npairs), k32((size_t)(mmax + 1) * npairs);
+    std::vector<double> pmm64((size_t)(mmax + 1) * npairs);
+    std::vector<int> k64((size_t)(mmax + 1) * npairs);
     auto split = [](double mant, long e, int S, double &y, int &k) {
         if (mant == 0.0) { y = 0.0; k = 0; return; }
         if (e >= 1 - S) { y = std::ldexp(mant, (int)e); k = 0; return; }
@@ -174,7 +177,6 @@ int plan_build(Plan &p, std::string &err)
             if (m % mres) continue;   // only the orders of the plan are stored
             const size_t o = (size_t)(m / mres) * npairs + j;
             split(mant, e, Scale<double>::S, pmm64[o], k64[o]);
-            split(mant, e, Scale<float>::S, pmm32d[o], k32[o]);
         }
     }
 
@@ -206,9 +208,7 @@ int plan_build(Plan &p, std::string &err)
     size_t bytes = padded<double2>(nlm) + padded<double>(nlm) + 3 * padded<double>(npairs) +
                    padded<double>((size_t)(mmax + 1) * npairs) + padded<int>((size_t)(mmax + 1) * npairs) +
                    2 * padded<double2>(H1);
-    bytes += padded<float2>(nlm) + padded<float>(nlm) + 3 * padded<float>(npairs) +
-             padded<float>((size_t)(mmax + 1) * npairs) + padded<int>((size_t)(mmax + 1) * npairs) +
-             2 * padded<float2>(H1);
+    bytes += padded<float2>(nlm) + padded<float>(nlm) + 3 * padded<float>(npairs) + 2 * padded<float2>(H1);
     bytes += padded<float4>(H1) + padded<int>(1);
     DevArena ar;
     cudaError_t ce = cudaGetDevice(&p.device);
@@ -242,7 +242,7 @@ int plan_build(Plan &p, std::string &err)
     ok &= up(p.t64.rtw, rtw.data(), sizeof(double) * 2 * H1);
 
     std::vector<float> ab32 = to_f32(ab), dc32 = to_f32(dc), x32 = to_f32(xp), s32 = to_f32(sp),
-                       w32 = to_f32(wp), pmm32 = to_f32(pmm32d), tw32 = to_f32(tw),
+                       w32 = to_f32(wp), tw32 = to_f32(tw),
                        rtw32 = to_f32(rtw);
     p.t32.ab = ar.take<float2>(nlm);
     ok &= up(p.t32.ab, ab32.data(), sizeof(float) * 2 * nlm);
@@ -254,10 +254,6 @@ int plan_build(Plan &p, std::string &err)
     ok &= up(p.t32.st, s32.data(), sizeof(float) * npairs);
     p.t32.wq = ar.take<float>(npairs);
     ok &= up(p.t32.wq, w32.data(), sizeof(float) * npairs);
-    p.t32.pmm = ar.take<float>((size_t)(mmax + 1) * npairs);
-    ok &= up(p.t32.pmm, pmm32.data(), sizeof(float) * pmm32.size());
-    p.t32.pmmk = ar.take<int>((size_t)(mmax + 1) * npairs);
-    ok &= up(p.t32.pmmk, k32.data(), sizeof(int) * k32.size());
     p.t32.tw = ar.take<float2>(H1);
     ok &= up(p.t32.tw, tw32.data(), sizeof(float) * 2 * H1);
     p.t32.rtw = ar.take<float2>(H1);
@@ -320,7 +316,7 @@ void free_seeds64(Plan &p)
     cudaFree(p.seeds64);
     p.seeds64 = nullptr;
     p.seeds64k = nullptr;
-    p.live64 = nullptr;
+    p.live64 = p.glive64 = nullptr;
     p.qs64 = p.abx64 = nullptr;
     p.eps64 = nullptr;
     p.hseg64 = nullptr;
@@ -341,17 +337,19 @@ int plan_seeds32(Plan &p, std::string &err)
     if (rc) return rc;
     const size_t nseg = plan_nseg(p);
     cudaError_t e = cudaMalloc(&p.seeds32, sizeof(float4) * nseg * (size_t)p.npairs);
-    if (e == cudaSuccess) e = cudaMalloc(&p.live32, sizeof(unsigned short) * (size_t)(p.mmax + 1) * p.npairs);
+    const size_t norder = (size_t)(p.mmax + 1) * p.npairs, ng = plan_groups(p);
+    if (e == cudaSuccess) e = cudaMalloc(&p.live32, sizeof(unsigned short) * (norder + 2 * ng));
+    if (e == cudaSuccess) p.glive32 = p.live32 + norder;
     if (e == cudaSuccess)
-        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, nullptr, p.live32, p.thr_cc32(),
-                                  0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, nullptr, p.live32, p.glive32,
+                                  p.glive32 + plan_groups(p), p.thr_cc32(), 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         cudaGetLastError();
         cudaFree(p.seeds32);
         cudaFree(p.live32);
         p.seeds32 = nullptr;
-        p.live32 = nullptr;
+        p.live32 = p.glive32 = nullptr;
         err = std::string("building FP32 recurrence seeds: ") + cudaGetErrorString(e);
         return SHT_ENOMEM;
     }
@@ -369,12 +367,13 @@ int plan_seeds64(Plan &p, std::string &err)
     const size_t nlmx = (size_t)p.nlm + p.mmax + 1;   // degrees to lmax + 1
     DevArena ar;
     ar.cap = padded<double2>(nstate) + padded<int>(nstate) + padded<unsigned short>(norder) +
-             2 * padded<double2>(nlmx) + padded<double>(nlmx) + padded<int>(nseg);
+             padded<unsigned short>(2 * plan_groups(p)) + 2 * padded<double2>(nlmx) + padded<double>(nlmx) + padded<int>(nseg);
     cudaError_t e = cudaMalloc(&ar.base, ar.cap);
     if (e == cudaSuccess) {
         p.seeds64 = ar.take<double2>(nstate);   // the allocation's base
         p.seeds64k = ar.take<int>(nstate);
         p.live64 = ar.take<unsigned short>(norder);
+        p.glive64 = ar.take<unsigned short>(2 * plan_groups(p));
         p.qs64 = ar.take<double2>(nlmx);
         p.abx64 = ar.take<double2>(nlmx);
         p.eps64 = ar.take<double>(nlmx);
@@ -382,8 +381,8 @@ int plan_seeds64(Plan &p, std::string &err)
         e = launch_build_qs(p.view64(), p.d_seg32, p.qs64, p.abx64, p.eps64, p.hseg64, 0);
     }
     if (e == cudaSuccess)
-        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.hseg64, p.live64,
-                                  p.thr_cc64(), 0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.hseg64, p.live64, p.glive64,
+                                  p.glive64 + plan_groups(p), p.thr_cc64(), 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -398,11 +397,11 @@ int plan_relive(Plan &p, std::string &err)
 {
     cudaError_t e = cudaSuccess;
     if (p.seeds32)
-        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, nullptr, p.live32, p.thr_cc32(),
-                                  0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, p.seeds32, nullptr, nullptr, nullptr, p.live32, p.glive32,
+                                  p.glive32 + plan_groups(p), p.thr_cc32(), 0);
     if (e == cudaSuccess && p.seeds64)
-        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.hseg64, p.live64,
-                                  p.thr_cc64(), 0);
+        e = launch_build_restarts(p.view64(), p.d_seg32, nullptr, p.seeds64, p.seeds64k, p.hseg64, p.live64, p.glive64,
+                                  p.glive64 + plan_groups(p), p.thr_cc64(), 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         err = std::string("rebuilding the polar tables: ") + cudaGetErrorString(e);
@@ -470,7 +469,7 @@ void plan_free(Plan &p)
     free_seeds64(p);
     p.seeds32 = nullptr;
     p.d_seg32 = nullptr;
-    p.live32 = nullptr;
+    p.live32 = p.glive32 = nullptr;
     for (cudaEvent_t e : p.timer.pool) cudaEventDestroy(e);
     p.timer.pool.clear();
     if (p.tables_base) cudaFree(p.tables_base);

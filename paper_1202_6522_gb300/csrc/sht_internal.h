@@ -12,13 +12,12 @@
 
 namespace sht {
 
-// Exponent step of the underflow rescaling (Sec. 3.5): a value is carried as
-// y * 2^(-S k) with an integer k >= 0.  While k > 0 the true value is below
-// 2^-S: it is left out of the Legendre sums but still advanced by the
-// recurrence.  Dropped terms are < 2^-240 (FP64) or 2^-64 (FP32).
+// Exponent step of the underflow rescaling (Sec. 3.5) of the FP64 recurrence: a
+// value is carried as y * 2^(-S k) with an integer k >= 0.  While k > 0 the true
+// value is below 2^-S: it is left out of the Legendre sums but still advanced by
+// the recurrence.  (The FP32 kernels rescale per segment, see legendre.cu.)
 template <typename T> struct Scale;
 template <> struct Scale<double> { static constexpr int S = 240; };
-template <> struct Scale<float> { static constexpr int S = 64; };
 
 template <typename T> struct Vec2;
 template <> struct Vec2<double> { using type = double2; };
@@ -33,8 +32,8 @@ struct Tables {
     T *x = nullptr;      // [npairs] cos(theta) of the northern node of each pair (>= 0)
     T *st = nullptr;     // [npairs] sin(theta)
     T *wq = nullptr;     // [npairs] Gauss weight of that node
-    T *pmm = nullptr;    // [mmax+1][npairs] P_m^m(x_p) * 2^(S k) (mantissa)
-    int *pmmk = nullptr; // [mmax+1][npairs] k (number of 2^S steps)
+    T *pmm = nullptr;    // FP64: [mmax+1][npairs] P_m^m(x_p) * 2^(S k) (mantissa)
+    int *pmmk = nullptr; // FP64: [mmax+1][npairs] k (number of 2^S steps)
     T2 *tw = nullptr;    // [nphi/2] e^{2 pi i k / nphi}
     T2 *rtw = nullptr;   // [H] four-step FFT twiddles: rtw[k1 N2 + n2] = e^{2 pi i n2 k1 / H}
 };
@@ -61,7 +60,7 @@ struct PlanView {
     int mres;                     // order stride: order index k is the order m = k mres
     const float4 *twdf;           // FP64 plans: tw as double-float pairs (re.hi, re.lo, im.hi, im.lo)
     // FP32 plans: restart states of the recurrence (see kSeedSeg), [segment][npairs]
-    // float4 (y1, y2, k as int bits, 0), segments of order index m from segoff[m].
+    // float4 (y1, y2, factor, 0) with P = factor y, segments of order index m from segoff[m].
     const float4 *seeds;
     const unsigned long long *segoff;
     // FP64 plans: the same states as (y1, y2) 2^hseg and k, [segment][npairs].
@@ -71,6 +70,10 @@ struct PlanView {
     // first kSeedSeg-degree segment holding a |P_n^m| at or above the
     // threshold (the segment count when none does), [mmax+1][npairs].
     const unsigned short *live;
+    // The same per group of 32 pairs, [mmax+1][ceil(npairs/32)]; and the first
+    // segment in which some value of the group enters sums at any threshold
+    // (the vector transforms have no threshold).
+    const unsigned short *glive, *glive_vec;
     // FP64 plans: recurrences of legendre64.cu for degrees m .. lmax + 1 of every
     // order, order index m from col_of_mres(lmax + 1, m, mres): (beta_n, s_n) of
     // Q_n = P_n / s_n, (a_n, b_n) of P_n, eps_n; and the state scale of each segment.
@@ -82,8 +85,7 @@ struct PlanView {
 
 // The FP32 Legendre kernels restart the recurrence of Sec. 3.2 every kSeedSeg
 // degrees from the state (P_{n0-1}, P_{n0-2}) computed by the FP64 recurrence,
-// carried in the exponent-scaled form of Sec. 3.5 (y * 2^(-64 k)), so that
-// FP32 rounding errors accumulate over at most kSeedSeg steps.
+// times a power of two where it is small (Sec. 3.5), so that FP32 rounding errors accumulate over at most kSeedSeg steps.
 constexpr int kSeedSeg = 32;
 
 // First packed index of order index k (order m = k mres): the degrees of the
@@ -128,9 +130,9 @@ enum Op {
 };
 
 // Kernel shapes chosen by sht_tune for one (precision, batch).  FP64: synth_lpt
-// is the warps per CTA, analys_lpt is not used (legendre64.cu).
+// is the warps per CTA (legendre64.cu).
 struct TunedShape {
-    int synth_lpt = 0, synth_bc = 0, analys_lpt = 0, analys_bc = 0;
+    int synth_lpt = 0, synth_bc = 0, analys_bc = 0;
     int auto_mode = 1;           // SHT_F32_AUTO: the fastest of SHT_F32, SHT_TC_BF16X3, SHT_TC_OTF
 };
 
@@ -186,6 +188,7 @@ struct Plan {
     double *eps64 = nullptr;
     int *hseg64 = nullptr;
     unsigned short *live32 = nullptr, *live64 = nullptr;   // first live segment per (m, pair), per precision
+    unsigned short *glive32 = nullptr, *glive64 = nullptr; // ... per (m, group of 32 pairs), scalar then vector
     bool polar_thr_set = false;                 // sht_set_polar_threshold was called
     // thresholds of the static polar optimisation of the CUDA-core kernels:
     // the set value, else 2^-40 (FP32) and 2^-64 (FP64, below the rounding of its sums)
@@ -219,20 +222,19 @@ int plan_relive(Plan &p, std::string &err);
 size_t seed_segment_offsets(int lmax, int mmax, int mres, std::vector<unsigned long long> &segoff);
 // One thread per (m, pair): FP32 states (seeds32) or FP64 states (seeds64,
 // seeds64k, scaled by 2^hseg of their segment), and the first segment holding
-// |P| >= thr (thr <= 0: segment 0).
+// |P| >= thr (thr <= 0: segment 0), per pair and per group of 32 pairs.
 cudaError_t launch_build_restarts(const PlanView<double> &pv, const unsigned long long *segoff, float4 *seeds32,
-                                  double2 *seeds64, int *seeds64k, const int *hseg, unsigned short *live, double thr,
-                                  cudaStream_t st);
+                                  double2 *seeds64, int *seeds64k, const int *hseg, unsigned short *live,
+                                  unsigned short *glive, unsigned short *glive_vec, double thr, cudaStream_t st);
 
 // Launchers (legendre.cu, legendre64.cu, fft.cu).  `eo` / `sd` are intermediate
 // buffers of [batch][mmax+1][npairs][2] complex values.
-// FP32.  Explicit kernel shapes (lpt pairs per thread, bc fields per CTA; 0 =
-// default).  Synthesis: lpt in {1,2,4}, bc in {1,2,4}; analysis: lpt in
-// {2,4,8}, bc in {1,2}.
+// FP32.  Explicit kernel shapes (lpt pairs per lane, bc fields per CTA; 0 =
+// default).  Synthesis: lpt in {1,2,4}, bc in {1,2,4}, not both 4; analysis: bc in {1,2}.
 cudaError_t launch_legendre_synth(const PlanView<float> &pv, const float *spec, float *eo, int batch, Op op, int lpt,
                                   int bc, cudaStream_t s);
-cudaError_t launch_legendre_analys(const PlanView<float> &pv, const float *sd, float *spec, int batch, Op op, int lpt,
-                                   int bc, cudaStream_t s);
+cudaError_t launch_legendre_analys(const PlanView<float> &pv, const float *sd, float *spec, int batch, Op op, int bc,
+                                   cudaStream_t s);
 cudaError_t launch_legendre_synth_vec(const PlanView<float> &pv, const float *S, const float *Tc, float *eot,
                                       float *eop, int batch, Op op, cudaStream_t s);
 cudaError_t launch_legendre_analys_vec(const PlanView<float> &pv, const float *sdt, const float *sdp, float *S,
@@ -300,8 +302,9 @@ cudaError_t tc_batch_legendre(Plan &p, bool synth, const float *in, float *out, 
 // Records an error message for sht_last_error and returns `code`.
 int set_error(int code, const std::string &msg);
 int batch_fft_group(int H, int npairs);
-constexpr int kBatchSynthPairs = 256;   // pairs per synthesis tile (128 threads x 2)
-constexpr int kBatchMaxPairs = 512;     // analysis CTA (256 threads x 2 pairs) limit
+constexpr int kBatchSynthPairs = 64;    // pairs per synthesis tile (32 lanes x 2)
+constexpr int kBatchAnalysSegs = 4;     // segments per analysis tile
+constexpr int kBatchMaxPairs = 512;
 
 // Tensor-core path (tc.cu).  `mres` is the plan's order stride everywhere:
 // order index m (0 .. mmax) is the order m mres.
