@@ -15,10 +15,16 @@
 // Tensor-core mode: the fields of one shape form a group whose spectra (a
 // gather kernel copies them in, or the results out) and intermediates are
 // contiguous, so each group's Legendre stage is one batched tcgen05
-// contraction against that plan's P panels; the FFTs stay one persistent
-// launch over all fields.  The captured graph then holds the pointer-table
-// copy, the gather (or scatter), one contraction per group and the FFT.  The
-// automatic mode times both and keeps the faster.
+// contraction against that plan's P panels.  The automatic mode times both and
+// keeps the faster.
+//
+// Up to kMaxGroups shapes, the FFTs are one launch per shape, and each shape's
+// copies, contraction and FFT a branch of the graph of their own: one shape's FFT
+// fills the SMs that another's contraction leaves.
+// (The persistent FFT kernel fetches its tile, the field's plan and pointers one
+// after the other before any data, and runs the registers and shared memory of
+// the largest length: 99 / 86 us for 96 fields of N = 63 .. 511, against 37 / 38
+// us for the four launches on their own.)  More shapes keep the persistent kernel.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -32,6 +38,8 @@
 #include "sht_internal.h"
 
 namespace {
+constexpr size_t kMaxGroups = 8;
+
 // One copy of the gather (synthesis) or scatter (analysis) of the tensor-core mode.
 struct BatchCopy {
     const float2 *src;
@@ -50,12 +58,28 @@ struct sht_batch_plan {
     std::vector<size_t> field_gspec;       // ... per field: its slot in d_gspec, floats
     std::vector<size_t> ginter_off;        // ... per group: its contiguous intermediate in d_inter, floats
     std::vector<size_t> inter_tc;          // ... per field: its intermediate in that layout
-    BatchCopy *h_copies = nullptr, *d_copies = nullptr;
+    // per call: pointer table of the group FFTs and copy list, fields in group order, one
+    // upload from the direction's own pinned staging
+    unsigned char *h_up[2] = {nullptr, nullptr}, *d_up = nullptr;
+    std::vector<size_t> group_first;       // first entry of each group in that order
+    std::vector<int> order;                // groups by falling size
+    bool grouped = false;                  // FFTs by group
+    sht::BatchPtrs *h_ptrs(int dir) const { return reinterpret_cast<sht::BatchPtrs *>(h_up[dir]); }
+    BatchCopy *h_copies(int dir) const
+    {
+        return reinterpret_cast<BatchCopy *>(h_up[dir] + sizeof(sht::BatchPtrs) * nfields);
+    }
+    const sht::BatchPtrs *d_ptrs() const { return reinterpret_cast<const sht::BatchPtrs *>(d_up); }
+    const BatchCopy *d_copies() const
+    {
+        return reinterpret_cast<const BatchCopy *>(d_up + sizeof(sht::BatchPtrs) * nfields);
+    }
+    size_t up_bytes() const { return (sizeof(sht::BatchPtrs) + sizeof(BatchCopy)) * nfields; }
     float tuned_ms[2] = {0.f, 0.f};        // automatic mode: round trip per path (CUDA cores, tensor cores)
     std::vector<std::unique_ptr<sht::Plan>> plans;   // one per distinct shape
     std::vector<int> field_plan;
     std::vector<int> lmax, nlat, nphi;
-    sht::BatchField *h_fields = nullptr;   // pinned staging of the pointer table
+    sht::BatchField *h_fields[2] = {nullptr, nullptr};   // pinned staging of the field table, per direction
     sht::BatchField *d_fields = nullptr;
     int4 *d_tiles = nullptr;               // [synth legendre | synth fft | analys fft | analys legendre]
     int ntile[4] = {0, 0, 0, 0};
@@ -66,7 +90,8 @@ struct sht_batch_plan {
     size_t fft_smem = 0;
     int ctas_legendre_syn = 0, ctas_legendre_ana = 0, ctas_fft = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};   // synthesis, analysis
-    cudaEvent_t done = nullptr;                      // last launch (guards h_fields reuse)
+    cudaEvent_t used[2] = {nullptr, nullptr};        // last launch of each direction (guards its staging)
+    cudaEvent_t done = nullptr;                      // last launch (guards the device buffers)
 };
 
 namespace {
@@ -79,9 +104,12 @@ void free_batch(sht_batch_plan *b)
     for (auto &g : b->graph)
         if (g) cudaGraphExecDestroy(g);
     if (b->done) cudaEventDestroy(b->done);
-    if (b->h_fields) cudaFreeHost(b->h_fields);
-    if (b->h_copies) cudaFreeHost(b->h_copies);
-    cudaFree(b->d_copies);
+    for (int dir = 0; dir < 2; ++dir) {
+        if (b->used[dir]) cudaEventDestroy(b->used[dir]);
+        if (b->h_fields[dir]) cudaFreeHost(b->h_fields[dir]);
+        if (b->h_up[dir]) cudaFreeHost(b->h_up[dir]);
+    }
+    cudaFree(b->d_up);
     cudaFree(b->d_gspec);
     cudaFree(b->d_fields);
     cudaFree(b->d_tiles);
@@ -92,32 +120,66 @@ void free_batch(sht_batch_plan *b)
     delete b;
 }
 
-// Gather / scatter of the tensor-core mode: blockIdx.y = copy.
+// Gather / scatter of the tensor-core mode: blockIdx.y = copy, kCopyPer complex
+// values per thread.  16 bytes at a time where source and destination lie alike
+// on 16 bytes (a field's spectrum starts on 8), all loads before the stores.
+constexpr int kCopyPer = 8;
 __global__ void __launch_bounds__(256) k_batch_copy(const BatchCopy *__restrict__ copies)
 {
     const BatchCopy c = copies[blockIdx.y];
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < c.n; i += (long long)gridDim.x * blockDim.x)
-        c.dst[i] = c.src[i];
+    const size_t sa = reinterpret_cast<size_t>(c.src) & 15, da = reinterpret_cast<size_t>(c.dst) & 15;
+    if (sa == da) {
+        const long long lead = sa ? 1 : 0, n4 = (c.n - lead) >> 1;
+        const float4 *src = reinterpret_cast<const float4 *>(c.src + lead);
+        float4 *dst = reinterpret_cast<float4 *>(c.dst + lead);
+        const long long i0 = (long long)blockIdx.x * (256 * kCopyPer / 2) + threadIdx.x;
+        float4 v[kCopyPer / 2];
+#pragma unroll
+        for (int u = 0; u < kCopyPer / 2; ++u)
+            if (i0 + 256 * u < n4) v[u] = src[i0 + 256 * u];
+#pragma unroll
+        for (int u = 0; u < kCopyPer / 2; ++u)
+            if (i0 + 256 * u < n4) dst[i0 + 256 * u] = v[u];
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            if (lead) c.dst[0] = c.src[0];
+            if (lead + 2 * n4 < c.n) c.dst[c.n - 1] = c.src[c.n - 1];
+        }
+        return;
+    }
+    const long long i0 = (long long)blockIdx.x * (256 * kCopyPer) + threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < kCopyPer; ++u)
+        if (i0 + 256 * u < c.n) c.dst[i0 + 256 * u] = c.src[i0 + 256 * u];
 }
 
-// Fill the pointer table (and the tensor-core mode's copy list) for one call.
+// Fill the per-call tables.
 void fill_fields(sht_batch_plan *b, bool synth, void *const *in, void *const *out)
 {
     const bool tc = b->mode == SHT_TC_BF16X3;
+    const int dir = synth ? 0 : 1;
+    for (size_t g = 0; g < b->group_fields.size(); ++g)
+        for (size_t i = 0; i < b->group_fields[g].size(); ++i) {
+            const int f = b->group_fields[g][i];
+            const size_t at = b->group_first[g] + i;
+            sht::BatchPtrs &q = b->h_ptrs(dir)[at];
+            q.in = static_cast<const float *>(in[f]);
+            q.out = static_cast<float *>(out[f]);
+            q.inter = b->d_inter + (tc ? b->inter_tc[f] : b->inter_off[f]);
+            if (!tc) continue;
+            BatchCopy &c = b->h_copies(dir)[at];
+            float2 *slot = reinterpret_cast<float2 *>(b->d_gspec + b->field_gspec[f]);
+            c.n = b->plans[g]->nlm;
+            c.src = synth ? static_cast<const float2 *>(in[f]) : slot;
+            c.dst = synth ? slot : static_cast<float2 *>(out[f]);
+        }
+    if (tc && b->grouped) return;   // only the persistent kernels read the field table
     for (int f = 0; f < b->nfields; ++f) {
-        sht::BatchField &bf = b->h_fields[f];
+        sht::BatchField &bf = b->h_fields[dir][f];
         const sht::Plan &p = *b->plans[b->field_plan[f]];
         bf.pv = p.view32();
         bf.in = static_cast<const float *>(in[f]);
         bf.out = static_cast<float *>(out[f]);
         bf.inter = b->d_inter + (tc ? b->inter_tc[f] : b->inter_off[f]);
-        if (tc) {
-            BatchCopy &c = b->h_copies[f];
-            float2 *slot = reinterpret_cast<float2 *>(b->d_gspec + b->field_gspec[f]);
-            c.n = p.nlm;
-            c.src = synth ? static_cast<const float2 *>(in[f]) : slot;
-            c.dst = synth ? slot : static_cast<float2 *>(out[f]);
-        }
         // row FFT tiles for power-of-two lengths <= 2^10, else the mixed-radix kernel
         const int H = p.nphi / 2;
         int logH = 0;
@@ -127,61 +189,105 @@ void fill_fields(sht_batch_plan *b, bool synth, void *const *in, void *const *ou
     }
 }
 
-cudaError_t launch_copies(sht_batch_plan *b, cudaStream_t s)
+// One group's copies, contraction and FFT.
+cudaError_t group_copies(sht_batch_plan *b, int g, cudaStream_t s)
 {
-    k_batch_copy<<<dim3(16, (unsigned)b->nfields), 256, 0, s>>>(b->d_copies);
+    const int n = b->plans[g]->nlm;
+    const dim3 grid((unsigned)((n + 256 * kCopyPer - 1) / (256 * kCopyPer)), (unsigned)b->group_fields[g].size());
+    k_batch_copy<<<grid, 256, 0, s>>>(b->d_copies() + b->group_first[g]);
     return cudaGetLastError();
 }
 
-// Tensor-core mode: one contraction per group of equal shape.
-cudaError_t group_contractions(sht_batch_plan *b, bool synth, cudaStream_t s)
+cudaError_t group_contraction(sht_batch_plan *b, bool synth, int g, cudaStream_t s)
 {
-    for (size_t g = 0; g < b->group_fields.size(); ++g) {
-        sht::Plan &p = *b->plans[g];
-        float *spec = b->d_gspec + b->gspec_off[g], *inter = b->d_inter + b->ginter_off[g];
-        const int nb = (int)b->group_fields[g].size();
-        cudaError_t e = synth ? sht::tc_batch_legendre(p, true, spec, inter, nb, s)
-                              : sht::tc_batch_legendre(p, false, inter, spec, nb, s);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    float *spec = b->d_gspec + b->gspec_off[g], *inter = b->d_inter + b->ginter_off[g];
+    const int nb = (int)b->group_fields[g].size();
+    return synth ? sht::tc_batch_legendre(*b->plans[g], true, spec, inter, nb, s)
+                 : sht::tc_batch_legendre(*b->plans[g], false, inter, spec, nb, s);
 }
 
-// Enqueue the steps of one direction on stream s.
-cudaError_t enqueue(sht_batch_plan *b, bool synth, cudaStream_t s)
+cudaError_t group_fft(sht_batch_plan *b, bool synth, int g, cudaStream_t s)
 {
-    cudaError_t e = cudaMemcpyAsync(b->d_fields, b->h_fields, sizeof(sht::BatchField) * b->nfields,
-                                    cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(b->d_counters, 0, 4 * sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    if (b->mode == SHT_TC_BF16X3) {
-        e = cudaMemcpyAsync(b->d_copies, b->h_copies, sizeof(BatchCopy) * b->nfields, cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) return e;
-        if (synth) {
-            if ((e = launch_copies(b, s)) != cudaSuccess) return e;
-            if ((e = group_contractions(b, true, s)) != cudaSuccess) return e;
-            return sht::launch_batch_fft(true, b->d_fields, b->d_tiles + b->tile_off[1], b->ntile[1],
-                                         b->d_counters + 1, b->ctas_fft, b->fft_smem, s);
+    return sht::launch_group_fft(synth, b->plans[g]->view32(), b->d_ptrs() + b->group_first[g],
+                                 (int)b->group_fields[g].size(), s);
+}
+
+// A stream per group beside `main` while a graph is captured (empty otherwise:
+// every step then runs on `main`).  Fork and join through events.
+struct Branches {
+    cudaStream_t main = nullptr;
+    std::vector<cudaStream_t> streams;
+    std::vector<cudaEvent_t> events;
+    cudaError_t err = cudaSuccess;
+
+    cudaStream_t of(int g) const { return streams.empty() ? main : streams[g]; }
+    // `to` goes on once what `from` holds so far is done
+    void after(cudaStream_t to, cudaStream_t from)
+    {
+        if (to == from || err != cudaSuccess) return;
+        cudaEvent_t ev = nullptr;
+        err = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (err != cudaSuccess) return;
+        events.push_back(ev);
+        err = cudaEventRecord(ev, from);
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(to, ev, 0);
+    }
+    void run(cudaError_t e) { if (err == cudaSuccess) err = e; }
+    cudaError_t open(cudaStream_t s, int groups, bool fork)
+    {
+        main = s;
+        for (int g = 0; g < groups && fork && err == cudaSuccess; ++g) {
+            cudaStream_t t = nullptr;
+            err = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
+            if (err == cudaSuccess) streams.push_back(t);
         }
-        e = sht::launch_batch_fft(false, b->d_fields, b->d_tiles + b->tile_off[2], b->ntile[2], b->d_counters + 2,
-                                  b->ctas_fft, b->fft_smem, s);
-        if (e != cudaSuccess) return e;
-        if ((e = group_contractions(b, false, s)) != cudaSuccess) return e;
-        return launch_copies(b, s);
+        return err;
     }
-    if (synth) {
-        e = sht::launch_batch_legendre(true, b->d_fields, b->d_tiles + b->tile_off[0], b->ntile[0], b->d_counters + 0,
-                                       b->ctas_legendre_syn, s);
-        if (e != cudaSuccess) return e;
-        return sht::launch_batch_fft(true, b->d_fields, b->d_tiles + b->tile_off[1], b->ntile[1], b->d_counters + 1,
-                                     b->ctas_fft, b->fft_smem, s);
+    ~Branches()
+    {
+        for (cudaEvent_t e : events) cudaEventDestroy(e);
+        for (cudaStream_t t : streams) cudaStreamDestroy(t);
     }
-    e = sht::launch_batch_fft(false, b->d_fields, b->d_tiles + b->tile_off[2], b->ntile[2], b->d_counters + 2,
-                              b->ctas_fft, b->fft_smem, s);
-    if (e != cudaSuccess) return e;
-    return sht::launch_batch_legendre(false, b->d_fields, b->d_tiles + b->tile_off[3], b->ntile[3], b->d_counters + 3,
-                                      b->ctas_legendre_ana, s);
+};
+
+// Enqueue the steps of one direction on stream s, those of a group on its branch.
+cudaError_t enqueue(sht_batch_plan *b, bool synth, cudaStream_t s, Branches &br)
+{
+    const bool tc = b->mode == SHT_TC_BF16X3;
+    const int ng = (int)b->plans.size();
+    br.run(cudaMemcpyAsync(b->d_up, b->h_up[synth ? 0 : 1], b->up_bytes(), cudaMemcpyHostToDevice, s));
+    if (!tc || !b->grouped) {
+        br.run(cudaMemcpyAsync(b->d_fields, b->h_fields[synth ? 0 : 1], sizeof(sht::BatchField) * b->nfields,
+                               cudaMemcpyHostToDevice, s));
+        br.run(cudaMemsetAsync(b->d_counters, 0, 4 * sizeof(int), s));
+    }
+    const auto persistent_fft = [&] {
+        const int k = synth ? 1 : 2;
+        br.run(sht::launch_batch_fft(synth, b->d_fields, b->d_tiles + b->tile_off[k], b->ntile[k], b->d_counters + k,
+                                     b->ctas_fft, b->fft_smem, s));
+    };
+    const auto legendre = [&] {
+        const int k = synth ? 0 : 3;
+        br.run(sht::launch_batch_legendre(synth, b->d_fields, b->d_tiles + b->tile_off[k], b->ntile[k],
+                                          b->d_counters + k, synth ? b->ctas_legendre_syn : b->ctas_legendre_ana, s));
+    };
+    // each group's steps follow one another on its branch, the largest group first
+    if (synth && !tc) legendre();
+    if (!synth && !b->grouped) persistent_fft();
+    for (int i = 0; i < ng && (tc || b->grouped); ++i) {
+        const int g = b->order[i];
+        cudaStream_t gs = br.of(g);
+        br.after(gs, s);
+        if (!synth && b->grouped) br.run(group_fft(b, false, g, gs));
+        if (tc && synth) br.run(group_copies(b, g, gs));
+        if (tc) br.run(group_contraction(b, synth, g, gs));
+        if (tc && !synth) br.run(group_copies(b, g, gs));
+        if (synth && b->grouped) br.run(group_fft(b, true, g, gs));
+    }
+    for (int g = 0; g < ng; ++g) br.after(s, br.of(g));
+    if (synth && !b->grouped) persistent_fft();
+    if (!synth && !tc) legendre();
+    return br.err;
 }
 
 int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int use_graph, void *stream)
@@ -194,11 +300,14 @@ int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int us
     if (cudaGetDevice(&dev) != cudaSuccess || dev != b->device)
         return bfail(SHT_EINVAL, "current CUDA device differs from the batch plan's device");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the previous launch copies h_fields when it runs: wait for it before overwriting
-    cudaError_t e = cudaEventSynchronize(b->done);
+    // this direction's previous launch copies its staging when it runs: the host
+    // waits for it before overwriting; the other direction's launch may still be
+    // running, and the stream waits for it before this one uses the device buffers
+    const int dir = synth ? 0 : 1;
+    cudaError_t e = cudaEventSynchronize(b->used[dir]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b->done, 0);
     if (e != cudaSuccess) return bfail(SHT_ECUDA, std::string("waiting for the previous batch call: ") + cudaGetErrorString(e));
     fill_fields(b, synth, in, out);
-    const int dir = synth ? 0 : 1;
     if (use_graph) {
         if (!b->graph[dir]) {
             cudaStream_t cs;
@@ -207,7 +316,9 @@ int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int us
             cudaGraph_t g = nullptr;
             e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
-                cudaError_t e2 = enqueue(b, synth, cs);
+                Branches br;
+                cudaError_t e2 = br.open(cs, (int)b->plans.size(), b->grouped);
+                if (e2 == cudaSuccess) e2 = enqueue(b, synth, cs, br);
                 e = cudaStreamEndCapture(cs, &g);
                 if (e == cudaSuccess) e = e2;
             }
@@ -221,8 +332,11 @@ int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int us
         }
         e = cudaGraphLaunch(b->graph[dir], s);
     } else {
-        e = enqueue(b, synth, s);
+        Branches br;
+        br.open(s, 0, false);
+        e = enqueue(b, synth, s, br);
     }
+    if (e == cudaSuccess) e = cudaEventRecord(b->used[dir], s);
     if (e == cudaSuccess) e = cudaEventRecord(b->done, s);
     if (e != cudaSuccess) return bfail(SHT_ECUDA, std::string("batch launch: ") + cudaGetErrorString(e));
     return SHT_OK;
@@ -344,6 +458,17 @@ int sht_batch_create_mode(int nfields, const int *lmax, const int *nlat, const i
     }
     b->group_fields.assign(b->plans.size(), std::vector<int>());
     for (int f = 0; f < nfields; ++f) b->group_fields[b->field_plan[f]].push_back(f);
+    b->grouped = b->plans.size() <= kMaxGroups;
+    size_t first = 0;
+    std::vector<double> work;   // of a group: panel bytes and data
+    for (size_t g = 0; g < b->plans.size(); ++g) {
+        const sht::Plan &p = *b->plans[g];
+        b->group_first.push_back(first);
+        first += b->group_fields[g].size();
+        b->order.push_back((int)g);
+        work.push_back((double)p.nlm * p.npairs * 4 + (double)b->group_fields[g].size() * p.nlat * p.nphi * 8);
+    }
+    std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) { return work[x] > work[y]; });
     // intermediates, tile lists (longest first)
     size_t inter = 0;
     std::vector<std::pair<double, int4>> syn, ffts, ana;
@@ -421,14 +546,18 @@ int sht_batch_create_mode(int nfields, const int *lmax, const int *nlat, const i
     b->ctas_legendre_syn = sms * 8;   // 128-thread CTAs
     b->ctas_legendre_ana = sms * 4;   // 128-thread CTAs of independent warps
     b->ctas_fft = sms * std::max(1, (int)std::min<size_t>(8, (200 * 1024) / std::max<size_t>(smem, 1)));
-    cudaError_t e = cudaMallocHost(&b->h_fields, sizeof(sht::BatchField) * nfields);
+    cudaError_t e = cudaSuccess;
+    for (int dir = 0; dir < 2; ++dir) {
+        if (e == cudaSuccess) e = cudaMallocHost(&b->h_fields[dir], sizeof(sht::BatchField) * nfields);
+        if (e == cudaSuccess) e = cudaMallocHost(&b->h_up[dir], b->up_bytes());
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->used[dir], cudaEventDisableTiming);
+    }
     if (e == cudaSuccess) e = cudaMalloc(&b->d_fields, sizeof(sht::BatchField) * nfields);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, sizeof(int4) * tiles.size());
     if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, 4 * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_inter, sizeof(float) * std::max<size_t>(inter, 64));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && tc_ok) e = cudaMallocHost(&b->h_copies, sizeof(BatchCopy) * nfields);
-    if (e == cudaSuccess && tc_ok) e = cudaMalloc(&b->d_copies, sizeof(BatchCopy) * nfields);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_up, b->up_bytes());
     if (e == cudaSuccess && tc_ok) e = cudaMalloc(&b->d_gspec, sizeof(float) * std::max<size_t>(gspec, 64));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming);
     if (e != cudaSuccess) {

@@ -1550,7 +1550,84 @@ cudaError_t launch_fft_analys_df(const PlanView<double> &pv, const double *grid,
 }
 
 // ---------------------------------------------------------------------------
-// Persistent FFT kernels for uneven batches (FP32, 256 threads, one field per tile).
+// FFTs of the fields of one shape of an uneven batch: the tiles of the regular
+// launches, with each field's buffers from a table (blockIdx.y = field).
+// ---------------------------------------------------------------------------
+namespace {
+
+template <int LOGH, bool SYNTH>
+__global__ void __launch_bounds__(64 * kRowPairs, 2)
+k_group_rows(PlanView<float> pv, const BatchPtrs *__restrict__ ptrs)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const BatchPtrs f = ptrs[blockIdx.y];
+    const int p0 = blockIdx.x * RowPairs<LOGH>::n;
+    if constexpr (SYNTH) fft_synth_rows_tile<LOGH>(pv, f.inter, f.out, 0, p0, OP_SYNTH, smem_raw);
+    else fft_analys_rows_tile<LOGH>(pv, f.in, f.inter, 0, p0, OP_ANALYS, 0, smem_raw);
+}
+
+template <bool MIXED, bool SYNTH>
+__global__ void __launch_bounds__(512)
+k_group_tiles(PlanView<float> pv, const BatchPtrs *__restrict__ ptrs, int G)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const BatchPtrs f = ptrs[blockIdx.y];
+    const int p0 = blockIdx.x * G;
+    if constexpr (SYNTH)
+        fft_synth_tile<float, MIXED>(pv, f.inter, f.out, 0, p0, G, OP_SYNTH, pv.fftplan, smem_raw);
+    else
+        fft_analys_tile<float, MIXED>(pv, f.in, f.inter, 0, p0, G, OP_ANALYS, 0, pv.fftplan, smem_raw);
+}
+
+template <int LOGH, bool SYNTH>
+cudaError_t group_rows(const PlanView<float> &pv, const BatchPtrs *ptrs, int nfields, cudaStream_t s)
+{
+    constexpr int RP = RowPairs<LOGH>::n;
+    const size_t smem = row_fft_smem(RowShape<LOGH>::LD, RP);
+    cudaError_t e = set_smem(k_group_rows<LOGH, SYNTH>, smem);
+    if (e != cudaSuccess) return e;
+    dim3 g((unsigned)((pv.npairs + RP - 1) / RP), (unsigned)nfields);
+    k_group_rows<LOGH, SYNTH><<<g, 64 * kRowPairs, smem, s>>>(pv, ptrs);
+    return cudaGetLastError();
+}
+
+template <bool MIXED, bool SYNTH>
+cudaError_t group_tiles(const PlanView<float> &pv, const BatchPtrs *ptrs, int nfields, cudaStream_t s)
+{
+    int G, threads;
+    size_t smem;
+    fft_shape<float>(pv.nphi / 2, 16, pv.npairs, nfields, G, threads, smem);
+    cudaError_t e = set_smem(k_group_tiles<MIXED, SYNTH>, smem);
+    if (e != cudaSuccess) return e;
+    dim3 g((unsigned)((pv.npairs + G - 1) / G), (unsigned)nfields);
+    k_group_tiles<MIXED, SYNTH><<<g, threads, smem, s>>>(pv, ptrs, G);
+    return cudaGetLastError();
+}
+
+template <bool SYNTH>
+cudaError_t group_fft(const PlanView<float> &pv, const BatchPtrs *ptrs, int nfields, cudaStream_t s)
+{
+    const int H = pv.nphi / 2;
+    if (!pow2(H)) return group_tiles<true, SYNTH>(pv, ptrs, nfields, s);
+    switch (ilog2(H)) {
+#define SHT_GROUP_CASE(L) case L: return group_rows<L, SYNTH>(pv, ptrs, nfields, s);
+        SHT_GROUP_CASE(0) SHT_GROUP_CASE(1) SHT_GROUP_CASE(2) SHT_GROUP_CASE(3) SHT_GROUP_CASE(4) SHT_GROUP_CASE(5)
+        SHT_GROUP_CASE(6) SHT_GROUP_CASE(7) SHT_GROUP_CASE(8) SHT_GROUP_CASE(9) SHT_GROUP_CASE(10)
+#undef SHT_GROUP_CASE
+    default: return group_tiles<false, SYNTH>(pv, ptrs, nfields, s);
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_group_fft(bool synth, const PlanView<float> &pv, const BatchPtrs *ptrs, int nfields, cudaStream_t s)
+{
+    return synth ? group_fft<true>(pv, ptrs, nfields, s) : group_fft<false>(pv, ptrs, nfields, s);
+}
+
+// ---------------------------------------------------------------------------
+// Persistent FFT kernel for uneven batches of many shapes (FP32, 256 threads, one
+// field per tile).
 // ---------------------------------------------------------------------------
 namespace {
 

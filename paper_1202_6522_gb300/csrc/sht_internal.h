@@ -291,6 +291,14 @@ cudaError_t launch_batch_legendre(bool synth, const BatchField *fields, const in
 cudaError_t launch_batch_fft(bool synth, const BatchField *fields, const int4 *tiles, int ntiles, int *counter,
                              int ctas, size_t smem, cudaStream_t s);
 size_t batch_fft_smem(int H, int G);
+// The fields of one shape (same plan) in one launch: field f reads ptrs[f].in and
+// writes ptrs[f].inter (analysis) or reads inter and writes out (synthesis).
+struct BatchPtrs {
+    const float *in;
+    float *out;
+    float *inter;
+};
+cudaError_t launch_group_fft(bool synth, const PlanView<float> &pv, const BatchPtrs *ptrs, int nfields, cudaStream_t s);
 cudaError_t batch_fft_prepare(size_t smem);   // once, outside any stream capture
 
 // Uneven batches on the tensor cores (capi.cu): panels + operand scratch of a
