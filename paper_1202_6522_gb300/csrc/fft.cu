@@ -224,16 +224,24 @@ struct RegDft<T2, 5, SIGN> {
 template <bool MIXED, int V = 16> struct PassRegs { static constexpr int n = !MIXED ? V : (V == 16 ? 20 : 6); };
 template <int V = 16> __host__ __device__ inline int row_tpr(int H) { return (H + V - 1) / V; }
 
-// Values per thread.  FP32: 16, two radix-16 passes with few barriers.  FP64 up
-// to H = 1024 (512 threads for two rows): 4.  The FP64 pipe takes a warp
-// instruction every ~64 cycles per SM quarter, so a row spread over four times
-// the threads keeps all four quarters busy where a launch has few rows, at the
-// same instruction count (radix 4: 28 FP64 instructions per 4 points and pass,
-// four passes; radix 16: 228 per 16 points, two passes).  One field of 256 x 512
-// points: 51 / 54 us with 16 values and 8 pairs per CTA (16 CTAs), 28 / 27 us
-// with one pair per CTA, 10.2 / 10.3 us with 4 values; 16 fields of 512 x 1024:
-// 373 / 417 -> 334 / 360 us (synthesis / analysis).
-template <typename T> inline int fft_values(int H) { return sizeof(T) == 8 && H <= 1024 ? 4 : 16; }
+// Values per thread.  FP64 up to H = 1024 (512 threads for two rows): 4.  The
+// FP64 pipe takes a warp instruction every ~64 cycles per SM quarter, so a row
+// spread over four times the threads keeps all four quarters busy where a launch
+// has few rows, at the same instruction count (radix 4: 28 FP64 instructions per 4
+// points and pass, four passes; radix 16: 228 per 16 points, two passes).  One
+// field of 256 x 512 points: 51 / 54 us with 16 values and 8 pairs per CTA (16
+// CTAs), 28 / 27 us with one pair per CTA, 10.2 / 10.3 us with 4 values; 16 fields
+// of 512 x 1024: 373 / 417 -> 334 / 360 us (synthesis / analysis).
+// FP32: 16, two radix-16 passes with few barriers; but 4 for mixed radices in the
+// synthesis up to H = 1024 and the analysis up to H = 256, where the 16-value
+// passes leave threads without items (6 fields of 288 x 384: 9.2 / 9.2 -> 6.2 /
+// 6.7 us; 32 of 384 x 1152: synthesis 80 -> 66 us, analysis 88 -> 93).
+template <typename T> inline int fft_values(int H, bool synth)
+{
+    const bool p2 = (H & (H - 1)) == 0;
+    if (sizeof(T) == 8) return H <= 1024 ? 4 : 16;
+    return !p2 && H <= (synth ? 1024 : 256) ? 4 : 16;
+}
 
 // One Stockham pass of radix RD over a row of length H held in `row` (padded
 // indices) or, for the first/last pass, in global memory.  Each thread owns
@@ -243,14 +251,25 @@ template <typename T> inline int fft_values(int H) { return sizeof(T) == 8 && H 
 // log2 of a power of two
 __device__ __forceinline__ int lg2(int v) { return __popc(v - 1); }
 
+// q / d for 0 <= q < 2^19 and d >= 1 with q / d < 2^13 by one FP32 product (an
+// integer division by a run-time value is a long instruction sequence): the
+// rounding of (q + 1/2) (1/d) moves it by less than 2^-22 q/d < 1 / (2 d), its
+// distance from an integer, while d q/d < 2^21.
+struct FastDiv {
+    float inv;
+    __device__ __forceinline__ explicit FastDiv(int d) : inv(1.0f / (float)d) {}
+    __device__ __forceinline__ int operator()(int q) const { return (int)(((float)q + 0.5f) * inv); }
+};
+
 // P2: every length involved is a power of two, so the index arithmetic is
-// masks and shifts (a division by a run-time value is a long instruction
-// sequence on the integer pipe, which the FFT kernels are short of).
+// masks and shifts.  r q0 < H in either form: q0 < H / RD.
 template <typename T2, int RD, int SIGN, int NR, bool P2, int V = 16>
 __device__ __forceinline__ void stockham_load(const T2 *src, bool global_src, int t, int TPR, int H, int Ns,
                                               const T2 *__restrict__ wtab, T2 (&v)[NR])
 {
     constexpr int IT = (V + RD - 1) / RD;
+    const FastDiv div(Ns);
+    const int wstep = P2 ? 0 : H / (Ns * RD);
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
         const int j = t + it * TPR;
@@ -262,10 +281,10 @@ __device__ __forceinline__ void stockham_load(const T2 *src, bool global_src, in
             a[r] = global_src ? src[idx] : src[padi(idx)];
         }
         if (Ns > 1) {
-            const int q0 = P2 ? (j & (Ns - 1)) << (lg2(H) - lg2(Ns) - lg2(RD)) : (j % Ns) * (H / (Ns * RD));
+            const int q0 = P2 ? (j & (Ns - 1)) << (lg2(H) - lg2(Ns) - lg2(RD)) : (j - div(j) * Ns) * wstep;
 #pragma unroll
             for (int r = 1; r < RD; ++r) {
-                T2 w = wtab[P2 ? (r * q0) & (H - 1) : (r * q0) % H];
+                T2 w = wtab[r * q0];
                 if (SIGN < 0) w = conj_(w);
                 a[r] = cmul(a[r], w);
             }
@@ -276,23 +295,26 @@ __device__ __forceinline__ void stockham_load(const T2 *src, bool global_src, in
     }
 }
 
-template <typename T2, int RD, bool P2>
-__device__ __forceinline__ int stockham_out(int j, int r, int Ns)
+// First output position of item j: y[(j / Ns) Ns RD + j mod Ns + r Ns].
+template <int RD, bool P2>
+__device__ __forceinline__ int stockham_out(int j, int Ns, const FastDiv &div)
 {
-    if (P2) return ((j & ~(Ns - 1)) * RD) + (j & (Ns - 1)) + r * Ns;
-    return (j / Ns) * Ns * RD + (j % Ns) + r * Ns;
+    if (P2) return ((j & ~(Ns - 1)) * RD) + (j & (Ns - 1));
+    return j + div(j) * Ns * (RD - 1);
 }
 
 template <typename T2, int RD, int NR, bool P2, int V = 16>
 __device__ __forceinline__ void stockham_store_smem(T2 *row, int t, int TPR, int H, int Ns, const T2 (&v)[NR])
 {
     constexpr int IT = (V + RD - 1) / RD;
+    const FastDiv div(Ns);
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
         const int j = t + it * TPR;
         if (j >= H / RD) break;
+        const int o = stockham_out<RD, P2>(j, Ns, div);
 #pragma unroll
-        for (int r = 0; r < RD; ++r) row[padi(stockham_out<T2, RD, P2>(j, r, Ns))] = v[it * RD + r];
+        for (int r = 0; r < RD; ++r) row[padi(o + r * Ns)] = v[it * RD + r];
     }
 }
 
@@ -412,8 +434,9 @@ __device__ __forceinline__ void fft_synth_tile(const PlanView<T> &pv, const T *_
 
     fill_wtab(wtab, pv.tw, H);
     // 1. spectra of the 2G rows, natural order, zero padded above mmax
+    const FastDiv byG(G), byHalf(H / 2 + 1);
     for (int q = threadIdx.x; q < G * H; q += blockDim.x) {
-        const int m = q / G, i = q - m * G;
+        const int m = byG(q), i = q - m * G;
         const int p = p0 + i;
         T2 XN = mk<T2>(T(0), T(0)), XS = XN;
         if (m <= mmax && p < npairs) {
@@ -431,7 +454,7 @@ __device__ __forceinline__ void fft_synth_tile(const PlanView<T> &pv, const T *_
     //    W = e^{2 pi i / (2H)}: Z_k = A + i P and, since W^{H-k} = -conj W^k,
     //    Z_{H-k} = conj A + i conj P (one product for both positions); X_H = 0
     for (int q = threadIdx.x; q < R * (H / 2 + 1); q += blockDim.x) {
-        const int r = q / (H / 2 + 1), k = q - r * (H / 2 + 1);
+        const int r = byHalf(q), k = q - r * (H / 2 + 1);
         T2 *row = buf + r * ld;
         if (k == 0) {
             const T2 X0 = row[0];
@@ -577,8 +600,9 @@ __device__ __forceinline__ void fft_analys_tile(const PlanView<T> &pv, const T *
         sd2[o + 1] = d;
     };
     const int mhalf = min(H / 2, mmax);
+    const FastDiv byG(G);
     for (int q = threadIdx.x; q < G * (mhalf + 1); q += blockDim.x) {
-        const int m = q / G, i = q - m * G;
+        const int m = byG(q), i = q - m * G;
         const int pp = p0 + i;
         if (pp >= npairs) continue;
         const int m2 = H - m;   // its partner, when it is another position and an order of the plan
@@ -714,13 +738,13 @@ __host__ __device__ constexpr size_t df_extra_smem(int G) { return (size_t)4 * (
 // Legendre output arrives as FP64 E, O; they are staged unconverted in the
 // rows while the pair's largest exponent is found, then converted in the
 // pre-twiddle.
-template <bool MIXED, int LOGH = 0>
+template <bool MIXED, int LOGH, int V>
 __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, const double *__restrict__ eo,
                                                   double *__restrict__ grid, int b, int p0, int G, int op,
-                                                  unsigned char *smem_raw)
+                                                  unsigned long long plan, unsigned char *smem_raw)
 {
     const int H = LOGH ? (1 << LOGH) : pv.nphi / 2, R = 2 * G;
-    const int TPR = row_tpr(H);
+    const int TPR = row_tpr<V>(H);
     const int ld = padi(H) + 1;
     dfl2 *wtab = reinterpret_cast<dfl2 *>(smem_raw);
     dfl2 *buf = wtab + H;
@@ -739,13 +763,12 @@ __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, co
     }
     __syncthreads();
     // 1. E (row 2i) and O (row 2i+1) of the G pairs in natural order, zero
-    //    above mmax, and the largest exponent per pair (G is a power of two
-    //    unless the plan has fewer pairs: shifts, not divisions, split q)
-    const bool gp2 = (G & (G - 1)) == 0;
-    const int lgG = __popc(G - 1);
+    //    above mmax, and the largest exponent per pair
+    const FastDiv byG(G), byHalf(H / 2 + 1);
     {
-        // the loads of U items are issued before their stores (latency, not bandwidth, is the limit here)
-        constexpr int U = 8;
+        // the loads of U items are issued before their stores (latency, not bandwidth, is the
+        // limit here); a thread of V = 4 has two items
+        constexpr int U = V == 4 ? 2 : 8;
         int cur = -1, emax = 0;
         for (int q0 = threadIdx.x; q0 < G * H; q0 += U * blockDim.x) {
             double2 E[U], O[U];
@@ -755,7 +778,7 @@ __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, co
                 E[u] = make_double2(0.0, 0.0);
                 O[u] = E[u];
                 if (q < G * H) {
-                    const int m = gp2 ? q >> lgG : q / G, i = q - m * G;
+                    const int m = byG(q), i = q - m * G;
                     const int p = p0 + i;
                     if (m <= mmax && p < npairs) {
                         const size_t o = (((size_t)b * (mmax + 1) + m) * npairs + p) * 2;
@@ -768,7 +791,7 @@ __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, co
             for (int u = 0; u < U; ++u) {
                 const int q = q0 + u * blockDim.x;
                 if (q >= G * H) break;
-                const int m = gp2 ? q >> lgG : q / G, i = q - m * G;
+                const int m = byG(q), i = q - m * G;
                 if (m == 0) { E[u].y = 0.0; O[u].y = 0.0; }
                 raw[(2 * i) * ld + padi(m)] = E[u];
                 raw[(2 * i + 1) * ld + padi(m)] = O[u];
@@ -786,7 +809,7 @@ __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, co
     // 2. X_N = E + O, X_S = E - O and the pre-twiddle, in double-float; a thread
     //    owns positions k and H - k of both rows of its pair (converted in place)
     for (int q = threadIdx.x; q < G * (H / 2 + 1); q += blockDim.x) {
-        const int i = q / (H / 2 + 1), k = q - i * (H / 2 + 1);
+        const int i = byHalf(q), k = q - i * (H / 2 + 1);
         const int u = s_e[i] - 1023;
         const int k2 = k == 0 ? 0 : H - k;
         const double2 *rE = raw + (2 * i) * ld, *rO = raw + (2 * i + 1) * ld;
@@ -828,6 +851,7 @@ __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, co
         out[idx] = make_double2(df2d(z.x, u), df2d(z.y, u));
     };
     if constexpr (LOGH == 10) {
+        static_assert(V == 16, "radix 4, 16, 16");
         // inverse complex FFT of length 1024: radix 4, 16, 16, the last from registers to the grid
         constexpr int NR = PassRegs<false>::n;
         dfl2 v[NR];
@@ -855,17 +879,17 @@ __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, co
         return;
     }
     int Ns = 1;
-    dfl2 v[PassRegs<MIXED>::n];
+    dfl2 v[PassRegs<MIXED, V>::n];
     for (int ps = 0;; ++ps) {
-        const int rd = fft_plan_radix(pv.fftplan, ps);
-        if (r < R) pass_load<dfl2, 1, MIXED>(rd, row, false, t, TPR, H, Ns, wtab, v);
+        const int rd = fft_plan_radix(plan, ps);
+        if (r < R) pass_load<dfl2, 1, MIXED, V>(rd, row, false, t, TPR, H, Ns, wtab, v);
         const bool last = Ns * rd == H;
         __syncthreads();
         if (last) {
-            if (live_row) last_pass_out<MIXED>(rd, v, t, TPR, H, put);
+            if (live_row) last_pass_out<MIXED, V>(rd, v, t, TPR, H, put);
             break;
         }
-        if (r < R) pass_store<dfl2, MIXED>(rd, row, t, TPR, H, Ns, v);
+        if (r < R) pass_store<dfl2, MIXED, V>(rd, row, t, TPR, H, Ns, v);
         __syncthreads();
         Ns *= rd;
     }
@@ -880,13 +904,14 @@ __device__ __forceinline__ void fft_synth_tile_df(const PlanView<double> &pv, co
 // spelled out (radix 4, 16, 16 for LOGH = 10, the plan's order), so the index
 // arithmetic folds and no code of other radices sits in the kernel (the
 // synthesis tile has the same form).
-template <bool MIXED, int LOGH = 0>
+template <bool MIXED, int LOGH, int V>
 __device__ __forceinline__ void fft_analys_tile_df(const PlanView<double> &pv, const double *__restrict__ grid,
                                                    double *__restrict__ sd, int b, int p0, int G, int op,
-                                                   int vector, int *__restrict__ fmax, unsigned char *smem_raw)
+                                                   int vector, int *__restrict__ fmax, unsigned long long plan,
+                                                   unsigned char *smem_raw)
 {
     const int H = LOGH ? (1 << LOGH) : pv.nphi / 2, R = 2 * G;
-    const int TPR = row_tpr(H);
+    const int TPR = row_tpr<V>(H);
     const int ld = padi(H) + 1;
     dfl2 *wtab = reinterpret_cast<dfl2 *>(smem_raw);
     dfl2 *buf = wtab + H;
@@ -912,12 +937,12 @@ __device__ __forceinline__ void fft_analys_tile_df(const PlanView<double> &pv, c
     const bool live_row = r < R && p < npairs && !((r & 1) && j == p);
     dfl2 *row = buf + (r < R ? r : 0) * ld;
     const double2 *in = reinterpret_cast<const double2 *>(grid) + ((size_t)b * nlat + (live_row ? j : 0)) * H;
-    // H <= 16 TPR: at most 16 values per thread
-    double2 x[16];
+    // H <= V TPR: at most V values per thread
+    double2 x[V];
     {
         int e = 0;
 #pragma unroll
-        for (int it = 0; it < 16; ++it) {
+        for (int it = 0; it < V; ++it) {
             const int k = t + it * TPR;
             x[it] = (live_row && k < H) ? in[k] : make_double2(0.0, 0.0);
             e = max(e, dexp2(x[it]));
@@ -928,13 +953,14 @@ __device__ __forceinline__ void fft_analys_tile_df(const PlanView<double> &pv, c
     if (r < R) {
         const int u = s_e[r >> 1] - 1023;
 #pragma unroll
-        for (int it = 0; it < 16; ++it) {
+        for (int it = 0; it < V; ++it) {
             const int k = t + it * TPR;
             if (k < H) row[padi(k)] = d2df2(x[it], u);
         }
     }
     __syncthreads();
     if constexpr (LOGH == 10) {
+        static_assert(V == 16, "radix 4, 16, 16");
         // forward complex FFT of length 1024: radix 4, 16, 16
         constexpr int NR = PassRegs<false>::n;
         dfl2 v[NR];
@@ -952,13 +978,13 @@ __device__ __forceinline__ void fft_analys_tile_df(const PlanView<double> &pv, c
     } else if (H > 1) {
         // forward complex FFT of length H
         int Ns = 1;
-        dfl2 v[PassRegs<MIXED>::n];
-        const int npass = fft_plan_npass(pv.fftplan);
+        dfl2 v[PassRegs<MIXED, V>::n];
+        const int npass = fft_plan_npass(plan);
         for (int ps = 0; ps < npass; ++ps) {
-            const int rd = fft_plan_radix(pv.fftplan, ps);
-            if (r < R) pass_load<dfl2, -1, MIXED>(rd, row, false, t, TPR, H, Ns, wtab, v);
+            const int rd = fft_plan_radix(plan, ps);
+            if (r < R) pass_load<dfl2, -1, MIXED, V>(rd, row, false, t, TPR, H, Ns, wtab, v);
             __syncthreads();
-            if (r < R) pass_store<dfl2, MIXED>(rd, row, t, TPR, H, Ns, v);
+            if (r < R) pass_store<dfl2, MIXED, V>(rd, row, t, TPR, H, Ns, v);
             __syncthreads();
             Ns *= rd;
         }
@@ -988,10 +1014,9 @@ __device__ __forceinline__ void fft_analys_tile_df(const PlanView<double> &pv, c
         ebits = max(ebits, (unsigned)max(dexp2(so), dexp2(dd)));
     };
     const int mhalf = min(H / 2, mmax);
-    const bool gp2 = (G & (G - 1)) == 0;
-    const int lgG = __popc(G - 1);
+    const FastDiv byG(G);
     for (int q = threadIdx.x; q < G * (mhalf + 1); q += blockDim.x) {
-        const int m = gp2 ? q >> lgG : q / G, i = q - m * G;
+        const int m = byG(q), i = q - m * G;
         const int pp = p0 + i;
         if (pp >= npairs) continue;
         const int m2 = H - m;   // its partner, when it is another position and an order of the plan
@@ -1002,7 +1027,7 @@ __device__ __forceinline__ void fft_analys_tile_df(const PlanView<double> &pv, c
         for (int h = 0; h < 2; ++h) {
             const dfl2 *rw = buf + (2 * i + h) * ld;
             const dfl2 Zk = rw[padi(m)];
-            const dfl2 Zc = conj_(rw[padi(MIXED ? (H - m) % H : (H - m) & (H - 1))]);
+            const dfl2 Zc = conj_(rw[padi(m == 0 ? 0 : m2)]);
             dfl2 E = cadd(Zk, Zc), O = csub(Zk, Zc);
             E.x = scale2(E.x, 0.5f);
             E.y = scale2(E.y, 0.5f);
@@ -1022,21 +1047,22 @@ __device__ __forceinline__ void fft_analys_tile_df(const PlanView<double> &pv, c
     }
 }
 
-template <bool MIXED, int LOGH = 0>
+template <bool MIXED, int LOGH, int V>
 __global__ void __launch_bounds__(512)
-k_fft_synth_df(PlanView<double> pv, const double *__restrict__ eo, double *__restrict__ grid, int G, int op)
+k_fft_synth_df(PlanView<double> pv, const double *__restrict__ eo, double *__restrict__ grid, int G, int op,
+               unsigned long long plan)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fft_synth_tile_df<MIXED, LOGH>(pv, eo, grid, blockIdx.y, blockIdx.x * G, G, op, smem_raw);
+    fft_synth_tile_df<MIXED, LOGH, V>(pv, eo, grid, blockIdx.y, blockIdx.x * G, G, op, plan, smem_raw);
 }
 
-template <bool MIXED, int LOGH = 0>
+template <bool MIXED, int LOGH, int V>
 __global__ void __launch_bounds__(512)
 k_fft_analys_df(PlanView<double> pv, const double *__restrict__ grid, double *__restrict__ sd, int G, int op,
-                int vector, int *__restrict__ fmax)
+                int vector, int *__restrict__ fmax, unsigned long long plan)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fft_analys_tile_df<MIXED, LOGH>(pv, grid, sd, blockIdx.y, blockIdx.x * G, G, op, vector, fmax, smem_raw);
+    fft_analys_tile_df<MIXED, LOGH, V>(pv, grid, sd, blockIdx.y, blockIdx.x * G, G, op, vector, fmax, plan, smem_raw);
 }
 
 // ---------------------------------------------------------------------------
@@ -1478,10 +1504,10 @@ cudaError_t launch_fft_synth(const PlanView<T> &pv, const T *eo, T *grid, int ba
     if constexpr (sizeof(T) == 4) {
         if (pow2(H) && logH <= kRowLogMax) return launch_rows_dispatch(logH, true, pv, eo, grid, batch, op, false, s);
     }
-    if constexpr (sizeof(T) == 8) {
-        if (fft_values<T>(H) == 4)
-            return pow2(H) ? synth_tiles<T, false, 4>(pv, eo, grid, batch, op, s)
-                           : synth_tiles<T, true, 4>(pv, eo, grid, batch, op, s);
+    if (fft_values<T>(H, true) == 4) {
+        if constexpr (sizeof(T) == 8)
+            if (pow2(H)) return synth_tiles<T, false, 4>(pv, eo, grid, batch, op, s);
+        return synth_tiles<T, true, 4>(pv, eo, grid, batch, op, s);
     }
     return pow2(H) ? synth_tiles<T, false, 16>(pv, eo, grid, batch, op, s)
                    : synth_tiles<T, true, 16>(pv, eo, grid, batch, op, s);
@@ -1496,57 +1522,82 @@ cudaError_t launch_fft_analys(const PlanView<T> &pv, const T *grid, T *sd, int b
         if (pow2(H) && logH <= kRowLogMax)
             return launch_rows_dispatch(logH, false, pv, grid, sd, batch, op, vector, s);
     }
-    if constexpr (sizeof(T) == 8) {
-        if (fft_values<T>(H) == 4)
-            return pow2(H) ? analys_tiles<T, false, 4>(pv, grid, sd, batch, op, vector, s)
-                           : analys_tiles<T, true, 4>(pv, grid, sd, batch, op, vector, s);
+    if (fft_values<T>(H, false) == 4) {
+        if constexpr (sizeof(T) == 8)
+            if (pow2(H)) return analys_tiles<T, false, 4>(pv, grid, sd, batch, op, vector, s);
+        return analys_tiles<T, true, 4>(pv, grid, sd, batch, op, vector, s);
     }
     return pow2(H) ? analys_tiles<T, false, 16>(pv, grid, sd, batch, op, vector, s)
                    : analys_tiles<T, true, 16>(pv, grid, sd, batch, op, vector, s);
 }
 
+namespace {
+
+// 4 values per thread instead of 16, up to H = 1024: always for mixed radices,
+// whose 16-value passes spill and leave threads without items (16 fields of 512 x
+// 1080: 183 / 188 -> 144 / 148 us, 5 of 361 x 720: 46 / 44 -> 27 / 26 us;
+// synthesis / analysis); for powers of two while the 16-value form has too few
+// warps, at most 320 threads per SM (2 fields of 512 x 1024: 26 / 22 -> 20 / 20 us),
+// above which its fewer passes win (16 fields: 96 against 110 us).
+bool df_few_values(int H, int npairs, int batch)
+{
+    return H <= 1024 && (!pow2(H) || (long)batch * npairs * 2 * row_tpr<16>(H) <= 320L * sm_count());
+}
+
+template <bool MIXED, int LOGH, int V>
+cudaError_t synth_df_go(const PlanView<double> &pv, const double *eo, double *grid, int batch, Op op, cudaStream_t s)
+{
+    const int H = pv.nphi / 2;
+    int G, threads;
+    size_t smem;
+    fft_shape<double>(H, V, pv.npairs, batch, G, threads, smem);
+    smem += df_extra_smem(G);
+    cudaError_t e = set_smem(k_fft_synth_df<MIXED, LOGH, V>, smem);
+    if (e != cudaSuccess) return e;
+    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
+    k_fft_synth_df<MIXED, LOGH, V><<<gridd, threads, smem, s>>>(pv, eo, grid, G, (int)op, fft_plan_of(H, V == 4 ? 2 : 4));
+    return cudaGetLastError();
+}
+
+template <bool MIXED, int LOGH, int V>
+cudaError_t analys_df_go(const PlanView<double> &pv, const double *grid, double *sd, int batch, Op op, bool vector,
+                         cudaStream_t s, int *fmax)
+{
+    const int H = pv.nphi / 2;
+    int G, threads;
+    size_t smem;
+    fft_shape<double>(H, V, pv.npairs, batch, G, threads, smem);
+    smem += df_extra_smem(G);
+    cudaError_t e = set_smem(k_fft_analys_df<MIXED, LOGH, V>, smem);
+    if (e != cudaSuccess) return e;
+    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
+    k_fft_analys_df<MIXED, LOGH, V><<<gridd, threads, smem, s>>>(pv, grid, sd, G, (int)op, vector ? 1 : 0, fmax,
+                                                                fft_plan_of(H, V == 4 ? 2 : 4));
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_fft_synth_df(const PlanView<double> &pv, const double *eo, double *grid, int batch, Op op,
                                 cudaStream_t s)
 {
     if (!pv.twdf) return cudaErrorInvalidValue;
-    int G, threads;
-    size_t smem;
-    fft_shape<double>(pv.nphi / 2, 16, pv.npairs, batch, G, threads, smem);
-    smem += df_extra_smem(G);
-    const bool mixed = !pow2(pv.nphi / 2), h1024 = pv.nphi == 2048;
-    cudaError_t e = mixed ? set_smem(k_fft_synth_df<true>, smem)
-                          : (h1024 ? set_smem(k_fft_synth_df<false, 10>, smem) : set_smem(k_fft_synth_df<false>, smem));
-    if (e != cudaSuccess) return e;
-    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
-    if (mixed)
-        k_fft_synth_df<true><<<gridd, threads, smem, s>>>(pv, eo, grid, G, (int)op);
-    else if (h1024)
-        k_fft_synth_df<false, 10><<<gridd, threads, smem, s>>>(pv, eo, grid, G, (int)op);
-    else
-        k_fft_synth_df<false><<<gridd, threads, smem, s>>>(pv, eo, grid, G, (int)op);
-    return cudaGetLastError();
+    const int H = pv.nphi / 2;
+    if (df_few_values(H, pv.npairs, batch))
+        return pow2(H) ? synth_df_go<false, 0, 4>(pv, eo, grid, batch, op, s) : synth_df_go<true, 0, 4>(pv, eo, grid, batch, op, s);
+    if (H == 1024) return synth_df_go<false, 10, 16>(pv, eo, grid, batch, op, s);
+    return pow2(H) ? synth_df_go<false, 0, 16>(pv, eo, grid, batch, op, s) : synth_df_go<true, 0, 16>(pv, eo, grid, batch, op, s);
 }
 
 cudaError_t launch_fft_analys_df(const PlanView<double> &pv, const double *grid, double *sd, int batch, Op op,
                                  bool vector, cudaStream_t s, int *fmax)
 {
     if (!pv.twdf) return cudaErrorInvalidValue;
-    int G, threads;
-    size_t smem;
-    fft_shape<double>(pv.nphi / 2, 16, pv.npairs, batch, G, threads, smem);
-    smem += df_extra_smem(G);
-    const bool mixed = !pow2(pv.nphi / 2), h1024 = pv.nphi == 2048;
-    cudaError_t e = mixed ? set_smem(k_fft_analys_df<true>, smem)
-                          : (h1024 ? set_smem(k_fft_analys_df<false, 10>, smem) : set_smem(k_fft_analys_df<false>, smem));
-    if (e != cudaSuccess) return e;
-    dim3 gridd((unsigned)((pv.npairs + G - 1) / G), (unsigned)batch);
-    if (mixed)
-        k_fft_analys_df<true><<<gridd, threads, smem, s>>>(pv, grid, sd, G, (int)op, vector ? 1 : 0, fmax);
-    else if (h1024)
-        k_fft_analys_df<false, 10><<<gridd, threads, smem, s>>>(pv, grid, sd, G, (int)op, vector ? 1 : 0, fmax);
-    else
-        k_fft_analys_df<false><<<gridd, threads, smem, s>>>(pv, grid, sd, G, (int)op, vector ? 1 : 0, fmax);
-    return cudaGetLastError();
+    const int H = pv.nphi / 2;
+    if (df_few_values(H, pv.npairs, batch))
+        return pow2(H) ? analys_df_go<false, 0, 4>(pv, grid, sd, batch, op, vector, s, fmax) : analys_df_go<true, 0, 4>(pv, grid, sd, batch, op, vector, s, fmax);
+    if (H == 1024) return analys_df_go<false, 10, 16>(pv, grid, sd, batch, op, vector, s, fmax);
+    return pow2(H) ? analys_df_go<false, 0, 16>(pv, grid, sd, batch, op, vector, s, fmax) : analys_df_go<true, 0, 16>(pv, grid, sd, batch, op, vector, s, fmax);
 }
 
 // ---------------------------------------------------------------------------
@@ -1566,17 +1617,17 @@ k_group_rows(PlanView<float> pv, const BatchPtrs *__restrict__ ptrs)
     else fft_analys_rows_tile<LOGH>(pv, f.in, f.inter, 0, p0, OP_ANALYS, 0, smem_raw);
 }
 
-template <bool MIXED, bool SYNTH>
+template <bool MIXED, bool SYNTH, int V>
 __global__ void __launch_bounds__(512)
-k_group_tiles(PlanView<float> pv, const BatchPtrs *__restrict__ ptrs, int G)
+k_group_tiles(PlanView<float> pv, const BatchPtrs *__restrict__ ptrs, int G, unsigned long long plan)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const BatchPtrs f = ptrs[blockIdx.y];
     const int p0 = blockIdx.x * G;
     if constexpr (SYNTH)
-        fft_synth_tile<float, MIXED>(pv, f.inter, f.out, 0, p0, G, OP_SYNTH, pv.fftplan, smem_raw);
+        fft_synth_tile<float, MIXED, V>(pv, f.inter, f.out, 0, p0, G, OP_SYNTH, plan, smem_raw);
     else
-        fft_analys_tile<float, MIXED>(pv, f.in, f.inter, 0, p0, G, OP_ANALYS, 0, pv.fftplan, smem_raw);
+        fft_analys_tile<float, MIXED, V>(pv, f.in, f.inter, 0, p0, G, OP_ANALYS, 0, plan, smem_raw);
 }
 
 template <int LOGH, bool SYNTH>
@@ -1591,16 +1642,17 @@ cudaError_t group_rows(const PlanView<float> &pv, const BatchPtrs *ptrs, int nfi
     return cudaGetLastError();
 }
 
-template <bool MIXED, bool SYNTH>
+template <bool MIXED, bool SYNTH, int V>
 cudaError_t group_tiles(const PlanView<float> &pv, const BatchPtrs *ptrs, int nfields, cudaStream_t s)
 {
+    const int H = pv.nphi / 2;
     int G, threads;
     size_t smem;
-    fft_shape<float>(pv.nphi / 2, 16, pv.npairs, nfields, G, threads, smem);
-    cudaError_t e = set_smem(k_group_tiles<MIXED, SYNTH>, smem);
+    fft_shape<float>(H, V, pv.npairs, nfields, G, threads, smem);
+    cudaError_t e = set_smem(k_group_tiles<MIXED, SYNTH, V>, smem);
     if (e != cudaSuccess) return e;
     dim3 g((unsigned)((pv.npairs + G - 1) / G), (unsigned)nfields);
-    k_group_tiles<MIXED, SYNTH><<<g, threads, smem, s>>>(pv, ptrs, G);
+    k_group_tiles<MIXED, SYNTH, V><<<g, threads, smem, s>>>(pv, ptrs, G, fft_plan_of(H, V == 4 ? 2 : 4));
     return cudaGetLastError();
 }
 
@@ -1608,13 +1660,15 @@ template <bool SYNTH>
 cudaError_t group_fft(const PlanView<float> &pv, const BatchPtrs *ptrs, int nfields, cudaStream_t s)
 {
     const int H = pv.nphi / 2;
-    if (!pow2(H)) return group_tiles<true, SYNTH>(pv, ptrs, nfields, s);
+    if (!pow2(H))
+        return fft_values<float>(H, SYNTH) == 4 ? group_tiles<true, SYNTH, 4>(pv, ptrs, nfields, s)
+                                                : group_tiles<true, SYNTH, 16>(pv, ptrs, nfields, s);
     switch (ilog2(H)) {
 #define SHT_GROUP_CASE(L) case L: return group_rows<L, SYNTH>(pv, ptrs, nfields, s);
         SHT_GROUP_CASE(0) SHT_GROUP_CASE(1) SHT_GROUP_CASE(2) SHT_GROUP_CASE(3) SHT_GROUP_CASE(4) SHT_GROUP_CASE(5)
         SHT_GROUP_CASE(6) SHT_GROUP_CASE(7) SHT_GROUP_CASE(8) SHT_GROUP_CASE(9) SHT_GROUP_CASE(10)
 #undef SHT_GROUP_CASE
-    default: return group_tiles<false, SYNTH>(pv, ptrs, nfields, s);
+    default: return group_tiles<false, SYNTH, 16>(pv, ptrs, nfields, s);
     }
 }
 
