@@ -507,7 +507,7 @@ template <typename T> constexpr int mode_of_type() { return sizeof(T) == 8 ? SHT
 cudaError_t legendre_synth(const sht::PlanView<double> &pv, const double *spec, double *eo, int batch, sht::Op op,
                            const sht::TunedShape &ts, cudaStream_t s)
 {
-    return sht::launch_synth64(pv, spec, eo, batch, op, ts.synth_lpt, ts.synth_bc, s);
+    return sht::launch_synth64(pv, spec, eo, batch, op, ts.synth_bc, s);
 }
 cudaError_t legendre_synth(const sht::PlanView<float> &pv, const float *spec, float *eo, int batch, sht::Op op,
                            const sht::TunedShape &ts, cudaStream_t s)
@@ -1280,16 +1280,16 @@ extern "C" int sht_tune(sht_handle h, int batch, int mode, double *report, void 
     double best_syn = 1e30, best_ana = 1e30;
     const int reps = 3;
     const int widths[5] = {1, 2, 4, 8, 16};   // fields per CTA (FP32: up to 4 and 2)
-    const int lpts_s[4] = {1, 2, 4, 8};
-    for (int li = 0; li < 4; ++li)
+    const int lpts_s[3] = {1, 2, 4};
+    for (int li = 0; li < 3; ++li)
         for (int bi = 0; bi < 5; ++bi) {
-            const int lpt = lpts_s[li], bc = widths[bi];   // FP64: lpt warps per CTA
+            const int lpt = lpts_s[li], bc = widths[bi];
             if (bc > batch && bc > 1) continue;
-            if (shape_mode == SHT_F64 ? (bc == 16 && lpt == 8) : (lpt > 4 || bc > 4 || lpt * bc > 8)) continue;
+            if (shape_mode == SHT_F64 ? li > 0 : (bc > 4 || lpt * bc > 8)) continue;
             bool ok = false;
             double ms;
             if (shape_mode == SHT_F64)
-                ms = time_ms([&] { return sht::launch_synth64(p.view64(), (const double *)spec, (double *)p.work, batch, sht::OP_SYNTH, lpt, bc, s); }, s, reps, ok);
+                ms = time_ms([&] { return sht::launch_synth64(p.view64(), (const double *)spec, (double *)p.work, batch, sht::OP_SYNTH, bc, s); }, s, reps, ok);
             else
                 ms = time_ms([&] { return sht::launch_legendre_synth(p.view32(), (const float *)spec, (float *)p.work, batch, sht::OP_SYNTH, lpt, bc, s); }, s, reps, ok);
             if (ok && ms < best_syn) { best_syn = ms; best.synth_lpt = lpt; best.synth_bc = bc; }
@@ -1427,7 +1427,7 @@ extern "C" int sht_synth_static(sht_handle h, const void *spec, void *grid, int 
     if (mode == SHT_F64) {
         const sht::PlanView<double> pv = h->p.view64();
         double *eo = static_cast<double *>(scratch);
-        rc = launched(sht::launch_synth64(pv, static_cast<const double *>(spec), eo, batch, sht::OP_SYNTH, 0, 0, s),
+        rc = launched(sht::launch_synth64(pv, static_cast<const double *>(spec), eo, batch, sht::OP_SYNTH, 0, s),
                       "legendre synthesis launch");
         if (rc) return rc;
         return launched(sht::launch_fft_synth<double>(pv, eo, static_cast<double *>(grid), batch, sht::OP_SYNTH, s),

@@ -91,34 +91,46 @@ __device__ __forceinline__ bool reaches_one(double q, int hs)
 }
 
 // ---------------------------------------------------------------------------
-// Scalar synthesis.  A CTA of W warps per (order m, 32 latitude pairs, BC
-// fields), one pair per lane; warp w takes the live segments w, w + W, ... and
-// the warps' sums meet in shared memory in a fixed order.  Splitting the
-// degrees over warps keeps the SMs busy where orders x pairs x fields are few
-// (one field at N = 255: 134 us with one CTA of 128 pairs per order, 43 us with
-// four warps per 32 pairs).  16 fields at N = 511: 1981 us with three
-// instructions per step and 8 fields, 1766 us with two and 16 fields (34 FP64
-// instructions per degree, pair and 16 fields; 0.86 of the pipe's rate).  vec: the
-// spectra run to degree lmax + 1, the recurrence is Sec. 3.2's, and the sums
-// are divided by sin(theta).
+// Scalar synthesis.  A CTA of four warps (one per SM quarter) per (order m, 32
+// latitude pairs, BC fields).  It takes the degrees four segments at a time: each
+// warp generates P of one segment, one pair per lane, and the segment's spectral
+// values times s_n into shared memory; then warp w sums the pairs 8 w .. 8 w + 7,
+// lane (slice, c) the products of component c (field, real/imaginary) over the
+// degrees of its slice.  With C = 2 BC components there are 32 / C slices, each
+// of one parity of n - m (16 fields: both, in turn), summed over at the end by a
+// butterfly.  The sums are spread evenly over the SM quarters whatever the
+// number of segments (2 x 16 vector fields at N = 127: 165 us with a warp per
+// segment and 16 fields, 130 us).  16 fields at N = 511: 1981 us with three
+// instructions per step and 8 fields, 1766 with two and 16 fields a warp, 1656 us;
+// one field at N = 255: 134 -> 42 us.  vec: the spectra run to degree lmax + 1,
+// the recurrence is Sec. 3.2's, and the sums are divided by sin(theta).
 // ---------------------------------------------------------------------------
-template <int BC, int W>
-__global__ void __launch_bounds__(32 * W)
+constexpr int kSynWarps = 4;
+constexpr int kSynRow = 34;   // row of the P tile: 32 pairs, 16-byte aligned rows on shifted banks
+template <int BC> constexpr size_t synth64_smem()
+{
+    return sizeof(double) * (kSynWarps * kSeedSeg * ((2 * BC + 2) + kSynRow));
+}
+
+template <int BC>
+__global__ void __launch_bounds__(32 * kSynWarps)
 k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restrict__ eo, int batch, int ngroups,
           int nchunk, int nsm, int vec, int op)
 {
-    extern __shared__ __align__(16) double2 s_mem[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    double2 *s_f = s_mem + w * 64 * BC;                                  // [BC][kMaxDeg]
+    constexpr int C = 2 * BC, SL = 32 / C, W = kSynWarps, FS = C + 2, PAR = SL == 1 ? 2 : 1, PW = 32 / W;
+    extern __shared__ __align__(16) double s_mem[];
+    double *s_f = s_mem;                              // [W kSeedSeg degrees][FS]
+    double *s_P = s_mem + W * kSeedSeg * FS;          // [W kSeedSeg degrees][kSynRow]
     __shared__ double s_a[W][kMaxDeg], s_beta[W][kMaxDeg];
     __shared__ int s_hs[W][kMaxDeg];
 
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int item = snake(blockIdx.x, gridDim.x, nsm);
     const int chunk = item % nchunk, rest = item / nchunk;
     const int g = rest % ngroups, m = rest / ngroups;
     const int b0 = chunk * BC;
     const int npairs = pv.npairs, Ls = pv.lmax - m * pv.mres + 1, L = Ls + vec;
-    const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg;
+    const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg, ntask = (L + kSeedSeg - 1) / kSeedSeg;
     const long colq = col_ext(pv, m, 1), col = col_ext(pv, m, vec);
     const size_t nlm = (size_t)pv.nlm + (size_t)vec * (pv.mmax + 1);
     const double2 *spec2 = reinterpret_cast<const double2 *>(spec);
@@ -127,120 +139,128 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restri
     const double x = valid ? pv.x[p] : 0.0;
     const int first = (vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g];
     const double insc = (op == OP_ANALYS_ADJ && m > 0) ? 0.5 : 1.0;   // adjoint of analysis: b / c_m
+    const int c = lane % C, slice = lane / C;
+    const int u = (w + item) & (W - 1);   // the segment of a block this warp generates (turned from CTA to CTA)
 
-    double er[BC], ei[BC], orr[BC], oi[BC];
+    double acc[PAR][PW];
 #pragma unroll
-    for (int b = 0; b < BC; ++b) er[b] = ei[b] = orr[b] = oi[b] = 0.0;
+    for (int q = 0; q < PW; ++q)
+#pragma unroll
+        for (int r = 0; r < PAR; ++r) acc[r][q] = 0.0;
 
-    for (int seg = first + w; seg < nseg; seg += W) {
-        const int n0 = seg * kSeedSeg;
-        const int cnt = seg == nseg - 1 ? L - n0 : kSeedSeg;
-        double y1 = 0.0, y2 = 0.0;
-        int k = 0;
-        if (valid) {
-            const size_t o = (size_t)(pv.segoff[m] + seg) * npairs + p;
-            const double2 v = __ldg(pv.seeds64 + o);
-            const double down = vec ? seg_down(pv, m, seg) : 1.0;
-            y1 = v.x * down;
-            y2 = v.y * down;
-            k = __ldg(pv.seeds64k + o);
-        }
-        __syncwarp();
-        for (int t = lane; t < ((cnt + 1) & ~1); t += 32) {
-            const Step st = step_of(pv, colq + n0 + t, t < cnt, vec);
-            s_a[w][t] = st.a;
-            s_beta[w][t] = st.b;
-            s_hs[w][t] = __double2hiint(st.s) - kHiOne;
-            const double sc = st.s * insc;
+    for (int sb = first; sb < ntask; sb += W) {
+        const int sg = sb + u;
+        if (sg < ntask) {
+            // `vec`: the degree lmax + 1 is a segment of its own when the order's
+            // degrees fill theirs; it continues the last one's recurrence
+            const bool tail = sg == nseg;
+            const int seg = tail ? nseg - 1 : sg;
+            const int cnt = min(kSeedSeg, L - sg * kSeedSeg);
+            const int nstep = tail ? kSeedSeg + 1 : (cnt + 15) & ~15;
+            double y1 = 0.0, y2 = 0.0;
+            int k = 0;
+            if (valid) {
+                const size_t o = (size_t)(pv.segoff[m] + seg) * npairs + p;
+                const double2 v = __ldg(pv.seeds64 + o);
+                const double down = vec ? seg_down(pv, m, seg) : 1.0;
+                y1 = v.x * down;
+                y2 = v.y * down;
+                k = __ldg(pv.seeds64k + o);
+            }
+            double fs = 1.0;   // s_n of this lane's degree
+            for (int t = lane; t < nstep; t += 32) {
+                const int d = seg * kSeedSeg + t;
+                const Step st = step_of(pv, colq + d, d < L, vec);
+                s_a[u][t] = st.a;
+                s_beta[u][t] = st.b;
+                s_hs[u][t] = __double2hiint(st.s) - kHiOne;
+                if (t < kSeedSeg) fs = st.s;
+            }
+            const double sc = vec ? 1.0 : fs * insc;
+            double *row = s_f + (u * kSeedSeg + lane) * FS;
 #pragma unroll
             for (int b = 0; b < BC; ++b) {
                 double2 f = make_double2(0.0, 0.0);
-                if (t < cnt && b0 + b < batch) {
-                    f = __ldg(spec2 + (size_t)(b0 + b) * nlm + col + n0 + t);
-                    f.x *= sc;
-                    f.y = m == 0 ? 0.0 : f.y * sc;
+                if (lane < cnt && b0 + b < batch) {
+                    f = __ldg(spec2 + (size_t)(b0 + b) * nlm + col + sg * kSeedSeg + lane);
+                    if (!vec) {
+                        f.x *= sc;
+                        f.y *= sc;
+                    }
+                    if (m == 0) f.y = 0.0;
                 }
-                s_f[b * kMaxDeg + t] = f;
+                *reinterpret_cast<double2 *>(row + 2 * b) = f;
             }
-        }
-        __syncwarp();
-        if (!__any_sync(kFull, k > 0)) {
-            for (int t = 0; t < cnt; t += 2) {
-                y2 = fma(vec ? s_a[w][t] * x : x, y1, s_beta[w][t] * y2);
-#pragma unroll
-                for (int b = 0; b < BC; ++b) {
-                    const double2 f = s_f[b * kMaxDeg + t];
-                    er[b] = fma(f.x, y2, er[b]);
-                    ei[b] = fma(f.y, y2, ei[b]);
-                }
-                y1 = fma(vec ? s_a[w][t + 1] * x : x, y2, s_beta[w][t + 1] * y1);
-#pragma unroll
-                for (int b = 0; b < BC; ++b) {
-                    const double2 f = s_f[b * kMaxDeg + t + 1];
-                    orr[b] = fma(f.x, y1, orr[b]);
-                    oi[b] = fma(f.y, y1, oi[b]);
-                }
-            }
-        } else {
-            // some pair of the warp still carries a scaled value (Sec. 3.5)
-            for (int t = 0; t < cnt; ++t) {
-                double yn = fma(vec ? s_a[w][t] * x : x, y1, s_beta[w][t] * y2);
+            __syncwarp();
+            double *Pt = s_P + u * kSeedSeg * kSynRow + lane;
+            const bool scaled = __any_sync(kFull, k > 0);
+            for (int t = 0; t < nstep; ++t) {
+                double yn = fma(vec ? s_a[u][t] * x : x, y1, s_beta[u][t] * y2);
                 y2 = y1;
-                if (k > 0 && reaches_one(yn, s_hs[w][t])) {
-                    yn *= kDown;
-                    y2 *= kDown;
-                    k -= 1;
+                double v = yn;
+                if (scaled) {   // some pair still carries a scaled value (Sec. 3.5)
+                    if (k > 0 && reaches_one(yn, s_hs[u][t])) {
+                        yn *= kDown;
+                        y2 *= kDown;
+                        k -= 1;
+                    }
+                    v = k == 0 ? yn : 0.0;
                 }
                 y1 = yn;
-                if (!__any_sync(kFull, k == 0)) continue;
-                const double c = k == 0 ? yn : 0.0;
-                const bool odd = t & 1;
+                if (!tail) Pt[t * kSynRow] = v;
+                else if (t == kSeedSeg) Pt[0] = v;
+                else if (t > 0 && t < 16) Pt[t * kSynRow] = 0.0;
+            }
+        }
+        __syncthreads();
+        // rows past the order's last degree, up to a multiple of 16, hold zeros times finite values
+        const int nd = min(W * kSeedSeg, L - sb * kSeedSeg);
+        const double *fd = s_f + slice * FS + c, *Pd = s_P + slice * kSynRow + PW * w;
+        const int nj = (nd + SL * PAR - 1) / (SL * PAR);
+#pragma unroll 2
+        for (int j = 0; j < nj; ++j) {
 #pragma unroll
-                for (int b = 0; b < BC; ++b) {
-                    const double2 f = s_f[b * kMaxDeg + t];
-                    if (odd) {
-                        orr[b] = fma(f.x, c, orr[b]);
-                        oi[b] = fma(f.y, c, oi[b]);
-                    } else {
-                        er[b] = fma(f.x, c, er[b]);
-                        ei[b] = fma(f.y, c, ei[b]);
-                    }
+            for (int r = 0; r < PAR; ++r) {
+                const double f = fd[(j * PAR + r) * SL * FS];
+                const double2 *P2 = reinterpret_cast<const double2 *>(Pd + (j * PAR + r) * SL * kSynRow);
+#pragma unroll
+                for (int q = 0; q < PW / 2; ++q) {
+                    const double2 v = P2[q];
+                    acc[r][2 * q] = fma(f, v.x, acc[r][2 * q]);
+                    acc[r][2 * q + 1] = fma(f, v.y, acc[r][2 * q + 1]);
                 }
             }
         }
+        __syncthreads();
     }
-
-    double2 *eo2 = reinterpret_cast<double2 *>(eo);
-    if (W == 1) {
-        if (!valid) return;
-        const double is = vec ? 1.0 / pv.st[p] : 1.0;
+    // over the slices of one parity (lane bits 2 C .. 16): a lane keeps half of its pairs each time
 #pragma unroll
-        for (int b = 0; b < BC; ++b) {
-            if (b0 + b >= batch) break;
-            const size_t o = (((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + p) * 2;
-            eo2[o] = make_double2(er[b] * is, ei[b] * is);
-            eo2[o + 1] = make_double2(orr[b] * is, oi[b] * is);
+    for (int o = 16; o >= 2 * C; o >>= 1) {
+        const int h = PW * o / 32;
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double send = up ? acc[0][q] : acc[0][q + h];
+            const double keep = up ? acc[0][q + h] : acc[0][q];
+            acc[0][q] = keep + __shfl_xor_sync(kFull, send, o);
         }
-        return;
     }
-    // the warps' sums, [warp][field][pair][E, O]
-    __syncwarp();
+    {
+        // [field][pair][E, O][part], in the P tile
+        constexpr int V = SL == 1 ? PW : PW * C / 16;   // pairs held
+        const int off = SL == 1 ? 0 : (lane & ~(2 * C - 1)) * PW / 32;
 #pragma unroll
-    for (int b = 0; b < BC; ++b) {
-        s_f[(b * 32 + lane) * 2] = make_double2(er[b], ei[b]);
-        s_f[(b * 32 + lane) * 2 + 1] = make_double2(orr[b], oi[b]);
+        for (int r = 0; r < PAR; ++r)
+#pragma unroll
+            for (int q = 0; q < V; ++q)
+                s_P[(((c >> 1) * 32 + PW * w + off + q) * 2 + (SL == 1 ? r : slice & 1)) * 2 + (c & 1)] = acc[r][q];
     }
     __syncthreads();
+    double2 *eo2 = reinterpret_cast<double2 *>(eo);
     for (int i = threadIdx.x; i < BC * 64; i += 32 * W) {
         const int b = i >> 6, q = g * 32 + ((i & 63) >> 1);
         if (b0 + b >= batch || q >= npairs) continue;
-        double2 v = s_mem[i];
-#pragma unroll
-        for (int u = 1; u < W; ++u) {
-            const double2 z = s_mem[u * 64 * BC + i];
-            v.x += z.x;
-            v.y += z.y;
-        }
+        double2 v = reinterpret_cast<const double2 *>(s_P)[i];
         if (vec) {
             const double is = 1.0 / pv.st[q];
             v.x *= is;
@@ -261,7 +281,9 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restri
 // slices per segment (none at 16 fields); a lane per pair instead needs an FP64
 // butterfly over all 32 lanes for every 16 / BC degrees -- with 96 pairs a third
 // on top of the sums -- and a warp per segment leaves SM quarters idle where
-// segments are few.  Every sum has a fixed order, so results are bitwise
+// segments are few.  16 fields at N = 511: 2357 us with lanes as pairs and 8
+// fields, 1633 us; 2 x 16 vector fields at N = 127: 926 -> 162 us; one field at
+// N = 255: 67 -> 44 us.  Every sum has a fixed order, so results are bitwise
 // reproducible.  The groups of 32 pairs before the first one with a live pair in
 // the segment (static polar optimisation, Sec. 3.1) are left out.
 //
@@ -487,8 +509,9 @@ k_vec64_join(PlanView<double> pv, const double2 *__restrict__ ab, double2 *__res
 // Plan tables: (beta_n, s_n), (a_n, b_n) and eps_n of every degree m .. lmax + 1
 // of every order, and per segment the exponent h of its states' scale.  s_n^2 is
 // the product of (4 j^2 - 1) / (j^2 - m^2) over the segment, formed in
-// double-double arithmetic (Dekker 1971).  Thread per (segment, order index
-// blockIdx.y).
+// double-double arithmetic (Dekker 1971).  A warp per (segment, order index
+// blockIdx.y), a degree per lane, the product by a scan (a thread per segment
+// took 100 us of divisions and roots one after the other).
 // ---------------------------------------------------------------------------
 struct dd { double h, l; };
 __device__ __forceinline__ dd dd_norm(double h, double l)
@@ -498,53 +521,40 @@ __device__ __forceinline__ dd dd_norm(double h, double l)
     r.l = l - (r.h - h);
     return r;
 }
-__device__ __forceinline__ dd dd_mul(dd a, double b)
+__device__ __forceinline__ dd dd_mul(dd a, dd b)
 {
-    const double p = a.h * b;
-    return dd_norm(p, fma(a.l, b, fma(a.h, b, -p)));
-}
-// the quotient, rounded
-__device__ __forceinline__ double dd_div(dd a, dd b)
-{
-    const double q = a.h / b.h;
-    return q + (fma(-q, b.h, a.h) + (a.l - q * b.l)) / b.h;
+    const double p = a.h * b.h;
+    return dd_norm(p, fma(a.l, b.h, fma(a.h, b.l, fma(a.h, b.h, -p))));
 }
 
-__global__ void __launch_bounds__(64)
+__global__ void __launch_bounds__(32)
 k_build_qs(PlanView<double> pv, const unsigned long long *__restrict__ segoff, double2 *__restrict__ qs,
            double2 *__restrict__ abx, double *__restrict__ eps, int *__restrict__ hseg)
 {
-    const int m = blockIdx.y, seg = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m = blockIdx.y, seg = blockIdx.x, lane = threadIdx.x;
     const double dm = m * pv.mres;
     const int Ls = pv.lmax - m * pv.mres + 1;
     const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg;
     if (seg >= nseg) return;
     const long colx = col_ext(pv, m, 1), col = col_ext(pv, m, 0);
-    const int i0 = seg * kSeedSeg, i1 = seg == nseg - 1 ? Ls + 1 : i0 + kSeedSeg;
-    const auto factor = [&](int i, dd &num, dd &den) {   // into s^2 at degree dm + i
-        const double n = dm + i;
-        num = dd_mul(num, 4.0 * n * n - 1.0);
-        den = dd_mul(den, n * n - dm * dm);
+    const int i0 = seg * kSeedSeg;
+    const auto ratio = [&](int i) {   // s_n^2 / s_{n-1}^2 at degree dm + i
+        dd r = {1.0, 0.0};
+        if (i == 0) return r;
+        const double n = dm + i, num = 4.0 * n * n - 1.0, den = n * n - dm * dm;   // exact
+        const double q = num / den;
+        return dd_norm(q, fma(-q, den, num) / den);
     };
-    dd num = {1.0, 0.0}, den = num;
-    for (int i = max(1, i0); i < min(Ls, i0 + kSeedSeg); ++i) factor(i, num, den);
-    const int h = ilogb(num.h / den.h) / 4;   // half of the growth of s
-    hseg[segoff[m] + seg] = h;
-    num.h = scalbn(1.0, -2 * h);
-    num.l = 0.0;
-    den.h = 1.0;
-    den.l = 0.0;
-    for (int i = i0; i < i1; ++i) {
+    const auto put = [&](int i, dd s2, int h) {
         const double n = dm + i, n1 = n - 1.0;
         if (i == 0) {   // Q_m is the start value P_m^m, handed over as Q_{m-2}
             qs[colx] = make_double2(1.0, scalbn(1.0, -h));
             abx[colx] = make_double2(0.0, 1.0);
             eps[colx] = 0.0;
-            continue;
+            return;
         }
-        factor(i, num, den);
         const double bb = i == 1 ? 0.0 : (n1 * n1 - dm * dm) / (4.0 * n1 * n1 - 1.0);   // eps_{n-1}^2
-        qs[colx + i] = make_double2(i == i0 ? -sqrt(bb) : -bb, sqrt(dd_div(num, den)));
+        qs[colx + i] = make_double2(i == i0 ? -sqrt(bb) : -bb, scalbn(sqrt(s2.h), -h));
         eps[colx + i] = sqrt((n * n - dm * dm) / (4.0 * n * n - 1.0));
         double2 ab;
         if (i < Ls)
@@ -555,7 +565,20 @@ k_build_qs(PlanView<double> pv, const unsigned long long *__restrict__ segoff, d
             ab = make_double2(sqrt((4.0 * n * n - 1.0) / (n * n - dm * dm)),
                               -sqrt((2.0 * n + 1.0) / (2.0 * n - 3.0) * (n1 * n1 - dm * dm) / (n * n - dm * dm)));
         abx[colx + i] = ab;
+    };
+    dd s2 = ratio(i0 + lane);
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+        dd u;
+        u.h = __shfl_up_sync(kFull, s2.h, o);
+        u.l = __shfl_up_sync(kFull, s2.l, o);
+        if (lane >= o) s2 = dd_mul(s2, u);
     }
+    // half of the growth of s over the segment's degrees
+    const int h = __shfl_sync(kFull, ilogb(s2.h) / 4, min(kSeedSeg, Ls - i0) - 1);
+    if (lane == 0) hseg[segoff[m] + seg] = h;
+    if (i0 + lane <= Ls) put(i0 + lane, s2, h);
+    if (lane == kSeedSeg - 1 && i0 + kSeedSeg == Ls) put(Ls, dd_mul(s2, ratio(Ls)), h);
 }
 
 inline int sm_count()
@@ -567,15 +590,23 @@ inline int sm_count()
     return sms;
 }
 
-// Fields per CTA: the width whose CTAs issue the fewest FP64 instructions per
-// degree and pair, 2 + 2 BC each (unused fields of the last CTA count); the
-// larger of equals.
-inline int pick_bc64(int batch, int most)
+// Fields per CTA {1, 2, 4, 8, 16}: the width with the shortest busiest SM -- CTAs
+// per SM, rounded up, times the FP64 instructions of one (2 per degree and 32
+// pairs to generate P, 2 per field to sum).
+inline int pick_width(long units, int batch)
 {
-    int best = 1;
-    for (int bc = 2; bc <= most; bc *= 2)
-        if ((long)((batch + bc - 1) / bc) * (2 + 2 * bc) <= (long)((batch + best - 1) / best) * (2 + 2 * best)) best = bc;
-    return best;
+    const long sms = sm_count();
+    long best = 0;
+    int bc = 1;
+    for (int f = 16; f >= 1; f /= 2) {
+        const long ctas = units * ((batch + f - 1) / f);
+        const long t = (ctas + sms - 1) / sms * (1 + f);
+        if (best == 0 || t < best) {
+            best = t;
+            bc = f;
+        }
+    }
+    return bc;
 }
 
 bool tables_ok(const PlanView<double> &pv)
@@ -583,44 +614,35 @@ bool tables_ok(const PlanView<double> &pv)
     return pv.segoff && pv.seeds64 && pv.seeds64k && pv.glive && pv.glive_vec && pv.qs && pv.abx && pv.eps && pv.hseg;
 }
 
-// A launch of the synthesis with W warps per CTA.
-template <int BC, int W>
+template <int BC>
 cudaError_t synth64_go(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, bool vec,
                        cudaStream_t s)
 {
     const int ng = (pv.npairs + 31) / 32, nc = (batch + BC - 1) / BC;
-    const size_t smem = sizeof(double2) * 64 * BC * W;
+    constexpr size_t smem = synth64_smem<BC>();
     if (smem > 40 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_synth64<BC, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_synth64<BC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     const long items = (long)(pv.mmax + 1) * ng * nc;
-    k_synth64<BC, W><<<(unsigned)items, 32 * W, smem, s>>>(pv, spec, eo, batch, ng, nc, sm_count(), vec ? 1 : 0,
-                                                          (int)op);
+    k_synth64<BC><<<(unsigned)items, 32 * kSynWarps, smem, s>>>(pv, spec, eo, batch, ng, nc, sm_count(), vec ? 1 : 0,
+                                                                (int)op);
     return cudaGetLastError();
 }
 
-// w: warps per CTA {1, 2, 4, 8} (0: enough for 16 warps per SM, at most one per
-// segment of order 0); bc: fields per CTA {1, 2, 4, 8, 16} (0: pick_bc64).
-cudaError_t synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int w, int bc,
-                    bool vec, cudaStream_t s)
+cudaError_t synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int bc, bool vec,
+                    cudaStream_t s)
 {
     if (!tables_ok(pv)) return cudaErrorInvalidValue;
-    if (bc <= 0) bc = pick_bc64(batch, 16);
-    if (w <= 0) {
-        const long units = (long)(pv.mmax + 1) * ((pv.npairs + 31) / 32) * ((batch + bc - 1) / bc);
-        const int nseg = (pv.lmax + kSeedSeg) / kSeedSeg;
-        w = 1;
-        while (w < 8 && w < nseg && units * w < 16L * sm_count() && !(bc == 16 && w == 4)) w *= 2;
+    if (bc <= 0) bc = pick_width((long)(pv.mmax + 1) * ((pv.npairs + 31) / 32), batch);
+    switch (bc) {
+    case 1: return synth64_go<1>(pv, spec, eo, batch, op, vec, s);
+    case 2: return synth64_go<2>(pv, spec, eo, batch, op, vec, s);
+    case 4: return synth64_go<4>(pv, spec, eo, batch, op, vec, s);
+    case 8: return synth64_go<8>(pv, spec, eo, batch, op, vec, s);
+    case 16: return synth64_go<16>(pv, spec, eo, batch, op, vec, s);
+    default: return cudaErrorInvalidValue;
     }
-#define SHT_SYN64(B, W_) if (bc == B && w == W_) return synth64_go<B, W_>(pv, spec, eo, batch, op, vec, s);
-    SHT_SYN64(1, 1) SHT_SYN64(1, 2) SHT_SYN64(1, 4) SHT_SYN64(1, 8)
-    SHT_SYN64(2, 1) SHT_SYN64(2, 2) SHT_SYN64(2, 4) SHT_SYN64(2, 8)
-    SHT_SYN64(4, 1) SHT_SYN64(4, 2) SHT_SYN64(4, 4) SHT_SYN64(4, 8)
-    SHT_SYN64(8, 1) SHT_SYN64(8, 2) SHT_SYN64(8, 4) SHT_SYN64(8, 8)
-    SHT_SYN64(16, 1) SHT_SYN64(16, 2) SHT_SYN64(16, 4)
-#undef SHT_SYN64
-    return cudaErrorInvalidValue;
 }
 
 template <int BC>
@@ -641,25 +663,11 @@ inline long segments(const PlanView<double> &pv)
     return n;
 }
 
-// bc: fields per CTA {1, 2, 4, 8, 16}; 0: the width with the shortest busiest
-// SM -- CTAs per SM, rounded up, times the FP64 instructions of one (2 per degree
-// and 32 pairs to generate P, 2 per field to sum).
 cudaError_t analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc, bool vec,
                      cudaStream_t s)
 {
     if (!tables_ok(pv)) return cudaErrorInvalidValue;
-    if (bc <= 0) {
-        const long sms = sm_count(), segs = segments(pv);
-        long best = 0;
-        for (int f = 16; f >= 1; f /= 2) {
-            const long ctas = segs * ((batch + f - 1) / f);
-            const long t = (ctas + sms - 1) / sms * (1 + f);
-            if (best == 0 || t < best) {
-                best = t;
-                bc = f;
-            }
-        }
-    }
+    if (bc <= 0) bc = pick_width(segments(pv), batch);
     switch (bc) {
     case 1: return analys64_go<1>(pv, sd, spec, batch, op, vec, s);
     case 2: return analys64_go<2>(pv, sd, spec, batch, op, vec, s);
@@ -676,15 +684,14 @@ cudaError_t launch_build_qs(const PlanView<double> &pv, const unsigned long long
                             double *eps, int *hseg, cudaStream_t st)
 {
     const int nseg = (pv.lmax + kSeedSeg) / kSeedSeg;
-    k_build_qs<<<dim3((unsigned)((nseg + 63) / 64), (unsigned)(pv.mmax + 1)), 64, 0, st>>>(pv, segoff, qs, abx, eps,
-                                                                                       hseg);
+    k_build_qs<<<dim3((unsigned)nseg, (unsigned)(pv.mmax + 1)), 32, 0, st>>>(pv, segoff, qs, abx, eps, hseg);
     return cudaGetLastError();
 }
 
-cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int w, int bc,
+cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int bc,
                            cudaStream_t s)
 {
-    return synth64(pv, spec, eo, batch, op, w, bc, false, s);
+    return synth64(pv, spec, eo, batch, op, bc, false, s);
 }
 
 cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc,
@@ -707,7 +714,7 @@ cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, cons
                                        reinterpret_cast<double2 *>(uw), batch, (int)op);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return synth64(pv, uw, eo, 2 * batch, OP_SYNTH, 0, 0, true, s);
+    return synth64(pv, uw, eo, 2 * batch, OP_SYNTH, 0, true, s);
 }
 
 cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *ab, double *S, double *Tc,

@@ -129,8 +129,7 @@ enum Op {
     OP_ANALYS_ADJ = 3   // adjoint of analysis (a weighted synthesis of b / c_m)
 };
 
-// Kernel shapes chosen by sht_tune for one (precision, batch).  FP64: synth_lpt
-// is the warps per CTA (legendre64.cu).
+// Kernel shapes chosen by sht_tune for one (precision, batch); synth_lpt FP32 only.
 struct TunedShape {
     int synth_lpt = 0, synth_bc = 0, analys_bc = 0;
     int auto_mode = 1;           // SHT_F32_AUTO: the fastest of SHT_F32, SHT_TC_BF16X3, SHT_TC_OTF
@@ -239,9 +238,8 @@ cudaError_t launch_legendre_synth_vec(const PlanView<float> &pv, const float *S,
                                       float *eop, int batch, Op op, cudaStream_t s);
 cudaError_t launch_legendre_analys_vec(const PlanView<float> &pv, const float *sdt, const float *sdp, float *S,
                                        float *Tc, int batch, Op op, cudaStream_t s);
-// FP64.  w: warps per CTA of the synthesis in {1,2,4,8}; bc: fields per CTA in
-// {1,2,4,8,16} (16 fields: w <= 4); 0 = default.
-cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int w, int bc,
+// FP64.  bc: fields per CTA in {1,2,4,8,16}; 0 = default.
+cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int bc,
                            cudaStream_t s);
 cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc,
                             cudaStream_t s);
