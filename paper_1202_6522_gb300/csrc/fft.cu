@@ -28,6 +28,32 @@ constexpr double kTwoPiD = 6.283185307179586476925286766559;
 template <typename T2> __device__ __forceinline__ T2 mk(decltype(T2::x) a, decltype(T2::x) b) { T2 r; r.x = a; r.y = b; return r; }
 template <typename T2> __device__ __forceinline__ T2 cadd(T2 a, T2 b) { return mk<T2>(a.x + b.x, a.y + b.y); }
 template <typename T2> __device__ __forceinline__ T2 csub(T2 a, T2 b) { return mk<T2>(a.x - b.x, a.y - b.y); }
+// FP32 complex sums as one packed instruction (add.f32x2 rounds each half as the
+// scalar instruction does): the FFTs are short of issue slots, not of FMA lanes.
+__device__ __forceinline__ unsigned long long pack2(float2 a)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long r)
+{
+    float2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
 template <typename T2> __device__ __forceinline__ T2 cmul(T2 a, T2 b)
 {
     return mk<T2>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -166,6 +192,14 @@ struct RegDft {
 #pragma unroll
         for (int k = 0; k < RD / 2; ++k) {
             const T2 t = (k == 0) ? o[k] : Tw64<T2, SIGN>::mul(k * (64 / RD), o[k]);
+            if constexpr (sizeof(T2) == sizeof(float2)) {
+                // +-i o: a swap, which scalar sums take for nothing
+                if (k * (64 / RD) != 16) {
+                    v[k] = add2(e[k], t);
+                    v[k + RD / 2] = sub2(e[k], t);
+                    continue;
+                }
+            }
             v[k] = cadd(e[k], t);
             v[k + RD / 2] = csub(e[k], t);
         }
@@ -251,6 +285,19 @@ template <typename T> inline int fft_values(int H, bool synth)
 // log2 of a power of two
 __device__ __forceinline__ int lg2(int v) { return __popc(v - 1); }
 
+template <typename T2> struct IsDf { static constexpr bool value = false; };
+template <> struct IsDf<dfl2> { static constexpr bool value = true; };
+// a + w b, and 2 a - s, by FMAs
+template <typename T2> __device__ __forceinline__ T2 fma_add(T2 a, T2 w, T2 b)
+{
+    return mk<T2>(fma(-w.y, b.y, fma(w.x, b.x, a.x)), fma(w.y, b.x, fma(w.x, b.y, a.y)));
+}
+template <typename T2> __device__ __forceinline__ T2 twice_less(T2 a, T2 s)
+{
+    using T = decltype(T2::x);
+    return mk<T2>(fma(T(2), a.x, -s.x), fma(T(2), a.y, -s.y));
+}
+
 // q / d for 0 <= q < 2^19 and d >= 1 with q / d < 2^13 by one FP32 product (an
 // integer division by a run-time value is a long instruction sequence): the
 // rounding of (q + 1/2) (1/d) moves it by less than 2^-22 q/d < 1 / (2 d), its
@@ -279,6 +326,26 @@ __device__ __forceinline__ void stockham_load(const T2 *src, bool global_src, in
         for (int r = 0; r < RD; ++r) {
             const int idx = j + r * (H / RD);
             a[r] = global_src ? src[idx] : src[padi(idx)];
+        }
+        if constexpr (sizeof(T2) == sizeof(double2) && RD == 4 && !IsDf<T2>::value) {
+            // FP64: the twiddles w, w^2 (w^3 = w w^2) fused into the butterflies, s = a + w b
+            // by four FMAs and a - w b = 2 a - s by two: 24 instructions instead of 28
+            if (Ns > 1) {
+                const int q0 = P2 ? (j & (Ns - 1)) << (lg2(H) - lg2(Ns) - 2) : (j - div(j) * Ns) * wstep;
+                T2 w1 = wtab[q0], w2 = wtab[2 * q0];
+                if (SIGN < 0) {
+                    w1 = conj_(w1);
+                    w2 = conj_(w2);
+                }
+                const T2 p = fma_add(a[0], w2, a[2]), q = twice_less(a[0], p);
+                const T2 u = fma_add(a[1], w2, a[3]), z = twice_less(a[1], u);
+                const T2 iz = SIGN > 0 ? mul_i(z) : mk<T2>(z.y, -z.x);
+                v[it * RD] = fma_add(p, w1, u);
+                v[it * RD + 2] = twice_less(p, v[it * RD]);
+                v[it * RD + 1] = fma_add(q, w1, iz);
+                v[it * RD + 3] = twice_less(q, v[it * RD + 1]);
+                continue;
+            }
         }
         if (Ns > 1) {
             const int q0 = P2 ? (j & (Ns - 1)) << (lg2(H) - lg2(Ns) - lg2(RD)) : (j - div(j) * Ns) * wstep;
