@@ -645,16 +645,17 @@ __global__ void __launch_bounds__(kWsThreads, kWsCtasPerSm) k_tc_ws(TcArgs a, co
 // field groups as adjacent CTAs of each (m, tile), so the later ones read the
 // panel chunks the first brought into L2.
 constexpr int kVecHalf = 32;
+constexpr int kVecThreads = 320;
 
 // Persistent: one CTA per SM walks its list of work items (order, tile,
 // field half), the entries sched[gridDim.x + 1 + k] for k in
-// [sched[blockIdx.x], sched[blockIdx.x + 1]) (schedule_lpt), with 192
-// threads: warps 0-3 run the epilogue, warp 4 lane 0 issues the MMAs, warp 5
-// lane 0 streams the P, dP and data chunks.  The ring of stages runs on across
+// [sched[blockIdx.x], sched[blockIdx.x + 1]) (schedule_lpt), with kVecThreads
+// threads: warps 0-3 and 6-9 run the epilogue, warp 4 lane 0 issues the MMAs,
+// warp 5 lane 0 streams the P, dP and data chunks.  The ring of stages runs on across
 // items, so the next item's chunks load while the epilogue drains the
 // accumulators; the next item's MMAs start once the epilogue has read them.
 template <bool SYNTH>
-__global__ void __launch_bounds__(192, 1) k_tc_vec(TcArgs a)
+__global__ void __launch_bounds__(kVecThreads, 1) k_tc_vec(TcArgs a)
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -700,7 +701,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_vec(TcArgs a)
             tc::mbar_init(&bar_mma[q], 1);
         }
         tc::mbar_init(bar_full, 1);
-        tc::mbar_init(bar_free, 4);   // one arrival per epilogue warp
+        tc::mbar_init(bar_free, 8);   // one arrival per epilogue warp
         tc::mbar_init(bar_done, 1);
         tc::mbar_fence_init();
         s_abort = 0;
@@ -806,8 +807,9 @@ __global__ void __launch_bounds__(192, 1) k_tc_vec(TcArgs a)
             (void)tc::mbar_wait_bounded(bar_done, 0, 100000000ull);
         }
     } else {
-        // ---------------- epilogue (warps 0-3: TMEM lanes 32 warp ..) ----------------
-        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+        // ------- epilogue (warps 0-3 and 6-9: TMEM lanes 32 (warp % 4) .., every other block of 16 columns) -------
+        const int wq = warp & 3, wg = warp < 4 ? 0 : 1;
+        const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
         unsigned j = 0;
         for (int kk = k0; kk < k1; ++kk) {
             const Item it = item_of(items[kk]);
@@ -821,62 +823,72 @@ __global__ void __launch_bounds__(192, 1) k_tc_vec(TcArgs a)
             const int m = it.m, L = it.L;
             const long col = col_of_mres(lmax, m, a.mres);
             const int fb0 = it.half * kVecHalf, nbh = min(kVecHalf, a.batch - fb0);
-            const int row = it.tile * kRows + warp * 32 + lane;
+            const int row = it.tile * kRows + wq * 32 + lane;
             const float fm = (float)(m * a.mres);
             float isn = 1.f;
             if (SYNTH && row < npairs) isn = 1.f / a.st[row];
-            for (int cls = 0; cls < 2; ++cls) {
-                for (int cb = 0; cb < NH; cb += 32) {
-                    float v[2][2][32];  // [acc][first|second quantity][col]
+            float sc[2] = {1.f, 1.f};   // analysis: scale of the degrees 2 row, 2 row + 1
+            if (!SYNTH) {
+#pragma unroll
+                for (int cls = 0; cls < 2; ++cls) {
+                    const int n = m * a.mres + 2 * row + cls;
+                    if (a.op == OP_SYNTH_ADJ) sc[cls] = (m > 0) ? 2.f : 1.f;
+                    else sc[cls] = (n == 0) ? 0.f : 1.f / ((float)n * (float)(n + 1));
+                }
+            }
+            for (int cb = 16 * wg; cb < NH; cb += 32) {
+                float v[2][2][2][16];  // [cls][acc][first|second quantity][col]
+#pragma unroll
+                for (int cls = 0; cls < 2; ++cls)
 #pragma unroll
                     for (int ac = 0; ac < 2; ++ac)
 #pragma unroll
                         for (int hf = 0; hf < 2; ++hf) {
                             if (it.nlive > 0) {
-                                tc::tmem_ld32(lane_base + (uint32_t)((cls * 2 + ac) * NV + hf * NH + cb), v[ac][hf]);
+                                tc::tmem_ld16(lane_base + (uint32_t)((cls * 2 + ac) * NV + hf * NH + cb),
+                                              v[cls][ac][hf]);
                             } else {
 #pragma unroll
-                                for (int i = 0; i < 32; ++i) v[ac][hf][i] = 0.f;
+                                for (int i = 0; i < 16; ++i) v[cls][ac][hf][i] = 0.f;
                             }
                         }
-                    if (cls == 1 && cb + 32 >= NH) {
-                        // the accumulators are read: the next item's MMAs may overwrite them
-                        tc::tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(bar_free);
+                if (cb + 32 >= NH) {
+                    // the warp's accumulators are read: once all warps' are, the next item's
+                    // MMAs may overwrite them
+                    tc::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(bar_free);
+                }
+#pragma unroll
+                for (int q = 0; q < 16; q += 2) {
+                    const int bl = (cb + q) >> 1;   // field within the half
+                    const int b = fb0 + bl;
+                    if (bl >= nbh) continue;
+                    float2 x0[2], x1[2];
+#pragma unroll
+                    for (int cls = 0; cls < 2; ++cls) {
+                        // sums of P and dP with the first (u) and second (w) quantity
+                        const float pur = v[cls][0][0][q], pui = v[cls][0][0][q + 1];
+                        const float pwr = v[cls][0][1][q], pwi = v[cls][0][1][q + 1];
+                        const float dur = v[cls][1][0][q], dui = v[cls][1][0][q + 1];
+                        const float dwr = v[cls][1][1][q], dwi = v[cls][1][1][q + 1];
+                        const float s = SYNTH ? isn : sc[cls];
+                        x0[cls] = make_float2(s * (dur + fm * pwi), s * (dui - fm * pwr));
+                        x1[cls] = make_float2(s * (dwr - fm * pui), s * (dwi + fm * pur));
                     }
-                    for (int q = 0; q < 32; q += 2) {
-                        const int bl = (cb + q) >> 1;   // field within the half
-                        if (bl >= nbh) break;
-                        const int b = fb0 + bl;
-                        if (SYNTH) {
-                            if (row >= npairs) continue;
-                            const float psr = v[0][0][q], psi = v[0][0][q + 1];   // sum P S
-                            const float ptr = v[0][1][q], pti = v[0][1][q + 1];   // sum P T
-                            const float dsr = v[1][0][q], dsi = v[1][0][q + 1];   // sum dP S
-                            const float dtr = v[1][1][q], dti = v[1][1][q + 1];   // sum dP T
-                            const size_t oi = (((size_t)b * (a.mmax + 1) + m) * npairs + row) * 2 + cls;
-                            reinterpret_cast<float2 *>(a.out0)[oi] =
-                                make_float2((dsr + fm * pti) * isn, (dsi - fm * ptr) * isn);
-                            reinterpret_cast<float2 *>(a.out1)[oi] =
-                                make_float2((dtr - fm * psi) * isn, (dti + fm * psr) * isn);
-                        } else {
+                    if (SYNTH) {
+                        if (row < npairs) {
+                            const size_t oi = ((size_t)b * (a.mmax + 1) + m) * npairs + row;
+                            reinterpret_cast<float4 *>(a.out0)[oi] = make_float4(x0[0].x, x0[0].y, x0[1].x, x0[1].y);
+                            reinterpret_cast<float4 *>(a.out1)[oi] = make_float4(x1[0].x, x1[0].y, x1[1].x, x1[1].y);
+                        }
+                    } else {
+#pragma unroll
+                        for (int cls = 0; cls < 2; ++cls) {
                             const int nn = 2 * row + cls;
                             if (nn >= L) continue;
-                            const int n = m * a.mres + nn;
-                            float sc;
-                            if (a.op == OP_SYNTH_ADJ) sc = (m > 0) ? 2.f : 1.f;
-                            else sc = (n == 0) ? 0.f : 1.f / ((float)n * (float)(n + 1));
-                            const float pthr = v[0][0][q], pthi = v[0][0][q + 1];   // P^T theta folds
-                            const float pphr = v[0][1][q], pphi = v[0][1][q + 1];   // P^T phi folds
-                            const float dthr = v[1][0][q], dthi = v[1][0][q + 1];   // dP^T theta folds
-                            const float dphr = v[1][1][q], dphi = v[1][1][q + 1];   // dP^T phi folds
-                            float2 sv = make_float2(sc * (dthr + fm * pphi), sc * (dthi - fm * pphr));
-                            float2 tv = make_float2(sc * (dphr - fm * pthi), sc * (dphi + fm * pthr));
-                            if (m == 0) {
-                                sv.y = 0.f;
-                                tv.y = 0.f;
-                            }
+                            const float2 sv = make_float2(x0[cls].x, m == 0 ? 0.f : x0[cls].y);
+                            const float2 tv = make_float2(x1[cls].x, m == 0 ? 0.f : x1[cls].y);
                             reinterpret_cast<float2 *>(a.out0)[(size_t)b * a.nlm + col + nn] = sv;
                             reinterpret_cast<float2 *>(a.out1)[(size_t)b * a.nlm + col + nn] = tv;
                         }
@@ -1777,11 +1789,11 @@ cudaError_t launch_tc_vec(bool synth, int lmax, int mmax, int mres, int npairs, 
     if (synth) {
         e = cudaFuncSetAttribute(k_tc_vec<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_tc_vec<true><<<(unsigned)nctas, 192, smem, st>>>(a);
+        k_tc_vec<true><<<(unsigned)nctas, kVecThreads, smem, st>>>(a);
     } else {
         e = cudaFuncSetAttribute(k_tc_vec<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_tc_vec<false><<<(unsigned)nctas, 192, smem, st>>>(a);
+        k_tc_vec<false><<<(unsigned)nctas, kVecThreads, smem, st>>>(a);
     }
     return cudaGetLastError();
 }
