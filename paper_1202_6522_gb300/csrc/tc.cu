@@ -138,26 +138,27 @@ k_build_panels(PlanView<double> pv, const unsigned long long *__restrict__ off_s
 // ---------------------------------------------------------------------------
 constexpr int kPrepThreads = 128;
 
-// Packs 8 bf16 values into one 16-byte core-matrix row.
-__device__ __forceinline__ uint4 pack8(const __nv_bfloat16 (&v)[8])
+// Writes the hi and lo parts of 8 consecutive K values of the operand rows row (re,
+// even) and row + 1 (im).  Each part's two 16-byte core-matrix rows are neighbours:
+// one 32-byte store, a whole sector (the operand starts on a 256-byte boundary).
+__device__ __forceinline__ void store32(unsigned char *p, const uint32_t (&a)[4], const uint32_t (&b)[4])
 {
-    uint4 r;
-    r.x = (uint32_t)__bfloat16_as_ushort(v[0]) | ((uint32_t)__bfloat16_as_ushort(v[1]) << 16);
-    r.y = (uint32_t)__bfloat16_as_ushort(v[2]) | ((uint32_t)__bfloat16_as_ushort(v[3]) << 16);
-    r.z = (uint32_t)__bfloat16_as_ushort(v[4]) | ((uint32_t)__bfloat16_as_ushort(v[5]) << 16);
-    r.w = (uint32_t)__bfloat16_as_ushort(v[6]) | ((uint32_t)__bfloat16_as_ushort(v[7]) << 16);
-    return r;
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a[0]), "r"(a[1]), "r"(a[2]),
+                 "r"(a[3]), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3])
+                 : "memory");
 }
-
-// Writes the hi and lo rows of 8 consecutive K values of one operand row.
-__device__ __forceinline__ void put_row8(unsigned char *bh, unsigned char *bl, int row, int h, const float (&v)[8])
+__device__ __forceinline__ void put_rows8(unsigned char *bh, unsigned char *bl, int row, int h, const float (&re)[8],
+                                          const float (&im)[8])
 {
-    __nv_bfloat16 hv[8], lv[8];
+    uint32_t rh[4], rl[4], ih[4], il[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) split_bf16(v[i], hv[i], lv[i]);
+    for (int i = 0; i < 4; ++i) {
+        split2(re[2 * i], re[2 * i + 1], rh[i], rl[i]);
+        split2(im[2 * i], im[2 * i + 1], ih[i], il[i]);
+    }
     const uint32_t o = blk_off(row, 8 * h);
-    *reinterpret_cast<uint4 *>(bh + o) = pack8(hv);
-    *reinterpret_cast<uint4 *>(bl + o) = pack8(lv);
+    store32(bh + o, rh, ih);
+    store32(bl + o, rl, il);
 }
 
 // One thread per 8 consecutive K positions of one field (and quantity): it
@@ -211,8 +212,7 @@ k_tc_prep(int synth, int vec, int lmax, int mmax, int mres, int npairs, int nlm,
         }
         unsigned char *bh = dat + (size_t)(cls * 2) * blk;
         const int r0 = q * NH + 2 * b;
-        put_row8(bh, bh + blk, r0, h, re);
-        put_row8(bh, bh + blk, r0 + 1, h, im);
+        put_rows8(bh, bh + blk, r0, h, re, im);
     } else {
         const int b = it % batch, q = it / batch;
         const float4 *A = reinterpret_cast<const float4 *>(q ? in1 : in0) + ((size_t)b * (mmax + 1) + m) * npairs;
@@ -223,20 +223,20 @@ k_tc_prep(int synth, int vec, int lmax, int mmax, int mres, int npairs, int nlm,
             v[i] = p < npairs ? A[p] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         const int r0 = q * NH + 2 * b;
-        float t[8];
+        float re[8], im[8];
         // class 0: s folds (x: re, y: im); class 1: d folds (z: re, w: im)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = v[i].x;
-        put_row8(dat, dat + blk, r0, h, t);
+        for (int i = 0; i < 8; ++i) {
+            re[i] = v[i].x;
+            im[i] = v[i].y;
+        }
+        put_rows8(dat, dat + blk, r0, h, re, im);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = v[i].y;
-        put_row8(dat, dat + blk, r0 + 1, h, t);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = v[i].z;
-        put_row8(dat + 2 * blk, dat + 3 * blk, r0, h, t);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = v[i].w;
-        put_row8(dat + 2 * blk, dat + 3 * blk, r0 + 1, h, t);
+        for (int i = 0; i < 8; ++i) {
+            re[i] = v[i].z;
+            im[i] = v[i].w;
+        }
+        put_rows8(dat + 2 * blk, dat + 3 * blk, r0, h, re, im);
     }
 }
 

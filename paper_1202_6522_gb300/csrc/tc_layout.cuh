@@ -28,12 +28,6 @@ __host__ __device__ __forceinline__ uint32_t blk_off(int row, int k)
 __host__ __device__ inline size_t data_chunk_bytes(int rows) { return 4 * (size_t)rows * kKc * 2; }
 
 // v = hi + lo with hi = bf16(v), lo = bf16(v - hi)
-__device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bfloat16 &lo)
-{
-    hi = __float2bfloat16_rn(v);
-    lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-}
-
 // v0, v1 -> bf16x2 hi and lo words (v0 in the low half) with v = hi + lo per element
 __device__ __forceinline__ void split2(float v0, float v1, uint32_t &hi, uint32_t &lo)
 {
