@@ -196,6 +196,8 @@ struct Plan {
     double otf_skip_s = 0, otf_skip_a = 0;      // on-the-fly mode: fraction of chunks skipped
     void *work = nullptr;            // scratch (grown on demand)
     size_t work_bytes = 0;
+    std::vector<void *> vspec;       // spectra of the FP64 vector transforms' scalar form; the last
+    size_t vspec_bytes = 0;          // one, of this size, is in use (see ensure_vspec)
     int device = 0;
     KernelTimer timer;
     std::vector<std::pair<long long, TunedShape>> tuned;   // key: mode * 2^32 + batch

@@ -84,3 +84,27 @@ def test_fp64_vector_strided_orders(lmax, mres, mmax):
         r = r.copy()
         r[:, 0] = 0        # the degree 0 has no vector part
         assert normwise(g.cpu().numpy(), r) < 1e-12
+
+
+def test_fp64_vector_graph_outlives_a_larger_call():
+    """A captured vector transform replays after a call with more fields, whose
+    intermediates fit the scratch that a scalar call left, took larger spectra."""
+    from paper_1202_6522_gb300 import SHT, build
+    build.build()
+    lmax, nlat, nphi = 40, 48, 96
+    sht = SHT(lmax, lmax, nlat, nphi, device=DEV)
+    dev = lambda v: torch.from_numpy(v).to(DEV)  # noqa: E731
+    a, b = (synthetic.spectrum(lmax, lmax, batch=9, seed=s, power=1.5) for s in (5, 6))
+    sht.synth_(dev(synthetic.spectrum(lmax, lmax, batch=64, seed=1, power=1.5)))
+    S, T = dev(a[:2]), dev(b[:2])
+    ref = [v.clone() for v in sht.synth_vec_(S, T)]
+    out = [torch.empty_like(v) for v in ref]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for o, v in zip(out, sht.synth_vec_(S, T)):
+            o.copy_(v)
+    sht.synth_vec_(dev(a), dev(b))
+    g.replay()
+    torch.cuda.synchronize()
+    for o, r in zip(out, ref):
+        assert torch.equal(o, r)
