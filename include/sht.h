@@ -72,15 +72,18 @@ enum {
 };
 
 enum {
-    SHT_F64 = 0,       /* FP64 throughout: the plain path.  Scalar transforms restart
-                        * the recurrence at every 32-degree segment they run, from
-                        * states the FP64 recurrence computes once per plan together
-                        * with the table of the static polar optimisation (built by
-                        * the first scalar call in this mode or by sht_reserve: 20 B
-                        * per latitude pair and 32 degrees, 175 MB at lmax = 1023). */
-    SHT_F32 = 1,       /* FP32 data and recurrence with the explicit exponent scale of
-                        * Sec. 3.5, restarted every 32 degrees from states the FP64
-                        * recurrence computes once per plan (built by the first call
+    SHT_F64 = 0,       /* FP64 throughout: the plain path.  The recurrence restarts at
+                        * every 32-degree segment, from states the FP64 recurrence
+                        * computes once per plan together with the table of the static
+                        * polar optimisation and the per-degree factors of the kernels
+                        * (built by the first call in this mode or by sht_reserve: 20 B
+                        * per latitude pair and 32 degrees, 175 MB at lmax = 1023, and
+                        * 40 B per coefficient).  Vector calls also take scratch for
+                        * the combined spectra of their two scalar transforms. */
+    SHT_F32 = 1,       /* FP32 data and recurrence restarted every 32 degrees from
+                        * states the FP64 recurrence computes once per plan, each held
+                        * with the power-of-two scale of its segment (the explicit
+                        * exponent of Sec. 3.5; built by the first call
                         * in this mode or by sht_reserve: 16 B per latitude pair and
                         * 32 degrees, (lmax+1)^2 ceil(nlat/2) / 4 bytes, 138 MB at
                         * lmax = 1023), so that FP32 rounding errors grow over at most
@@ -236,8 +239,8 @@ SHT_API int sht_sync_status(sht_handle h, void *stream);
 SHT_API int sht_synth_static(sht_handle h, const void *spec, void *grid, int batch, int mode, void *stream);
 
 /* Runtime tuning, after the paper's runtime tuning (Sec. 3.2): time the
- * candidate kernel shapes of the Legendre stage (latitude pairs per thread x
- * fields per CTA) for `batch` fields in `mode` (SHT_F64 or SHT_F32) and keep
+ * candidate kernel shapes of the Legendre stage (fields per CTA and, for FP32
+ * synthesis, latitude pairs per thread) for `batch` fields in `mode` (SHT_F64 or SHT_F32) and keep
  * the fastest for later calls with that batch size.  With SHT_F32_AUTO it also
  * times full round trips of the FP32 CUDA-core path, the tensor-core path with
  * precomputed panels and the tensor-core path with on-the-fly P_n^m (the
@@ -269,9 +272,11 @@ SHT_API int sht_batch_create(int nfields, const int *lmax, const int *nlat, cons
  * stage of each group of equal shape as one batched tensor-core contraction
  * against that shape's P panels (built here, ~(N+1)^3 bytes per direction per
  * shape), the group's spectra gathered into (synthesis) or scattered from
- * (analysis) a contiguous buffer by one copy kernel, the FFTs one persistent
- * kernel over all fields -- the graph then holds the copies, one contraction
- * per group and the FFT; SHT_F32_AUTO times a round trip of both on zero
+ * (analysis) a contiguous buffer, and the group's FFTs in a launch of their own.
+ * With up to 8 shapes each group's copies, contraction and FFT are a branch of
+ * the graph (without a graph they follow each other on the stream); beyond
+ * that one copy kernel and one persistent FFT kernel run over all fields.
+ * SHT_F32_AUTO times a round trip of both on zero
  * fields here (a few launches, synchronising) and keeps the faster.  Errors as
  * sht_batch_create, SHT_EINVAL for another mode, and the tensor-core
  * preparation's (SHT_ENOMEM) for SHT_TC_BF16X3. */
