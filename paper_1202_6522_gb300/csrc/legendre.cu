@@ -834,19 +834,23 @@ namespace {
 constexpr int kLeast32 = -70;   // FP32 leaves out segments with every |P| below 2^kLeast32
 
 // y 2^(-240 k) = P; emax: floor(log2) of the segment's largest |P|.  A state of
-// at least 2^-62 is stored as it is.  A smaller one can grow by up to 2^149 over
+// at least 2^-63 is stored as it is.  A smaller one can grow by up to 2^149 over
 // 32 degrees (order 4095): it is stored times the power of two that takes the
 // segment's largest value to about 2^50, which leaves every value and the factor
 // in FP32's normal range; the recurrence rounds the same at either scale.
+// Exponents from the high words and powers of two from integers: the FP64 pipe is
+// left to the recurrence.
 __device__ float4 fp32_state(double y1, double y2, int k, int emax)
 {
     constexpr int kTop = 50;
-    const double mx = fmax(fabs(y1), fabs(y2));
-    if (mx == 0.0 || emax < kLeast32) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const int h = max(__double2hiint(y1) & 0x7fffffff, __double2hiint(y2) & 0x7fffffff);
+    if (h < 0x100000 || emax < kLeast32) return make_float4(0.f, 0.f, 0.f, 0.f);
     const int down = -Scale<double>::S * k;
-    if (ilogb(mx) + down >= -63) return make_float4((float)scalbn(y1, down), (float)scalbn(y2, down), 1.f, 0.f);
-    const int e = kTop - emax;
-    return make_float4((float)scalbn(y1, down + e), (float)scalbn(y2, down + e), (float)scalbn(1.0, -e), 0.f);
+    if (k == 0 && (h >> 20) - 1023 >= -63) return make_float4((float)y1, (float)y2, 1.f, 0.f);
+    // 0 below FP64's range, where the states are below FP32's all the same
+    const int e = kTop - emax, field = 1023 + down + e;
+    const double f = field > 0 ? __hiloint2double(min(field, 2046) << 20, 0) : 0.0;
+    return make_float4((float)(y1 * f), (float)(y2 * f), __int_as_float((127 - e) << 23), 0.f);
 }
 
 __global__ void __launch_bounds__(128)
