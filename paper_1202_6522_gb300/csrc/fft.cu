@@ -261,11 +261,12 @@ template <int V = 16> __host__ __device__ inline int row_tpr(int H) { return (H 
 // Values per thread.  FP64 up to H = 1024 (512 threads for two rows): 4.  The
 // FP64 pipe takes a warp instruction every ~64 cycles per SM quarter, so a row
 // spread over four times the threads keeps all four quarters busy where a launch
-// has few rows, at the same instruction count (radix 4: 28 FP64 instructions per 4
+// has few rows, at the same instruction count (radix 4: 24 FP64 instructions per 4
 // points and pass, four passes; radix 16: 228 per 16 points, two passes).  One
 // field of 256 x 512 points: 51 / 54 us with 16 values and 8 pairs per CTA (16
 // CTAs), 28 / 27 us with one pair per CTA, 10.2 / 10.3 us with 4 values; 16 fields
-// of 512 x 1024: 373 / 417 -> 334 / 360 us (synthesis / analysis).
+// of 512 x 1024: 373 / 417 -> 308 / 317 us (synthesis / analysis; FP64 pipe 88 %
+// active), of which 43 / 44 us are the twiddles fused into the radix-4 FMAs.
 // FP32: 16, two radix-16 passes with few barriers; but 4 for mixed radices in the
 // synthesis up to H = 1024 and the analysis up to H = 256, where the 16-value
 // passes leave threads without items (6 fields of 288 x 384: 9.2 / 9.2 -> 6.2 /

@@ -654,6 +654,10 @@ constexpr int kVecThreads = 320;
 // warp 5 lane 0 streams the P, dP and data chunks.  The ring of stages runs on across
 // items, so the next item's chunks load while the epilogue drains the
 // accumulators; the next item's MMAs start once the epilogue has read them.
+// Bound by HBM and the epilogue in turn (the accumulators fill the tensor memory,
+// so they can't be doubled): a warp reads blocks of 16 columns of all accumulators
+// and stores both parities of a pair as 16 bytes.  N = 511, 64 fields: 171 / 164 us
+// with four epilogue warps, parity by parity, 138 / 151 us (synthesis / analysis).
 template <bool SYNTH>
 __global__ void __launch_bounds__(kVecThreads, 1) k_tc_vec(TcArgs a)
 {
