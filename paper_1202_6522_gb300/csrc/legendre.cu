@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include <climits>
+#include <type_traits>
 
 #include "sht_internal.h"
 
@@ -344,29 +345,33 @@ __device__ __forceinline__ void analys_segment(const PlanView<float> &pv, const 
         for (int b = 0; b < BC; ++b) f[b] = r[1 + b][lane];
         fetch();
         float y1 = st.x, y2 = st.y;
-        if (__any_sync(kFull, st.z != 1.f)) {   // states stored scaled: the factor into the folds
+        // one group of pairs; `scaled`: P = factor y
+        const auto add = [&](auto scaled) {
+            constexpr bool kScaled = decltype(scaled)::value;
 #pragma unroll
-            for (int b = 0; b < BC; ++b)
-                f[b] = make_float4(f[b].x * st.z, f[b].y * st.z, f[b].z * st.z, f[b].w * st.z);
-        }
+            for (int tb = 0; tb < kSeedSeg; tb += 8) {
+                if (tb >= cnt) break;   // rows past cnt are zero
 #pragma unroll
-        for (int tb = 0; tb < kSeedSeg; tb += 8) {
-            if (tb >= cnt) break;   // rows past cnt are zero
+                for (int t = tb; t < tb + 8; t += 2) {
+                    const float4 ab = sm.ab[t >> 1];
+                    y2 = next_p(ab.x, ab.y, x, y1, y2);
+                    y1 = next_p(ab.z, ab.w, x, y2, y1);
+                    const float c0 = kScaled ? y2 * st.z : y2, c1 = kScaled ? y1 * st.z : y1;
 #pragma unroll
-            for (int t = tb; t < tb + 8; t += 2) {
-                const float4 ab = sm.ab[t >> 1];
-                y2 = next_p(ab.x, ab.y, x, y1, y2);
-                y1 = next_p(ab.z, ab.w, x, y2, y1);
-#pragma unroll
-                for (int b = 0; b < BC; ++b) {
-                    float *a = acc + t * C + 2 * b;
-                    a[0] = fmaf(y2, f[b].x, a[0]);
-                    a[1] = fmaf(y2, f[b].y, a[1]);
-                    a[C] = fmaf(y1, f[b].z, a[C]);
-                    a[C + 1] = fmaf(y1, f[b].w, a[C + 1]);
+                    for (int b = 0; b < BC; ++b) {
+                        float *a = acc + t * C + 2 * b;
+                        a[0] = fmaf(c0, f[b].x, a[0]);
+                        a[1] = fmaf(c0, f[b].y, a[1]);
+                        a[C] = fmaf(c1, f[b].z, a[C]);
+                        a[C + 1] = fmaf(c1, f[b].w, a[C + 1]);
+                    }
                 }
             }
-        }
+        };
+        // the factor goes to P, not to the folds: times the folds of small data it leaves
+        // the FP32 range, though P times fold does not
+        if (__any_sync(kFull, st.z != 1.f)) add(std::true_type());
+        else add(std::false_type());
     }
     cp_async_wait<0>();
     warp_transpose_reduce<kSeedSeg * C>(acc, lane);
@@ -647,31 +652,36 @@ k_analys_vec(PlanView<float> pv, const float *__restrict__ sdt, const float *__r
         cp_async_wait<kRing - 2>();
         const float4 (&r)[3][32] = sm.ring[(slot + 1) & (kRing - 1)];   // the oldest
         const float4 st = r[0][lane];
-        float4 vt = r[1][lane], vp = r[2][lane];   // (s, d) of theta and phi
+        const float4 vt = r[1][lane], vp = r[2][lane];   // (s, d) of theta and phi
         fetch();
         float y1 = st.x, y2 = st.y;
-        if (__any_sync(kFull, st.z != 1.f)) {   // states stored scaled: the factor into the folds
-            vt = make_float4(vt.x * st.z, vt.y * st.z, vt.z * st.z, vt.w * st.z);
-            vp = make_float4(vp.x * st.z, vp.y * st.z, vp.z * st.z, vp.w * st.z);
-        }
         const float4 mt = make_float4(fm * vt.x, fm * vt.y, fm * vt.z, fm * vt.w);
         const float4 mp = make_float4(fm * vp.x, fm * vp.y, fm * vp.z, fm * vp.w);
+        const auto add = [&](auto scaled) {   // as in analys_segment
+            constexpr bool kScaled = decltype(scaled)::value;
 #pragma unroll
-        for (int tb = 0; tb < kSeedSeg; tb += 8) {
-            if (tb >= cnt) break;   // rows past cnt are zero
+            for (int tb = 0; tb < kSeedSeg; tb += 8) {
+                if (tb >= cnt) break;   // rows past cnt are zero
 #pragma unroll
-            for (int t = tb; t < tb + 8; ++t) {
-                float c, cd;
-                vec_step(sm.rec[t], x, y1, y2, c, cd);
-                // n - m even: P even -> s folds, dP odd -> d folds; odd: the other way round
-                const bool odd = t & 1;
-                float *a = acc + 4 * t;
-                a[0] = fmaf(cd, odd ? vt.x : vt.z, fmaf(c, odd ? mp.w : mp.y, a[0]));
-                a[1] = fmaf(cd, odd ? vt.y : vt.w, fmaf(-c, odd ? mp.z : mp.x, a[1]));
-                a[2] = fmaf(cd, odd ? vp.x : vp.z, fmaf(-c, odd ? mt.w : mt.y, a[2]));
-                a[3] = fmaf(cd, odd ? vp.y : vp.w, fmaf(c, odd ? mt.z : mt.x, a[3]));
+                for (int t = tb; t < tb + 8; ++t) {
+                    float c, cd;
+                    vec_step(sm.rec[t], x, y1, y2, c, cd);
+                    if (kScaled) {
+                        c *= st.z;
+                        cd *= st.z;
+                    }
+                    // n - m even: P even -> s folds, dP odd -> d folds; odd: the other way round
+                    const bool odd = t & 1;
+                    float *a = acc + 4 * t;
+                    a[0] = fmaf(cd, odd ? vt.x : vt.z, fmaf(c, odd ? mp.w : mp.y, a[0]));
+                    a[1] = fmaf(cd, odd ? vt.y : vt.w, fmaf(-c, odd ? mp.z : mp.x, a[1]));
+                    a[2] = fmaf(cd, odd ? vp.x : vp.z, fmaf(-c, odd ? mt.w : mt.y, a[2]));
+                    a[3] = fmaf(cd, odd ? vp.y : vp.w, fmaf(c, odd ? mt.z : mt.x, a[3]));
+                }
             }
-        }
+        };
+        if (__any_sync(kFull, st.z != 1.f)) add(std::true_type());   // states stored scaled: P = factor y
+        else add(std::false_type());
     }
     cp_async_wait<0>();
     warp_transpose_reduce<kSeedSeg * 4>(acc, lane);
