@@ -59,15 +59,21 @@ struct sht_batch_plan {
     std::vector<size_t> ginter_off;        // ... per group: its contiguous intermediate in d_inter, floats
     std::vector<size_t> inter_tc;          // ... per field: its intermediate in that layout
     // per call: pointer table of the group FFTs and copy list, fields in group order, one
-    // upload from the direction's own pinned staging
-    unsigned char *h_up[2] = {nullptr, nullptr}, *d_up = nullptr;
+    // upload from the direction's own pinned staging, beside the field table's
+    struct Staging {
+        unsigned char *up = nullptr;
+        sht::BatchField *fields = nullptr;
+    };
+    Staging stage[2];
+    std::vector<Staging> captured;         // of calls that a caller captured into a graph of its own
+    unsigned char *d_up = nullptr;
     std::vector<size_t> group_first;       // first entry of each group in that order
     std::vector<int> order;                // groups by falling size
     bool grouped = false;                  // FFTs by group
-    sht::BatchPtrs *h_ptrs(int dir) const { return reinterpret_cast<sht::BatchPtrs *>(h_up[dir]); }
-    BatchCopy *h_copies(int dir) const
+    sht::BatchPtrs *h_ptrs(const Staging &st) const { return reinterpret_cast<sht::BatchPtrs *>(st.up); }
+    BatchCopy *h_copies(const Staging &st) const
     {
-        return reinterpret_cast<BatchCopy *>(h_up[dir] + sizeof(sht::BatchPtrs) * nfields);
+        return reinterpret_cast<BatchCopy *>(st.up + sizeof(sht::BatchPtrs) * nfields);
     }
     const sht::BatchPtrs *d_ptrs() const { return reinterpret_cast<const sht::BatchPtrs *>(d_up); }
     const BatchCopy *d_copies() const
@@ -75,11 +81,21 @@ struct sht_batch_plan {
         return reinterpret_cast<const BatchCopy *>(d_up + sizeof(sht::BatchPtrs) * nfields);
     }
     size_t up_bytes() const { return (sizeof(sht::BatchPtrs) + sizeof(BatchCopy)) * nfields; }
+    cudaError_t alloc(Staging &st) const
+    {
+        cudaError_t e = cudaMallocHost(&st.fields, sizeof(sht::BatchField) * nfields);
+        return e == cudaSuccess ? cudaMallocHost(&st.up, up_bytes()) : e;
+    }
+    static void release(Staging &st)
+    {
+        if (st.fields) cudaFreeHost(st.fields);
+        if (st.up) cudaFreeHost(st.up);
+        st = Staging();
+    }
     float tuned_ms[2] = {0.f, 0.f};        // automatic mode: round trip per path (CUDA cores, tensor cores)
     std::vector<std::unique_ptr<sht::Plan>> plans;   // one per distinct shape
     std::vector<int> field_plan;
     std::vector<int> lmax, nlat, nphi;
-    sht::BatchField *h_fields[2] = {nullptr, nullptr};   // pinned staging of the field table, per direction
     sht::BatchField *d_fields = nullptr;
     int4 *d_tiles = nullptr;               // [synth legendre | synth fft | analys fft | analys legendre]
     int ntile[4] = {0, 0, 0, 0};
@@ -106,9 +122,9 @@ void free_batch(sht_batch_plan *b)
     if (b->done) cudaEventDestroy(b->done);
     for (int dir = 0; dir < 2; ++dir) {
         if (b->used[dir]) cudaEventDestroy(b->used[dir]);
-        if (b->h_fields[dir]) cudaFreeHost(b->h_fields[dir]);
-        if (b->h_up[dir]) cudaFreeHost(b->h_up[dir]);
+        b->release(b->stage[dir]);
     }
+    for (auto &st : b->captured) b->release(st);
     cudaFree(b->d_up);
     cudaFree(b->d_gspec);
     cudaFree(b->d_fields);
@@ -153,20 +169,19 @@ __global__ void __launch_bounds__(256) k_batch_copy(const BatchCopy *__restrict_
 }
 
 // Fill the per-call tables.
-void fill_fields(sht_batch_plan *b, bool synth, void *const *in, void *const *out)
+void fill_fields(sht_batch_plan *b, bool synth, void *const *in, void *const *out, const sht_batch_plan::Staging &st)
 {
     const bool tc = b->mode == SHT_TC_BF16X3;
-    const int dir = synth ? 0 : 1;
     for (size_t g = 0; g < b->group_fields.size(); ++g)
         for (size_t i = 0; i < b->group_fields[g].size(); ++i) {
             const int f = b->group_fields[g][i];
             const size_t at = b->group_first[g] + i;
-            sht::BatchPtrs &q = b->h_ptrs(dir)[at];
+            sht::BatchPtrs &q = b->h_ptrs(st)[at];
             q.in = static_cast<const float *>(in[f]);
             q.out = static_cast<float *>(out[f]);
             q.inter = b->d_inter + (tc ? b->inter_tc[f] : b->inter_off[f]);
             if (!tc) continue;
-            BatchCopy &c = b->h_copies(dir)[at];
+            BatchCopy &c = b->h_copies(st)[at];
             float2 *slot = reinterpret_cast<float2 *>(b->d_gspec + b->field_gspec[f]);
             c.n = b->plans[g]->nlm;
             c.src = synth ? static_cast<const float2 *>(in[f]) : slot;
@@ -174,7 +189,7 @@ void fill_fields(sht_batch_plan *b, bool synth, void *const *in, void *const *ou
         }
     if (tc && b->grouped) return;   // only the persistent kernels read the field table
     for (int f = 0; f < b->nfields; ++f) {
-        sht::BatchField &bf = b->h_fields[dir][f];
+        sht::BatchField &bf = st.fields[f];
         const sht::Plan &p = *b->plans[b->field_plan[f]];
         bf.pv = p.view32();
         bf.in = static_cast<const float *>(in[f]);
@@ -251,13 +266,13 @@ struct Branches {
 };
 
 // Enqueue the steps of one direction on stream s, those of a group on its branch.
-cudaError_t enqueue(sht_batch_plan *b, bool synth, cudaStream_t s, Branches &br)
+cudaError_t enqueue(sht_batch_plan *b, bool synth, cudaStream_t s, Branches &br, const sht_batch_plan::Staging &st)
 {
     const bool tc = b->mode == SHT_TC_BF16X3;
     const int ng = (int)b->plans.size();
-    br.run(cudaMemcpyAsync(b->d_up, b->h_up[synth ? 0 : 1], b->up_bytes(), cudaMemcpyHostToDevice, s));
+    br.run(cudaMemcpyAsync(b->d_up, st.up, b->up_bytes(), cudaMemcpyHostToDevice, s));
     if (!tc || !b->grouped) {
-        br.run(cudaMemcpyAsync(b->d_fields, b->h_fields[synth ? 0 : 1], sizeof(sht::BatchField) * b->nfields,
+        br.run(cudaMemcpyAsync(b->d_fields, st.fields, sizeof(sht::BatchField) * b->nfields,
                                cudaMemcpyHostToDevice, s));
         br.run(cudaMemsetAsync(b->d_counters, 0, 4 * sizeof(int), s));
     }
@@ -304,10 +319,28 @@ int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int us
     // waits for it before overwriting; the other direction's launch may still be
     // running, and the stream waits for it before this one uses the device buffers
     const int dir = synth ? 0 : 1;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap == cudaStreamCaptureStatusActive) {
+        // into the caller's graph, whose replays read the staging again: one of the call's own, kept
+        // with the plan, and no events, which would tie the graph to calls outside of it
+        sht_batch_plan::Staging st;
+        cudaError_t e = b->alloc(st);
+        if (e == cudaSuccess) {
+            fill_fields(b, synth, in, out, st);
+            Branches br;
+            br.open(s, 0, false);
+            e = enqueue(b, synth, s, br, st);
+        }
+        b->captured.push_back(st);
+        if (e != cudaSuccess) return bfail(SHT_ECUDA, std::string("batch launch under capture: ") + cudaGetErrorString(e));
+        return SHT_OK;
+    }
+    const sht_batch_plan::Staging &st = b->stage[dir];
     cudaError_t e = cudaEventSynchronize(b->used[dir]);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b->done, 0);
     if (e != cudaSuccess) return bfail(SHT_ECUDA, std::string("waiting for the previous batch call: ") + cudaGetErrorString(e));
-    fill_fields(b, synth, in, out);
+    fill_fields(b, synth, in, out, st);
     if (use_graph) {
         if (!b->graph[dir]) {
             cudaStream_t cs;
@@ -318,7 +351,7 @@ int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int us
             if (e == cudaSuccess) {
                 Branches br;
                 cudaError_t e2 = br.open(cs, (int)b->plans.size(), b->grouped);
-                if (e2 == cudaSuccess) e2 = enqueue(b, synth, cs, br);
+                if (e2 == cudaSuccess) e2 = enqueue(b, synth, cs, br, st);
                 e = cudaStreamEndCapture(cs, &g);
                 if (e == cudaSuccess) e = e2;
             }
@@ -334,7 +367,7 @@ int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int us
     } else {
         Branches br;
         br.open(s, 0, false);
-        e = enqueue(b, synth, s, br);
+        e = enqueue(b, synth, s, br, st);
     }
     if (e == cudaSuccess) e = cudaEventRecord(b->used[dir], s);
     if (e == cudaSuccess) e = cudaEventRecord(b->done, s);
@@ -548,8 +581,7 @@ int sht_batch_create_mode(int nfields, const int *lmax, const int *nlat, const i
     b->ctas_fft = sms * std::max(1, (int)std::min<size_t>(8, (200 * 1024) / std::max<size_t>(smem, 1)));
     cudaError_t e = cudaSuccess;
     for (int dir = 0; dir < 2; ++dir) {
-        if (e == cudaSuccess) e = cudaMallocHost(&b->h_fields[dir], sizeof(sht::BatchField) * nfields);
-        if (e == cudaSuccess) e = cudaMallocHost(&b->h_up[dir], b->up_bytes());
+        if (e == cudaSuccess) e = b->alloc(b->stage[dir]);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->used[dir], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaMalloc(&b->d_fields, sizeof(sht::BatchField) * nfields);
