@@ -204,13 +204,18 @@ void fill_fields(sht_batch_plan *b, bool synth, void *const *in, void *const *ou
     }
 }
 
+// Copies of `count` fields from entry `first` of the list, of at most n values each.
+cudaError_t copies(sht_batch_plan *b, size_t first, size_t count, int n, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((n + 256 * kCopyPer - 1) / (256 * kCopyPer)), (unsigned)count);
+    k_batch_copy<<<grid, 256, 0, s>>>(b->d_copies() + first);
+    return cudaGetLastError();
+}
+
 // One group's copies, contraction and FFT.
 cudaError_t group_copies(sht_batch_plan *b, int g, cudaStream_t s)
 {
-    const int n = b->plans[g]->nlm;
-    const dim3 grid((unsigned)((n + 256 * kCopyPer - 1) / (256 * kCopyPer)), (unsigned)b->group_fields[g].size());
-    k_batch_copy<<<grid, 256, 0, s>>>(b->d_copies() + b->group_first[g]);
-    return cudaGetLastError();
+    return copies(b, b->group_first[g], b->group_fields[g].size(), b->plans[g]->nlm, s);
 }
 
 cudaError_t group_contraction(sht_batch_plan *b, bool synth, int g, cudaStream_t s)
@@ -281,6 +286,11 @@ cudaError_t enqueue(sht_batch_plan *b, bool synth, cudaStream_t s, Branches &br,
         br.run(sht::launch_batch_fft(synth, b->d_fields, b->d_tiles + b->tile_off[k], b->ntile[k], b->d_counters + k,
                                      b->ctas_fft, b->fft_smem, s));
     };
+    const auto all_copies = [&] {   // blocks past the end of a shorter field return at once
+        int n = 0;
+        for (const auto &p : b->plans) n = std::max(n, p->nlm);
+        br.run(copies(b, 0, (size_t)b->nfields, n, s));
+    };
     const auto legendre = [&] {
         const int k = synth ? 0 : 3;
         br.run(sht::launch_batch_legendre(synth, b->d_fields, b->d_tiles + b->tile_off[k], b->ntile[k],
@@ -289,17 +299,19 @@ cudaError_t enqueue(sht_batch_plan *b, bool synth, cudaStream_t s, Branches &br,
     // each group's steps follow one another on its branch, the largest group first
     if (synth && !tc) legendre();
     if (!synth && !b->grouped) persistent_fft();
+    if (synth && tc && !b->grouped) all_copies();
     for (int i = 0; i < ng && (tc || b->grouped); ++i) {
         const int g = b->order[i];
         cudaStream_t gs = br.of(g);
         br.after(gs, s);
         if (!synth && b->grouped) br.run(group_fft(b, false, g, gs));
-        if (tc && synth) br.run(group_copies(b, g, gs));
+        if (tc && synth && b->grouped) br.run(group_copies(b, g, gs));
         if (tc) br.run(group_contraction(b, synth, g, gs));
-        if (tc && !synth) br.run(group_copies(b, g, gs));
+        if (tc && !synth && b->grouped) br.run(group_copies(b, g, gs));
         if (synth && b->grouped) br.run(group_fft(b, true, g, gs));
     }
     for (int g = 0; g < ng; ++g) br.after(s, br.of(g));
+    if (!synth && tc && !b->grouped) all_copies();
     if (synth && !b->grouped) persistent_fft();
     if (!synth && !tc) legendre();
     return br.err;
