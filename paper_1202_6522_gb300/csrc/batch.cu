@@ -70,6 +70,7 @@ struct sht_batch_plan {
     std::vector<size_t> group_first;       // first entry of each group in that order
     std::vector<int> order;                // groups by falling size
     bool grouped = false;                  // FFTs by group
+    std::vector<unsigned long long> fft_plan[2];   // per direction and shape: passes of the persistent FFT kernel's tiles
     sht::BatchPtrs *h_ptrs(const Staging &st) const { return reinterpret_cast<sht::BatchPtrs *>(st.up); }
     BatchCopy *h_copies(const Staging &st) const
     {
@@ -192,6 +193,7 @@ void fill_fields(sht_batch_plan *b, bool synth, void *const *in, void *const *ou
         sht::BatchField &bf = st.fields[f];
         const sht::Plan &p = *b->plans[b->field_plan[f]];
         bf.pv = p.view32();
+        bf.pv.fftplan = b->fft_plan[synth ? 0 : 1][b->field_plan[f]];
         bf.in = static_cast<const float *>(in[f]);
         bf.out = static_cast<float *>(out[f]);
         bf.inter = b->d_inter + (tc ? b->inter_tc[f] : b->inter_off[f]);
@@ -511,6 +513,7 @@ int sht_batch_create_mode(int nfields, const int *lmax, const int *nlat, const i
         b->group_first.push_back(first);
         first += b->group_fields[g].size();
         b->order.push_back((int)g);
+        for (int dir = 0; dir < 2; ++dir) b->fft_plan[dir].push_back(sht::tile_fft_plan32(p.nphi / 2, dir == 0));
         work.push_back((double)p.nlm * p.npairs * 4 + (double)b->group_fields[g].size() * p.nlat * p.nphi * 8);
     }
     std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) { return work[x] > work[y]; });

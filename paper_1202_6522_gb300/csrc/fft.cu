@@ -1808,6 +1808,8 @@ size_t batch_fft_smem(int H, int G)
     return (size_t)H * sizeof(float2) + (size_t)2 * G * row_bytes + (size_t)G * sizeof(float);
 }
 
+unsigned long long tile_fft_plan32(int H, bool synth) { return fft_plan_of(H, fft_values<float>(H, synth) == 4 ? 2 : 4); }
+
 cudaError_t batch_fft_prepare(size_t smem) { return set_smem(k_batch_fft, smem); }
 
 cudaError_t launch_batch_fft(bool synth, const BatchField *fields, const int4 *tiles, int ntiles, int *counter,

@@ -291,6 +291,9 @@ cudaError_t launch_batch_legendre(bool synth, const BatchField *fields, const in
 cudaError_t launch_batch_fft(bool synth, const BatchField *fields, const int4 *tiles, int ntiles, int *counter,
                              int ctas, size_t smem, cudaStream_t s);
 size_t batch_fft_smem(int H, int G);
+// Passes of the FP32 tile FFT of length H as the per-field launches run them: the
+// persistent kernel takes the same, so that its results equal theirs bit for bit.
+unsigned long long tile_fft_plan32(int H, bool synth);
 // The fields of one shape (same plan) in one launch: field f reads ptrs[f].in and
 // writes ptrs[f].inter (analysis) or reads inter and writes out (synthesis).
 struct BatchPtrs {
