@@ -276,7 +276,7 @@ SHT_API int sht_batch_create(int nfields, const int *lmax, const int *nlat, cons
  * With up to 8 shapes each group's copies, contraction and FFT are a branch of
  * the graph (without a graph they follow each other on the stream); beyond
  * that one copy kernel and one persistent FFT kernel run over all fields.
- * SHT_F32_AUTO times a round trip of both on zero
+ * SHT_F32_AUTO times a round trip of both, as graphs, on zero
  * fields here (a few launches, synchronising) and keeps the faster.  Errors as
  * sht_batch_create, SHT_EINVAL for another mode, and the tensor-core
  * preparation's (SHT_ENOMEM) for SHT_TC_BF16X3. */
