@@ -78,8 +78,8 @@ enum {
                         * polar optimisation and the per-degree factors of the kernels
                         * (built by the first call in this mode or by sht_reserve: 20 B
                         * per latitude pair and 32 degrees, 175 MB at lmax = 1023, and
-                        * 40 B per coefficient).  Vector calls also take scratch for
-                        * the combined spectra of their two scalar transforms. */
+                        * 40 B per coefficient).  Vector calls form the spectra of two
+                        * scalar transforms in their output arrays before they fill them. */
     SHT_F32 = 1,       /* FP32 data and recurrence restarted every 32 degrees from
                         * states the FP64 recurrence computes once per plan, each held
                         * with the power-of-two scale of its segment (the explicit

@@ -423,9 +423,13 @@ size_t tc_work_bytes(const sht::Plan &p, int batch, bool vec)
     return tc_data_offset(p, batch, vec) + sht::tc_data_bytes(p.mmax, p.npairs, p.tc_nchunk_s, nb, vec);
 }
 
+// With room for what the FP64 vector transforms keep behind two intermediates, 1 / (2
+// npairs) of them: a scratch that holds the intermediates holds that too, whichever
+// call it was made for.
 int ensure_work(sht::Plan &p, size_t bytes)
 {
     if (bytes <= p.work_bytes) return SHT_OK;
+    bytes += bytes / (2 * (size_t)p.npairs) + 256;
     if (p.work) {
         cudaError_t e = cudaFree(p.work);  // cudaFree waits for work using the old buffer
         p.work = nullptr;
@@ -556,27 +560,11 @@ int run_analys(sht::Plan &p, const sht::PlanView<T> &pv, const void *grid, void 
     });
 }
 
-// Vector transforms on the CUDA cores: two intermediates (theta, phi).
-size_t vec_work_bytes(const sht::Plan &p, int batch, int mode) { return 2 * inter_bytes(p, batch, mode); }
-
-// FP64 vector transforms: the spectra of their scalar form.  In a buffer of their
-// own, so that a call whose intermediates fit the scratch does not move it; a
-// buffer that got too small stays until the plan is destroyed, since a captured
-// graph may hold it, and each is at least twice its predecessor.
-int ensure_vspec(sht::Plan &p, int batch)
+// Vector transforms on the CUDA cores: two intermediates (theta, phi) and, in FP64,
+// the degree lmax + 1 of the combined spectra behind them.
+size_t vec_work_bytes(const sht::Plan &p, int batch, int mode)
 {
-    const size_t need = sht::vec64_spec_bytes(p.nlm, p.mmax, batch);
-    if (need <= p.vspec_bytes) return SHT_OK;
-    const size_t twice = 2 * p.vspec_bytes, bytes = need > twice ? need : twice;
-    void *buf = nullptr;
-    cudaError_t e = cudaMalloc(&buf, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fail(SHT_ENOMEM, std::string("cudaMalloc(vector spectra): ") + cudaGetErrorString(e));
-    }
-    p.vspec.push_back(buf);
-    p.vspec_bytes = bytes;
-    return SHT_OK;
+    return 2 * inter_bytes(p, batch, mode) + (mode == SHT_F64 ? sht::vec64_top_bytes(p.mmax, batch) : 0);
 }
 
 template <typename T>
@@ -588,7 +576,8 @@ int run_synth_vec(sht::Plan &p, const sht::PlanView<T> &pv, const void *S, const
     int rc = timed(p, SHT_K_LEGENDRE_SYNTH_VEC, s, "legendre vector synthesis launch", [&] {
         const T *Si = static_cast<const T *>(S), *Ti = static_cast<const T *>(Tc);
         if constexpr (sizeof(T) == sizeof(double))
-            return sht::launch_synth_vec64(pv, Si, Ti, static_cast<T *>(p.vspec.back()), eot, batch, op, s);
+            return sht::launch_synth_vec64(pv, Si, Ti, static_cast<T *>(vt), static_cast<T *>(vp),
+                                           eop + (eop - eot), eot, batch, op, s);
         else
             return sht::launch_legendre_synth_vec(pv, Si, Ti, eot, eop, batch, op, s);
     });
@@ -617,7 +606,7 @@ int run_analys_vec(sht::Plan &p, const sht::PlanView<T> &pv, const void *vt, con
     return timed(p, SHT_K_LEGENDRE_ANALYS_VEC, s, "legendre vector analysis launch", [&] {
         T *So = static_cast<T *>(S), *To = static_cast<T *>(Tc);
         if constexpr (sizeof(T) == sizeof(double))
-            return sht::launch_analys_vec64(pv, sdt, static_cast<T *>(p.vspec.back()), So, To, batch, op, s);
+            return sht::launch_analys_vec64(pv, sdt, sdp + (sdp - sdt), So, To, batch, op, s);
         else
             return sht::launch_legendre_analys_vec(pv, sdt, sdp, So, To, batch, op, s);
     });
@@ -708,7 +697,7 @@ int vector_s2g(sht_handle h, const void *S, const void *T, void *vt, void *vp, i
         return run_synth_vec_tc(h->p, S, T, vt, vp, batch, op, s);
     }
     if (mode == SHT_F32 && (rc = ensure_seeds32(h->p))) return rc;
-    if (mode == SHT_F64 && ((rc = ensure_seeds64(h->p)) || (rc = ensure_vspec(h->p, batch)))) return rc;
+    if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
     if ((rc = ensure_work(h->p, vec_work_bytes(h->p, batch, mode)))) return rc;
     if (mode == SHT_F64) return run_synth_vec<double>(h->p, h->p.view64(), S, T, vt, vp, batch, op, s);
     return run_synth_vec<float>(h->p, h->p.view32(), S, T, vt, vp, batch, op, s);
@@ -728,7 +717,7 @@ int vector_g2s(sht_handle h, const void *vt, const void *vp, void *S, void *T, i
         return run_analys_vec_tc(h->p, vt, vp, S, T, batch, op, s);
     }
     if (mode == SHT_F32 && (rc = ensure_seeds32(h->p))) return rc;
-    if (mode == SHT_F64 && ((rc = ensure_seeds64(h->p)) || (rc = ensure_vspec(h->p, batch)))) return rc;
+    if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
     if ((rc = ensure_work(h->p, vec_work_bytes(h->p, batch, mode)))) return rc;
     if (mode == SHT_F64) return run_analys_vec<double>(h->p, h->p.view64(), vt, vp, S, T, batch, op, s);
     return run_analys_vec<float>(h->p, h->p.view32(), vt, vp, S, T, batch, op, s);
@@ -1028,7 +1017,7 @@ int sht_reserve(sht_handle h, int batch, int mode)
         return ensure_work(h->p, tc64_work_bytes(h->p, batch));
     }
     if ((mode == SHT_F32 || mode == SHT_F32_AUTO) && (rc = ensure_seeds32(h->p))) return rc;
-    if (mode == SHT_F64 && ((rc = ensure_seeds64(h->p)) || (rc = ensure_vspec(h->p, batch)))) return rc;
+    if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
     return ensure_work(h->p, vec_work_bytes(h->p, batch, mode));
 }
 

@@ -57,6 +57,18 @@ __device__ __forceinline__ int snake(int i, int total, int nsm)
     return first + len - 1 - (i - first);
 }
 
+// Spectra of a vector transform's scalar form: the degrees m .. lmax of U (or A) and
+// of W (B) as [nb][nlm] each, and the degree lmax + 1 of both as [2 nb][mmax + 1].
+// Field f of the scalar form is U of field f, then W of field f - nb.
+struct VecSpec {
+    double2 *u, *w, *top;
+    int nb;
+    __device__ __forceinline__ double2 *field(int f, int nlm) const
+    {
+        return f < nb ? u + (size_t)f * nlm : w + (size_t)(f - nb) * nlm;
+    }
+};
+
 // One step of the recurrence, y_n = a x y_{n-1} + b y_{n-2}, and the factor s_n of
 // the value: (beta_n, s_n) of Q_n, where a = 1 is left out by the caller, or
 // (a_n, b_n) of P_n itself (`plain`).  Zeros past the order's last degree.
@@ -114,8 +126,8 @@ template <int BC> constexpr size_t synth64_smem()
 
 template <int BC>
 __global__ void __launch_bounds__(32 * kSynWarps)
-k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restrict__ eo, int batch, int ngroups,
-          int nchunk, int nsm, int vec, int op)
+k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, double *__restrict__ eo, int batch,
+          int ngroups, int nchunk, int nsm, int vec, int op)
 {
     constexpr int C = 2 * BC, SL = 32 / C, W = kSynWarps, FS = C + 2, PAR = SL == 1 ? 2 : 1, PW = 32 / W;
     extern __shared__ __align__(16) double s_mem[];
@@ -131,8 +143,7 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restri
     const int b0 = chunk * BC;
     const int npairs = pv.npairs, Ls = pv.lmax - m * pv.mres + 1, L = Ls + vec;
     const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg, ntask = (L + kSeedSeg - 1) / kSeedSeg;
-    const long colq = col_ext(pv, m, 1), col = col_ext(pv, m, vec);
-    const size_t nlm = (size_t)pv.nlm + (size_t)vec * (pv.mmax + 1);
+    const long colq = col_ext(pv, m, 1), col = col_ext(pv, m, 0);
     const double2 *spec2 = reinterpret_cast<const double2 *>(spec);
     const int p = g * 32 + lane;
     const bool valid = p < npairs;
@@ -182,7 +193,9 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, double *__restri
             for (int b = 0; b < BC; ++b) {
                 double2 f = make_double2(0.0, 0.0);
                 if (lane < cnt && b0 + b < batch) {
-                    f = __ldg(spec2 + (size_t)(b0 + b) * nlm + col + sg * kSeedSeg + lane);
+                    const int i = sg * kSeedSeg + lane;
+                    const double2 *src = vec ? vs.field(b0 + b, pv.nlm) : spec2 + (size_t)(b0 + b) * pv.nlm;
+                    f = __ldg(i < Ls ? src + col + i : vs.top + (size_t)(b0 + b) * (pv.mmax + 1) + m);
                     if (!vec) {
                         f.x *= sc;
                         f.y *= sc;
@@ -295,7 +308,8 @@ constexpr int kAnaWarps = 4;
 
 template <int BC>
 __global__ void __launch_bounds__(32 * kAnaWarps)
-k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restrict__ spec, int batch, int vec, int op)
+k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restrict__ spec, VecSpec vs, int batch,
+           int vec, int op)
 {
     constexpr int C = 2 * BC, SL = 32 / C, W = kAnaWarps, DB = kSeedSeg / W;
     constexpr int NQ = W * 32 / SL;   // pairs of a slice per block of 128
@@ -314,8 +328,7 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
     if (n0 >= L) return;
     const int cnt = min(kSeedSeg, L - n0);
     const int nstep = tail ? kSeedSeg + 1 : (cnt + DB - 1) & ~(DB - 1);
-    const long colq = col_ext(pv, m, 1) + seg * kSeedSeg, col = col_ext(pv, m, vec) + n0;
-    const size_t nlm = (size_t)pv.nlm + (size_t)vec * (pv.mmax + 1);
+    const long colq = col_ext(pv, m, 1) + seg * kSeedSeg, col = col_ext(pv, m, 0) + n0;
     if (threadIdx.x == 0) s_g0 = ngroups;
     if (threadIdx.x < nstep) {
         const int t = threadIdx.x;
@@ -432,25 +445,28 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
     // P_n = s_n Q_n; c_m for the adjoint of synthesis
     const double sc = (vec ? 1.0 : __ldg(&pv.qs[colq + lane].y)) * ((op == OP_SYNTH_ADJ && m > 0) ? 2.0 : 1.0);
     double2 *spec2 = reinterpret_cast<double2 *>(spec);
-    for (int i = w; i < BC && b0 + i < batch; i += W)
-        spec2[(size_t)(b0 + i) * nlm + col + lane] =
-            make_double2(s_P[0][lane][2 * i] * sc, m == 0 ? 0.0 : s_P[0][lane][2 * i + 1] * sc);
+    for (int i = w; i < BC && b0 + i < batch; i += W) {
+        double2 *dst = vec ? vs.field(b0 + i, pv.nlm) : spec2 + (size_t)(b0 + i) * pv.nlm;
+        dst = n0 + lane < Ls ? dst + col + lane : vs.top + (size_t)(b0 + i) * (pv.mmax + 1) + m;
+        *dst = make_double2(s_P[0][lane][2 * i] * sc, m == 0 ? 0.0 : s_P[0][lane][2 * i + 1] * sc);
+    }
 }
 
 // ---------------------------------------------------------------------------
 // Vector transforms: spectra in and out of the scalar sums (see the head of
-// this file).  Thread per (degree, order index m = blockIdx.y, field blockIdx.z).
+// this file).  U and W (degrees to lmax) are written where the grids will be,
+// which the FFT fills last: nlm <= nlat nphi / 2.  A and B come in the place of S
+// and T.  Only the degree lmax + 1 needs room of its own (VecSpec::top).
 // ---------------------------------------------------------------------------
+// Thread per (degree, order index m = blockIdx.y, field blockIdx.z).
 __global__ void __launch_bounds__(128)
-k_vec64_split(PlanView<double> pv, const double2 *__restrict__ S, const double2 *__restrict__ T,
-              double2 *__restrict__ uw, int batch, int op)
+k_vec64_split(PlanView<double> pv, const double2 *__restrict__ S, const double2 *__restrict__ T, VecSpec vs, int op)
 {
     const int m = blockIdx.y, b = blockIdx.z, dm = m * pv.mres;
     const int L = pv.lmax - dm + 1;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;   // degree k = dm + i, up to lmax + 1
     if (i > L) return;
     const long col = col_ext(pv, m, 0), colx = col_ext(pv, m, 1);
-    const size_t nlmx = (size_t)pv.nlm + pv.mmax + 1;
     const double2 *Sb = S + (size_t)b * pv.nlm + col, *Tb = T + (size_t)b * pv.nlm + col;
     const double k = dm + i;
     // adjoint of analysis: b / (c_m n (n + 1)), nothing at n = 0
@@ -473,36 +489,61 @@ k_vec64_split(PlanView<double> pv, const double2 *__restrict__ S, const double2 
     U.y = lo * Sl.y - hi * Sh.y - dm * Tc.x;
     W.x = lo * Tl.x - hi * Th.x - dm * Sc.y;
     W.y = lo * Tl.y - hi * Th.y + dm * Sc.x;
-    uw[(size_t)b * nlmx + colx + i] = U;
-    uw[(size_t)(batch + b) * nlmx + colx + i] = W;
+    if (i < L) {
+        vs.u[(size_t)b * pv.nlm + col + i] = U;
+        vs.w[(size_t)b * pv.nlm + col + i] = W;
+    } else {
+        vs.top[(size_t)b * (pv.mmax + 1) + m] = U;
+        vs.top[(size_t)(vs.nb + b) * (pv.mmax + 1) + m] = W;
+    }
 }
 
-__global__ void __launch_bounds__(128)
-k_vec64_join(PlanView<double> pv, const double2 *__restrict__ ab, double2 *__restrict__ S, double2 *__restrict__ T,
-             int batch, int op)
+// In place; a CTA per (order index m = blockIdx.x, field blockIdx.y) takes the degrees
+// blockDim.x at a time, each block's values read before any is overwritten, and the
+// last of a block handed on to the next.
+__global__ void __launch_bounds__(128) k_vec64_join(PlanView<double> pv, VecSpec vs, int op)
 {
-    const int m = blockIdx.y, b = blockIdx.z, dm = m * pv.mres;
+    __shared__ double2 s_last[2][2];   // A and B of the degree before the block, of this and the next
+    const int m = blockIdx.x, b = blockIdx.y, dm = m * pv.mres;
     const int L = pv.lmax - dm + 1;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // degree n = dm + i
-    if (i >= L) return;
     const long col = col_ext(pv, m, 0), colx = col_ext(pv, m, 1);
-    const size_t nlmx = (size_t)pv.nlm + pv.mmax + 1;
-    const double2 *A = ab + (size_t)b * nlmx + colx, *B = ab + (size_t)(batch + b) * nlmx + colx;
-    const double n = dm + i;
-    const double hi = n * pv.eps[colx + i + 1], lo = i > 0 ? (n + 1.0) * pv.eps[colx + i] : 0.0;
-    const double2 Ah = A[i + 1], Ac = A[i], Bh = B[i + 1], Bc = B[i];
-    const double2 z = make_double2(0.0, 0.0), Al = i > 0 ? A[i - 1] : z, Bl = i > 0 ? B[i - 1] : z;
-    double sc;
-    if (op == OP_SYNTH_ADJ) sc = m > 0 ? 2.0 : 1.0;
-    else sc = n == 0.0 ? 0.0 : 1.0 / (n * (n + 1.0));
-    double2 s, t;
-    s.x = sc * (hi * Ah.x - lo * Al.x + dm * Bc.y);
-    s.y = sc * (hi * Ah.y - lo * Al.y - dm * Bc.x);
-    t.x = sc * (hi * Bh.x - lo * Bl.x - dm * Ac.y);
-    t.y = sc * (hi * Bh.y - lo * Bl.y + dm * Ac.x);
-    if (m == 0) s.y = t.y = 0.0;
-    S[(size_t)b * pv.nlm + col + i] = s;
-    T[(size_t)b * pv.nlm + col + i] = t;
+    double2 *A = vs.u + (size_t)b * pv.nlm + col, *B = vs.w + (size_t)b * pv.nlm + col;
+    const double2 At = vs.top[(size_t)b * (pv.mmax + 1) + m], Bt = vs.top[(size_t)(vs.nb + b) * (pv.mmax + 1) + m];
+    const double2 z = make_double2(0.0, 0.0);
+    if (threadIdx.x < 2) s_last[0][threadIdx.x] = z;
+    __syncthreads();
+    for (int i0 = 0, q = 0; i0 < L; i0 += blockDim.x, q ^= 1) {
+        const int i = i0 + threadIdx.x;   // degree n = dm + i
+        const bool in = i < L;
+        double2 Al = z, Ac = z, Ah = z, Bl = z, Bc = z, Bh = z;
+        if (in) {
+            Ac = A[i];
+            Bc = B[i];
+            Ah = i + 1 < L ? A[i + 1] : At;
+            Bh = i + 1 < L ? B[i + 1] : Bt;
+            Al = threadIdx.x > 0 ? A[i - 1] : s_last[q][0];
+            Bl = threadIdx.x > 0 ? B[i - 1] : s_last[q][1];
+        }
+        if (threadIdx.x == blockDim.x - 1) {
+            s_last[q ^ 1][0] = Ac;
+            s_last[q ^ 1][1] = Bc;
+        }
+        __syncthreads();
+        if (!in) continue;
+        const double n = dm + i;
+        const double hi = n * pv.eps[colx + i + 1], lo = i > 0 ? (n + 1.0) * pv.eps[colx + i] : 0.0;
+        double sc;
+        if (op == OP_SYNTH_ADJ) sc = m > 0 ? 2.0 : 1.0;
+        else sc = n == 0.0 ? 0.0 : 1.0 / (n * (n + 1.0));
+        double2 s, t;
+        s.x = sc * (hi * Ah.x - lo * Al.x + dm * Bc.y);
+        s.y = sc * (hi * Ah.y - lo * Al.y - dm * Bc.x);
+        t.x = sc * (hi * Bh.x - lo * Bl.x - dm * Ac.y);
+        t.y = sc * (hi * Bh.y - lo * Bl.y + dm * Ac.x);
+        if (m == 0) s.y = t.y = 0.0;
+        A[i] = s;
+        B[i] = t;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -615,7 +656,7 @@ bool tables_ok(const PlanView<double> &pv)
 }
 
 template <int BC>
-cudaError_t synth64_go(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, bool vec,
+cudaError_t synth64_go(const PlanView<double> &pv, const double *spec, const VecSpec *vs, double *eo, int batch, Op op,
                        cudaStream_t s)
 {
     const int ng = (pv.npairs + 31) / 32, nc = (batch + BC - 1) / BC;
@@ -625,33 +666,34 @@ cudaError_t synth64_go(const PlanView<double> &pv, const double *spec, double *e
         if (e != cudaSuccess) return e;
     }
     const long items = (long)(pv.mmax + 1) * ng * nc;
-    k_synth64<BC><<<(unsigned)items, 32 * kSynWarps, smem, s>>>(pv, spec, eo, batch, ng, nc, sm_count(), vec ? 1 : 0,
-                                                                (int)op);
+    k_synth64<BC><<<(unsigned)items, 32 * kSynWarps, smem, s>>>(pv, spec, vs ? *vs : VecSpec(), eo, batch, ng, nc,
+                                                                sm_count(), vs ? 1 : 0, (int)op);
     return cudaGetLastError();
 }
 
-cudaError_t synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int bc, bool vec,
-                    cudaStream_t s)
+// Scalar from `spec`, or with `vs` the scalar form of a vector transform, from its spectra.
+cudaError_t synth64(const PlanView<double> &pv, const double *spec, const VecSpec *vs, double *eo, int batch, Op op,
+                    int bc, cudaStream_t s)
 {
     if (!tables_ok(pv)) return cudaErrorInvalidValue;
     if (bc <= 0) bc = pick_width((long)(pv.mmax + 1) * ((pv.npairs + 31) / 32), batch);
     switch (bc) {
-    case 1: return synth64_go<1>(pv, spec, eo, batch, op, vec, s);
-    case 2: return synth64_go<2>(pv, spec, eo, batch, op, vec, s);
-    case 4: return synth64_go<4>(pv, spec, eo, batch, op, vec, s);
-    case 8: return synth64_go<8>(pv, spec, eo, batch, op, vec, s);
-    case 16: return synth64_go<16>(pv, spec, eo, batch, op, vec, s);
+    case 1: return synth64_go<1>(pv, spec, vs, eo, batch, op, s);
+    case 2: return synth64_go<2>(pv, spec, vs, eo, batch, op, s);
+    case 4: return synth64_go<4>(pv, spec, vs, eo, batch, op, s);
+    case 8: return synth64_go<8>(pv, spec, vs, eo, batch, op, s);
+    case 16: return synth64_go<16>(pv, spec, vs, eo, batch, op, s);
     default: return cudaErrorInvalidValue;
     }
 }
 
 template <int BC>
-cudaError_t analys64_go(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, bool vec,
-                        cudaStream_t s)
+cudaError_t analys64_go(const PlanView<double> &pv, const double *sd, double *spec, const VecSpec *vs, int batch,
+                        Op op, cudaStream_t s)
 {
-    const dim3 grid((unsigned)((pv.lmax + (vec ? 1 : 0) + kSeedSeg) / kSeedSeg), (unsigned)(pv.mmax + 1),
+    const dim3 grid((unsigned)((pv.lmax + (vs ? 1 : 0) + kSeedSeg) / kSeedSeg), (unsigned)(pv.mmax + 1),
                     (unsigned)((batch + BC - 1) / BC));
-    k_analys64<BC><<<grid, 32 * kAnaWarps, 0, s>>>(pv, sd, spec, batch, vec ? 1 : 0, (int)op);
+    k_analys64<BC><<<grid, 32 * kAnaWarps, 0, s>>>(pv, sd, spec, vs ? *vs : VecSpec(), batch, vs ? 1 : 0, (int)op);
     return cudaGetLastError();
 }
 
@@ -663,17 +705,17 @@ inline long segments(const PlanView<double> &pv)
     return n;
 }
 
-cudaError_t analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc, bool vec,
-                     cudaStream_t s)
+cudaError_t analys64(const PlanView<double> &pv, const double *sd, double *spec, const VecSpec *vs, int batch, Op op,
+                     int bc, cudaStream_t s)
 {
     if (!tables_ok(pv)) return cudaErrorInvalidValue;
     if (bc <= 0) bc = pick_width(segments(pv), batch);
     switch (bc) {
-    case 1: return analys64_go<1>(pv, sd, spec, batch, op, vec, s);
-    case 2: return analys64_go<2>(pv, sd, spec, batch, op, vec, s);
-    case 4: return analys64_go<4>(pv, sd, spec, batch, op, vec, s);
-    case 8: return analys64_go<8>(pv, sd, spec, batch, op, vec, s);
-    case 16: return analys64_go<16>(pv, sd, spec, batch, op, vec, s);
+    case 1: return analys64_go<1>(pv, sd, spec, vs, batch, op, s);
+    case 2: return analys64_go<2>(pv, sd, spec, vs, batch, op, s);
+    case 4: return analys64_go<4>(pv, sd, spec, vs, batch, op, s);
+    case 8: return analys64_go<8>(pv, sd, spec, vs, batch, op, s);
+    case 16: return analys64_go<16>(pv, sd, spec, vs, batch, op, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -691,40 +733,39 @@ cudaError_t launch_build_qs(const PlanView<double> &pv, const unsigned long long
 cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, double *eo, int batch, Op op, int bc,
                            cudaStream_t s)
 {
-    return synth64(pv, spec, eo, batch, op, bc, false, s);
+    return synth64(pv, spec, nullptr, eo, batch, op, bc, s);
 }
 
 cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc,
                             cudaStream_t s)
 {
-    return analys64(pv, sd, spec, batch, op, bc, false, s);
+    return analys64(pv, sd, spec, nullptr, batch, op, bc, s);
 }
 
-size_t vec64_spec_bytes(int nlm, int mmax, int batch)
-{
-    return (size_t)2 * batch * ((size_t)nlm + mmax + 1) * sizeof(double2);
-}
+size_t vec64_top_bytes(int mmax, int batch) { return (size_t)2 * batch * (mmax + 1) * sizeof(double2); }
 
-cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *uw, double *eo,
-                               int batch, Op op, cudaStream_t s)
+cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *vt, double *vp,
+                               double *top, double *eo, int batch, Op op, cudaStream_t s)
 {
     if (!tables_ok(pv)) return cudaErrorInvalidValue;
+    const VecSpec vs = {reinterpret_cast<double2 *>(vt), reinterpret_cast<double2 *>(vp),
+                        reinterpret_cast<double2 *>(top), batch};
     const dim3 grid((unsigned)((pv.lmax + 2 + 127) / 128), (unsigned)(pv.mmax + 1), (unsigned)batch);
     k_vec64_split<<<grid, 128, 0, s>>>(pv, reinterpret_cast<const double2 *>(S), reinterpret_cast<const double2 *>(Tc),
-                                       reinterpret_cast<double2 *>(uw), batch, (int)op);
+                                       vs, (int)op);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return synth64(pv, uw, eo, 2 * batch, OP_SYNTH, 0, true, s);
+    return synth64(pv, nullptr, &vs, eo, 2 * batch, OP_SYNTH, 0, s);
 }
 
-cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *ab, double *S, double *Tc,
+cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *top, double *S, double *Tc,
                                 int batch, Op op, cudaStream_t s)
 {
-    cudaError_t e = analys64(pv, sd, ab, 2 * batch, OP_ANALYS, 0, true, s);
+    const VecSpec vs = {reinterpret_cast<double2 *>(S), reinterpret_cast<double2 *>(Tc),
+                        reinterpret_cast<double2 *>(top), batch};
+    cudaError_t e = analys64(pv, sd, nullptr, &vs, 2 * batch, OP_ANALYS, 0, s);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((pv.lmax + 1 + 127) / 128), (unsigned)(pv.mmax + 1), (unsigned)batch);
-    k_vec64_join<<<grid, 128, 0, s>>>(pv, reinterpret_cast<const double2 *>(ab), reinterpret_cast<double2 *>(S),
-                                      reinterpret_cast<double2 *>(Tc), batch, (int)op);
+    k_vec64_join<<<dim3((unsigned)(pv.mmax + 1), (unsigned)batch), 128, 0, s>>>(pv, vs, (int)op);
     return cudaGetLastError();
 }
 

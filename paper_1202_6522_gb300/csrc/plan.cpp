@@ -474,9 +474,6 @@ void plan_free(Plan &p)
     p.timer.pool.clear();
     if (p.tables_base) cudaFree(p.tables_base);
     if (p.work) cudaFree(p.work);
-    for (void *b : p.vspec) cudaFree(b);
-    p.vspec.clear();
-    p.vspec_bytes = 0;
     if (p.panel_s) cudaFree(p.panel_s);
     if (p.panel_a) cudaFree(p.panel_a);
     if (p.d_off_s) cudaFree(p.d_off_s);

@@ -196,8 +196,6 @@ struct Plan {
     double otf_skip_s = 0, otf_skip_a = 0;      // on-the-fly mode: fraction of chunks skipped
     void *work = nullptr;            // scratch (grown on demand)
     size_t work_bytes = 0;
-    std::vector<void *> vspec;       // spectra of the FP64 vector transforms' scalar form; the last
-    size_t vspec_bytes = 0;          // one, of this size, is in use (see ensure_vspec)
     int device = 0;
     KernelTimer timer;
     std::vector<std::pair<long long, TunedShape>> tuned;   // key: mode * 2^32 + batch
@@ -245,12 +243,13 @@ cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, doubl
                            cudaStream_t s);
 cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc,
                             cudaStream_t s);
-// Vector transforms as scalar ones of 2 batch fields: `uw` / `ab` are scratch
-// of vec64_spec_bytes; eo / sd hold the theta fields, then the phi fields.
-size_t vec64_spec_bytes(int nlm, int mmax, int batch);
-cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *uw, double *eo,
-                               int batch, Op op, cudaStream_t s);
-cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *ab, double *S, double *Tc,
+// Vector transforms as scalar ones of 2 batch fields.  eo / sd hold the theta
+// fields, then the phi fields; `top` is scratch of vec64_top_bytes, and the
+// synthesis overwrites the grids vt, vp, which its FFTs fill afterwards.
+size_t vec64_top_bytes(int mmax, int batch);
+cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *vt, double *vp,
+                               double *top, double *eo, int batch, Op op, cudaStream_t s);
+cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *top, double *S, double *Tc,
                                 int batch, Op op, cudaStream_t s);
 // Fills the plan's qs, abx, eps and hseg tables (the view's are not used).
 cudaError_t launch_build_qs(const PlanView<double> &pv, const unsigned long long *segoff, double2 *qs, double2 *abx,
