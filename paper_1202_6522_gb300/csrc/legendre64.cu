@@ -107,21 +107,25 @@ __device__ __forceinline__ bool reaches_one(double q, int hs)
 // latitude pairs, BC fields).  It takes the degrees four segments at a time: each
 // warp generates P of one segment, one pair per lane, and the segment's spectral
 // values times s_n into shared memory; then warp w sums the pairs 8 w .. 8 w + 7,
-// lane (slice, c) the products of component c (field, real/imaginary) over the
-// degrees of its slice.  With C = 2 BC components there are 32 / C slices, each
-// of one parity of n - m (16 fields: both, in turn), summed over at the end by a
-// butterfly.  The sums are spread evenly over the SM quarters whatever the
+// lane (pairs, parity, c) the products of component c (field, real/imaginary) over
+// the degrees of one parity of n - m.  With C = 2 BC components 16 / C lanes share
+// the 8 pairs of a component and parity (16 fields: a lane takes both parities).
+// Every sum runs over the degrees in order whatever BC is, so a field's result
+// does not depend on the batch it comes in (lanes as slices of the degrees took
+// the same time).  The sums are spread evenly over the SM quarters whatever the
 // number of segments (2 x 16 vector fields at N = 127: 165 us with a warp per
 // segment and 16 fields, 130 us).  16 fields at N = 511: 1981 us with three
-// instructions per step and 8 fields, 1766 with two and 16 fields a warp, 1656 us;
+// instructions per step and 8 fields, 1766 with two and 16 fields a warp, 1653 us;
 // one field at N = 255: 134 -> 42 us.  vec: the spectra run to degree lmax + 1,
 // the recurrence is Sec. 3.2's, and the sums are divided by sin(theta).
 // ---------------------------------------------------------------------------
 constexpr int kSynWarps = 4;
-constexpr int kSynRow = 34;   // row of the P tile: 32 pairs, 16-byte aligned rows on shifted banks
+// row of the P tile: 32 pairs, 16-byte aligned rows on shifted banks (two rows by four
+// lanes of one pair each at 1 field)
+template <int BC> constexpr int kSynRow = BC == 1 ? 36 : 34;
 template <int BC> constexpr size_t synth64_smem()
 {
-    return sizeof(double) * (kSynWarps * kSeedSeg * ((2 * BC + 2) + kSynRow));
+    return sizeof(double) * (kSynWarps * kSeedSeg * ((2 * BC + 2) + kSynRow<BC>));
 }
 
 template <int BC>
@@ -129,10 +133,12 @@ __global__ void __launch_bounds__(32 * kSynWarps)
 k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, double *__restrict__ eo, int batch,
           int ngroups, int nchunk, int nsm, int vec, int op)
 {
-    constexpr int C = 2 * BC, SL = 32 / C, W = kSynWarps, FS = C + 2, PAR = SL == 1 ? 2 : 1, PW = 32 / W;
+    // PW pairs per warp; a lane takes NP of them and PAR parities
+    constexpr int C = 2 * BC, W = kSynWarps, FS = C + 2, PW = 32 / W, PAR = C == 32 ? 2 : 1, NP = C == 32 ? PW : PW * C / 16;
+    constexpr int kRow = kSynRow<BC>;
     extern __shared__ __align__(16) double s_mem[];
     double *s_f = s_mem;                              // [W kSeedSeg degrees][FS]
-    double *s_P = s_mem + W * kSeedSeg * FS;          // [W kSeedSeg degrees][kSynRow]
+    double *s_P = s_mem + W * kSeedSeg * FS;          // [W kSeedSeg degrees][kRow]
     __shared__ double s_a[W][kMaxDeg], s_beta[W][kMaxDeg];
     __shared__ int s_hs[W][kMaxDeg];
 
@@ -150,12 +156,12 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
     const double x = valid ? pv.x[p] : 0.0;
     const int first = (vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g];
     const double insc = (op == OP_ANALYS_ADJ && m > 0) ? 0.5 : 1.0;   // adjoint of analysis: b / c_m
-    const int c = lane % C, slice = lane / C;
+    const int c = lane % C, par = PAR == 2 ? 0 : (lane / C) & 1, pq = PW * w + (PAR == 2 ? 0 : lane / (2 * C)) * NP;
     const int u = (w + item) & (W - 1);   // the segment of a block this warp generates (turned from CTA to CTA)
 
-    double acc[PAR][PW];
+    double acc[PAR][NP];
 #pragma unroll
-    for (int q = 0; q < PW; ++q)
+    for (int q = 0; q < NP; ++q)
 #pragma unroll
         for (int r = 0; r < PAR; ++r) acc[r][q] = 0.0;
 
@@ -189,13 +195,18 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
             }
             const double sc = vec ? 1.0 : fs * insc;
             double *row = s_f + (u * kSeedSeg + lane) * FS;
+            // this lane's degree of field f: at (f < nb ? pa : pb) + f * step
+            const int i = sg * kSeedSeg + lane;
+            const bool top = i == Ls;
+            const int nb = vec ? vs.nb : batch;
+            const size_t step = top ? pv.mmax + 1 : pv.nlm;
+            const double2 *pa = top ? vs.top + m : (vec ? vs.u : spec2) + col + i;
+            const double2 *pb = top ? pa : vs.w + col + i - (size_t)nb * pv.nlm;
 #pragma unroll
             for (int b = 0; b < BC; ++b) {
                 double2 f = make_double2(0.0, 0.0);
                 if (lane < cnt && b0 + b < batch) {
-                    const int i = sg * kSeedSeg + lane;
-                    const double2 *src = vec ? vs.field(b0 + b, pv.nlm) : spec2 + (size_t)(b0 + b) * pv.nlm;
-                    f = __ldg(i < Ls ? src + col + i : vs.top + (size_t)(b0 + b) * (pv.mmax + 1) + m);
+                    f = __ldg((b0 + b < nb ? pa : pb) + (size_t)(b0 + b) * step);
                     if (!vec) {
                         f.x *= sc;
                         f.y *= sc;
@@ -205,7 +216,7 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
                 *reinterpret_cast<double2 *>(row + 2 * b) = f;
             }
             __syncwarp();
-            double *Pt = s_P + u * kSeedSeg * kSynRow + lane;
+            double *Pt = s_P + u * kSeedSeg * kRow + lane;
             const bool scaled = __any_sync(kFull, k > 0);
             for (int t = 0; t < nstep; ++t) {
                 double yn = fma(vec ? s_a[u][t] * x : x, y1, s_beta[u][t] * y2);
@@ -220,54 +231,41 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
                     v = k == 0 ? yn : 0.0;
                 }
                 y1 = yn;
-                if (!tail) Pt[t * kSynRow] = v;
+                if (!tail) Pt[t * kRow] = v;
                 else if (t == kSeedSeg) Pt[0] = v;
-                else if (t > 0 && t < 16) Pt[t * kSynRow] = 0.0;
+                else if (t > 0 && t < 16) Pt[t * kRow] = 0.0;
             }
         }
         __syncthreads();
         // rows past the order's last degree, up to a multiple of 16, hold zeros times finite values
         const int nd = min(W * kSeedSeg, L - sb * kSeedSeg);
-        const double *fd = s_f + slice * FS + c, *Pd = s_P + slice * kSynRow + PW * w;
-        const int nj = (nd + SL * PAR - 1) / (SL * PAR);
-#pragma unroll 2
+        const double *fd = s_f + par * FS + c, *Pd = s_P + par * kRow + pq;
+        const int nj = (nd + 1) / 2;
+#pragma unroll (NP >= 8 ? 2 : 16 / NP)
         for (int j = 0; j < nj; ++j) {
 #pragma unroll
             for (int r = 0; r < PAR; ++r) {
-                const double f = fd[(j * PAR + r) * SL * FS];
-                const double2 *P2 = reinterpret_cast<const double2 *>(Pd + (j * PAR + r) * SL * kSynRow);
+                const double f = fd[(2 * j + r) * FS];
+                const double *Pj = Pd + (2 * j + r) * kRow;
+                if constexpr (NP == 1) {
+                    acc[r][0] = fma(f, Pj[0], acc[r][0]);
+                } else {
 #pragma unroll
-                for (int q = 0; q < PW / 2; ++q) {
-                    const double2 v = P2[q];
-                    acc[r][2 * q] = fma(f, v.x, acc[r][2 * q]);
-                    acc[r][2 * q + 1] = fma(f, v.y, acc[r][2 * q + 1]);
+                    for (int q = 0; q < NP / 2; ++q) {
+                        const double2 v = reinterpret_cast<const double2 *>(Pj)[q];
+                        acc[r][2 * q] = fma(f, v.x, acc[r][2 * q]);
+                        acc[r][2 * q + 1] = fma(f, v.y, acc[r][2 * q + 1]);
+                    }
                 }
             }
         }
         __syncthreads();
     }
-    // over the slices of one parity (lane bits 2 C .. 16): a lane keeps half of its pairs each time
+    // [field][pair][E, O][part], in the P tile
 #pragma unroll
-    for (int o = 16; o >= 2 * C; o >>= 1) {
-        const int h = PW * o / 32;
-        const bool up = (lane & o) != 0;
+    for (int r = 0; r < PAR; ++r)
 #pragma unroll
-        for (int q = 0; q < h; ++q) {
-            const double send = up ? acc[0][q] : acc[0][q + h];
-            const double keep = up ? acc[0][q + h] : acc[0][q];
-            acc[0][q] = keep + __shfl_xor_sync(kFull, send, o);
-        }
-    }
-    {
-        // [field][pair][E, O][part], in the P tile
-        constexpr int V = SL == 1 ? PW : PW * C / 16;   // pairs held
-        const int off = SL == 1 ? 0 : (lane & ~(2 * C - 1)) * PW / 32;
-#pragma unroll
-        for (int r = 0; r < PAR; ++r)
-#pragma unroll
-            for (int q = 0; q < V; ++q)
-                s_P[(((c >> 1) * 32 + PW * w + off + q) * 2 + (SL == 1 ? r : slice & 1)) * 2 + (c & 1)] = acc[r][q];
-    }
+        for (int q = 0; q < NP; ++q) s_P[(((c >> 1) * 32 + pq + q) * 2 + par + r) * 2 + (c & 1)] = acc[r][q];
     __syncthreads();
     double2 *eo2 = reinterpret_cast<double2 *>(eo);
     for (int i = threadIdx.x; i < BC * 64; i += 32 * W) {
@@ -288,17 +286,19 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
 // segment of kSeedSeg degrees, BC fields).  It takes the latitude pairs 128 at a
 // time: each warp generates P of the segment for 32 of them, one pair per lane,
 // into shared memory; then warp w sums degrees 8 w .. 8 w + 7 over all 128,
-// lane (slice, c) the products of component c (field, real/imaginary) over the
-// pairs of its slice, one accumulator per degree.  With C = 2 BC components there
-// are 32 / C slices, so the sum over latitudes needs one butterfly over the
-// slices per segment (none at 16 fields); a lane per pair instead needs an FP64
-// butterfly over all 32 lanes for every 16 / BC degrees -- with 96 pairs a third
-// on top of the sums -- and a warp per segment leaves SM quarters idle where
-// segments are few.  16 fields at N = 511: 2357 us with lanes as pairs and 8
-// fields, 1633 us; 2 x 16 vector fields at N = 127: 926 -> 162 us; one field at
-// N = 255: 67 -> 44 us.  Every sum has a fixed order, so results are bitwise
-// reproducible.  The groups of 32 pairs before the first one with a live pair in
-// the segment (static polar optimisation, Sec. 3.1) are left out.
+// lane (degrees, half, c) the products of component c (field, real/imaginary) over
+// the even or the odd pairs.  With C = 2 BC components 16 / C lanes share the 8
+// degrees of a component and half (16 fields: a lane takes both halves), and the
+// sum over latitudes needs one exchange per degree; a lane per pair instead needs
+// an FP64 butterfly over all 32 lanes for every 16 / BC degrees -- with 96 pairs a
+// third on top of the sums -- and a warp per segment leaves SM quarters idle where
+// segments are few.  Every half is summed over its pairs in order whatever BC is,
+// so a field's result does not depend on the batch it comes in.  16 fields at
+// N = 511: 2357 us with lanes as pairs and 8 fields, 1644 us (1636 with lanes as
+// slices of the pairs, 32 / C of them, whose sums depended on BC); 2 x 16 vector
+// fields at N = 127: 926 -> 164 us; one field at N = 255: 67 -> 43 us.  The groups
+// of 32 pairs before the first one with a live pair in the segment (static polar
+// optimisation, Sec. 3.1) are left out.
 //
 // blockIdx: x segment (with `vec`, see k_synth64, the degree lmax + 1 is one
 // more, alone in its block when the order's degrees fill their segments: it
@@ -311,8 +311,10 @@ __global__ void __launch_bounds__(32 * kAnaWarps)
 k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restrict__ spec, VecSpec vs, int batch,
            int vec, int op)
 {
-    constexpr int C = 2 * BC, SL = 32 / C, W = kAnaWarps, DB = kSeedSeg / W;
-    constexpr int NQ = W * 32 / SL;   // pairs of a slice per block of 128
+    // DB degrees per warp; a lane takes ND of them and HV halves of the pairs (the even, the odd ones)
+    constexpr int C = 2 * BC, W = kAnaWarps, DB = kSeedSeg / W, HV = C == 32 ? 2 : 1, ND = C == 32 ? DB : DB * C / 16;
+    // folds in flight: pairs of a half ahead of the sums, one fold per pair where a lane has one degree
+    constexpr int AH = 16 / ND / HV, NF = ND == 1 ? 1 : 2;
     __shared__ double s_P[W][kSeedSeg][33];
     __shared__ double s_a[kSeedSeg + DB], s_beta[kSeedSeg + DB];
     __shared__ int s_hs[kSeedSeg + DB];
@@ -348,13 +350,17 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
     __syncthreads();
     const int g0 = s_g0;
 
-    // this lane's component and slice of the pairs, this warp's degrees
-    const int c = lane % C, slice = lane / C, b = b0 + (c >> 1), d0 = w * DB;
-    const double *fold = sd + ((size_t)b * (pv.mmax + 1) + m) * npairs * 4 + (c & 1);   // s at 4 q, d at 4 q + 2
-    const bool has = b < batch && d0 < cnt;
-    double acc[DB];
+    // this lane's component, half and degrees
+    const int c = lane % C, half = HV == 2 ? 0 : (lane / C) & 1, b = b0 + (c >> 1);
+    const int dw = w * DB, d0 = dw + (HV == 2 ? 0 : lane / (2 * C)) * ND;
+    // s at 4 q, d at 4 q + 2 (a lane with one degree: the one its parity takes)
+    const double *fold = sd + ((size_t)b * (pv.mmax + 1) + m) * npairs * 4 + (c & 1) + (ND == 1 ? 2 * (d0 & 1) : 0);
+    const bool has = b < batch && dw < cnt;
+    double acc[HV][ND];
 #pragma unroll
-    for (int t = 0; t < DB; ++t) acc[t] = 0.0;
+    for (int h = 0; h < HV; ++h)
+#pragma unroll
+        for (int t = 0; t < ND; ++t) acc[h][t] = 0.0;
 
     for (int gb = g0; gb < ngroups; gb += W) {
         const int p = (gb + w) * 32 + lane;
@@ -370,15 +376,19 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
             y2 = v.y * down;
             k = __ldg(pv.seeds64k + o);
         }
-        // the folds of the slice's pairs, two pairs ahead of the sums
-        const int q0 = gb * 32 + slice;
-        double sv[2], dv[2];
+        // the folds, AH pairs of a half ahead of the sums
+        const int nq = min(64, (npairs - gb * 32 + 1) / 2);   // pairs of a half in this block
+        double fv[AH][HV][NF];
+        const auto fetch = [&](int j, int h, double (&f)[NF]) {
+            const int q = gb * 32 + 2 * j + half + h;
+            const bool in = has && j < nq && q < npairs;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int q = q0 + u * SL;
-            sv[u] = has && q < npairs ? __ldg(fold + (size_t)q * 4) : 0.0;
-            dv[u] = has && q < npairs ? __ldg(fold + (size_t)q * 4 + 2) : 0.0;
-        }
+            for (int i = 0; i < NF; ++i) f[i] = in ? __ldg(fold + (size_t)q * 4 + 2 * i) : 0.0;
+        };
+#pragma unroll
+        for (int u = 0; u < AH; ++u)
+#pragma unroll
+            for (int h = 0; h < HV; ++h) fetch(u, h, fv[u][h]);
         __syncthreads();   // the last block's sums are done with s_P
         if (gb + w < ngroups) {
             const bool scaled = __any_sync(kFull, k > 0);
@@ -400,46 +410,35 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
             }
         }
         __syncthreads();
-        if (d0 < cnt) {
-            const int nq = min(NQ, (npairs - gb * 32 + SL - 1) / SL);
-#pragma unroll 2
-            for (int j = 0; j < nq; ++j) {
-                const int r = j * SL + slice;   // pair within the block
-                const double *P = &s_P[r >> 5][d0][r & 31];
-                const double s = sv[j & 1], d = dv[j & 1];
-                const int q = q0 + (j + 2) * SL;
-                sv[j & 1] = has && j + 2 < nq && q < npairs ? __ldg(fold + (size_t)q * 4) : 0.0;
-                dv[j & 1] = has && j + 2 < nq && q < npairs ? __ldg(fold + (size_t)q * 4 + 2) : 0.0;
+        if (dw < cnt) {
+            const auto add = [&](int j, double (&f)[HV][NF]) {
 #pragma unroll
-                for (int t = 0; t < DB; ++t) acc[t] = fma(P[t * 33], (t & 1) ? d : s, acc[t]);
-            }
+                for (int h = 0; h < HV; ++h) {
+                    const int r = 2 * j + half + h;   // pair within the block
+                    const double *P = &s_P[r >> 5][d0][r & 31];
+                    const double s = f[h][0], d = f[h][NF - 1];
+                    if (ND == DB) fetch(j + AH, h, f[h]);   // (few pairs ahead: before the sums)
+#pragma unroll
+                    for (int t = 0; t < ND; ++t) acc[h][t] = fma(P[t * 33], (t & 1) ? d : s, acc[h][t]);
+                    if (ND < DB) fetch(j + AH, h, f[h]);
+                }
+            };
+            int j = 0;
+#pragma unroll 1
+            for (; j + AH <= nq; j += AH)
+#pragma unroll
+                for (int u = 0; u < AH; ++u) add(j + u, fv[u]);
+#pragma unroll
+            for (int u = 0; u < AH - 1; ++u)
+                if (j + u < nq) add(j + u, fv[u]);
         }
     }
-    // over the slices (lane bits C .. 16): while a lane holds several degrees it
-    // keeps half of them, then both lanes of a pair keep the sum
+    // even and odd pairs
 #pragma unroll
-    for (int o = 16; o >= C; o >>= 1) {
-        const int h = DB * o / 32;   // degrees kept (0: one degree left, add)
-        if (h > 0) {
-            const bool up = (lane & o) != 0;
-#pragma unroll
-            for (int t = 0; t < h; ++t) {
-                const double send = up ? acc[t] : acc[t + h];
-                const double keep = up ? acc[t + h] : acc[t];
-                acc[t] = keep + __shfl_xor_sync(kFull, send, o);
-            }
-        } else {
-            acc[0] += __shfl_xor_sync(kFull, acc[0], o);
-        }
-    }
+    for (int t = 0; t < ND; ++t) acc[0][t] += HV == 2 ? acc[HV - 1][t] : __shfl_xor_sync(kFull, acc[0][t], C & 31);
     __syncthreads();
-    {
-        // degrees held: DB C / 32 (at least one) from the kept halves' offset
-        constexpr int V = DB * C / 32 > 0 ? DB * C / 32 : 1;
-        const int off = (lane & ~(C - 1)) * DB / 32 / V * V;
 #pragma unroll
-        for (int t = 0; t < V; ++t) s_P[0][d0 + off + t][c] = acc[t];
-    }
+    for (int t = 0; t < ND; ++t) s_P[0][d0 + t][c] = acc[0][t];   // the same from either half's lane
     __syncthreads();
     if (lane >= cnt) return;
     // P_n = s_n Q_n; c_m for the adjoint of synthesis
