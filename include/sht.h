@@ -79,7 +79,9 @@ enum {
                         * (built by the first call in this mode or by sht_reserve: 20 B
                         * per latitude pair and 32 degrees, 175 MB at lmax = 1023, and
                         * 40 B per coefficient).  Vector calls form the spectra of two
-                        * scalar transforms in their output arrays before they fill them. */
+                        * scalar transforms in their output arrays before they fill them,
+                        * and run without the tables, slower, where these cannot be had:
+                        * in a first call that is captured, or for want of memory. */
     SHT_F32 = 1,       /* FP32 data and recurrence restarted every 32 degrees from
                         * states the FP64 recurrence computes once per plan, each held
                         * with the power-of-two scale of its segment (the explicit

@@ -295,6 +295,18 @@ int ensure_seeds64(sht::Plan &p)
     return rc ? fail(rc, err) : SHT_OK;
 }
 
+// FP64 vector transforms run without the tables where these cannot be had: under
+// capture, or for want of memory (legendre64.cu).
+int vector_tables64(sht::Plan &p, cudaStream_t s)
+{
+    if (p.seeds64) return SHT_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap == cudaStreamCaptureStatusActive) return SHT_OK;
+    const int rc = ensure_seeds64(p);
+    return rc == SHT_ENOMEM ? SHT_OK : rc;
+}
+
 size_t elem_size(int mode) { return (mode == SHT_F64 || mode == SHT_TC_F64) ? sizeof(double) : sizeof(float); }
 
 // FP64-accurate tensor-core mode: digit-slice panels (about 6 (lmax+1)^3
@@ -697,7 +709,7 @@ int vector_s2g(sht_handle h, const void *S, const void *T, void *vt, void *vp, i
         return run_synth_vec_tc(h->p, S, T, vt, vp, batch, op, s);
     }
     if (mode == SHT_F32 && (rc = ensure_seeds32(h->p))) return rc;
-    if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
+    if (mode == SHT_F64 && (rc = vector_tables64(h->p, s))) return rc;
     if ((rc = ensure_work(h->p, vec_work_bytes(h->p, batch, mode)))) return rc;
     if (mode == SHT_F64) return run_synth_vec<double>(h->p, h->p.view64(), S, T, vt, vp, batch, op, s);
     return run_synth_vec<float>(h->p, h->p.view32(), S, T, vt, vp, batch, op, s);
@@ -717,7 +729,7 @@ int vector_g2s(sht_handle h, const void *vt, const void *vp, void *S, void *T, i
         return run_analys_vec_tc(h->p, vt, vp, S, T, batch, op, s);
     }
     if (mode == SHT_F32 && (rc = ensure_seeds32(h->p))) return rc;
-    if (mode == SHT_F64 && (rc = ensure_seeds64(h->p))) return rc;
+    if (mode == SHT_F64 && (rc = vector_tables64(h->p, s))) return rc;
     if ((rc = ensure_work(h->p, vec_work_bytes(h->p, batch, mode)))) return rc;
     if (mode == SHT_F64) return run_analys_vec<double>(h->p, h->p.view64(), vt, vp, S, T, batch, op, s);
     return run_analys_vec<float>(h->p, h->p.view32(), vt, vp, S, T, batch, op, s);
@@ -1014,6 +1026,7 @@ int sht_reserve(sht_handle h, int batch, int mode)
     }
     if (mode == SHT_TC_F64) {
         if ((rc = ensure_panels64(h->p))) return rc;
+        if ((rc = vector_tables64(h->p, 0))) return rc;   // vector calls of this mode run SHT_F64
         return ensure_work(h->p, tc64_work_bytes(h->p, batch));
     }
     if ((mode == SHT_F32 || mode == SHT_F32_AUTO) && (rc = ensure_seeds32(h->p))) return rc;

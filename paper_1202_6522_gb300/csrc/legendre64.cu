@@ -69,15 +69,43 @@ struct VecSpec {
     }
 };
 
+// (a_n, b_n) of Sec. 3.2 at degree m mres + i, i = 0 .. L (degree lmax + 1), and eps_n.
+__device__ double2 plain_ab(const PlanView<double> &pv, int m, int i)
+{
+    const double dm = m * pv.mres, n = dm + i, n1 = n - 1.0;
+    if (i == 0) return make_double2(0.0, 1.0);   // the start value P_m^m, handed over as P_{m-2}
+    if (i < pv.lmax - m * pv.mres + 1) return pv.ab[col_ext(pv, m, 0) + i];
+    if (i == 1) return make_double2(sqrt(2.0 * dm + 3.0), 0.0);
+    return make_double2(sqrt((4.0 * n * n - 1.0) / (n * n - dm * dm)),
+                        -sqrt((2.0 * n + 1.0) / (2.0 * n - 3.0) * (n1 * n1 - dm * dm) / (n * n - dm * dm)));
+}
+__device__ double plain_eps(const PlanView<double> &pv, int m, int i)
+{
+    const double dm = m * pv.mres, n = dm + i;
+    return i == 0 ? 0.0 : sqrt((n * n - dm * dm) / (4.0 * n * n - 1.0));
+}
+
+// A vector transform whose plan has no tables -- a first call that is captured, in
+// which nothing can be allocated, or tables that do not fit -- computes them as it
+// goes: (a_n, b_n), eps_n and the segments' states, stepped to from P_m^m.  The
+// same values bit for bit, at the cost of the steps (a segment in the middle of an
+// order of 32 S degrees takes 16 S of them).  The kernels' parameter TAB.
+__device__ __forceinline__ double eps_at(const PlanView<double> &pv, long colx, int m, int i)
+{
+    return pv.eps ? pv.eps[colx + i] : plain_eps(pv, m, i);
+}
+
 // One step of the recurrence, y_n = a x y_{n-1} + b y_{n-2}, and the factor s_n of
-// the value: (beta_n, s_n) of Q_n, where a = 1 is left out by the caller, or
-// (a_n, b_n) of P_n itself (`plain`).  Zeros past the order's last degree.
+// the value, at degree m mres + i: (beta_n, s_n) of Q_n, where a = 1 is left out by
+// the caller, or (a_n, b_n) of P_n itself (`plain`).  Zeros past the order's last degree.
+// col: the order's first index in the tables.
 struct Step { double a, b, s; };
-__device__ __forceinline__ Step step_of(const PlanView<double> &pv, long i, bool in, bool plain)
+template <bool TAB>
+__device__ __forceinline__ Step step_of(const PlanView<double> &pv, long col, int m, int i, bool in, bool plain)
 {
     Step r = {0.0, 0.0, 0.0};
     if (!in) return r;
-    const double2 v = __ldg((plain ? pv.abx : pv.qs) + i);
+    const double2 v = TAB ? __ldg((plain ? pv.abx : pv.qs) + col + i) : plain_ab(pv, m, i);
     if (plain) {
         r.a = v.x;
         r.b = v.y;
@@ -89,10 +117,34 @@ __device__ __forceinline__ Step step_of(const PlanView<double> &pv, long i, bool
     return r;
 }
 
-// The power of two that takes a segment's stored state back to P.
-__device__ __forceinline__ double seg_down(const PlanView<double> &pv, int m, int seg)
+// The state entering a segment for pair p, y 2^(-240 k): of Q, or of P (`plain`).
+struct State { double y1, y2; int k; };
+__device__ State stepped_state(const PlanView<double> &pv, int m, int seg, int p)
 {
-    return __hiloint2double((1023 - __ldg(pv.hseg + pv.segoff[m] + seg)) << 20, 0);
+    const double x = pv.x[p];
+    State v = {0.0, pv.pmm[(size_t)m * pv.npairs + p], pv.pmmk[(size_t)m * pv.npairs + p]};
+    const double2 *ab = pv.ab + col_ext(pv, m, 0);
+    for (int i = 0; i < seg * kSeedSeg; ++i) {   // as k_build_restarts
+        const double yn = fma(ab[i].x * x, v.y1, ab[i].y * v.y2);
+        v.y2 = v.y1;
+        v.y1 = yn;
+        if (v.k > 0 && (__double2hiint(yn) & 0x7fffffff) >= kHiOne) {
+            v.y1 *= kDown;
+            v.y2 *= kDown;
+            v.k -= 1;
+        }
+    }
+    return v;
+}
+template <bool TAB>
+__device__ __forceinline__ State state_of(const PlanView<double> &pv, int m, int seg, int p, bool plain)
+{
+    if (!TAB) return stepped_state(pv, m, seg, p);
+    const size_t i = pv.segoff[m] + seg, o = i * pv.npairs + p;
+    const double2 v = __ldg(pv.seeds64 + o);
+    // the power of two that takes the segment's stored state back to P
+    const double down = plain ? __hiloint2double((1023 - __ldg(pv.hseg + i)) << 20, 0) : 1.0;
+    return State{v.x * down, v.y * down, __ldg(pv.seeds64k + o)};
 }
 
 // |Q| s >= 1 to within the 2^-20 of the high words' sum (a rescaling test: see
@@ -128,7 +180,7 @@ template <int BC> constexpr size_t synth64_smem()
     return sizeof(double) * (kSynWarps * kSeedSeg * ((2 * BC + 2) + kSynRow<BC>));
 }
 
-template <int BC>
+template <int BC, bool TAB>
 __global__ void __launch_bounds__(32 * kSynWarps)
 k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, double *__restrict__ eo, int batch,
           int ngroups, int nchunk, int nsm, int vec, int op)
@@ -154,7 +206,7 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
     const int p = g * 32 + lane;
     const bool valid = p < npairs;
     const double x = valid ? pv.x[p] : 0.0;
-    const int first = (vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g];
+    const int first = TAB ? (vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g] : 0;
     const double insc = (op == OP_ANALYS_ADJ && m > 0) ? 0.5 : 1.0;   // adjoint of analysis: b / c_m
     const int c = lane % C, par = PAR == 2 ? 0 : (lane / C) & 1, pq = PW * w + (PAR == 2 ? 0 : lane / (2 * C)) * NP;
     const int u = (w + item) & (W - 1);   // the segment of a block this warp generates (turned from CTA to CTA)
@@ -177,17 +229,15 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
             double y1 = 0.0, y2 = 0.0;
             int k = 0;
             if (valid) {
-                const size_t o = (size_t)(pv.segoff[m] + seg) * npairs + p;
-                const double2 v = __ldg(pv.seeds64 + o);
-                const double down = vec ? seg_down(pv, m, seg) : 1.0;
-                y1 = v.x * down;
-                y2 = v.y * down;
-                k = __ldg(pv.seeds64k + o);
+                const State v = state_of<TAB>(pv, m, seg, p, vec);
+                y1 = v.y1;
+                y2 = v.y2;
+                k = v.k;
             }
             double fs = 1.0;   // s_n of this lane's degree
             for (int t = lane; t < nstep; t += 32) {
                 const int d = seg * kSeedSeg + t;
-                const Step st = step_of(pv, colq + d, d < L, vec);
+                const Step st = step_of<TAB>(pv, colq, m, d, d < L, vec);
                 s_a[u][t] = st.a;
                 s_beta[u][t] = st.b;
                 s_hs[u][t] = __double2hiint(st.s) - kHiOne;
@@ -306,7 +356,7 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
 // ---------------------------------------------------------------------------
 constexpr int kAnaWarps = 4;
 
-template <int BC>
+template <int BC, bool TAB>
 __global__ void __launch_bounds__(32 * kAnaWarps)
 k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restrict__ spec, VecSpec vs, int batch,
            int vec, int op)
@@ -334,7 +384,7 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
     if (threadIdx.x == 0) s_g0 = ngroups;
     if (threadIdx.x < nstep) {
         const int t = threadIdx.x;
-        const Step st = step_of(pv, colq + t, seg * kSeedSeg + t < L, vec);
+        const Step st = step_of<TAB>(pv, colq - seg * kSeedSeg, m, seg * kSeedSeg + t, seg * kSeedSeg + t < L, vec);
         s_a[t] = st.a;
         s_beta[t] = st.b;
         s_hs[t] = __double2hiint(st.s) - kHiOne;
@@ -343,7 +393,7 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
         for (int t = 1; t < DB; ++t) s_P[w][t][lane] = 0.0;
     __syncthreads();
     for (int g = threadIdx.x; g < ngroups; g += 32 * W)
-        if ((vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g] <= seg) {
+        if (!TAB || (vec ? pv.glive_vec : pv.glive)[(size_t)m * ngroups + g] <= seg) {
             atomicMin(&s_g0, g);
             break;
         }
@@ -368,13 +418,11 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
         double x = 0.0, y1 = 0.0, y2 = 0.0;
         int k = 0;
         if (valid) {
-            const size_t o = (size_t)(pv.segoff[m] + seg) * npairs + p;
-            const double2 v = __ldg(pv.seeds64 + o);
+            const State v = state_of<TAB>(pv, m, seg, p, vec);
             x = pv.x[p];
-            const double down = vec ? seg_down(pv, m, seg) : 1.0;
-            y1 = v.x * down;
-            y2 = v.y * down;
-            k = __ldg(pv.seeds64k + o);
+            y1 = v.y1;
+            y2 = v.y2;
+            k = v.k;
         }
         // the folds, AH pairs of a half ahead of the sums
         const int nq = min(64, (npairs - gb * 32 + 1) / 2);   // pairs of a half in this block
@@ -480,7 +528,7 @@ k_vec64_split(PlanView<double> pv, const double2 *__restrict__ S, const double2 
         }
         return v;
     };
-    const double lo = (k - 1.0) * pv.eps[colx + i], hi = i < L ? (k + 2.0) * pv.eps[colx + i + 1] : 0.0;
+    const double lo = (k - 1.0) * eps_at(pv, colx, m, i), hi = i < L ? (k + 2.0) * eps_at(pv, colx, m, i + 1) : 0.0;
     const double2 Sl = load(Sb, i - 1), Sc = load(Sb, i), Sh = load(Sb, i + 1);
     const double2 Tl = load(Tb, i - 1), Tc = load(Tb, i), Th = load(Tb, i + 1);
     double2 U, W;
@@ -530,7 +578,7 @@ __global__ void __launch_bounds__(128) k_vec64_join(PlanView<double> pv, VecSpec
         __syncthreads();
         if (!in) continue;
         const double n = dm + i;
-        const double hi = n * pv.eps[colx + i + 1], lo = i > 0 ? (n + 1.0) * pv.eps[colx + i] : 0.0;
+        const double hi = n * eps_at(pv, colx, m, i + 1), lo = i > 0 ? (n + 1.0) * eps_at(pv, colx, m, i) : 0.0;
         double sc;
         if (op == OP_SYNTH_ADJ) sc = m > 0 ? 2.0 : 1.0;
         else sc = n == 0.0 ? 0.0 : 1.0 / (n * (n + 1.0));
@@ -576,7 +624,7 @@ k_build_qs(PlanView<double> pv, const unsigned long long *__restrict__ segoff, d
     const int Ls = pv.lmax - m * pv.mres + 1;
     const int nseg = (Ls + kSeedSeg - 1) / kSeedSeg;
     if (seg >= nseg) return;
-    const long colx = col_ext(pv, m, 1), col = col_ext(pv, m, 0);
+    const long colx = col_ext(pv, m, 1);
     const int i0 = seg * kSeedSeg;
     const auto ratio = [&](int i) {   // s_n^2 / s_{n-1}^2 at degree dm + i
         dd r = {1.0, 0.0};
@@ -589,22 +637,14 @@ k_build_qs(PlanView<double> pv, const unsigned long long *__restrict__ segoff, d
         const double n = dm + i, n1 = n - 1.0;
         if (i == 0) {   // Q_m is the start value P_m^m, handed over as Q_{m-2}
             qs[colx] = make_double2(1.0, scalbn(1.0, -h));
-            abx[colx] = make_double2(0.0, 1.0);
+            abx[colx] = plain_ab(pv, m, 0);
             eps[colx] = 0.0;
             return;
         }
         const double bb = i == 1 ? 0.0 : (n1 * n1 - dm * dm) / (4.0 * n1 * n1 - 1.0);   // eps_{n-1}^2
         qs[colx + i] = make_double2(i == i0 ? -sqrt(bb) : -bb, scalbn(sqrt(s2.h), -h));
-        eps[colx + i] = sqrt((n * n - dm * dm) / (4.0 * n * n - 1.0));
-        double2 ab;
-        if (i < Ls)
-            ab = pv.ab[col + i];
-        else if (i == 1)
-            ab = make_double2(sqrt(2.0 * dm + 3.0), 0.0);
-        else
-            ab = make_double2(sqrt((4.0 * n * n - 1.0) / (n * n - dm * dm)),
-                              -sqrt((2.0 * n + 1.0) / (2.0 * n - 3.0) * (n1 * n1 - dm * dm) / (n * n - dm * dm)));
-        abx[colx + i] = ab;
+        eps[colx + i] = plain_eps(pv, m, i);
+        abx[colx + i] = plain_ab(pv, m, i);
     };
     dd s2 = ratio(i0 + lane);
 #pragma unroll
@@ -649,23 +689,25 @@ inline int pick_width(long units, int batch)
     return bc;
 }
 
-bool tables_ok(const PlanView<double> &pv)
+// All of the tables, or with `vec` none of them.
+bool tables_ok(const PlanView<double> &pv, bool vec)
 {
+    if (vec && !pv.seeds64) return pv.ab && pv.pmm && pv.pmmk && !pv.eps;
     return pv.segoff && pv.seeds64 && pv.seeds64k && pv.glive && pv.glive_vec && pv.qs && pv.abx && pv.eps && pv.hseg;
 }
 
-template <int BC>
+template <int BC, bool TAB = true>
 cudaError_t synth64_go(const PlanView<double> &pv, const double *spec, const VecSpec *vs, double *eo, int batch, Op op,
                        cudaStream_t s)
 {
     const int ng = (pv.npairs + 31) / 32, nc = (batch + BC - 1) / BC;
     constexpr size_t smem = synth64_smem<BC>();
     if (smem > 40 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_synth64<BC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_synth64<BC, TAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     const long items = (long)(pv.mmax + 1) * ng * nc;
-    k_synth64<BC><<<(unsigned)items, 32 * kSynWarps, smem, s>>>(pv, spec, vs ? *vs : VecSpec(), eo, batch, ng, nc,
+    k_synth64<BC, TAB><<<(unsigned)items, 32 * kSynWarps, smem, s>>>(pv, spec, vs ? *vs : VecSpec(), eo, batch, ng, nc,
                                                                 sm_count(), vs ? 1 : 0, (int)op);
     return cudaGetLastError();
 }
@@ -674,7 +716,8 @@ cudaError_t synth64_go(const PlanView<double> &pv, const double *spec, const Vec
 cudaError_t synth64(const PlanView<double> &pv, const double *spec, const VecSpec *vs, double *eo, int batch, Op op,
                     int bc, cudaStream_t s)
 {
-    if (!tables_ok(pv)) return cudaErrorInvalidValue;
+    if (!tables_ok(pv, vs != nullptr)) return cudaErrorInvalidValue;
+    if (!pv.seeds64) return synth64_go<8, false>(pv, spec, vs, eo, batch, op, s);
     if (bc <= 0) bc = pick_width((long)(pv.mmax + 1) * ((pv.npairs + 31) / 32), batch);
     switch (bc) {
     case 1: return synth64_go<1>(pv, spec, vs, eo, batch, op, s);
@@ -686,13 +729,13 @@ cudaError_t synth64(const PlanView<double> &pv, const double *spec, const VecSpe
     }
 }
 
-template <int BC>
+template <int BC, bool TAB = true>
 cudaError_t analys64_go(const PlanView<double> &pv, const double *sd, double *spec, const VecSpec *vs, int batch,
                         Op op, cudaStream_t s)
 {
     const dim3 grid((unsigned)((pv.lmax + (vs ? 1 : 0) + kSeedSeg) / kSeedSeg), (unsigned)(pv.mmax + 1),
                     (unsigned)((batch + BC - 1) / BC));
-    k_analys64<BC><<<grid, 32 * kAnaWarps, 0, s>>>(pv, sd, spec, vs ? *vs : VecSpec(), batch, vs ? 1 : 0, (int)op);
+    k_analys64<BC, TAB><<<grid, 32 * kAnaWarps, 0, s>>>(pv, sd, spec, vs ? *vs : VecSpec(), batch, vs ? 1 : 0, (int)op);
     return cudaGetLastError();
 }
 
@@ -707,7 +750,8 @@ inline long segments(const PlanView<double> &pv)
 cudaError_t analys64(const PlanView<double> &pv, const double *sd, double *spec, const VecSpec *vs, int batch, Op op,
                      int bc, cudaStream_t s)
 {
-    if (!tables_ok(pv)) return cudaErrorInvalidValue;
+    if (!tables_ok(pv, vs != nullptr)) return cudaErrorInvalidValue;
+    if (!pv.seeds64) return analys64_go<8, false>(pv, sd, spec, vs, batch, op, s);
     if (bc <= 0) bc = pick_width(segments(pv), batch);
     switch (bc) {
     case 1: return analys64_go<1>(pv, sd, spec, vs, batch, op, s);
@@ -746,7 +790,7 @@ size_t vec64_top_bytes(int mmax, int batch) { return (size_t)2 * batch * (mmax +
 cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *vt, double *vp,
                                double *top, double *eo, int batch, Op op, cudaStream_t s)
 {
-    if (!tables_ok(pv)) return cudaErrorInvalidValue;
+    if (!tables_ok(pv, true)) return cudaErrorInvalidValue;
     const VecSpec vs = {reinterpret_cast<double2 *>(vt), reinterpret_cast<double2 *>(vp),
                         reinterpret_cast<double2 *>(top), batch};
     const dim3 grid((unsigned)((pv.lmax + 2 + 127) / 128), (unsigned)(pv.mmax + 1), (unsigned)batch);

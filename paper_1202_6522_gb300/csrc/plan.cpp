@@ -98,7 +98,7 @@ PlanView<double> Plan::view64() const
 {
     PlanView<double> v{lmax, mmax, nlat, nphi, npairs, nlm,
                        t64.ab, t64.dc, t64.x, t64.st, t64.wq, t64.pmm, t64.pmmk, t64.tw, t64.rtw, fft_plan_of(nphi / 2), mres, twdf,
-                       nullptr, d_seg32, seeds64, seeds64k, live64, glive64, glive64 + plan_groups(*this), qs64, abx64, eps64, hseg64};
+                       nullptr, d_seg32, seeds64, seeds64k, live64, glive64, glive64 ? glive64 + plan_groups(*this) : nullptr, qs64, abx64, eps64, hseg64};
     return v;
 }
 
