@@ -1601,16 +1601,17 @@ cudaError_t launch_fft_analys(const PlanView<T> &pv, const T *grid, T *sd, int b
 
 namespace {
 
-// 4 values per thread instead of 16, up to H = 1024: always for mixed radices,
-// whose 16-value passes spill and leave threads without items (16 fields of 512 x
-// 1080: 183 / 188 -> 144 / 148 us, 5 of 361 x 720: 46 / 44 -> 27 / 26 us;
-// synthesis / analysis); for powers of two while the 16-value form has too few
-// warps, at most 320 threads per SM (2 fields of 512 x 1024: 26 / 22 -> 20 / 20 us),
-// above which its fewer passes win (16 fields: 96 against 110 us).
-bool df_few_values(int H, int npairs, int batch)
-{
-    return H <= 1024 && (!pow2(H) || (long)batch * npairs * 2 * row_tpr<16>(H) <= 320L * sm_count());
-}
+// 4 values per thread instead of 16: for mixed radices up to H = 1024, whose 16-value
+// passes spill and leave threads without items (16 fields of 512 x 1080: 183 / 188 ->
+// 144 / 148 us, 5 of 361 x 720: 46 / 44 -> 27 / 26 us; synthesis / analysis), and for
+// powers of two up to H = 512, where a launch has too few warps of 16 values (512 x
+// 1024: one field 28.7 / 27.2 -> 16.6 / 19.0 us, four 39.7 / 37.9 -> 35.5 / 40.0, but
+// 16 100 / 103 -> 113 / 117; 256 x 512: 16.5 / 19.0 -> 11.0 / 12.9 and, 16 fields,
+// 31.1 / 33.9 -> 30.7 / 33.9).  By the length alone: a field's result must not depend
+// on its batch.  At H = 1024 16 values win from one field on (39.4 / 36.1 us against
+// 43.0 / 45.5).  Errors are smaller with 4 (N = 511: 2.87e-14 against 2.94e-14,
+// analysis 2.05e-14 against 2.19e-14).
+bool df_few_values(int H) { return H <= (pow2(H) ? 512 : 1024); }
 
 template <bool MIXED, int LOGH, int V>
 cudaError_t synth_df_go(const PlanView<double> &pv, const double *eo, double *grid, int batch, Op op, cudaStream_t s)
@@ -1651,7 +1652,7 @@ cudaError_t launch_fft_synth_df(const PlanView<double> &pv, const double *eo, do
 {
     if (!pv.twdf) return cudaErrorInvalidValue;
     const int H = pv.nphi / 2;
-    if (df_few_values(H, pv.npairs, batch))
+    if (df_few_values(H))
         return pow2(H) ? synth_df_go<false, 0, 4>(pv, eo, grid, batch, op, s) : synth_df_go<true, 0, 4>(pv, eo, grid, batch, op, s);
     if (H == 1024) return synth_df_go<false, 10, 16>(pv, eo, grid, batch, op, s);
     return pow2(H) ? synth_df_go<false, 0, 16>(pv, eo, grid, batch, op, s) : synth_df_go<true, 0, 16>(pv, eo, grid, batch, op, s);
@@ -1662,7 +1663,7 @@ cudaError_t launch_fft_analys_df(const PlanView<double> &pv, const double *grid,
 {
     if (!pv.twdf) return cudaErrorInvalidValue;
     const int H = pv.nphi / 2;
-    if (df_few_values(H, pv.npairs, batch))
+    if (df_few_values(H))
         return pow2(H) ? analys_df_go<false, 0, 4>(pv, grid, sd, batch, op, vector, s, fmax) : analys_df_go<true, 0, 4>(pv, grid, sd, batch, op, vector, s, fmax);
     if (H == 1024) return analys_df_go<false, 10, 16>(pv, grid, sd, batch, op, vector, s, fmax);
     return pow2(H) ? analys_df_go<false, 0, 16>(pv, grid, sd, batch, op, vector, s, fmax) : analys_df_go<true, 0, 16>(pv, grid, sd, batch, op, vector, s, fmax);

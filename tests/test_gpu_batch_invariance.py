@@ -50,3 +50,17 @@ def test_field_alone_and_in_batches(setup, name):
         ref = _list(getattr(oracle, name)(LMAX, LMAX, NLAT, NPHI, *[a[b:b + 1] for a in args]))
         for f, r in zip(full, ref):
             assert normwise(f[b].cpu().numpy(), np.asarray(r)[0]) <= fp64_bound(LMAX)
+
+
+@pytest.mark.parametrize("lmax,nlat,nphi", [(255, 256, 512), (100, 101, 240)])
+@pytest.mark.parametrize("name", NAMES[:4])
+def test_tensor_core_field_alone_and_in_batches(name, lmax, nlat, nphi):
+    """SHT_TC_F64: the contraction is exact in integers, the FFTs double-float."""
+    from paper_1202_6522_gb300 import SHT
+    sht = SHT(lmax, lmax, nlat, nphi, device=DEV, fp64_path="tc")
+    spec = torch.from_numpy(synthetic.spectrum(lmax, batch=19, seed=1)).to(DEV)
+    grid = torch.from_numpy(synthetic.grid(nlat, nphi, batch=19, seed=3)).to(DEV)
+    x = _args(name, [spec], [grid])[0]
+    full = getattr(sht, name + "_")(x)
+    for lo, hi in ((0, 1), (2, 5), (8, 19)):
+        assert torch.equal(getattr(sht, name + "_")(x[lo:hi].contiguous()), full[lo:hi])
