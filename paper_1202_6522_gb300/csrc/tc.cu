@@ -261,7 +261,6 @@ struct TcArgs {
     unsigned long long data_half;          // vector: bytes of one half's data operand
     const float *in;                       // raw FP32 s/d folds (warp-specialised analysis)
     int fused;                             // synthesis: spectra converted in the kernel (tensor map)
-    int wide;                              // scalar: form of the MMAs (ws_tmem_cols)
     const unsigned char *panel, *dpanel;   // dpanel: vector transforms only
     const unsigned long long *off;         // per-order panel byte offsets
     const int *c0;                         // per (m, tile): first chunk above the polar threshold
@@ -328,10 +327,17 @@ __host__ __device__ inline size_t ws_smem_bytes(int rows, int batch, int stages,
 // wide: per parity, A_hi x [B_hi ; B_lo] as one MMA of N = 2 NC (columns
 // [hi.hi + lo.hi | hi.lo], summed by the epilogue) plus A_lo x B_hi, 4 MMAs per
 // chunk; else 3 MMAs of N = NC per parity into NC columns, half the TMEM.
+// Up to 16 fields (NC = 32) the wide accumulators fit kWsCtasPerSm times into TMEM,
+// with 17 .. 32 twice.  Three CTAs of the narrow form are faster there (N = 511, 24
+// fields: 44.5 / 43.2 us against 51.3 / 46.9; N = 1023: 207 / 201 against 226 / 211;
+// synthesis / analysis), but it adds hi.lo to the sums of hi.hi: errors of 5.57e-6
+// against 5.20e-6 (22 fields, N = 511), and a field differs from itself in a batch
+// of 16.
+__host__ __device__ inline bool ws_wide(int NC) { return NC <= 64; }
 // TMEM columns of a CTA (a power of two): two parities.
-__host__ __device__ inline uint32_t ws_tmem_cols(int NC, bool wide)
+__host__ __device__ inline uint32_t ws_tmem_cols(int NC)
 {
-    const int c = 2 * (wide ? 2 * NC : NC);
+    const int c = 2 * (ws_wide(NC) ? 2 * NC : NC);
     return c <= 64 ? 64 : (c <= 128 ? 128 : (c <= 256 ? 256 : 512));
 }
 
@@ -363,9 +369,9 @@ __global__ void __launch_bounds__(kWsThreads, kWsCtasPerSm) k_tc_ws(TcArgs a, co
     const unsigned char *panel = a.panel + a.off[m] + (size_t)tile * nchunks * kChunkPanel;
     const int cstart = a.c0 ? a.c0[m * a.ntiles + tile] : 0;
     const int nlive = nchunks - cstart;
-    const bool wide = a.wide;
+    const bool wide = ws_wide(NC);
     const int pcols = wide ? 2 * NC : NC;   // accumulator columns per parity
-    const uint32_t ncols = ws_tmem_cols(NC, wide);
+    const uint32_t ncols = ws_tmem_cols(NC);
 
     if (tid == 0) {
         for (int q = 0; q < S; ++q) {
@@ -1702,17 +1708,9 @@ cudaError_t launch_tc_legendre(bool synth, int lmax, int mmax, int mres, int npa
     tc_tile_counts(lmax, npairs, ts, ta);
     a.ntiles = synth ? ts : ta;
     const unsigned blocks = (unsigned)((mmax + 1) * a.ntiles);
-    // Up to 16 fields the wide MMAs fit kWsCtasPerSm CTAs' accumulators into TMEM.
-    // With 17 .. 32 they take 256 columns, two CTAs per SM: right for launches of
-    // at most two CTAs per SM (24 fields at N = 255: 11.1 / 10.5 us against 12.3 /
-    // 11.5), while larger ones need the third CTA in flight (N = 511: 38.7 / 40.0 us
-    // against 45.5 / 42.7; N = 1023: 203 / 198 against 223 / 208; synthesis / analysis).
-    int dev = 0, sms = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    a.wide = rows <= 32 || (rows <= 64 && blocks <= 2u * (unsigned)sms) ? 1 : 0;
     // CTAs of up to 3 stages (228 KB per SM, 1 KB reserved per CTA, a little static
     // shared memory), as many as TMEM holds; wider batches fall back to fewer CTAs
-    const int per_sm = std::min(kWsCtasPerSm, std::max(1, 512 / (int)ws_tmem_cols(rows, a.wide)));
+    const int per_sm = std::min(kWsCtasPerSm, std::max(1, 512 / (int)ws_tmem_cols(rows)));
     const size_t cap = (size_t)228 * 1024 / per_sm - 1024 - 256;
     int stages = 3;
     while (stages > 2 && ws_smem_bytes(rows, batch, stages, synth) > cap) --stages;

@@ -64,3 +64,20 @@ def test_tensor_core_field_alone_and_in_batches(name, lmax, nlat, nphi):
     full = getattr(sht, name + "_")(x)
     for lo, hi in ((0, 1), (2, 5), (8, 19)):
         assert torch.equal(getattr(sht, name + "_")(x[lo:hi].contiguous()), full[lo:hi])
+
+
+@pytest.mark.parametrize("lmax", [63, 511])
+@pytest.mark.parametrize("name", ["synth_", "analys_"])
+def test_split_bf16_up_to_32_fields(name, lmax):
+    """Split-bf16 products: up to 32 fields the sums of each product have columns of
+    their own, and a field is the same in any such batch."""
+    from paper_1202_6522_gb300 import SHT
+    nlat, nphi = lmax + 1, 2 * (lmax + 1)
+    sht = SHT(lmax, lmax, nlat, nphi, device=DEV, fp32_path="tc")
+    if name == "synth_":
+        x = torch.from_numpy(synthetic.spectrum(lmax, batch=32, seed=1).astype(np.complex64)).to(DEV)
+    else:
+        x = torch.from_numpy(synthetic.grid(nlat, nphi, batch=32, seed=3).astype(np.float32)).to(DEV)
+    full = getattr(sht, name)(x)
+    for lo, hi in ((0, 1), (0, 16), (15, 32), (3, 27)):
+        assert torch.equal(getattr(sht, name)(x[lo:hi].contiguous()), full[lo:hi])
