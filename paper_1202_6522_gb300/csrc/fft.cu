@@ -261,12 +261,11 @@ template <int V = 16> __host__ __device__ inline int row_tpr(int H) { return (H 
 // Values per thread.  FP64 up to H = 1024 (512 threads for two rows): 4.  The
 // FP64 pipe takes a warp instruction every ~64 cycles per SM quarter, so a row
 // spread over four times the threads keeps all four quarters busy where a launch
-// has few rows, at the same instruction count (radix 4: 24 FP64 instructions per 4
-// points and pass, four passes; radix 16: 228 per 16 points, two passes).  One
+// has few rows, at about the same instruction count (radix 4: 28 FP64 instructions per
+// 4 points and pass, four passes; radix 16: 228 per 16 points, two passes).  One
 // field of 256 x 512 points: 51 / 54 us with 16 values and 8 pairs per CTA (16
 // CTAs), 28 / 27 us with one pair per CTA, 10.2 / 10.3 us with 4 values; 16 fields
-// of 512 x 1024: 373 / 417 -> 308 / 317 us (synthesis / analysis; FP64 pipe 88 %
-// active), of which 43 / 44 us are the twiddles fused into the radix-4 FMAs.
+// of 512 x 1024: 373 / 417 -> 341 / 350 us (synthesis / analysis).
 // FP32: 16, two radix-16 passes with few barriers; but 4 for mixed radices in the
 // synthesis up to H = 1024 and the analysis up to H = 256, where the 16-value
 // passes leave threads without items (6 fields of 288 x 384: 9.2 / 9.2 -> 6.2 /
@@ -288,15 +287,10 @@ __device__ __forceinline__ int lg2(int v) { return __popc(v - 1); }
 
 template <typename T2> struct IsDf { static constexpr bool value = false; };
 template <> struct IsDf<dfl2> { static constexpr bool value = true; };
-// a + w b, and 2 a - s, by FMAs
+// a + w b by FMAs
 template <typename T2> __device__ __forceinline__ T2 fma_add(T2 a, T2 w, T2 b)
 {
     return mk<T2>(fma(-w.y, b.y, fma(w.x, b.x, a.x)), fma(w.y, b.x, fma(w.x, b.y, a.y)));
-}
-template <typename T2> __device__ __forceinline__ T2 twice_less(T2 a, T2 s)
-{
-    using T = decltype(T2::x);
-    return mk<T2>(fma(T(2), a.x, -s.x), fma(T(2), a.y, -s.y));
 }
 
 // q / d for 0 <= q < 2^19 and d >= 1 with q / d < 2^13 by one FP32 product (an
@@ -329,22 +323,27 @@ __device__ __forceinline__ void stockham_load(const T2 *src, bool global_src, in
             a[r] = global_src ? src[idx] : src[padi(idx)];
         }
         if constexpr (sizeof(T2) == sizeof(double2) && RD == 4 && !IsDf<T2>::value) {
-            // FP64: the twiddles w, w^2 (w^3 = w w^2) fused into the butterflies, s = a + w b
-            // by four FMAs and a - w b = 2 a - s by two: 24 instructions instead of 28
+            // FP64: two of the three twiddles into the butterflies' first sums, a +- w b by
+            // FMAs: 28 instructions as with the products apart, and two roundings less.  24
+            // instructions (w^3 as w w^2, a - w b as 2 a - s) took 9 % less time, but their
+            // errors are 12 % above those of the products apart, these 2 % below (emulated,
+            // H = 16 .. 1024: 2.23e-16, 1.95e-16 and 1.99e-16 at H = 1024).
             if (Ns > 1) {
                 const int q0 = P2 ? (j & (Ns - 1)) << (lg2(H) - lg2(Ns) - 2) : (j - div(j) * Ns) * wstep;
-                T2 w1 = wtab[q0], w2 = wtab[2 * q0];
+                T2 w1 = wtab[q0], w2 = wtab[2 * q0], w3 = wtab[3 * q0];
                 if (SIGN < 0) {
                     w1 = conj_(w1);
                     w2 = conj_(w2);
+                    w3 = conj_(w3);
                 }
-                const T2 p = fma_add(a[0], w2, a[2]), q = twice_less(a[0], p);
-                const T2 u = fma_add(a[1], w2, a[3]), z = twice_less(a[1], u);
+                const T2 b = cmul(a[1], w1);
+                const T2 p = fma_add(a[0], w2, a[2]), q = fma_add(a[0], mk<T2>(-w2.x, -w2.y), a[2]);
+                const T2 u = fma_add(b, w3, a[3]), z = fma_add(b, mk<T2>(-w3.x, -w3.y), a[3]);
                 const T2 iz = SIGN > 0 ? mul_i(z) : mk<T2>(z.y, -z.x);
-                v[it * RD] = fma_add(p, w1, u);
-                v[it * RD + 2] = twice_less(p, v[it * RD]);
-                v[it * RD + 1] = fma_add(q, w1, iz);
-                v[it * RD + 3] = twice_less(q, v[it * RD + 1]);
+                v[it * RD] = cadd(p, u);
+                v[it * RD + 2] = csub(p, u);
+                v[it * RD + 1] = cadd(q, iz);
+                v[it * RD + 3] = csub(q, iz);
                 continue;
             }
         }
