@@ -435,13 +435,9 @@ size_t tc_work_bytes(const sht::Plan &p, int batch, bool vec)
     return tc_data_offset(p, batch, vec) + sht::tc_data_bytes(p.mmax, p.npairs, p.tc_nchunk_s, nb, vec);
 }
 
-// With room for what the FP64 vector transforms keep behind two intermediates, 1 / (2
-// npairs) of them: a scratch that holds the intermediates holds that too, whichever
-// call it was made for.
 int ensure_work(sht::Plan &p, size_t bytes)
 {
     if (bytes <= p.work_bytes) return SHT_OK;
-    bytes += bytes / (2 * (size_t)p.npairs) + 256;
     if (p.work) {
         cudaError_t e = cudaFree(p.work);  // cudaFree waits for work using the old buffer
         p.work = nullptr;
@@ -572,12 +568,8 @@ int run_analys(sht::Plan &p, const sht::PlanView<T> &pv, const void *grid, void 
     });
 }
 
-// Vector transforms on the CUDA cores: two intermediates (theta, phi) and, in FP64,
-// the degree lmax + 1 of the combined spectra behind them.
-size_t vec_work_bytes(const sht::Plan &p, int batch, int mode)
-{
-    return 2 * inter_bytes(p, batch, mode) + (mode == SHT_F64 ? sht::vec64_top_bytes(p.mmax, batch) : 0);
-}
+// Vector transforms on the CUDA cores: two intermediates (theta, phi).
+size_t vec_work_bytes(const sht::Plan &p, int batch, int mode) { return 2 * inter_bytes(p, batch, mode); }
 
 template <typename T>
 int run_synth_vec(sht::Plan &p, const sht::PlanView<T> &pv, const void *S, const void *Tc, void *vt, void *vp,
@@ -589,7 +581,7 @@ int run_synth_vec(sht::Plan &p, const sht::PlanView<T> &pv, const void *S, const
         const T *Si = static_cast<const T *>(S), *Ti = static_cast<const T *>(Tc);
         if constexpr (sizeof(T) == sizeof(double))
             return sht::launch_synth_vec64(pv, Si, Ti, static_cast<T *>(vt), static_cast<T *>(vp),
-                                           eop + (eop - eot), eot, batch, op, s);
+                                           p.top64, eot, batch, op, s);
         else
             return sht::launch_legendre_synth_vec(pv, Si, Ti, eot, eop, batch, op, s);
     });
@@ -618,7 +610,7 @@ int run_analys_vec(sht::Plan &p, const sht::PlanView<T> &pv, const void *vt, con
     return timed(p, SHT_K_LEGENDRE_ANALYS_VEC, s, "legendre vector analysis launch", [&] {
         T *So = static_cast<T *>(S), *To = static_cast<T *>(Tc);
         if constexpr (sizeof(T) == sizeof(double))
-            return sht::launch_analys_vec64(pv, sdt, sdp + (sdp - sdt), So, To, batch, op, s);
+            return sht::launch_analys_vec64(pv, sdt, p.top64, So, To, batch, op, s);
         else
             return sht::launch_legendre_analys_vec(pv, sdt, sdp, So, To, batch, op, s);
     });

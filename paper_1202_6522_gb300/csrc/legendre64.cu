@@ -58,11 +58,13 @@ __device__ __forceinline__ int snake(int i, int total, int nsm)
 }
 
 // Spectra of a vector transform's scalar form: the degrees m .. lmax of U (or A) and
-// of W (B) as [nb][nlm] each, and the degree lmax + 1 of both as [2 nb][mmax + 1].
-// Field f of the scalar form is U of field f, then W of field f - nb.
+// of W (B) as [nb][nlm] each, and the degree lmax + 1 of both as [2 nb][mmax + 1], for
+// a group of nb <= kVec64Group fields.  Field f of the scalar form is U of field f,
+// then W of field f - nb; its E/O or folds are field f + lo, or f + hi, of the call's.
 struct VecSpec {
     double2 *u, *w, *top;
-    int nb;
+    int nb, lo, hi;
+    __device__ __forceinline__ int inter(int f) const { return f + (f < nb ? lo : hi); }
     __device__ __forceinline__ double2 *field(int f, int nlm) const
     {
         return f < nb ? u + (size_t)f * nlm : w + (size_t)(f - nb) * nlm;
@@ -327,7 +329,7 @@ k_synth64(PlanView<double> pv, const double *__restrict__ spec, VecSpec vs, doub
             v.x *= is;
             v.y *= is;
         }
-        eo2[(((size_t)(b0 + b) * (pv.mmax + 1) + m) * npairs + q) * 2 + (i & 1)] = v;
+        eo2[(((size_t)vs.inter(b0 + b) * (pv.mmax + 1) + m) * npairs + q) * 2 + (i & 1)] = v;
     }
 }
 
@@ -404,7 +406,7 @@ k_analys64(PlanView<double> pv, const double *__restrict__ sd, double *__restric
     const int c = lane % C, half = HV == 2 ? 0 : (lane / C) & 1, b = b0 + (c >> 1);
     const int dw = w * DB, d0 = dw + (HV == 2 ? 0 : lane / (2 * C)) * ND;
     // s at 4 q, d at 4 q + 2 (a lane with one degree: the one its parity takes)
-    const double *fold = sd + ((size_t)b * (pv.mmax + 1) + m) * npairs * 4 + (c & 1) + (ND == 1 ? 2 * (d0 & 1) : 0);
+    const double *fold = sd + ((size_t)vs.inter(b) * (pv.mmax + 1) + m) * npairs * 4 + (c & 1) + (ND == 1 ? 2 * (d0 & 1) : 0);
     const bool has = b < batch && dw < cnt;
     double acc[HV][ND];
 #pragma unroll
@@ -785,31 +787,40 @@ cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double
     return analys64(pv, sd, spec, nullptr, batch, op, bc, s);
 }
 
-size_t vec64_top_bytes(int mmax, int batch) { return (size_t)2 * batch * (mmax + 1) * sizeof(double2); }
-
 cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *vt, double *vp,
-                               double *top, double *eo, int batch, Op op, cudaStream_t s)
+                               double2 *top, double *eo, int batch, Op op, cudaStream_t s)
 {
     if (!tables_ok(pv, true)) return cudaErrorInvalidValue;
-    const VecSpec vs = {reinterpret_cast<double2 *>(vt), reinterpret_cast<double2 *>(vp),
-                        reinterpret_cast<double2 *>(top), batch};
-    const dim3 grid((unsigned)((pv.lmax + 2 + 127) / 128), (unsigned)(pv.mmax + 1), (unsigned)batch);
-    k_vec64_split<<<grid, 128, 0, s>>>(pv, reinterpret_cast<const double2 *>(S), reinterpret_cast<const double2 *>(Tc),
-                                       vs, (int)op);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return synth64(pv, nullptr, &vs, eo, 2 * batch, OP_SYNTH, 0, s);
+    const size_t ngrid = (size_t)pv.nlat * pv.nphi, nspec = (size_t)pv.nlm * 2;
+    cudaError_t e = cudaSuccess;
+    for (int b0 = 0; b0 < batch && e == cudaSuccess; b0 += kVec64Group) {
+        const int nb = batch - b0 < kVec64Group ? batch - b0 : kVec64Group;
+        const VecSpec vs = {reinterpret_cast<double2 *>(vt + b0 * ngrid), reinterpret_cast<double2 *>(vp + b0 * ngrid),
+                            top, nb, b0, batch + b0 - nb};
+        const dim3 grid((unsigned)((pv.lmax + 2 + 127) / 128), (unsigned)(pv.mmax + 1), (unsigned)nb);
+        k_vec64_split<<<grid, 128, 0, s>>>(pv, reinterpret_cast<const double2 *>(S + b0 * nspec),
+                                           reinterpret_cast<const double2 *>(Tc + b0 * nspec), vs, (int)op);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = synth64(pv, nullptr, &vs, eo, 2 * nb, OP_SYNTH, 0, s);
+    }
+    return e;
 }
 
-cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *top, double *S, double *Tc,
+cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double2 *top, double *S, double *Tc,
                                 int batch, Op op, cudaStream_t s)
 {
-    const VecSpec vs = {reinterpret_cast<double2 *>(S), reinterpret_cast<double2 *>(Tc),
-                        reinterpret_cast<double2 *>(top), batch};
-    cudaError_t e = analys64(pv, sd, nullptr, &vs, 2 * batch, OP_ANALYS, 0, s);
-    if (e != cudaSuccess) return e;
-    k_vec64_join<<<dim3((unsigned)(pv.mmax + 1), (unsigned)batch), 128, 0, s>>>(pv, vs, (int)op);
-    return cudaGetLastError();
+    const size_t nspec = (size_t)pv.nlm * 2;
+    cudaError_t e = cudaSuccess;
+    for (int b0 = 0; b0 < batch && e == cudaSuccess; b0 += kVec64Group) {
+        const int nb = batch - b0 < kVec64Group ? batch - b0 : kVec64Group;
+        const VecSpec vs = {reinterpret_cast<double2 *>(S + b0 * nspec), reinterpret_cast<double2 *>(Tc + b0 * nspec),
+                            top, nb, b0, batch + b0 - nb};
+        e = analys64(pv, sd, nullptr, &vs, 2 * nb, OP_ANALYS, 0, s);
+        if (e != cudaSuccess) break;
+        k_vec64_join<<<dim3((unsigned)(pv.mmax + 1), (unsigned)nb), 128, 0, s>>>(pv, vs, (int)op);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 }  // namespace sht

@@ -207,7 +207,7 @@ int plan_build(Plan &p, std::string &err)
     // One device allocation holding both precisions' tables.
     size_t bytes = padded<double2>(nlm) + padded<double>(nlm) + 3 * padded<double>(npairs) +
                    padded<double>((size_t)(mmax + 1) * npairs) + padded<int>((size_t)(mmax + 1) * npairs) +
-                   2 * padded<double2>(H1);
+                   2 * padded<double2>(H1) + padded<double2>((size_t)2 * kVec64Group * (mmax + 1));
     bytes += padded<float2>(nlm) + padded<float>(nlm) + 3 * padded<float>(npairs) + 2 * padded<float2>(H1);
     bytes += padded<float4>(H1) + padded<int>(1);
     DevArena ar;
@@ -238,6 +238,7 @@ int plan_build(Plan &p, std::string &err)
     ok &= up(p.t64.pmmk, k64.data(), sizeof(int) * k64.size());
     p.t64.tw = ar.take<double2>(H1);
     ok &= up(p.t64.tw, tw.data(), sizeof(double) * 2 * H1);
+    p.top64 = ar.take<double2>((size_t)2 * kVec64Group * (mmax + 1));
     p.t64.rtw = ar.take<double2>(H1);
     ok &= up(p.t64.rtw, rtw.data(), sizeof(double) * 2 * H1);
 

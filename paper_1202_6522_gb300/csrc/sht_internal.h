@@ -194,6 +194,7 @@ struct Plan {
     float thr_cc32() const { return polar_thr_set ? polar_thr : 0x1p-40f; }
     float thr_cc64() const { return polar_thr_set ? polar_thr : 0x1p-64f; }
     double otf_skip_s = 0, otf_skip_a = 0;      // on-the-fly mode: fraction of chunks skipped
+    double2 *top64 = nullptr;        // FP64 vector transforms: degree lmax + 1 of a group's spectra, [2 kVec64Group][mmax+1]
     void *work = nullptr;            // scratch (grown on demand)
     size_t work_bytes = 0;
     int device = 0;
@@ -243,13 +244,13 @@ cudaError_t launch_synth64(const PlanView<double> &pv, const double *spec, doubl
                            cudaStream_t s);
 cudaError_t launch_analys64(const PlanView<double> &pv, const double *sd, double *spec, int batch, Op op, int bc,
                             cudaStream_t s);
-// Vector transforms as scalar ones of 2 batch fields.  eo / sd hold the theta
-// fields, then the phi fields; `top` is scratch of vec64_top_bytes, and the
+// Vector transforms as scalar ones of twice the fields, kVec64Group fields at a time.
+// eo / sd hold the theta fields, then the phi fields; `top` is the plan's, and the
 // synthesis overwrites the grids vt, vp, which its FFTs fill afterwards.
-size_t vec64_top_bytes(int mmax, int batch);
+constexpr int kVec64Group = 32;
 cudaError_t launch_synth_vec64(const PlanView<double> &pv, const double *S, const double *Tc, double *vt, double *vp,
-                               double *top, double *eo, int batch, Op op, cudaStream_t s);
-cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double *top, double *S, double *Tc,
+                               double2 *top, double *eo, int batch, Op op, cudaStream_t s);
+cudaError_t launch_analys_vec64(const PlanView<double> &pv, const double *sd, double2 *top, double *S, double *Tc,
                                 int batch, Op op, cudaStream_t s);
 // Fills the plan's qs, abx, eps and hseg tables (the view's are not used).
 cudaError_t launch_build_qs(const PlanView<double> &pv, const unsigned long long *segoff, double2 *qs, double2 *abx,

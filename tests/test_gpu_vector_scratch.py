@@ -34,7 +34,7 @@ def _captured(fn):
 
 
 @pytest.mark.parametrize("name", ["synth_vec_", "analys_vec_", "synth_vec_adj_", "analys_vec_adj_"])
-@pytest.mark.parametrize("lmax,nlat,nphi,batch", [(63, 64, 128, 2), (0, 1, 2, 3), (33, 41, 90, 5)])
+@pytest.mark.parametrize("lmax,nlat,nphi,batch", [(63, 64, 128, 2), (0, 1, 2, 3), (33, 41, 90, 5), (40, 41, 96, 70)])
 def test_captured_after_a_scalar_call(lib, name, lmax, nlat, nphi, batch):
     """A scalar call of twice as many fields leaves the scratch a vector call takes."""
     sht = lib.SHT(lmax, lmax, nlat, nphi, device=DEV)
