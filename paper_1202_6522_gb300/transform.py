@@ -15,8 +15,9 @@ from . import _capi as C
 
 
 # The current stream's handle by device index: torch.cuda.current_stream(d).cuda_stream
-# without the Stream object (2 us of a small transform's 27 us on the host).
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# without the Stream object (2 us of a small transform's 27 us on the host).  A torch
+# built without CUDA does not have it, nor a device for a plan.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _next_pow2(v: int) -> int:
