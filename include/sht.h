@@ -81,7 +81,11 @@ enum {
                         * 40 B per coefficient).  Vector calls form the spectra of two
                         * scalar transforms in their output arrays before they fill them,
                         * and run without the tables, slower, where these cannot be had:
-                        * in a first call that is captured, or for want of memory. */
+                        * in a first call that is captured, or for want of memory.
+                        * Scalar sums run on P_n^m divided by the growth of the recurrence
+                        * within its segment, up to 2^75 either way, so data and results
+                        * have to keep that distance from the ends of the FP64 range
+                        * (about 1e-285 .. 1e285). */
     SHT_F32 = 1,       /* FP32 data and recurrence restarted every 32 degrees from
                         * states the FP64 recurrence computes once per plan, each held
                         * with the power-of-two scale of its segment (the explicit

@@ -609,7 +609,7 @@ __device__ __forceinline__ void fft_analys_tile(const PlanView<T> &pv, const T *
             if (op == OP_ANALYS) wf *= pv.wq[pp];
             if (vector) wf /= pv.st[pp];
         }
-        s_w[i] = wf * T(0.5);   // the halves of E and O below
+        s_w[i] = wf;
     }
     __syncthreads();
     const int r = threadIdx.x / TPR, t = threadIdx.x - r * TPR;
@@ -649,7 +649,9 @@ __device__ __forceinline__ void fft_analys_tile(const PlanView<T> &pv, const T *
     __syncthreads();
     // post-twiddle, fold north/south, weight.  Positions m and H - m share their
     // terms: with E = Z_m + conj Z_{H-m}, Od = (Z_m - conj Z_{H-m}) / i and
-    // P = W^{-m} Od (W = e^{2 pi i / (2H)}), 2 X_m = E + P and 2 X_{H-m} = conj(E - P).
+    // P = W^{-m} Od / 2 (W = e^{2 pi i / (2H)}), X_m = E / 2 + P and X_{H-m} = conj(E / 2 - P),
+    // the halves in the twiddle and the sums' FMAs (not in the weight: 2 X_m needs
+    // twice the range).
     T2 *sd2 = reinterpret_cast<T2 *>(sd);
     const auto emit = [&](int m, int i, int pp, const T2 (&X)[2]) {
         const T wf = s_w[i];
@@ -675,15 +677,16 @@ __device__ __forceinline__ void fft_analys_tile(const PlanView<T> &pv, const T *
         const int m2 = H - m;   // its partner, when it is another position and an order of the plan
         const bool two = m2 != m && m2 < H && m2 <= mmax;
         T2 X[2], X2[2];
+        const T2 w = mk<T2>(T(0.5) * pv.tw[m].x, T(-0.5) * pv.tw[m].y);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const T2 *rw = buf + (2 * i + h) * ld;
             const T2 Zk = rw[padi(m)];
             const T2 Zc = conj_(rw[padi(m == 0 ? 0 : m2)]);
             const T2 E = cadd(Zk, Zc), O = csub(Zk, Zc);
-            const T2 P = cmul(conj_(pv.tw[m]), mk<T2>(O.y, -O.x));
-            X[h] = cadd(E, P);
-            X2[h] = conj_(csub(E, P));
+            const T2 P = cmul(w, mk<T2>(O.y, -O.x));
+            X[h] = mk<T2>(fma(T(0.5), E.x, P.x), fma(T(0.5), E.y, P.y));
+            X2[h] = mk<T2>(fma(T(0.5), E.x, -P.x), -fma(T(0.5), E.y, -P.y));
         }
         emit(m, i, pp, X);
         if (two) emit(m2, i, pp, X2);
