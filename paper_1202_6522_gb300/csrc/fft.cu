@@ -1481,16 +1481,6 @@ cudaError_t launch_rows_dispatch(int logH, bool synth, const PlanView<float> &pv
 inline int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 inline bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
-// SMs of the current device.
-inline int sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 152;
-    return sms;
-}
-
 // Threads per row and pairs per CTA: TPR = ceil(H/16) threads per row and
 // enough rows for 256 threads, capped so the CTA's buffer stays <= 96 KB.
 // (512-thread CTAs read the intermediate in longer runs but fit one CTA per

@@ -13,7 +13,7 @@
 // pair per lane, restarted at every segment of kSeedSeg degrees from the state
 // the FP64 recurrence computed once per plan (the FP32 recurrence alone loses
 // accuracy with n).  Underflow (Sec. 3.5) is taken care of per segment: where the
-// values entering it are below 2^-62, the state is stored times a power of two
+// values entering it are below 2^-63, the state is stored times a power of two
 // that keeps the whole segment in the FP32 range, together with the factor that
 // takes it back (0 where no |P| of the segment reaches 2^-70), so the recurrence
 // itself tests nothing.  Since segments do not depend on one another, they are

@@ -663,15 +663,6 @@ k_build_qs(PlanView<double> pv, const unsigned long long *__restrict__ segoff, d
     if (lane == kSeedSeg - 1 && i0 + kSeedSeg == Ls) put(Ls, dd_mul(s2, ratio(Ls)), h);
 }
 
-inline int sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 152;
-    return sms;
-}
-
 // Fields per CTA {1, 2, 4, 8, 16}: the width with the shortest busiest SM -- CTAs
 // per SM, rounded up, times the FP64 instructions of one (2 per degree and 32
 // pairs to generate P, 2 per field to sum).

@@ -12,6 +12,16 @@
 
 namespace sht {
 
+// SMs of the current device.
+inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 152;
+    return sms;
+}
+
 // Exponent step of the underflow rescaling (Sec. 3.5) of the FP64 recurrence: a
 // value is carried as y * 2^(-S k) with an integer k >= 0.  While k > 0 the true
 // value is below 2^-S: it is left out of the Legendre sums but still advanced by

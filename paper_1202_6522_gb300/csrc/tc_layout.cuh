@@ -27,8 +27,8 @@ __host__ __device__ __forceinline__ uint32_t blk_off(int row, int k)
 // bytes of one data chunk of `rows` rows: [2 classes][hi|lo] blocks
 __host__ __device__ inline size_t data_chunk_bytes(int rows) { return 4 * (size_t)rows * kKc * 2; }
 
-// v = hi + lo with hi = bf16(v), lo = bf16(v - hi)
-// v0, v1 -> bf16x2 hi and lo words (v0 in the low half) with v = hi + lo per element
+// v0, v1 -> bf16x2 hi and lo words (v0 in the low half) with v = hi + lo per element,
+// hi = bf16(v), lo = bf16(v - hi)
 __device__ __forceinline__ void split2(float v0, float v1, uint32_t &hi, uint32_t &lo)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
