@@ -339,6 +339,8 @@ int run(sht_batch_plan *b, bool synth, void *const *in, void *const *out, int us
     const int dir = synth ? 0 : 1;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap == cudaStreamCaptureStatusActive && use_graph)
+        return bfail(SHT_ECUDA, "a batch graph cannot be launched into a stream capture: call with use_graph = 0");
     if (cap == cudaStreamCaptureStatusActive) {
         // into the caller's graph, whose replays read the staging again: one of the call's own, kept
         // with the plan, and no events, which would tie the graph to calls outside of it

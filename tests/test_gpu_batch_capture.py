@@ -12,6 +12,23 @@ DEV = "cuda:0"
 LMAX = [31, 9, 31, 63]
 
 
+def test_graph_launch_stays_refused():
+    from paper_1202_6522_gb300 import UnevenBatch, _capi as C, build
+    build.build()
+    ub = UnevenBatch(LMAX, use_graph=True, path="f32")
+    specs = [torch.from_numpy(synthetic.spectrum(l, seed=i).astype(np.complex64)).to(DEV) for i, l in enumerate(LMAX)]
+    grids = ub.synth_(specs)
+    ref = [v.clone() for v in grids]
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        with pytest.raises(C.SHTError):
+            ub.synth_(specs, out=grids)
+        specs[0] + 1      # (a graph of something)
+    for u, v in zip(ub.synth_(specs), ref):
+        assert torch.equal(u, v)
+
+
 @pytest.mark.parametrize("path", ["f32", "tc"])
 def test_replay_after_other_calls(path):
     from paper_1202_6522_gb300 import UnevenBatch, build
