@@ -269,8 +269,11 @@ SHT_API int sht_tune(sht_handle h, int batch, int mode, double *report, void *st
  * afterwards; the capture happens on a private stream.
  * Limits: nphi = 2 x 2^a 3^b 5^c in [2, 4096], nlat <= 1024.
  * spec[f] / grid[f]: device pointers of field f ([nlm_f] complex floats and
- * [nlat_f][nphi_f] floats).  A call waits on the host until the previous call
- * on this batch plan has started its pointer-table copy. */
+ * [nlat_f][nphi_f] floats).  A call waits on the host until the previous call of
+ * its direction on this batch plan has finished, and its work waits on the device for
+ * the plan's last call, on whichever stream.  Under a relaxed stream capture, with
+ * use_graph = 0, it allocates staging of its own, which the plan keeps; the order of
+ * the graph's replays with other calls on the plan is then the caller's. */
 typedef struct sht_batch_plan *sht_batch;
 SHT_API int sht_batch_create(int nfields, const int *lmax, const int *nlat, const int *nphi, sht_batch *out);
 /* The same with a choice of path (Sec. 3.2's runtime choice, for batches):
